@@ -1150,12 +1150,12 @@ CUtensorMapSwizzle swizzle_for_bytes(unsigned row_bytes)
 thread_local int t_f16 = 0;      // element type of the tensor maps being encoded: 0 bf16, 1 fp16
 
 bool encode(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
-            const cuuint32_t* box, unsigned inner_bytes)
+            const cuuint32_t* box, unsigned inner_bytes, bool f32 = false)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint32_t ones[5] = {1, 1, 1, 1, 1};
-    return fn(m, t_f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(ptr), dims, strides_bytes, box,
+    return fn(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : t_f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(ptr), dims, strides_bytes, box,
               ones, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for_bytes(inner_bytes), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -1702,6 +1702,11 @@ bool tmap_encode_16(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t*
 {
     t_f16 = f16;
     return encode(m, rank, ptr, dims, strides_bytes, box, inner_bytes);
+}
+bool tmap_encode_f32(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
+                     const cuuint32_t* box, unsigned inner_bytes)
+{
+    return encode(m, rank, ptr, dims, strides_bytes, box, inner_bytes, true);
 }
 int sm_count() { return num_sms(); }
 

@@ -1,4 +1,5 @@
-// fp32 convolution layer: implicit GEMM on the FP32 pipes (FFMA), register tiled.
+// fp32 convolution layer: implicit GEMM on the FP32 pipes (FFMA), register tiled; and the choice between this kernel and
+// the one on the tensor cores.
 //
 // GEMM view of the layer (Section II of the paper: every output pixel is the sum over
 // input layers of a KxK kernel applied to a window): rows = output pixels (n, h, w),
@@ -325,6 +326,24 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
     p.out_c_offset = d.out_c_offset; p.out_c_total = d.out_c_total; p.relu = d.relu;
 
     const bool vec = (d.Cin % 4 == 0);
+    {
+        // The tensor-core kernel (conv_f32_tc.cu) starts and ends more slowly (5 us against 2) but is up to four times as
+        // fast on long reductions with many layers; this one keeps the small layers (SqueezeNet at batch 1: fire2's
+        // expand-1x1 2.9 us against 5.3, its squeeze 5.4 against 7.2) and those bound by memory with few layers.  Estimate
+        // for this kernel, fitted to SqueezeNet's layers at batch 1 .. 256: latency of the reduction loop, FFMA rate, or
+        // bytes.  Measured at batch 256, this kernel / the other: conv1 2687 / 1054 us, fire4's expand-3x3 1296 / 394,
+        // conv10 1256 / 353, fire8's squeeze 234 / 132, fire2's squeeze 123 / 150, its expand-1x1 88 / 107.
+        const float rate = 37.2e6f * (vec ? 0.58f : 0.44f);                       // multiply-adds per us
+        float us = 0.035f * (float)Kdim;
+        const float fma_us = (float)M * (float)d.Cout * (float)Kdim / rate;
+        const float mem_us = 4.f * ((float)d.N * d.H * d.W * d.Cin + (float)M * d.Cout) / 2.7e6f;
+        if (fma_us > us) us = fma_us;
+        if (mem_us > us) us = mem_us;
+        if (6.1f + 0.45f * (float)((Kdim + 31) / 32) < 2.f + us) {      // (the other kernel's time for one tile: not worth a plan if above)
+            const int rc = launch_conv_f32_tc(d, 2.f + us, stream);
+            if (rc != SQN_ERR_UNSUPPORTED) return rc;
+        }
+    }
     // output-layer tile: the candidate that wastes the fewest padded columns, larger on ties
     const int cand[6] = {128, 96, 64, 48, 32, 16};
     int best = 128;

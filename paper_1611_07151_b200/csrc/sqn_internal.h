@@ -30,8 +30,11 @@ void note_launch(int n = 1);
 // Device status word shared by all kernels (0 = fine, else an sqn_status).
 int* device_status_word();
 
-// fp32 path: register-tiled FFMA implicit GEMM, any (K, S, pad, Cin, Cout).
+// fp32 path, any (K, S, pad, Cin, Cout): on the tensor cores with every operand split exactly into three bf16 numbers, or
+// on the FFMA pipes, whichever is estimated to be faster for the shape (see launch_conv_f32).
 int launch_conv_f32(const ConvDesc& d, cudaStream_t stream);
+// The tensor-core kernel; SQN_ERR_UNSUPPORTED where it does not apply or where its own estimate is above limit_us.
+int launch_conv_f32_tc(const ConvDesc& d, float limit_us, cudaStream_t stream);
 
 // bf16 path: tcgen05/TMEM implicit GEMM fed by TMA.
 // Returns SQN_ERR_UNSUPPORTED for shapes outside its family.

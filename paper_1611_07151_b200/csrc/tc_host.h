@@ -11,6 +11,10 @@ namespace sqn {
 bool tmap_encode_16(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
                     const cuuint32_t* box, unsigned inner_bytes, int f16);
 
+// The same for 32-bit floating-point elements.
+bool tmap_encode_f32(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
+                     const cuuint32_t* box, unsigned inner_bytes);
+
 int sm_count();     // SMs of the current device
 
 }  // namespace sqn

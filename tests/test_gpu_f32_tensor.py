@@ -1,0 +1,79 @@
+"""The exact path's tensor-core kernel (every fp32 operand as three bf16 numbers) against the oracle, at the sizes where its
+tiles, chunks and dispatch branches end.  The shapes are large enough for the dispatch to take it.
+
+Bound per output, S = sum of |kernel * input| over the window: the products left out are below 2^-22 of the operands'
+product; a segment of 32 products is cut to 24 bits in two steps of at most 2^-23 of what it holds, the segments are added
+with rounded additions (2^-24 each), and so are corrections and bias."""
+import numpy as np
+import pytest
+
+from oracle import ref
+from paper_1611_07151_b200 import binding as B
+from paper_1611_07151_b200 import synth
+import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+F32 = B.SQN_F32
+
+# (N, Cin, Cout, H, K, S, pad)
+SHAPES = [
+    (40, 128, 32, 55, 1, 1, 0),     # kernels kept in shared memory, a quarter of the MMA rows live
+    (11, 260, 130, 27, 1, 1, 0),    # streamed kernels, last chunk of 4, two columns of tiles, ragged everywhere
+    (3, 512, 1000, 13, 1, 1, 0),    # eight columns of tiles
+    (24, 16, 64, 55, 3, 1, 1),      # patch, units of 16 reduction elements
+    (9, 48, 192, 27, 3, 1, 1),      # patch, last chunk of 16, 96 layers per column
+    (8, 64, 130, 33, 3, 1, 1),      # patch, streamed kernels
+    (6, 36, 70, 40, 5, 1, 2),       # 5x5 patch, chunk of 4
+    (4, 32, 64, 60, 3, 1, 0),       # no padding
+    (6, 32, 96, 41, 2, 1, 1),       # even kernel, output larger than the input
+    (2, 3, 96, 111, 7, 2, 0),       # staged windows, layers not a multiple of 4
+    (8, 64, 128, 33, 3, 2, 1),      # staged windows in 16-byte pieces, several blocks of layers
+    (4, 35, 72, 45, 3, 2, 1),       # ... in 4-byte pieces, kernels by copies
+    (12, 130, 128, 28, 1, 2, 0),    # windows apart from one another
+    (1, 64, 64, 300, 3, 1, 1),      # rows too long for the patch
+]
+
+
+def bound(x, w, b, S, pad, K, C):
+    z = np.zeros_like(b)
+    terms = ref.conv2d(np.abs(x), np.abs(w), z, S=S, pad=pad, relu=False).astype(np.float64)
+    return (2.0 ** -22 + 2 * 2.0 ** -23 + (K * K * C / 32 + 4) * 2.0 ** -24) * (terms + np.abs(b)[None, :, None, None])
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_tensor_core_kernel_within_rounding(shape):
+    N, C, M, H, K, S, pad = shape
+    rng = np.random.default_rng(sum(shape))
+    x = rng.standard_normal((N, C, H, H - 2)).astype(np.float32)
+    w, b = synth.draw_conv_params(rng, C, M, K)
+    exp = ref.conv2d(x, w, b, S=S, pad=pad, relu=False)
+    got = G.gpu_conv(x, w, b, S, pad, False, F32)
+    assert got.shape == exp.shape
+    assert (np.abs(got.astype(np.float64) - exp) <= bound(x, w, b, S, pad, K, C)).all()
+
+
+@pytest.mark.parametrize("offset,total", [(8, 160), (3, 135)])     # 16-byte stores, 4-byte stores
+def test_tensor_core_kernel_writes_its_slice_only(offset, total):
+    x, w, b = synth.conv_layer_case(8, 12, 128, 128, 29, 3)
+    exp = ref.conv2d(x, w, b, S=1, pad=1, relu=True)
+    got = G.gpu_conv(x, w, b, 1, 1, True, F32, c_offset=offset, c_total=total, fill=-7.0)
+    assert (np.abs(got[:, offset:offset + 128].astype(np.float64) - exp) <= bound(x, w, b, 1, 1, 3, 128)).all()
+    assert (got[:, :offset] == -7.0).all() and (got[:, offset + 128:] == -7.0).all()
+
+
+@pytest.mark.parametrize("K", [1, 3])
+def test_exact_sums_stay_exact_and_infinities_come_through(K):
+    """One kernel element per output layer: the outputs are input values, to the last bit; and an infinity, a NaN and the
+    largest float end up where multiply-adds put them."""
+    rng = np.random.default_rng(5)
+    N, C, H = 16, 160, 27
+    x = rng.standard_normal((N, C, H, H)).astype(np.float32)
+    w = np.zeros((C, C, K, K), np.float32)
+    w[np.arange(C), rng.permutation(C), K // 2, K // 2] = 1.0
+    b = np.zeros(C, np.float32)
+    exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=False)
+    np.testing.assert_array_equal(G.gpu_conv(x, w, b, 1, K // 2, False, F32), exp)
+    x[1, 5, 3, 4], x[2, 7, 20, 20], x[3, 9, 0, 0] = np.inf, np.nan, np.finfo(np.float32).max
+    with np.errstate(invalid="ignore"):
+        exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=False)
+    np.testing.assert_array_equal(G.gpu_conv(x, w, b, 1, K // 2, False, F32), exp)
