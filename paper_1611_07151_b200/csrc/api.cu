@@ -25,7 +25,7 @@ bool chained_launch_enabled()
     return on;
 }
 
-// The two expands of a fire layer go out as one launch (bf16) unless SQN_PAIR_LAUNCH=0.
+// The two expands of a fire layer go out as one launch (16-bit types; fp32 where they are small) unless SQN_PAIR_LAUNCH=0.
 bool pair_launch_enabled()
 {
     static const bool on = [] {
@@ -157,6 +157,7 @@ int run_expands(const ConvDesc& d1_in, const ConvDesc& d3_in, int dtype, cudaStr
         }
         if (rc != SQN_ERR_UNSUPPORTED) return rc;
     }
+    if (dtype == SQN_F32 && pair_launch_enabled() && !d1.pool && !d3.pool) return launch_conv_f32_pair(d1, d3, stream, paired);
     const int rc = run_conv(d1, dtype, nullptr, 0, stream);
     return rc != SQN_OK ? rc : run_conv(d3, dtype, nullptr, 0, stream);
 }
@@ -565,6 +566,7 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
         if (is16(dt)) {
             if ((rc = stem_bf16(d)) != SQN_OK) return rc;
         } else {
+            d.params_static = 1;
             if ((rc = launch_conv_f32(d, st)) != SQN_OK) return rc;
         }
         mark("conv1");
@@ -666,7 +668,7 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
             }
         }
         if (!fused_pool) {
-            if (is16(dt) && pair_launch_enabled()) {
+            if (pair_launch_enabled()) {
                 if ((rc = run_expands(d1, d3, dt, st, nullptr)) != SQN_OK) return rc;
                 mark((nm + "_e1+e3").c_str());
             } else {

@@ -326,24 +326,6 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
     p.out_c_offset = d.out_c_offset; p.out_c_total = d.out_c_total; p.relu = d.relu;
 
     const bool vec = (d.Cin % 4 == 0);
-    {
-        // The tensor-core kernel (conv_f32_tc.cu) starts and ends more slowly (5 us against 2) but is up to four times as
-        // fast on long reductions with many layers; this one keeps the small layers (SqueezeNet at batch 1: fire2's
-        // expand-1x1 2.9 us against 5.3, its squeeze 5.4 against 7.2) and those bound by memory with few layers.  Estimate
-        // for this kernel, fitted to SqueezeNet's layers at batch 1 .. 256: latency of the reduction loop, FFMA rate, or
-        // bytes.  Measured at batch 256, this kernel / the other: conv1 2687 / 1054 us, fire4's expand-3x3 1296 / 394,
-        // conv10 1256 / 353, fire8's squeeze 234 / 132, fire2's squeeze 123 / 150, its expand-1x1 88 / 107.
-        const float rate = 37.2e6f * (vec ? 0.58f : 0.44f);                       // multiply-adds per us
-        float us = 0.035f * (float)Kdim;
-        const float fma_us = (float)M * (float)d.Cout * (float)Kdim / rate;
-        const float mem_us = 4.f * ((float)d.N * d.H * d.W * d.Cin + (float)M * d.Cout) / 2.7e6f;
-        if (fma_us > us) us = fma_us;
-        if (mem_us > us) us = mem_us;
-        if (6.1f + 0.45f * (float)((Kdim + 31) / 32) < 2.f + us) {      // (the other kernel's time for one tile: not worth a plan if above)
-            const int rc = launch_conv_f32_tc(d, 2.f + us, stream);
-            if (rc != SQN_ERR_UNSUPPORTED) return rc;
-        }
-    }
     // output-layer tile: the candidate that wastes the fewest padded columns, larger on ties
     const int cand[6] = {128, 96, 64, 48, 32, 16};
     int best = 128;
@@ -377,6 +359,31 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
             if (best_t < 0 || t < best_t) { best_t = t; bm = sh.bm; bn = sh.bn; }
         }
     }
+    {
+        // Which of the three fp32 kernels: by estimated time.  This one: rounds of CTAs at 0.6 of the FFMA rate (0.45 with
+        // 4-byte loads), the latency of the reduction loop, or bytes.  Measured, this kernel / the small layers' / the tensor
+        // cores' -- batch 1: fire9's squeeze 19.6 / 4.7 / 18.0 us, fire6's expand-3x3 16.4 / 6.4 / 15.5, fire4's 14.5 / 11.3 /
+        // 12.6, conv1 25.7 / 31 / 17.4; batch 16: fire4's expand-3x3 99 / 109 / 33, its expand-1x1 17.2 / 34 / 11.5, fire2's
+        // expand-1x1 6.9 / 15.6 / 10.0; batch 256: conv1 2687 / - / 1054, fire4's expand-3x3 1296 / - / 394, conv10 1256 / - /
+        // 353, fire2's squeeze 123 / - / 150, its expand-1x1 88 / - / 107.
+        const double eff = bm == 128 ? (bn == 128 ? 1.0 : bn == 96 ? 0.95 : bn == 64 ? 0.85 : 0.75)
+                         : bm == 256 ? (bn == 32 ? 0.85 : 0.6) : (bn == 128 ? 0.85 : bn == 64 ? 0.6 : 0.4);
+        const double area = (double)((ctas_of(bm, bn) + sms - 1) / sms) * bm * bn / eff;
+        float us = (float)(area * (double)Kdim / (128.0 * 1965.0 * (vec ? 0.6 : 0.45)));
+        const float lat_us = 0.035f * (float)Kdim, mem_us = 4.f * ((float)d.N * d.H * d.W * d.Cin + (float)M * d.Cout) / 2.7e6f;
+        if (lat_us > us) us = lat_us;
+        if (mem_us > us) us = mem_us;
+        us += 2.f;
+        const float small_us = f32_small_estimate(d), other_us = small_us < us ? small_us : us;
+        if (6.1f + 0.45f * (float)((Kdim + 31) / 32) < other_us) {      // (one tile of the tensor-core kernel: not worth a plan if above)
+            const int rc = launch_conv_f32_tc(d, other_us, stream);
+            if (rc != SQN_ERR_UNSUPPORTED) return rc;
+        }
+        if (small_us < us) {
+            const int rc = launch_conv_f32_small(&d, 1, stream);
+            if (rc != SQN_ERR_UNSUPPORTED) return rc;
+        }
+    }
     switch (bm * 1000 + bn) {
         case 128128: return launch_cfg<128, 128, 4, 2>(p, vec, stream);
         case 128096: return launch_cfg<128, 96, 2, 3>(p, vec, stream);
@@ -388,6 +395,23 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
         case 64064: return launch_cfg<64, 64, 2, 1>(p, vec, stream);
         default: return launch_cfg<64, 32, 1, 1>(p, vec, stream);
     }
+}
+
+// One launch for two layers saves a launch's start and end (2 us of the squeezes' and expands' 3 to 12 at batch 1: fp32
+// forward of one image 168 -> 158 us, fire4 17.7 -> 15.4) as long as the small layers' kernel suits both; the line is where
+// its estimate meets the tensor-core kernel's on fire4's and fire8's expand-3x3.
+int launch_conv_f32_pair(const ConvDesc& a, const ConvDesc& b, cudaStream_t stream, bool* paired)
+{
+    if (paired) *paired = false;
+    int rc = SQN_ERR_UNSUPPORTED;
+    if (f32_small_estimate(a) < 14.f && f32_small_estimate(b) < 14.f) {
+        const ConvDesc two[2] = {b, a};             // the longer reduction's tiles first
+        rc = launch_conv_f32_small(two, 2, stream);
+        if (rc == SQN_OK && paired) *paired = true;
+    }
+    if (rc != SQN_ERR_UNSUPPORTED) return rc;
+    rc = launch_conv_f32(a, stream);
+    return rc != SQN_OK ? rc : launch_conv_f32(b, stream);
 }
 
 }  // namespace sqn

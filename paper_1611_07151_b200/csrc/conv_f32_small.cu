@@ -1,0 +1,307 @@
+// fp32 convolution for small layers (one image, few pixels): FFMA implicit GEMM with the reduction split over the warps of a
+// CTA.
+//
+// With few output tiles a layer's time is the latency of its reduction loop: load a tile of operands, synchronise, multiply,
+// one step after another (conv_f32.cu: 1100 clocks per 16 reduction elements when every SM has one CTA).  Here every warp of a
+// CTA owns a slice of the reduction -- chunks of 16 elements warp, warp + SL, ... -- and the whole output tile: it copies its
+// chunks asynchronously into a ring of its own, waits for nobody else, and the warps' partial sums are added once at the end,
+// in a fixed order.  Operand rows are stored as they lie in memory (reduction index contiguous, 80-byte pitch): a thread
+// takes four reduction elements of its 8 pixels and 4 layers with twelve 16-byte reads, free of bank conflicts, for 128
+// multiply-adds.  Two layers that read the same input (the expands of a fire layer) go out as one grid.
+#include <cstring>
+
+#include "f32_common.cuh"
+#include "sqn_internal.h"
+
+namespace sqn {
+namespace {
+
+constexpr int SK = 16;                  // reduction elements per chunk
+constexpr int SPITCH = SK + 4;          // floats per operand row: rows of consecutive threads fall into different banks
+
+struct F32SmallParams {
+    const float* in;
+    const float* w;
+    const float* bias;
+    float* out;
+    int* status;
+    int Cin, H, W, Cout, K, S, pad, OW, OHW, M, Kdim;
+    int out_c_offset, out_c_total, relu;
+    FastDiv div_ohw, div_ow, div_cin, div_k;
+    int chunks;
+    int n_tiles, blocks;
+    int vec_store, early;
+};
+
+// TY x TX threads of a warp, RM x 4 outputs each: tiles of RM*TY pixels x 4*TX layers.
+template <int TY, int RM, int SL, int ST, bool VEC>
+__device__ __forceinline__ void conv_f32_small_body(const F32SmallParams& p, const int bid)
+{
+    constexpr int TX = 32 / TY, TM = RM * TY, TN = 4 * TX, ROWS = TM + TN;
+    constexpr int SLOT = ROWS * SPITCH;                         // floats per ring slot
+    extern __shared__ __align__(16) float sm_small[];
+    __shared__ int3 rows[VEC ? 1 : TM];                         // scalar path: {offset, first row, first column} of every pixel's window
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ty = lane / TX, tx = lane % TX;
+    const int mt = bid / p.n_tiles, n0 = (bid - mt * p.n_tiles) * TN, m0 = mt * TM;
+    float* ring = sm_small + warp * (ST * SLOT);
+    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+
+    auto window = [&](int m, int& off, int& ih, int& iw) {      // window of output pixel m
+        if (m < p.M) {
+            const int img = fast_div(m, p.div_ohw), r = m - img * p.OHW;
+            const int oh = fast_div(r, p.div_ow), ow = r - oh * p.OW;
+            ih = oh * p.S - p.pad; iw = ow * p.S - p.pad;
+            off = ((img * p.H + ih) * p.W + iw) * p.Cin;
+        } else { off = 0; ih = -(1 << 30); iw = 0; }
+    };
+    constexpr int NA = VEC ? TM / 8 : 1;
+    int a_off[NA], a_ih[NA], a_iw[NA];
+    if (VEC) {
+#pragma unroll
+        for (int j = 0; j < NA; ++j) window(m0 + (lane >> 2) + 8 * j, a_off[j], a_ih[j], a_iw[j]);
+    } else {
+        for (int r = tid; r < TM; r += 32 * SL) {
+            int3 v;
+            window(m0 + r, v.x, v.y, v.z);
+            rows[r] = v;
+        }
+        __syncthreads();
+    }
+    // one chunk of the reduction into ring slot `slot`: pixels and kernels apart, so that kernels may be asked for early
+    auto load_w = [&](int ch, int slot) {
+        const uint32_t dst = ring_s + (uint32_t)(slot * SLOT + TM * SPITCH) * 4u;
+        if (VEC) {
+            const int k = ch * SK + 4 * (lane & 3);
+#pragma unroll
+            for (int j = 0; j < TN / 8; ++j) {
+                const int r = (lane >> 2) + 8 * j;
+                const bool ok = k < p.Kdim && n0 + r < p.Cout;
+                cp_async_16(dst + (uint32_t)(r * SPITCH + 4 * (lane & 3)) * 4u, ok ? p.w + (size_t)(n0 + r) * p.Kdim + k : p.w, ok);
+            }
+        } else {
+            const int k = ch * SK + (lane & 15);
+#pragma unroll
+            for (int j = 0; j < TN / 2; ++j) {
+                const int r = (lane >> 4) + 2 * j;
+                const bool ok = k < p.Kdim && n0 + r < p.Cout;
+                cp_async_4(dst + (uint32_t)(r * SPITCH + (lane & 15)) * 4u, ok ? p.w + (size_t)(n0 + r) * p.Kdim + k : p.w, ok);
+            }
+        }
+    };
+    auto load_x = [&](int ch, int slot) {
+        const uint32_t dst = ring_s + (uint32_t)(slot * SLOT) * 4u;
+        const int k = ch * SK + (VEC ? 4 * (lane & 3) : lane & 15);
+        const int t = fast_div(k, p.div_cin), c = k - t * p.Cin, kh = fast_div(t, p.div_k), kw = t - kh * p.K;
+        const int off = (kh * p.W + kw) * p.Cin + c;
+        if (VEC) {
+#pragma unroll
+            for (int j = 0; j < NA; ++j) {
+                const bool ok = k < p.Kdim && (unsigned)(a_ih[j] + kh) < (unsigned)p.H && (unsigned)(a_iw[j] + kw) < (unsigned)p.W;
+                cp_async_16(dst + (uint32_t)(((lane >> 2) + 8 * j) * SPITCH + 4 * (lane & 3)) * 4u, ok ? p.in + (a_off[j] + off) : p.in, ok);
+            }
+        } else {
+#pragma unroll 8
+            for (int j = 0; j < TM / 2; ++j) {
+                const int r = (lane >> 4) + 2 * j;
+                const int3 v = rows[r];
+                const bool ok = k < p.Kdim && (unsigned)(v.y + kh) < (unsigned)p.H && (unsigned)(v.z + kw) < (unsigned)p.W;
+                cp_async_4(dst + (uint32_t)(r * SPITCH + (lane & 15)) * 4u, ok ? p.in + (v.x + off) : p.in, ok);
+            }
+        }
+    };
+
+    const int mine = p.chunks > warp ? (p.chunks - warp + SL - 1) / SL : 0;
+    // the first chunks' kernels may be fetched before the grid ahead has finished (a net's own parameters)
+    if (!p.early) chain_wait();
+#pragma unroll
+    for (int i = 0; i < ST - 1; ++i)
+        if (i < mine) load_w(warp + SL * i, i);
+    if (p.early) chain_wait();
+#pragma unroll
+    for (int i = 0; i < ST - 1; ++i) {
+        if (i < mine) load_x(warp + SL * i, i);
+        cp_async_commit();
+    }
+    float acc[RM][4];
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int i = 0, slot = 0; i < mine; ++i) {
+        cp_async_wait<ST - 2>();
+        __syncwarp();                   // chunk i is here for every lane, and every lane has done with chunk i - 1's slot
+        {
+            const int nx = i + ST - 1;
+            const int ns = slot == 0 ? ST - 1 : slot - 1;
+            if (nx < mine) { load_w(warp + SL * nx, ns); load_x(warp + SL * nx, ns); }
+            cp_async_commit();
+        }
+        const float* xs = ring + slot * SLOT + ty * SPITCH;
+        const float* ws = ring + slot * SLOT + (TM + tx) * SPITCH;
+#pragma unroll
+        for (int kk = 0; kk < SK; kk += 4) {
+            float4 a[RM], b[4];
+#pragma unroll
+            for (int r = 0; r < RM; ++r) a[r] = *reinterpret_cast<const float4*>(xs + r * TY * SPITCH + kk);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) b[c] = *reinterpret_cast<const float4*>(ws + c * TX * SPITCH + kk);
+#pragma unroll
+            for (int r = 0; r < RM; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    acc[r][c] = fmaf(a[r].x, b[c].x, acc[r][c]);
+                    acc[r][c] = fmaf(a[r].y, b[c].y, acc[r][c]);
+                    acc[r][c] = fmaf(a[r].z, b[c].z, acc[r][c]);
+                    acc[r][c] = fmaf(a[r].w, b[c].w, acc[r][c]);
+                }
+        }
+        if (++slot == ST) slot = 0;
+    }
+    cp_async_wait<0>();
+    __syncwarp();
+    // partial sums into the warp's own ring, then all warps' sums in order
+    constexpr int RP = TN + 4;
+    static_assert(TM * RP <= ST * SLOT, "the partial sums fit the ring");
+#pragma unroll
+    for (int r = 0; r < RM; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ring[(ty + TY * r) * RP + tx + TX * c] = acc[r][c];
+    __syncthreads();
+#pragma unroll
+    for (int i0 = 0; i0 < TM * TN / 4; i0 += 32 * SL) {
+        const int i = tid + i0;
+        if (i >= TM * TN / 4) break;
+        const int r = i / (TN / 4), l4 = 4 * (i % (TN / 4));
+        const int m = m0 + r, n = n0 + l4;
+        if (m >= p.M || n >= p.Cout) continue;
+        float4 v = *reinterpret_cast<const float4*>(sm_small + r * RP + l4);
+#pragma unroll
+        for (int s = 1; s < SL; ++s) {
+            const float4 q = *reinterpret_cast<const float4*>(sm_small + s * (ST * SLOT) + r * RP + l4);
+            v.x += q.x; v.y += q.y; v.z += q.z; v.w += q.w;
+        }
+        const float* bias = p.bias + n;
+        v.x += __ldg(bias);
+        if (n + 1 < p.Cout) v.y += __ldg(bias + 1);
+        if (n + 2 < p.Cout) v.z += __ldg(bias + 2);
+        if (n + 3 < p.Cout) v.w += __ldg(bias + 3);
+        if (p.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+        if (!sqn_dbg_ok(m >= 0 && p.out_c_offset + n < p.out_c_total, p.status)) continue;
+        float* dst = p.out + (size_t)m * p.out_c_total + p.out_c_offset + n;
+        if (p.vec_store && n + 4 <= p.Cout) *reinterpret_cast<float4*>(dst) = v;
+        else {
+            dst[0] = v.x;
+            if (n + 1 < p.Cout) dst[1] = v.y;
+            if (n + 2 < p.Cout) dst[2] = v.z;
+            if (n + 3 < p.Cout) dst[3] = v.w;
+        }
+    }
+}
+
+template <int TY, int RM, int SL, int ST, bool VEC>
+__global__ void __launch_bounds__(32 * SL, 16 / SL)
+conv_f32_small_kernel(const __grid_constant__ F32SmallParams p0, const __grid_constant__ F32SmallParams p1)
+{
+    chain_release();
+    if ((int)blockIdx.x < p0.blocks) conv_f32_small_body<TY, RM, SL, ST, VEC>(p0, (int)blockIdx.x);
+    else conv_f32_small_body<TY, RM, SL, ST, VEC>(p1, (int)blockIdx.x - p0.blocks);
+}
+
+bool fill(const ConvDesc& d, int tm, int tn, F32SmallParams* p)
+{
+    std::memset(p, 0, sizeof(*p));
+    const long long M = (long long)d.N * d.OH * d.OW, Kdim = (long long)d.K * d.K * d.Cin;
+    if (M > 0x7fffffffLL - 512 || Kdim > 0x7fffffffLL - 64 || (long long)d.N * d.H * d.W * d.Cin > 0x3fffffffLL) return false;
+    if (((long long)d.K * d.W + d.K) * d.Cin + (long long)d.pad * (d.W + 1) * d.Cin > 0x3fffffffLL) return false;
+    p->in = static_cast<const float*>(d.in); p->w = static_cast<const float*>(d.w); p->bias = d.bias;
+    p->out = static_cast<float*>(d.out); p->status = device_status_word();
+    p->Cin = d.Cin; p->H = d.H; p->W = d.W; p->Cout = d.Cout; p->K = d.K; p->S = d.S; p->pad = d.pad;
+    p->OW = d.OW; p->OHW = d.OH * d.OW; p->M = (int)M; p->Kdim = (int)Kdim;
+    p->out_c_offset = d.out_c_offset; p->out_c_total = d.out_c_total; p->relu = d.relu;
+    p->div_ohw = make_div(p->OHW); p->div_ow = make_div(p->OW); p->div_cin = make_div(p->Cin); p->div_k = make_div(p->K);
+    p->chunks = (p->Kdim + SK - 1) / SK;
+    p->n_tiles = (d.Cout + tn - 1) / tn;
+    const long long blocks = ((M + tm - 1) / tm) * p->n_tiles;
+    if (blocks > 0x3fffffffLL) return false;
+    p->blocks = (int)blocks;
+    p->vec_store = d.out_c_offset % 4 == 0 && d.out_c_total % 4 == 0;
+    p->early = d.params_static;
+    return true;
+}
+
+template <int TY, int RM, int SL, int ST, bool VEC>
+cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
+{
+    constexpr size_t smem = (size_t)SL * ST * (RM * TY + 128 / TY) * SPITCH * 4;
+    static const cudaError_t attr_rc =
+        cudaFuncSetAttribute(conv_f32_small_kernel<TY, RM, SL, ST, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr_rc != cudaSuccess) return attr_rc;
+    return launch_chained(conv_f32_small_kernel<TY, RM, SL, ST, VEC>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
+}
+
+// Tile, warps and ring for a layer (or two) of so many tiles; measured on SqueezeNet's layers at batch 1 and 4:
+//  - half as many pixels per thread where the larger tiles would leave half of the SMs without a CTA (fire9's squeeze 6.9 ->
+//    4.7 us, fire5's 4.2 -> 3.2);
+//  - eight warps and three slots per warp where every SM gets one CTA at most, two slots where two CTAs per SM make it one
+//    wave (fire8's expand-3x3 at batch 1, 184 tiles: 14.1 -> 12.5 us), else four warps and three slots.
+struct SmallConfig { bool narrow; int rm, tm, tn; };
+
+SmallConfig config_of(const ConvDesc* d, int n)
+{
+    SmallConfig c;
+    c.narrow = d[0].Cout <= 16 && (n == 1 || d[1].Cout <= 16);
+    c.tn = c.narrow ? 16 : 32;
+    c.rm = 8;
+    long long blocks = 0;
+    for (int i = 0; i < n; ++i)
+        blocks += (((long long)d[i].N * d[i].OH * d[i].OW + (c.narrow ? 63 : 31)) / (c.narrow ? 64 : 32)) * ((d[i].Cout + c.tn - 1) / c.tn);
+    if (blocks <= 74) c.rm = 4;
+    c.tm = (c.narrow ? 8 : 4) * c.rm;
+    return c;
+}
+
+template <int TY, int RM, bool VEC>
+cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
+{
+    const int blocks = a.blocks + b.blocks;
+    const bool deep = a.chunks > 2 || (b.blocks && b.chunks > 2);       // (more than two warps have chunks)
+    if (deep && blocks <= 148) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
+    if (deep && blocks <= 296) return launch<TY, RM, 8, 2, VEC>(a, b, stream);
+    return launch<TY, RM, 4, 3, VEC>(a, b, stream);
+}
+
+}  // namespace
+
+// Microseconds, fitted to SqueezeNet's layers at batch 1 and 4 (within 25 %): a launch, then the busiest SM's tiles at 260
+// clocks per chunk (150 with the smaller tile; 750 where the operands come in pieces of 4 bytes).
+float f32_small_estimate(const ConvDesc& d)
+{
+    const SmallConfig c = config_of(&d, 1);
+    const long long blocks = (((long long)d.N * d.OH * d.OW + c.tm - 1) / c.tm) * ((d.Cout + c.tn - 1) / c.tn);
+    const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
+    const float us = (float)((blocks + 147) / 148) * (chunks * (d.Cin % 4 != 0 ? 750.f : c.rm == 4 ? 150.f : 260.f) + 450.f) / 1965.f;
+    return 2.2f + (blocks > 296 ? 1.2f * us : us);
+}
+
+int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
+{
+    const SmallConfig c = config_of(d, n);
+    bool vec = true;
+    F32SmallParams p[2];
+    for (int i = 0; i < n; ++i) {
+        if (!fill(d[i], c.tm, c.tn, &p[i])) return SQN_ERR_UNSUPPORTED;
+        vec = vec && d[i].Cin % 4 == 0;
+    }
+    if (n == 1) { p[1] = p[0]; p[1].blocks = 0; }
+    cudaError_t rc;
+    if (c.rm == 8) rc = c.narrow ? (vec ? launch_ty<8, 8, true>(p[0], p[1], stream) : launch_ty<8, 8, false>(p[0], p[1], stream))
+                                 : (vec ? launch_ty<4, 8, true>(p[0], p[1], stream) : launch_ty<4, 8, false>(p[0], p[1], stream));
+    else rc = c.narrow ? (vec ? launch_ty<8, 4, true>(p[0], p[1], stream) : launch_ty<8, 4, false>(p[0], p[1], stream))
+                       : (vec ? launch_ty<4, 4, true>(p[0], p[1], stream) : launch_ty<4, 4, false>(p[0], p[1], stream));
+    if (rc != cudaSuccess) return SQN_ERR_CUDA;
+    note_launch();
+    return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
+}
+
+}  // namespace sqn

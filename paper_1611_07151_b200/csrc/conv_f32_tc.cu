@@ -41,6 +41,7 @@
 //   27      MMA issuer (one elected lane), on the scheduler with the least other work
 #include <cstring>
 
+#include "f32_common.cuh"
 #include "ptx_sm100.cuh"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
@@ -72,8 +73,6 @@ enum { FT_FLAT = 0, FT_PATCH = 1, FT_BOX = 2 };
 // Kernels: split once per CTA and kept packed in shared memory; streamed for every tile by TMA boxes; streamed by copies of
 // 4 bytes (BOX, where the rows are no TMA tensor).
 enum { FT_W_PACKED = 0, FT_W_BOXES = 1, FT_W_COPIES = 2 };
-
-struct FastDiv { unsigned mul; int shift; };        // n / d for 0 <= n < 2^31 (mul = 0: d = 1)
 
 struct F32TcParams {
     const float* in;
@@ -126,20 +125,6 @@ struct F32TcShared {
     volatile int abort_flag;
 };
 
-__device__ __forceinline__ int fast_div(int n, FastDiv d)
-{
-    return d.mul ? (int)(__umulhi((unsigned)n, d.mul) >> d.shift) : n;
-}
-
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, bool ok)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_4(uint32_t dst, const void* src, bool ok)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
 // Two values as three packed bf16 pairs whose sums are the values (see the head of the file).
@@ -829,17 +814,6 @@ struct F32TcPlan {
     F32TcParams p;
     size_t smem;
 };
-
-FastDiv make_div(int d)
-{
-    FastDiv f = {0u, 0};
-    if (d <= 1) return f;
-    int l = 0;
-    while ((1ll << l) < d) ++l;
-    f.mul = (unsigned)(((1ull << (31 + l)) + (unsigned)d - 1) / (unsigned)d);
-    f.shift = l - 1;
-    return f;
-}
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 inline size_t up1k(size_t v) { return (v + 1023) / 1024 * 1024; }

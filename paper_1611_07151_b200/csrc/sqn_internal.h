@@ -30,11 +30,18 @@ void note_launch(int n = 1);
 // Device status word shared by all kernels (0 = fine, else an sqn_status).
 int* device_status_word();
 
-// fp32 path, any (K, S, pad, Cin, Cout): on the tensor cores with every operand split exactly into three bf16 numbers, or
-// on the FFMA pipes, whichever is estimated to be faster for the shape (see launch_conv_f32).
+// fp32 path, any (K, S, pad, Cin, Cout): three kernels, whichever is estimated to be the fastest for the shape (see
+// launch_conv_f32 in conv_f32.cu).
 int launch_conv_f32(const ConvDesc& d, cudaStream_t stream);
-// The tensor-core kernel; SQN_ERR_UNSUPPORTED where it does not apply or where its own estimate is above limit_us.
+// Two layers that read the same input: one launch where both are small, else two.  *paired (may be null) tells which.
+int launch_conv_f32_pair(const ConvDesc& a, const ConvDesc& b, cudaStream_t stream, bool* paired);
+// On the tensor cores, every operand split exactly into three bf16 numbers; SQN_ERR_UNSUPPORTED where the kernel does not
+// apply or where its own estimate is above limit_us.
 int launch_conv_f32_tc(const ConvDesc& d, float limit_us, cudaStream_t stream);
+// n (1 or 2) small layers in one launch, the reduction split over a CTA's warps (SQN_ERR_UNSUPPORTED: sizes beyond its
+// 32-bit offsets), and its time in microseconds.
+int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream);
+float f32_small_estimate(const ConvDesc& d);
 
 // bf16 path: tcgen05/TMEM implicit GEMM fed by TMA.
 // Returns SQN_ERR_UNSUPPORTED for shapes outside its family.
