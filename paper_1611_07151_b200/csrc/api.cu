@@ -9,6 +9,7 @@
 #include <vector>
 
 #include <cuda_fp16.h>
+#include <unistd.h>
 
 #include "sqn_internal.h"
 
@@ -16,6 +17,13 @@ namespace sqn {
 
 static std::atomic<unsigned long long> g_launches{0};
 void note_launch(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
+bool tuning_env_present()
+{
+    for (char** e = environ; e && *e; ++e)
+        if ((*e)[0] == 'S' && std::strncmp(*e, "SQN_", 4) == 0) return true;
+    return false;
+}
+
 bool chained_launch_enabled()
 {
     static const bool on = [] {
@@ -329,7 +337,8 @@ const FireSpec kFire[8] = {
     {"fire5", 256, 32, 128, 27, false}, {"fire6", 256, 48, 192, 27, false}, {"fire7", 384, 48, 192, 27, false},
     {"fire8", 384, 64, 256, 27, true},  {"fire9", 512, 64, 256, 13, false}};
 
-struct Slot { std::string name; int C, H, W; size_t offset; };   // offset in bytes for batch 1 element counts below
+struct Slot { std::string name; int C, H, W; };
+constexpr int MAX_SLOTS = 24;
 
 }  // namespace
 
@@ -339,6 +348,7 @@ struct sqn_net {
     int dtype;
     int max_batch;
     std::vector<Slot> slots;   // per-image element counts; byte offsets are computed per batch
+    int i_conv1, i_pool1, i_conv10, i_sq[8], i_out[8], i_pool[8];      // places in `slots` (i_pool: -1 where no pool follows)
     // optional per-launch timing: a ring of event rows, one row per forward
     int prof_slots = 0;
     long long prof_forwards = 0;
@@ -362,27 +372,31 @@ constexpr int IMG = 227;
 
 void build_slots(sqn_net* net)
 {
-    auto add = [&](const std::string& n, int C, int H, int W) { net->slots.push_back({n, C, H, W, 0}); };
-    add("conv1", 96, 111, 111);
-    add("pool1", 96, 55, 55);
-    for (const FireSpec& f : kFire) {
-        add(std::string(f.name) + "_sq", f.s, f.hw, f.hw);
-        add(f.name, 2 * f.e, f.hw, f.hw);
-        if (f.pool_after) add(std::string("pool") + (f.name + 4), 2 * f.e, (f.hw - 3) / 2 + 1, (f.hw - 3) / 2 + 1);
+    auto add = [&](const std::string& n, int C, int H, int W) {
+        net->slots.push_back({n, C, H, W});
+        return (int)net->slots.size() - 1;
+    };
+    net->i_conv1 = add("conv1", 96, 111, 111);
+    net->i_pool1 = add("pool1", 96, 55, 55);
+    for (int i = 0; i < 8; ++i) {
+        const FireSpec& f = kFire[i];
+        net->i_sq[i] = add(std::string(f.name) + "_sq", f.s, f.hw, f.hw);
+        net->i_out[i] = add(f.name, 2 * f.e, f.hw, f.hw);
+        net->i_pool[i] = f.pool_after ? add(std::string("pool") + (f.name + 4), 2 * f.e, (f.hw - 3) / 2 + 1, (f.hw - 3) / 2 + 1) : -1;
     }
-    add("conv10", 1000, 13, 13);
+    net->i_conv10 = add("conv10", 1000, 13, 13);
 }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Byte offset of every slot inside the workspace for a given batch; returns total bytes.
-size_t layout(const sqn_net* net, int batch, std::vector<size_t>* offs, size_t* stem_off)
+// Byte offset of every slot inside the workspace for a given batch (offs: MAX_SLOTS places, may be null); returns total bytes.
+size_t layout(const sqn_net* net, int batch, size_t* offs, size_t* stem_off)
 {
     size_t cur = 0;
     const size_t es = esize(net->dtype);
-    if (offs) offs->clear();
+    size_t i = 0;
     for (const Slot& s : net->slots) {
-        if (offs) offs->push_back(cur);
+        if (offs) offs[i++] = cur;
         cur = align_up(cur + (size_t)batch * s.C * s.H * s.W * es, 1024);
     }
     if (stem_off) *stem_off = cur;
@@ -479,8 +493,8 @@ extern "C" int squeezenet_layer_output(const sqn_net* net, const char* name, voi
     for (int f = 0; f < 8; ++f)
         if ((net->fused_fire_mask >> f & 1u) && std::string(kFire[f].name) + "_sq" == name)
             return SQN_ERR_UNSUPPORTED;   // kept in shared memory by the fused fire kernel of the last forward
-    std::vector<size_t> offs;
-    layout(net, batch, &offs, nullptr);
+    size_t offs[MAX_SLOTS];
+    layout(net, batch, offs, nullptr);
     *ptr = static_cast<char*>(workspace) + offs[i];
     if (C) *C = net->slots[i].C;
     if (H) *H = net->slots[i].H;
@@ -510,20 +524,19 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
     if (!aligned16(in_nhwc) || !aligned16(workspace)) return SQN_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int dt = net->dtype;
-    std::vector<size_t> offs;
-    size_t stem_off = 0;
-    const size_t total = layout(net, batch, &offs, &stem_off);
+    size_t offs[MAX_SLOTS], stem_off = 0;
+    const size_t total = layout(net, batch, offs, &stem_off);
     char* ws = static_cast<char*>(workspace);
-    auto buf = [&](const std::string& name) -> void* { return ws + offs[find_slot(net, name.c_str())]; };
+    auto buf = [&](int slot) -> void* { return ws + offs[slot]; };
 
     // per-launch timing (off unless squeezenet_profile enabled it)
     const bool prof = net->prof_slots > 0;
     std::vector<cudaEvent_t>* row = prof ? &net->prof_events[net->prof_forwards % net->prof_slots] : nullptr;
     const bool first = prof && net->prof_names.empty();
     size_t mark_i = 0;
-    auto mark = [&](const char* name) {
+    auto mark = [&](const char* name, const char* suffix = "") {
         if (!prof) return;
-        if (first) net->prof_names.push_back(name);
+        if (first) net->prof_names.push_back(std::string(name) + suffix);
         if (row->size() <= mark_i) {
             cudaEvent_t e;
             cudaEventCreate(&e);
@@ -555,13 +568,13 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
     };
     if (fuse_pools) {
         // stem and its max-pool in one kernel: the 96x111x111 map never goes to memory
-        rc = make_conv_desc(in_nhwc, net->w[0], net->b[0], buf("pool1"), 3, 96, IMG, IMG, 7, 2, 0, batch, 1, 0, 0, &d);
+        rc = make_conv_desc(in_nhwc, net->w[0], net->b[0], buf(net->i_pool1), 3, 96, IMG, IMG, 7, 2, 0, batch, 1, 0, 0, &d);
         if (rc != SQN_OK) return rc;
         d.pool = 1;
         if ((rc = stem_bf16(d)) != SQN_OK) return rc;
         mark("conv1+pool1");
     } else {
-        rc = make_conv_desc(in_nhwc, net->w[0], net->b[0], buf("conv1"), 3, 96, IMG, IMG, 7, 2, 0, batch, 1, 0, 0, &d);
+        rc = make_conv_desc(in_nhwc, net->w[0], net->b[0], buf(net->i_conv1), 3, 96, IMG, IMG, 7, 2, 0, batch, 1, 0, 0, &d);
         if (rc != SQN_OK) return rc;
         if (is16(dt)) {
             if ((rc = stem_bf16(d)) != SQN_OK) return rc;
@@ -570,16 +583,16 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
             if ((rc = launch_conv_f32(d, st)) != SQN_OK) return rc;
         }
         mark("conv1");
-        if ((rc = launch_maxpool3x3s2(buf("conv1"), buf("pool1"), 96, 111, 111, batch, dt, st)) != SQN_OK) return rc;
+        if ((rc = launch_maxpool3x3s2(buf(net->i_conv1), buf(net->i_pool1), 96, 111, 111, batch, dt, st)) != SQN_OK) return rc;
         mark("pool1");
     }
 
-    const void* cur = buf("pool1");
+    const void* cur = buf(net->i_pool1);
     net->fused_fire_mask = 0;
     for (int i = 0; i < 8; ++i) {
         const FireSpec& f = kFire[i];
-        void* sq = buf(std::string(f.name) + "_sq");
-        void* out = buf(f.name);
+        void* sq = buf(net->i_sq[i]);
+        void* out = buf(net->i_out[i]);
         ConvDesc dsq, d1, d3;
         rc = make_conv_desc(cur, net->w[1 + 3 * i], net->b[1 + 3 * i], sq, f.cin, f.s, f.hw, f.hw, 1, 1, 0, batch, 1, 0,
                             0, &dsq);
@@ -593,19 +606,17 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
         // the net's kernels and bias are not written by anything this forward enqueues
         dsq.params_static = d1.params_static = d3.params_static = 1;
         dsq.f16 = d1.f16 = d3.f16 = f16;
-        const std::string nm(f.name);
         // bf16: squeeze and both expands as one kernel where it applies (no pool behind the layer)
         if (is16(dt) && fused_fire_enabled() && !(f.pool_after && fuse_pools)) {
             rc = launch_fire_fused_bf16(dsq, d1, d3, st);
             if (rc == SQN_OK) {
                 net->fused_fire_mask |= 1u << i;
-                mark((nm + "_fused").c_str());
+                mark(f.name, "_fused");
                 cur = out;
                 if (f.pool_after) {
-                    const std::string pn = std::string("pool") + (f.name + 4);
-                    void* po = buf(pn);
+                    void* po = buf(net->i_pool[i]);
                     if ((rc = launch_maxpool3x3s2(cur, po, 2 * f.e, f.hw, f.hw, batch, dt, st)) != SQN_OK) return rc;
-                    mark(pn.c_str());
+                    mark("pool", f.name + 4);
                     cur = po;
                 }
                 continue;
@@ -613,14 +624,13 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
             if (rc != SQN_ERR_UNSUPPORTED) return rc;
         }
         if ((rc = run_conv(dsq, dt, nullptr, 0, st)) != SQN_OK) return rc;
-        mark((nm + "_sq").c_str());
+        mark(f.name, "_sq");
         // bf16: where a max-pool follows and the expands' kernels fit in shared memory, both expands pool
         // in their epilogues and write their halves of the pooled map; the unpooled map is never stored
         bool fused_pool = false;
         if (f.pool_after && fuse_pools) {
-            const std::string pn = std::string("pool") + (f.name + 4);
             ConvDesc p1 = d1, p3 = d3;
-            p1.out = p3.out = buf(pn);
+            p1.out = p3.out = buf(net->i_pool[i]);
             p1.pool = p3.pool = 1;
             // the pooled kernels take up to 128 output layers: wider expands (fire8: 256) go out in slices of 128
             const int parts = f.e > 128 && f.e % 128 == 0 ? f.e / 128 : 1;
@@ -654,41 +664,40 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
                     }
                     for (int h = 0; h < parts && !done; ++h)
                         if ((rc = run_expands(q1[h], q3[h], dt, st, nullptr)) != SQN_OK) return rc;
-                    mark((nm + "_e1+e3+pool").c_str());
+                    mark(f.name, "_e1+e3+pool");
                 } else {
                     for (int h = 0; h < parts; ++h)
                         if ((rc = run_conv(q1[h], dt, nullptr, 0, st)) != SQN_OK) return rc;
-                    mark((nm + "_e1+pool").c_str());
+                    mark(f.name, "_e1+pool");
                     for (int h = 0; h < parts; ++h)
                         if ((rc = run_conv(q3[h], dt, nullptr, 0, st)) != SQN_OK) return rc;
-                    mark((nm + "_e3+pool").c_str());
+                    mark(f.name, "_e3+pool");
                 }
-                cur = buf(pn);
+                cur = buf(net->i_pool[i]);
                 fused_pool = true;
             }
         }
         if (!fused_pool) {
             if (pair_launch_enabled()) {
                 if ((rc = run_expands(d1, d3, dt, st, nullptr)) != SQN_OK) return rc;
-                mark((nm + "_e1+e3").c_str());
+                mark(f.name, "_e1+e3");
             } else {
                 if ((rc = run_conv(d1, dt, nullptr, 0, st)) != SQN_OK) return rc;
-                mark((nm + "_e1").c_str());
+                mark(f.name, "_e1");
                 if ((rc = run_conv(d3, dt, nullptr, 0, st)) != SQN_OK) return rc;
-                mark((nm + "_e3").c_str());
+                mark(f.name, "_e3");
             }
             cur = out;
             if (f.pool_after) {
-                const std::string pn = std::string("pool") + (f.name + 4);
-                void* po = buf(pn);
+                void* po = buf(net->i_pool[i]);
                 if ((rc = launch_maxpool3x3s2(cur, po, 2 * f.e, f.hw, f.hw, batch, dt, st)) != SQN_OK) return rc;
-                mark(pn.c_str());
+                mark("pool", f.name + 4);
                 cur = po;
             }
         }
     }
     // conv10 1x1 + ReLU, global average, softmax
-    rc = make_conv_desc(cur, net->w[25], net->b[25], buf("conv10"), 512, 1000, 13, 13, 1, 1, 0, batch, 1, 0, 0, &d);
+    rc = make_conv_desc(cur, net->w[25], net->b[25], buf(net->i_conv10), 512, 1000, 13, 13, 1, 1, 0, batch, 1, 0, 0, &d);
     if (rc != SQN_OK) return rc;
     d.params_static = 1;
     d.f16 = f16;
@@ -711,7 +720,7 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
     }
     if ((rc = run_conv(d, dt, nullptr, 0, st)) != SQN_OK) return rc;
     mark("conv10");
-    rc = launch_avgpool_softmax(buf("conv10"), static_cast<float*>(logits_f32), static_cast<float*>(probs_f32), 1000,
+    rc = launch_avgpool_softmax(buf(net->i_conv10), static_cast<float*>(logits_f32), static_cast<float*>(probs_f32), 1000,
                                 13, 13, batch, dt, st);
     if (rc != SQN_OK) return rc;
     mark("head");

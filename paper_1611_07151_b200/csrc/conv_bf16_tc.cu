@@ -33,11 +33,11 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <map>
 #include <cstddef>
+#include <memory>
 #include <mutex>
-#include <string>
 
+#include "plan_cache.h"
 #include "ptx_sm100.cuh"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
@@ -1637,11 +1637,10 @@ struct PlanKey {
     const void *in, *w, *bias, *out, *ws;
     const void *rw, *rbias;     // the rider's kernels and bias (conv_pool_kernel), else null
     int v[14];
-    int r_c_off;
+    int r_c_off, dev;
 };
 
-std::mutex g_plan_mu;
-std::map<std::string, Plan> g_plans;
+PlanCache<PlanKey, Plan> g_plans(4096);
 
 // SQN_POOL_ISSUERS in the environment (tuning aid: 1 or 2 issuer warps for a pooled convolution without a rider), 0 if unset
 int pool_issuers_env()
@@ -1654,7 +1653,7 @@ int pool_issuers_env()
 // force_halves / force_cw != 0: the plan of that kernel variant (CTAs per SM, store chunk width) instead of the
 // layer's own best one, so that it can share a launch with another layer's plan.
 int cached_plan(const ConvDesc& d, bool stem, const void* a_ptr, const void* w_ptr, int Hp, int Wp, const void* ws,
-                Plan* out, int force_halves = 0, int force_cw = 0)
+                std::shared_ptr<const Plan>* out, int force_halves = 0, int force_cw = 0)
 {
     PlanKey k;
     std::memset(&k, 0, sizeof(k));
@@ -1663,34 +1662,16 @@ int cached_plan(const ConvDesc& d, bool stem, const void* a_ptr, const void* w_p
     const int v[14] = {d.N, d.Cin, d.H, d.W, d.Cout, d.K, d.S, d.pad, d.out_c_offset, d.out_c_total, d.relu | (d.pool << 1) | (d.params_static << 2) | (d.stem_prepacked << 3) | (d.f16 << 4),
                        (stem ? 1 : 0) | (force_halves << 4) | ((force_cw & 0xffff) << 8) | (pool_issuers_env() << 24), Hp, Wp};
     std::memcpy(k.v, v, sizeof(v));
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::string key(reinterpret_cast<const char*>(&k), sizeof(k));
-    key.push_back((char)dev);
-    {
-        std::lock_guard<std::mutex> lock(g_plan_mu);
-        auto it = g_plans.find(key);
-        if (it != g_plans.end()) { *out = it->second; return SQN_OK; }
-    }
-    Plan plan;
-    int rc;
-    if (force_halves != 0) {
+    cudaGetDevice(&k.dev);
+    return g_plans.get(k, out, [&](Plan* plan) {
+        if (force_halves == 0) return build_plan(d, stem, a_ptr, w_ptr, Hp, Wp, plan);
         t_force_cw = force_cw < 0 ? 0 : force_cw;
         t_pool_npix = force_cw == -128 ? 128 : 256;       // (pooled layers: the tile size instead of a chunk width)
-        rc = build_plan_cfg(d, stem, a_ptr, w_ptr, Hp, Wp, force_halves, &plan);
+        const int rc = build_plan_cfg(d, stem, a_ptr, w_ptr, Hp, Wp, force_halves, plan);
         t_force_cw = 0;
         t_pool_npix = 256;
-    } else {
-        rc = build_plan(d, stem, a_ptr, w_ptr, Hp, Wp, &plan);
-    }
-    if (rc != SQN_OK) return rc;
-    {
-        std::lock_guard<std::mutex> lock(g_plan_mu);
-        if (g_plans.size() > 4096) g_plans.clear();
-        g_plans[key] = plan;
-    }
-    *out = plan;
-    return SQN_OK;
+        return rc;
+    });
 }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -1727,17 +1708,17 @@ int conv_bf16_supported(const ConvDesc& d)
 // layer, the analogue of the paper's thread-granularity study (Section III-D, Tables 1 and 3).
 int launch_conv_bf16(const ConvDesc& d, cudaStream_t stream)
 {
-    Plan plan;
+    std::shared_ptr<const Plan> plan;
     int ctas = 0, cw = 0;
     const char* v = d.pool ? nullptr : std::getenv("SQN_TC_VARIANT");
     if (v && std::sscanf(v, "%d,%d", &ctas, &cw) == 2 && (ctas == 1 || ctas == 2) && (cw == 16 || cw == 32 || cw == 64)) {
         const int rc = cached_plan(d, false, d.in, d.w, 0, 0, nullptr, &plan, ctas == 1 ? 2 : 1, cw);
         if (rc != SQN_OK) return SQN_ERR_UNSUPPORTED;
-        return launch_plan(plan, stream);
+        return launch_plan(*plan, stream);
     }
     const int rc = cached_plan(d, false, d.in, d.w, 0, 0, nullptr, &plan);
     if (rc != SQN_OK) return rc;
-    return launch_plan(plan, stream);
+    return launch_plan(*plan, stream);
 }
 
 // Two layers that do not depend on one another (the two expands of a fire layer: same input, disjoint layer slices
@@ -1747,41 +1728,41 @@ int launch_conv_bf16(const ConvDesc& d, cudaStream_t stream)
 int launch_conv_bf16_pair(const ConvDesc& small, const ConvDesc& big, cudaStream_t stream)
 {
     if (small.pool != big.pool) return SQN_ERR_UNSUPPORTED;
-    Plan pb, ps;
+    std::shared_ptr<const Plan> pb, ps;
     int rc = cached_plan(big, false, big.in, big.w, 0, 0, nullptr, &pb);
     if (rc != SQN_OK) return rc;
     rc = cached_plan(small, false, small.in, small.w, 0, 0, nullptr, &ps);
     if (rc != SQN_OK) return rc;
-    if (big.pool && ps.p.npix != pb.p.npix) {          // both with the smaller tiles
+    if (big.pool && ps->p.npix != pb->p.npix) {          // both with the smaller tiles
         if (cached_plan(big, false, big.in, big.w, 0, 0, nullptr, &pb, 2, -128) != SQN_OK ||
             cached_plan(small, false, small.in, small.w, 0, 0, nullptr, &ps, 2, -128) != SQN_OK)
             return SQN_ERR_UNSUPPORTED;
     }
-    if (!big.pool && (ps.split != pb.split || ps.p.CW != pb.p.CW)) {
-        rc = cached_plan(small, false, small.in, small.w, 0, 0, nullptr, &ps, pb.halves, pb.p.CW);
+    if (!big.pool && (ps->split != pb->split || ps->p.CW != pb->p.CW)) {
+        rc = cached_plan(small, false, small.in, small.w, 0, 0, nullptr, &ps, pb->halves, pb->p.CW);
         if (rc != SQN_OK) return SQN_ERR_UNSUPPORTED;
     }
-    return launch_plan2(pb, ps, stream);
+    return launch_plan2(*pb, *ps, stream);
 }
 
 // Four pooled layers that read the same input (two slices of each expand of a fire layer) in ONE launch, in the order
 // given (the heavy ones first); all with the 128-pixel tiles.  SQN_ERR_UNSUPPORTED if one of them cannot be planned so.
 int launch_conv_bf16_pool4(const ConvDesc* d, cudaStream_t stream)
 {
-    Plan pl[4];
+    std::shared_ptr<const Plan> pl[4];
     size_t smem = 0;
     int grid = 0;
     for (int i = 0; i < 4; ++i) {
-        if (!d[i].pool || cached_plan(d[i], false, d[i].in, d[i].w, 0, 0, nullptr, &pl[i], 2, -128) != SQN_OK || pl[i].p.npix != 128)
+        if (!d[i].pool || cached_plan(d[i], false, d[i].in, d[i].w, 0, 0, nullptr, &pl[i], 2, -128) != SQN_OK || pl[i]->p.npix != 128)
             return SQN_ERR_UNSUPPORTED;
-        if (pl[i].smem > smem) smem = pl[i].smem;
-        grid += pl[i].grid;
+        if (pl[i]->smem > smem) smem = pl[i]->smem;
+        grid += pl[i]->grid;
     }
     static const cudaError_t attr_rc =
         cudaFuncSetAttribute(conv_pool_kernel4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT);
     if (attr_rc != cudaSuccess) return SQN_ERR_CUDA;
-    const cudaError_t rc = launch_chained(conv_pool_kernel4, dim3((unsigned)grid), dim3(POOLT_THREADS), smem, stream, pl[0].a, pl[0].b,
-                                          pl[0].p, pl[1].a, pl[1].b, pl[1].p, pl[2].a, pl[2].b, pl[2].p, pl[3].a, pl[3].b, pl[3].p);
+    const cudaError_t rc = launch_chained(conv_pool_kernel4, dim3((unsigned)grid), dim3(POOLT_THREADS), smem, stream, pl[0]->a, pl[0]->b,
+                                          pl[0]->p, pl[1]->a, pl[1]->b, pl[1]->p, pl[2]->a, pl[2]->b, pl[2]->p, pl[3]->a, pl[3]->b, pl[3]->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
@@ -1793,25 +1774,25 @@ int launch_conv_bf16_pool4(const ConvDesc* d, cudaStream_t stream)
 int launch_conv_bf16_pool_riders(const ConvDesc* big, const ConvDesc* rider, int n, cudaStream_t stream)
 {
     if (n < 1 || n > 2) return SQN_ERR_UNSUPPORTED;
-    Plan pl[2];
+    std::shared_ptr<const Plan> pl[2];
     for (int i = 0; i < n; ++i) {
         if (!big[i].pool || !rider[i].pool) return SQN_ERR_UNSUPPORTED;
         t_rider = &rider[i];
         int rc = cached_plan(big[i], false, big[i].in, big[i].w, 0, 0, nullptr, &pl[i], 2, -128);      // (the 128-pixel tiles)
-        if (rc == SQN_OK && n == 2 && i == 1 && pl[1].p.npix != pl[0].p.npix)
+        if (rc == SQN_OK && n == 2 && i == 1 && pl[1]->p.npix != pl[0]->p.npix)
             rc = SQN_ERR_UNSUPPORTED;
         t_rider = nullptr;
         if (rc != SQN_OK) return rc == SQN_ERR_CUDA ? rc : SQN_ERR_UNSUPPORTED;
-        if (!pl[i].p.rider) return SQN_ERR_UNSUPPORTED;
+        if (!pl[i]->p.rider) return SQN_ERR_UNSUPPORTED;
     }
-    return n == 1 ? launch_plan(pl[0], stream) : launch_plan2(pl[0], pl[1], stream);
+    return n == 1 ? launch_plan(*pl[0], stream) : launch_plan2(*pl[0], *pl[1], stream);
 }
 
 // Host-only feasibility test of the fused max-pool for a layer (shared-memory budget, shape rules).
 bool conv_bf16_pool_fits(const ConvDesc& d)
 {
     if (!d.pool || conv_bf16_supported(d) != SQN_OK) return false;
-    Plan plan;
+    std::shared_ptr<const Plan> plan;
     return cached_plan(d, false, d.in, d.w, 0, 0, nullptr, &plan) == SQN_OK;
 }
 
@@ -1869,10 +1850,10 @@ int launch_stem_conv_bf16(const ConvDesc& d, void* workspace, size_t workspace_b
     if (rc != SQN_OK) return rc;
     const int Hp = stem_packed_rows(d.H), Wp = stem_packed_cols(d.W);
     unsigned char* ws = static_cast<unsigned char*>(workspace);
-    Plan plan;
+    std::shared_ptr<const Plan> plan;
     rc = cached_plan(d, true, ws, ws + align_up((size_t)d.N * Hp * Wp * 8, 1024), Hp, Wp, workspace, &plan);
     if (rc != SQN_OK) return rc;
-    return launch_plan(plan, stream);
+    return launch_plan(*plan, stream);
 }
 
 int launch_stem_conv_bf16_prepacked(const ConvDesc& d, cudaStream_t stream)
@@ -1880,10 +1861,10 @@ int launch_stem_conv_bf16_prepacked(const ConvDesc& d, cudaStream_t stream)
     if (!d.stem_prepacked) return SQN_ERR_BADARG;
     if (d.Cout % 16 != 0 || d.Cout > 256) return SQN_ERR_UNSUPPORTED;
     if (d.out_c_offset % 8 != 0 || d.out_c_total % 8 != 0) return SQN_ERR_ALIGN;
-    Plan plan;
+    std::shared_ptr<const Plan> plan;
     const int rc = cached_plan(d, true, d.in, d.w, stem_packed_rows(d.H), stem_packed_cols(d.W), nullptr, &plan);
     if (rc != SQN_OK) return rc;
-    return launch_plan(plan, stream);
+    return launch_plan(*plan, stream);
 }
 
 }  // namespace sqn

@@ -9,6 +9,7 @@
 // an 8 x TN block of the output tile (the paper's "thread granularity" g, Section III-D,
 // carried to two dimensions: a loaded window value is reused TN times, a kernel value 8 times).
 #include "sqn_internal.h"
+#include "tc_host.h"
 
 namespace sqn {
 namespace {
@@ -340,12 +341,7 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
     // FFMA efficiency of the thread tile (8 x TN: fewer output layers per thread mean more shared-memory loads per
     // FFMA).  The sum over the reduction index runs in the same order for every tile shape, so the values do not
     // depend on this choice.
-    int sms = 148;
-    {
-        int dev = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 148;
-    }
+    const int sms = sm_count();
     auto ctas_of = [&](int tm, int tn) { return ((M + tm - 1) / tm) * (long long)((d.Cout + tn - 1) / tn); };
     int bm = best <= 32 ? 256 : 128, bn = best;
     if (ctas_of(bm, bn) < sms) {

@@ -16,10 +16,9 @@
 
 #include <cstdlib>
 #include <cstring>
-#include <map>
-#include <mutex>
-#include <string>
+#include <memory>
 
+#include "plan_cache.h"
 #include "ptx_sm100.cuh"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
@@ -245,8 +244,7 @@ struct HeadKey {
     int v[8];
 };
 
-std::mutex g_head_mu;
-std::map<std::string, HeadPlan> g_head_plans;
+PlanCache<HeadKey, HeadPlan> g_head_plans(1024);
 
 int build_head_plan(const ConvDesc& d, float* logits, HeadPlan* plan)
 {
@@ -321,26 +319,14 @@ int launch_conv_avgpool_bf16(const ConvDesc& d, float* logits, cudaStream_t stre
     cudaGetDevice(&dev);
     const int v[8] = {d.N, d.Cin, d.H, d.W, d.Cout, d.relu | (d.params_static << 1) | (d.f16 << 2), dev, d.K | (d.S << 8) | (d.pad << 16)};
     std::memcpy(k.v, v, sizeof(v));
-    const std::string key(reinterpret_cast<const char*>(&k), sizeof(k));
-    HeadPlan plan;
-    bool have = false;
-    {
-        std::lock_guard<std::mutex> lock(g_head_mu);
-        auto it = g_head_plans.find(key);
-        if (it != g_head_plans.end()) { plan = it->second; have = true; }
-    }
-    if (!have) {
-        const int rc = build_head_plan(d, logits, &plan);
-        if (rc != SQN_OK) return rc;
-        std::lock_guard<std::mutex> lock(g_head_mu);
-        if (g_head_plans.size() > 1024) g_head_plans.clear();
-        g_head_plans[key] = plan;
-    }
+    std::shared_ptr<const HeadPlan> plan;
+    const int prc = g_head_plans.get(k, &plan, [&](HeadPlan* p) { return build_head_plan(d, logits, p); });
+    if (prc != SQN_OK) return prc;
     static const cudaError_t attr_rc =
         cudaFuncSetAttribute(conv_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM_LIMIT);
     if (attr_rc != cudaSuccess) return SQN_ERR_CUDA;
-    const cudaError_t rc = launch_chained(conv_head_kernel, dim3((unsigned)plan.grid), dim3(CH_THREADS), plan.smem, stream, plan.x,
-                                          plan.w, plan.p);
+    const cudaError_t rc = launch_chained(conv_head_kernel, dim3((unsigned)plan->grid), dim3(CH_THREADS), plan->smem, stream, plan->x,
+                                          plan->w, plan->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;

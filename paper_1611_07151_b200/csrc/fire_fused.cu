@@ -30,10 +30,9 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
-#include <map>
-#include <mutex>
-#include <string>
+#include <memory>
 
+#include "plan_cache.h"
 #include "ptx_sm100.cuh"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
@@ -930,8 +929,7 @@ struct FireKey {
     int v[12];
 };
 
-std::mutex g_fire_mu;
-std::map<std::string, FirePlan> g_fire_plans;
+PlanCache<FireKey, FirePlan> g_fire_plans(1024);
 
 int launch_fire(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, cudaStream_t stream)
 {
@@ -947,37 +945,25 @@ int launch_fire(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, cud
     k.b1 = d1.bias; k.b3 = d3.bias; k.out = d1.out;
     int dev = 0;
     cudaGetDevice(&dev);
-    const char* bv = std::getenv("SQN_FIRE_BAND");
-    const char* ev = std::getenv("SQN_FIRE_ESLOTS");
-    const char* cv = std::getenv("SQN_FIRE_CS");
-    const char* pv = std::getenv("SQN_FIRE_PATCHES");
-    const int band = (bv ? std::atoi(bv) : 0) + 1000 * (ev ? std::atoi(ev) : 0) + 100000 * (cv ? std::atoi(cv) : 0) + 1000000 * (pv ? std::atoi(pv) : 0);
+    int band = 0;                       // the tuning aids that were in force
+    if (tuning_env_present()) {
+        auto num = [](const char* name) { const char* v = std::getenv(name); return v ? std::atoi(v) : 0; };
+        band = num("SQN_FIRE_BAND") + 1000 * num("SQN_FIRE_ESLOTS") + 100000 * num("SQN_FIRE_CS") + 1000000 * num("SQN_FIRE_PATCHES");
+    }
     const int v[12] = {d1.N, dsq ? dsq->Cin : -1, d1.H, d1.W, d1.Cin, d1.Cout, d3.Cout, d1.out_c_total,
                        (dsq ? dsq->params_static : 0) | (d1.params_static << 1) | (d3.params_static << 2), dev, band, d1.f16};
     std::memcpy(k.v, v, sizeof(v));
-    const std::string key(reinterpret_cast<const char*>(&k), sizeof(k));
-    FirePlan plan;
-    bool have = false;
-    {
-        std::lock_guard<std::mutex> lock(g_fire_mu);
-        auto it = g_fire_plans.find(key);
-        if (it != g_fire_plans.end()) { plan = it->second; have = true; }
-    }
-    if (!have) {
-        const int rc = build_fire_plan(dsq, d1, d3, &plan);
-        if (rc != SQN_OK) return rc;
-        std::lock_guard<std::mutex> lock(g_fire_mu);
-        if (g_fire_plans.size() > 1024) g_fire_plans.clear();
-        g_fire_plans[key] = plan;
-    }
+    std::shared_ptr<const FirePlan> plan;
+    const int prc = g_fire_plans.get(k, &plan, [&](FirePlan* p) { return build_fire_plan(dsq, d1, d3, p); });
+    if (prc != SQN_OK) return prc;
     // (the 16-bit type is a compile-time constant of the kernel: the epilogues' conversion loops are straight-line code)
     static const cudaError_t attr_rc0 =
         cudaFuncSetAttribute(fire_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FF_SMEM_LIMIT);
     static const cudaError_t attr_rc1 =
         cudaFuncSetAttribute(fire_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FF_SMEM_LIMIT);
     if (attr_rc0 != cudaSuccess || attr_rc1 != cudaSuccess) return SQN_ERR_CUDA;
-    const cudaError_t rc = launch_chained(plan.p.f16 ? fire_fused_kernel<true> : fire_fused_kernel<false>, dim3((unsigned)plan.p.grid),
-                                          dim3(FF_THREADS), plan.smem, stream, plan.x, plan.wsq, plan.w3, plan.w1, plan.o, plan.p);
+    const cudaError_t rc = launch_chained(plan->p.f16 ? fire_fused_kernel<true> : fire_fused_kernel<false>, dim3((unsigned)plan->p.grid),
+                                          dim3(FF_THREADS), plan->smem, stream, plan->x, plan->wsq, plan->w3, plan->w1, plan->o, plan->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;

@@ -27,6 +27,9 @@ struct ConvDesc {
 // Launch counter (host side): every kernel launch goes through note_launch().
 void note_launch(int n = 1);
 
+// False when no variable of the environment starts with SQN_: none of the tuning aids need be asked for.
+bool tuning_env_present();
+
 // Device status word shared by all kernels (0 = fine, else an sqn_status).
 int* device_status_word();
 
