@@ -127,6 +127,37 @@ int make_conv_desc(const void* in, const void* w, const void* bias, void* out, i
 
 inline bool is_stem_shape(const ConvDesc& d) { return d.K == 7 && d.S == 2 && d.pad == 0 && d.Cin == 3; }
 
+// A single 16-bit layer on the small-layer kernel?  Where its estimate is below that of a tcgen05 kernel with no more tiles than
+// SMs, 3.6 us and 5 ns per reduction element (one image of a bottleneck's 512 -> 512 3x3 layer at 7 x 7: 10.7 us against 26.4;
+// 256 -> 256 at 14 x 14: 6.6 against 15.3; 512 -> 1000 1x1 at 13 x 13: 4.8 against 8.5; five images of 128 -> 128 at 28 x 28 stay).
+// Layers that the pooled kernels take as well (up to 128 output layers, in groups of 32) keep the kernels whose sums add up
+// in the same order with and without a pool.
+bool small_conv(const ConvDesc& d)
+{
+    if (d.pool || (d.Cout <= 128 && d.Cout % 32 == 0)) return false;
+    return mma_small_estimate(&d, 1) < 3.6f + 0.005f * d.K * d.K * d.Cin && !(tuning_env_present() && std::getenv("SQN_TC_VARIANT"));
+}
+
+// A fire layer on the small-layer kernel, the squeeze and then both expands in one launch?  Estimates of the other paths with no
+// more tiles than SMs, K the reduction of both steps: 6.5 + 0.008 K us in one kernel (fire2 to fire5 at one image: 8.3 to
+// 10.8 us, here 5.7 to 8.8; at two images fire2 is 8.7 there and 9.1 here), else 10 + 0.0045 K us (fire6 to fire9 at one
+// image: 13.8 to 14.5 us, here 6.4 to 8.4; fire9 at eight images 15.3 and 11.5, fire8 at four 15.2 and 15.4).
+bool small_fire(const ConvDesc& dsq, const ConvDesc& d1, const ConvDesc& d3, bool fuses)
+{
+    const float k = (float)dsq.Cin + 9.f * d3.Cin, other = fuses ? 6.5f + 0.008f * k : 10.f + 0.0045f * k;
+    const float sq = mma_small_estimate(&dsq, 1);
+    if (sq >= other) return false;
+    const ConvDesc two[2] = {d3, d1};
+    return sq + mma_small_estimate(two, 2) < other;
+}
+
+// (the 3x3 expand first: its tiles take longer)
+int launch_small_expands(const ConvDesc& d1, const ConvDesc& d3, cudaStream_t stream)
+{
+    const ConvDesc two[2] = {d3, d1};
+    return launch_conv_mma_small(two, 2, stream);
+}
+
 int run_conv(const ConvDesc& d_in, int dtype, void* ws, size_t ws_bytes, cudaStream_t stream)
 {
     if (dtype == SQN_F32) return d_in.pool ? SQN_ERR_UNSUPPORTED : launch_conv_f32(d_in, stream);
@@ -198,6 +229,11 @@ extern "C" int conv_forward_ex(const void* in, const void* weights, const void* 
         if (d.OH < 3 || d.OW < 3) return SQN_ERR_BADARG;
         d.pool = 1;
     }
+    if (is16(o.dtype) && !is_stem_shape(d) && conv_bf16_supported(d) == SQN_OK && small_conv(d)) {
+        d.f16 = o.dtype == SQN_F16 ? 1 : 0;
+        const int src = launch_conv_mma_small(&d, 1, static_cast<cudaStream_t>(o.stream));
+        if (src != SQN_ERR_UNSUPPORTED) return src;
+    }
     return run_conv(d, o.dtype, o.workspace, o.workspace_bytes, static_cast<cudaStream_t>(o.stream));
 }
 
@@ -243,6 +279,11 @@ extern "C" int fire_forward(const void* in, const void* w_sq, const void* b_sq, 
     if (is16(dtype) && fused_fire_enabled()) {
         rc = launch_fire_fused_bf16(dsq, d1, d3, st);       // one kernel, squeeze_scratch stays untouched
         if (rc != SQN_ERR_UNSUPPORTED) return rc;
+        if (small_fire(dsq, d1, d3, false)) {
+            rc = launch_conv_mma_small(&dsq, 1, st);
+            if (rc == SQN_OK) return launch_small_expands(d1, d3, st);
+            if (rc != SQN_ERR_UNSUPPORTED) return rc;
+        }
     }
     if ((rc = run_conv(dsq, dtype, nullptr, 0, st)) != SQN_OK) return rc;
     return run_expands(d1, d3, dtype, st, nullptr);
@@ -606,12 +647,20 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
         // the net's kernels and bias are not written by anything this forward enqueues
         dsq.params_static = d1.params_static = d3.params_static = 1;
         dsq.f16 = d1.f16 = d3.f16 = f16;
-        // bf16: squeeze and both expands as one kernel where it applies (no pool behind the layer)
+        // bf16: squeeze and both expands as one kernel where it applies (no pool behind the layer), or on the small-layer kernel
         if (is16(dt) && fused_fire_enabled() && !(f.pool_after && fuse_pools)) {
-            rc = launch_fire_fused_bf16(dsq, d1, d3, st);
+            const bool fuses = fire_fuses(dsq, d1, d3), small = small_fire(dsq, d1, d3, fuses);
+            if (small) {
+                rc = launch_conv_mma_small(&dsq, 1, st);
+                if (rc == SQN_OK) {
+                    mark(f.name, "_sq");
+                    rc = launch_small_expands(d1, d3, st);
+                }
+            } else rc = fuses ? launch_fire_fused_bf16(dsq, d1, d3, st) : SQN_ERR_UNSUPPORTED;
             if (rc == SQN_OK) {
-                net->fused_fire_mask |= 1u << i;
-                mark(f.name, "_fused");
+                // (a layer that the one kernel takes does not show its squeeze map at any batch)
+                if (fuses) net->fused_fire_mask |= 1u << i;
+                mark(f.name, small ? "_e1+e3" : "_fused");
                 cur = out;
                 if (f.pool_after) {
                     void* po = buf(net->i_pool[i]);

@@ -931,7 +931,7 @@ struct FireKey {
 
 PlanCache<FireKey, FirePlan> g_fire_plans(1024);
 
-int launch_fire(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, cudaStream_t stream)
+int fire_plan(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, std::shared_ptr<const FirePlan>* plan)
 {
     if (d1.K != 1 || d3.K != 3 || d3.pad != 1 || d1.S != 1 || d3.S != 1 || !d1.relu || !d3.relu || d1.pool || d3.pool ||
         d1.in != d3.in || d1.Cin != d3.Cin || d1.H != d3.H || d1.W != d3.W || d1.N != d3.N)
@@ -953,8 +953,13 @@ int launch_fire(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, cud
     const int v[12] = {d1.N, dsq ? dsq->Cin : -1, d1.H, d1.W, d1.Cin, d1.Cout, d3.Cout, d1.out_c_total,
                        (dsq ? dsq->params_static : 0) | (d1.params_static << 1) | (d3.params_static << 2), dev, band, d1.f16};
     std::memcpy(k.v, v, sizeof(v));
+    return g_fire_plans.get(k, plan, [&](FirePlan* p) { return build_fire_plan(dsq, d1, d3, p); });
+}
+
+int launch_fire(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, cudaStream_t stream)
+{
     std::shared_ptr<const FirePlan> plan;
-    const int prc = g_fire_plans.get(k, &plan, [&](FirePlan* p) { return build_fire_plan(dsq, d1, d3, p); });
+    const int prc = fire_plan(dsq, d1, d3, &plan);
     if (prc != SQN_OK) return prc;
     // (the 16-bit type is a compile-time constant of the kernel: the epilogues' conversion loops are straight-line code)
     static const cudaError_t attr_rc0 =
@@ -982,6 +987,12 @@ bool fused_fire_enabled()
 int launch_fire_fused_bf16(const ConvDesc& dsq, const ConvDesc& d1, const ConvDesc& d3, cudaStream_t stream)
 {
     return launch_fire(&dsq, d1, d3, stream);
+}
+
+bool fire_fuses(const ConvDesc& dsq, const ConvDesc& d1, const ConvDesc& d3)
+{
+    std::shared_ptr<const FirePlan> plan;
+    return fire_plan(&dsq, d1, d3, &plan) == SQN_OK;
 }
 
 // Both expands of a fire layer on a stored squeeze map in one launch of the same kernel (its expand pipeline alone, the

@@ -50,6 +50,10 @@ float f32_small_estimate(const ConvDesc& d);
 // Returns SQN_ERR_UNSUPPORTED for shapes outside its family.
 int conv_bf16_supported(const ConvDesc& d);
 int launch_conv_bf16(const ConvDesc& d, cudaStream_t stream);
+// n (1 or 2) small layers in one launch on the warp-level matrix instructions (SQN_ERR_UNSUPPORTED: sizes beyond its 32-bit
+// offsets), and its time in microseconds (1e30 where it does not apply).
+int launch_conv_mma_small(const ConvDesc* d, int n, cudaStream_t stream);
+float mma_small_estimate(const ConvDesc* d, int n);
 // Two independent layers in one launch (first `big`'s CTAs, then `small`'s); SQN_ERR_UNSUPPORTED if they share no
 // kernel variant.
 int launch_conv_bf16_pair(const ConvDesc& small, const ConvDesc& big, cudaStream_t stream);
@@ -71,6 +75,7 @@ inline int stem_packed_cols(int W) { return (W + 2) / 2 * 2; }
 // where that kernel does not apply.  SQN_FUSED_FIRE=0 in the environment turns it off.
 bool fused_fire_enabled();
 int launch_fire_fused_bf16(const ConvDesc& dsq, const ConvDesc& d1, const ConvDesc& d3, cudaStream_t stream);
+bool fire_fuses(const ConvDesc& dsq, const ConvDesc& d1, const ConvDesc& d3);   // true for the shapes that it takes
 // Both expands on a stored squeeze map with the same kernel's expand pipeline (SQN_ERR_UNSUPPORTED where it does not apply).
 int launch_fire_expands_bf16(const ConvDesc& d1, const ConvDesc& d3, cudaStream_t stream);
 
