@@ -2,10 +2,11 @@
 // CTA, warp-level matrix instructions (mma.sync m16n8k16, fp32 accumulation).
 //
 // A layer of one image is a few microseconds of latency, not work: the tcgen05 kernels spend them on tensor maps, TMEM,
-// barriers and hand-overs between roles (fire9 at one image, squeeze and both expands: 14.5 us there, 6.1 here; fire2 8.6, 6.1).  Here there is nothing to set up: every warp copies its own chunks of 32
-// reduction elements asynchronously into its own ring (16-byte pieces, rows of 80 bytes: no bank conflicts), waits for nobody
-// else, multiplies the whole 32 x 32 output tile by them, and the warps' partial sums are added once at the end, in a fixed
-// order, with bias and ReLU in fp32.  Two layers that read the same input (the expands of a fire layer) go out as one grid.
+// barriers and hand-overs between roles (fire9 at one image, squeeze and both expands: 14.5 us there, 6.1 here; fire2 8.6,
+// 6.1).  Here there is nothing to set up: every warp copies its own chunks of 32 reduction elements asynchronously into its
+// own ring (16-byte pieces, rows of 80 bytes: no bank conflicts), waits for nobody else, multiplies the whole 32 x 32 output
+// tile by them, and the warps' partial sums are added once at the end, in a fixed order, with bias and ReLU in fp32.  Two
+// layers that read the same input (the expands of a fire layer) go out as one grid.
 #include <cmath>
 #include <cstring>
 
@@ -35,22 +36,6 @@ struct MmaSmallParams {
     int n_tiles, blocks;
     int early;
 };
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-template <bool F16>
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    if (F16)
-        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-    else
-        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 template <bool F16, int SL, int ST>
 __device__ __forceinline__ void conv_mma_small_body(const MmaSmallParams& p, const int bid)
