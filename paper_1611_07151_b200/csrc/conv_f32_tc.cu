@@ -25,11 +25,12 @@
 //           once per tap, and a tap is an MMA whose descriptor starts that many rows further into the split patch
 //   BOX     anything else: the input window of a tile of bw x bh output pixels is staged in shared memory as it is (zeros
 //           outside the map), im2col rows are read from there through a table of offsets
-// What bounds it (ablations at batch 256): layers whose kernels stay on the SM, instruction issue (28 warps share four
-// schedulers, a chunk costs the splitting warps some 300 instructions); layers whose kernels are streamed (K*K*Cin of 288 and
-// more with 128 layers), the kernels' way from the L2: 16 KB per unit at the L2's 16 bytes per clock and SM are 1000 clocks,
-// its MMAs 770.  Against the FFMA kernel, batch 256: conv1 1054 us (2687), fire2's expand-3x3 235 (373), fire4's 394 (1296),
-// fire6's 293 (675), fire8's 363 (1237), conv10 353 (1256), fire8's squeeze 132 (234); the tensor pipe is busy 40 .. 55 %.
+// What bounds it (clock traces and ablations at batch 256): instructions.  28 warps in six roles run straight-line code that
+// does not stay in the schedulers' instruction caches, some six clocks per instruction and warp, so a unit costs what the
+// slowest role's instructions for it cost: the issuing warp 1300 clocks (its 12 MMAs: 830), the splitting groups 1000 to 1350,
+// the epilogue 1100; and once per tile 3200 to 4200 for bias, ReLU and stores, during which the two segment accumulators
+// cover two units.  Against the FFMA kernel, batch 256: conv1 1011 us (2687), fire2's expand-3x3 230 (373), fire4's 381
+// (1296), fire6's 294 (675), fire8's 345 (1237), conv10 315 (1256), fire8's squeeze 114 (234), fire4's expand-1x1 89 (204).
 // Warps (one persistent CTA per SM, all of its tiles in one column of output layers):
 //   0..7    two groups of four split pixels into bf16 planes, written as swizzled K-major operand tiles (FLAT, BOX: the
 //           groups take the chunks of 32 reduction elements in turn; PATCH: each takes half of the patch's rows)
@@ -94,6 +95,7 @@ struct F32TcParams {
     int chunks, ksteps_last;    // pixel chunks of a tile, MMA k-steps of the last one
     int seg;                    // (chunk, tap) units whose w0*x0 products are summed on the tensor core before they are added in registers
     int kres;                   // 1: at most FT_KSLOTS units: the kernels stay in TMEM
+    int tstore;                 // FLAT where vec_store holds and Cout is a multiple of 4: pixels per TMA store of the epilogue (0: no TMA)
     int vec_store;              // 1: output rows and this layer's slice are 16-byte aligned
     int early;                  // 1: kernels and bias may be read before the wait for the grid ahead
     int ra, sa, sb;             // slots: split pixels, pixel boxes, kernel boxes
@@ -118,8 +120,12 @@ struct F32TcShared {
     unsigned long long a_full[FT_MAX_RA], a_empty[FT_MAX_RA];
     unsigned long long sa_full[FT_MAX_SA], sa_empty[FT_MAX_SA];
     unsigned long long sb_full[FT_MAX_SB], sb_empty[FT_MAX_SB];
-    unsigned long long k_full[FT_KSLOTS], k_empty[FT_KSLOTS];
-    unsigned long long seg_full[2], seg_empty[2];
+    unsigned long long k_full[FT_KSLOTS];
+    // done[u % 4]: the MMAs of unit u of the CTA's sequence have finished.  One commit per unit serves the kernel groups (slot
+    // u % 2 is free), the pixel groups of FLAT and BOX (a chunk is a unit) and the epilogue (a segment ends with a unit): each
+    // waits for units in order and none can be passed by four units, so two phases are never confused.
+    unsigned long long done[4];
+    unsigned long long seg_empty[2];
     unsigned long long gx_empty;
     unsigned tmem_base;
     volatile int abort_flag;
@@ -221,7 +227,7 @@ __device__ __noinline__ float plain_dot(const F32TcParams& p, int m, int n)
 // with all modes and twice as much unrolled epilogue in one kernel they evicted one another from the instruction cache
 // (expand-3x3 of fire2 at batch 256: 413 us instead of 300 at the time).
 template <int MODE>
-__device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const CUtensorMap& tmW, const F32TcParams& p, const int bid)
+__device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const CUtensorMap& tmW, const CUtensorMap& tmO, const F32TcParams& p, const int bid)
 {
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -242,16 +248,15 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
         for (int s = 0; s < FT_MAX_RA; ++s) { mbar_init(smem_u32(&sh->a_full[s]), px_warps); mbar_init(smem_u32(&sh->a_empty[s]), 1); }
         for (int s = 0; s < FT_MAX_SA; ++s) { mbar_init(smem_u32(&sh->sa_full[s]), 1); mbar_init(smem_u32(&sh->sa_empty[s]), px_warps); }
         for (int s = 0; s < FT_MAX_SB; ++s) { mbar_init(smem_u32(&sh->sb_full[s]), 1); mbar_init(smem_u32(&sh->sb_empty[s]), 4); }
-        for (int s = 0; s < FT_KSLOTS; ++s) { mbar_init(smem_u32(&sh->k_full[s]), 4); mbar_init(smem_u32(&sh->k_empty[s]), 1); }
-        for (int a = 0; a < 2; ++a) {
-            mbar_init(smem_u32(&sh->seg_full[a]), 1);
-            mbar_init(smem_u32(&sh->seg_empty[a]), 2 * live_quads);
-        }
+        for (int s = 0; s < FT_KSLOTS; ++s) { mbar_init(smem_u32(&sh->k_full[s]), 4); }
+        for (int u = 0; u < 4; ++u) mbar_init(smem_u32(&sh->done[u]), 1);
+        for (int a = 0; a < 2; ++a) mbar_init(smem_u32(&sh->seg_empty[a]), 2 * live_quads);
         mbar_init(smem_u32(&sh->gx_empty), 2 * live_quads);
         sh->abort_flag = 0;
         fence_mbar_init();
         if (p.sa) prefetch_tensormap(&tmX);
         if (p.wsrc == FT_W_BOXES) prefetch_tensormap(&tmW);
+        if (MODE == FT_FLAT && p.tstore) prefetch_tensormap(&tmO);
     }
     if (warp == FT_W_MMA) {
         tmem_alloc(smem_u32(&sh->tmem_base), 512);
@@ -268,6 +273,10 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
     volatile int* abort_flag = &sh->abort_flag;
+    const uint32_t done = smem_u32(sh->done);
+    auto wait_done = [&](int u) {           // all lanes of a warp; units before the first have finished
+        return u < 0 || __all_sync(0xffffffffu, wait_bar(done + 8u * ((uint32_t)u & 3u), ((uint32_t)u >> 2) & 1u, abort_flag, p.status));
+    };
     // Global memory that the grid ahead may have written or may still read is touched after chain_wait() only.
 
     if (warp < FT_W_KER) {
@@ -311,14 +320,14 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
         } else if (MODE == FT_FLAT) {
             const int total = my_tiles * p.chunks;
             int s = grp, st = grp;
-            uint32_t ph = 0, sph = 0;
+            uint32_t sph = 0;
             for (int a = grp; a < total; a += 2) {
                 if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&sh->sa_full[st]), sph, abort_flag, p.status))) break;
                 const uint32_t src = base + p.off_sa + (uint32_t)st * p.stage_a + (uint32_t)r0 * 128u + (uint32_t)q * 16u;
                 float4 v[FT_NA];
 #pragma unroll
                 for (int j = 0; j < FT_NA; ++j) v[j] = ld_shared_v4(src + (uint32_t)(16 * 128 * j));
-                if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&sh->a_empty[s]), ph ^ 1u, abort_flag, p.status))) break;
+                if (!wait_done(a - p.ra)) break;
                 const uint32_t slot = base + (uint32_t)s * p.slot_a + my_quad;
 #pragma unroll
                 for (int j = 0; j < FT_NA; ++j) store_split(slot + (uint32_t)(16 * j * FT_ROW), p.plane_a, v[j]);
@@ -329,7 +338,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                     mbar_arrive(smem_u32(&sh->sa_empty[st]));
                 }
                 s += 2;
-                if (s >= p.ra) { s -= p.ra; ph ^= 1u; }
+                if (s >= p.ra) s -= p.ra;
                 st += 2;
                 if (st >= p.sa) { st -= p.sa; sph ^= 1u; }
             }
@@ -379,7 +388,6 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             if (steps > 0) fill(0);
             bool ok = true;                             // (a group that gives up still takes part in the barriers)
             int a = 0, s = 0;                           // chunk of the CTA's sequence, its slot
-            uint32_t ph = 0;
             for (int step = 0; step < steps; ++step) {
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
                 bar_sync(1, 2 * FT_GT);                 // box filled by all; all have read the box of the step before
@@ -401,7 +409,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                                 v[j] = make_float4(ld_shared_f32(o0 + rowoff[j]), ld_shared_f32(o1 + rowoff[j]), ld_shared_f32(o2 + rowoff[j]),
                                                    ld_shared_f32(o3 + rowoff[j]));
                         }
-                        ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->a_empty[s]), ph ^ 1u, abort_flag, p.status));
+                        ok = wait_done(a - p.ra);
                         if (ok) {
                             const uint32_t slot = base + (uint32_t)s * p.slot_a + my_quad;
 #pragma unroll
@@ -411,7 +419,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                             if (lane == 0) mbar_arrive(smem_u32(&sh->a_full[s]));
                         }
                     }
-                    if (++s == p.ra) { s = 0; ph ^= 1u; }
+                    if (++s == p.ra) s = 0;
                 }
             }
         }
@@ -478,7 +486,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
         bool ok = true;
         const bool idle = p.wsrc == FT_W_PACKED && quad * 32 >= p.wrows;                          // no rows to give: whatever is in these lanes of TMEM is never read
         int st = grp, unit = grp % units, sl = 0;       // box slot, unit of the tile
-        uint32_t kph = 0, sph = 0;
+        uint32_t sph = 0;
         if (p.sb && st >= p.sb) { st -= p.sb; sph ^= 1u; }
         for (int u = grp; u < total; u += 2) {
             uint32_t h[16], m[16], l[16];
@@ -521,7 +529,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                     while (st >= p.sb) { st -= p.sb; sph ^= 1u; }
                 }
             }
-            if (ok) ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->k_empty[grp]), kph ^ 1u, abort_flag, p.status));
+            if (ok) ok = wait_done(u - FT_KSLOTS);
             if (ok) {
                 tc_fence_after();
                 if (idle) {
@@ -539,7 +547,6 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&sh->k_full[grp]));
             } else if (MODE != FT_BOX || p.wsrc != FT_W_COPIES) break;      // (with the copies the warps meet at a barrier in every turn)
-            kph ^= 1u;
             unit = next_unit;
         }
         if (MODE == FT_BOX) asm volatile("cp.async.wait_all;" ::: "memory");
@@ -553,23 +560,18 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
         const int wl = n_live - quad * 32 < 32 ? n_live - quad * 32 : 32;       // output layers of this warp
         const bool vec = p.vec_store && wl % 4 == 0;
         float* out_w = p.out + p.out_c_offset + nw;
-        const uint32_t stg = base + p.off_epi + (uint32_t)(warp - FT_W_EPI) * 2048u;
+        const uint32_t stg0 = base + p.off_epi + (uint32_t)(quad * 2 + half) * (MODE == FT_FLAT && p.tstore ? (uint32_t)p.tstore * 128u : 2048u);
         if (!p.early) chain_wait();
-        auto bias_of = [&](int e) { return 4 * (lane & 7) + e < wl ? __ldg(p.bias + nw + 4 * (lane & 7) + e) : 0.f; };
-        const float4 bias4 = make_float4(bias_of(0), bias_of(1), bias_of(2), bias_of(3));
+        const float bias = lane < wl ? __ldg(p.bias + nw + lane) : 0.f;
+        const float least = p.relu ? 0.f : -INFINITY;
         // 16 staged pixels -> memory; lane l of mc has the output pixel of staged row l - first
-        float nan = 0.f;                                // 0 as long as all outputs are finite
-        auto copy_out = [&](int mc, int first) {
+        auto copy_out = [&](uint32_t stg, int mc, int first) {
             const int l4 = 4 * (lane & 7);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
+                const float4 v = ld_shared_v4(stg + (uint32_t)(512 * i + 16 * lane));
                 int m = __shfl_sync(0xffffffffu, mc, first + 4 * i + (lane >> 3));
-                float4 v = ld_shared_v4(stg + (uint32_t)(512 * i + 16 * lane));
                 if (l4 >= wl || !sqn_dbg_ok(m < p.M && p.out_c_offset + nw + l4 < p.out_c_total, p.status)) m = -1;
-                const float z = fmaf(v.x, 0.f, v.y * 0.f) + fmaf(v.z, 0.f, v.w * 0.f);
-                if (m >= 0) nan += z;
-                v.x += bias4.x; v.y += bias4.y; v.z += bias4.z; v.w += bias4.w;
-                if (p.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
                 float* dst = out_w + (size_t)m * p.out_c_total + l4;
                 if (vec) {
                     if (m >= 0) *reinterpret_cast<float4*>(dst) = v;
@@ -598,9 +600,9 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             return tile * FT_N + c < p.M ? tile * FT_N + c : -1;
         };
         bool ok = quad < live_quads;                    // (warps without output layers are not counted by the barriers)
-        int b = 0;
-        uint32_t bph = 0;
-        for (int t = 0; t < my_tiles && ok; ++t) {
+        int b = 0, first_unit = 0;
+        const int units = p.chunks * p.taps;
+        for (int t = 0; t < my_tiles && ok; ++t, first_unit += units) {
             float acc[64];
             // output pixels of columns lane and lane + 32 of this warp's half
             const int mc0 = pixel_of(mt0 + t * p.m_step, half * 64 + lane), mc1 = pixel_of(mt0 + t * p.m_step, half * 64 + 32 + lane);
@@ -610,7 +612,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             for (int i = 0; i <= nseg; ++i) {
                 const bool corr = i == nseg - 1;
                 if (i < nseg) {
-                    ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->seg_full[b]), bph, abort_flag, p.status));
+                    ok = wait_done(first_unit + (corr ? units : (i + 1) * p.seg) - 1);
                     if (!ok) break;
                     tc_fence_after();
                 }
@@ -627,22 +629,44 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(corr ? &sh->gx_empty : &sh->seg_empty[b]));
-                if (!corr) { if (++b == 2) { b = 0; bph ^= 1u; } }
+                if (!corr) b ^= 1;
             }
             if (!ok) break;
-            // 16 pixels at a time through a staging tile (a pixel's 32 layers are a row), then in a short loop of 16-byte
-            // pieces, eight lanes per pixel, to memory
+            // bias and ReLU here, where a thread has one layer and 64 independent pixels, then 16 pixels at a time through a
+            // staging tile (a pixel's 32 layers are a row) and in 16-byte pieces, eight lanes per pixel, to memory; FLAT, whose
+            // pixels are consecutive: 32 or 64 pixels, then a TMA store.  Only two warps per 32 layers have rows to store, so
+            // the length of this chain is a tile's time where the reduction is short (fire2's 1x1 expand at batch 256 with
+            // bias and ReLU after the staging tile and no TMA 107 us, so 80; a bulk copy per pixel instead of the 16-byte
+            // pieces: fire2's expand-3x3 310 us instead of 230, conv1 1358 instead of 1011)
+            float nan = 0.f;                            // 0 as long as all outputs are finite
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 16) {
+                // (TMA: a staging tile of 32 or 64 pixels, free again when the store before has read it)
+                const uint32_t stg = stg0 + (MODE == FT_FLAT && p.tstore ? (uint32_t)(c0 & (p.tstore - 1)) * 128u : 0u);
+                if (MODE == FT_FLAT && lane == 0 && p.tstore && (c0 & (p.tstore - 1)) == 0) tma_store_wait_read();
                 __syncwarp();
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(stg + (uint32_t)(128 * j + 4 * lane)), "f"(acc[c0 + j]) : "memory");
-                __syncwarp();
-                copy_out(c0 & 32 ? mc1 : mc0, c0 & 16);
+                for (int j = 0; j < 16; ++j) {
+                    nan = fmaf(acc[c0 + j], 0.f, nan);
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(stg + (uint32_t)(128 * j + 4 * lane)), "f"(fmaxf(acc[c0 + j] + bias, least)) : "memory");
+                }
+                if (MODE == FT_FLAT && p.tstore) {
+                    if (((c0 + 16) & (p.tstore - 1)) == 0) {
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            const int m = (mt0 + t * p.m_step) * FT_N + half * 64 + c0 + 16 - p.tstore;
+                            if (m < p.M) tma_store_2d(&tmO, stg0, nw, m);
+                            tma_store_commit();
+                        }
+                    }
+                } else {
+                    __syncwarp();
+                    copy_out(stg, c0 & 32 ? mc1 : mc0, c0 & 16);
+                }
             }
-            if (__any_sync(0xffffffffu, nan != 0.f)) {  // something was not finite: this warp's outputs with fp32 multiply-adds
-                nan = 0.f;
+            if (__any_sync(0xffffffffu, lane < wl && nan != 0.f)) {      // something was not finite: this warp's outputs with fp32 multiply-adds
+                if (MODE == FT_FLAT && p.tstore && lane == 0) tma_store_wait_all();
                 __syncwarp();
                 for (int c = 0; c < 64; ++c) {
                     const int m = pixel_of(mt0 + t * p.m_step, half * 64 + c);
@@ -652,76 +676,90 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                 }
             }
         }
+        if (MODE == FT_FLAT && p.tstore && lane == 0) tma_store_wait_all();
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");       // (of 28 x 32 x 72 registers: 104 for the epilogue, 64 for the groups that split)
         if (warp == FT_W_MMA) {
             // -------------------------------------------------------------------- MMA issuer
+            // This warp's own instructions are what a unit takes at least (a barrier that is ready cost 150 to 350 clocks, a commit
+            // 120, in all 1800 clocks a unit against 830 of MMAs): so the barriers of a unit are tried together, and one
+            // commit serves all who wait for it.
             const uint32_t hi = (uint32_t)(make_kmajor_desc(0, FT_ROW, 8 * FT_ROW) >> 32);
             const uint32_t idesc = make_idesc_bf16(128, FT_N);
             const uint32_t PX = p.plane_a >> 4;             // plane pitch in 16-byte units
             auto desc = [&](uint32_t a16) { return ((uint64_t)hi << 32) | (uint64_t)(a16 | 0x10000u); };
-            bool ok = true;
-            const int units = p.chunks * p.taps;
-            int s = 0, ks = 0, b = 0;
-            uint32_t ph = 0, kph = 0, bph = 0, gph = 1;
+            const uint32_t a_full = smem_u32(sh->a_full), k_full = smem_u32(sh->k_full), seg_empty = smem_u32(sh->seg_empty);
             const uint32_t gx = tmem_base + FT_COL_GX;
+            const int units = p.chunks * p.taps, seg = p.seg;
+            bool ok = true;
+            uint32_t s = 0, ks = 0, b = 0, g = 0;
+            uint32_t ph = 0, kph = 0, bph = 1, gph = 1;
             for (int t = 0; t < my_tiles && ok; ++t) {
                 int in_seg = 0, u = 0;
                 for (int ch = 0; ch < p.chunks && ok; ++ch) {
-                    ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->a_full[s]), ph, abort_flag, p.status));
-                    if (!ok) break;
-                    const uint32_t slot = (base + (uint32_t)s * p.slot_a) >> 4;
-                    const int steps = ch == p.chunks - 1 ? p.ksteps_last : 2;
-                    int tap_row = 0, kw = 0;                // row of the patch the tap starts at
-                    for (int tap = 0; tap < p.taps; ++tap, ++u) {
-                        if (in_seg == 0) ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->seg_empty[b]), bph ^ 1u, abort_flag, p.status));
-                        if (!ok) break;
-                        if (!p.kres || t == 0) ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->k_full[ks]), kph, abort_flag, p.status));
-                        if (!ok) break;
-                        tc_fence_after();
-                        const bool seg_end = u == units - 1 || in_seg == p.seg - 1;
-                        const uint32_t g0 = tmem_base + (uint32_t)(b * FT_N);
-                        const uint64_t d0 = desc(slot + (uint32_t)tap_row * (FT_ROW >> 4)), d1 = d0 + PX, d2 = d1 + PX;      // the planes
-                        const uint32_t w = tmem_base + FT_COL_W + (uint32_t)ks * FT_W_COLS;
-                        if (elect_one()) {
-                            mma_bf16_ts(g0, w, d0, idesc, in_seg ? 1u : 0u);
-                            if (steps == 2) mma_bf16_ts(g0, w + 8u, d0 + 2u, idesc, 1u);
+                    uint32_t lo = (base + s * p.slot_a) >> 4;
+                    const bool two = ch != p.chunks - 1 || p.ksteps_last == 2;
+                    int kw = 0;
+                    for (int tap = 0; tap < p.taps; ++tap, ++u, ++g) {
+                        const uint32_t af = a_full + 8u * s, se = seg_empty + 8u * b, kf = k_full + 8u * ks;
+                        const bool need_a = tap == 0, need_s = in_seg == 0, need_k = !p.kres || t == 0;
+                        bool ready = !need_a || mbar_try_wait(af, ph);
+                        ready &= !need_s || mbar_try_wait(se, bph);
+                        ready &= !need_k || mbar_try_wait(kf, kph);
+                        if (!__all_sync(0xffffffffu, ready)) {
+                            ok = !need_a || wait_bar(af, ph, abort_flag, p.status);
+                            ok = ok && (!need_s || wait_bar(se, bph, abort_flag, p.status));
+                            ok = __all_sync(0xffffffffu, ok && (!need_k || wait_bar(kf, kph, abort_flag, p.status)));
+                            if (!ok) break;
                         }
-                        __syncwarp();
-                        if (u == 0) {                       // the corrections of the tile before have been read
+                        tc_fence_after();
+                        const uint32_t g0 = tmem_base + b * FT_N, w = tmem_base + FT_COL_W + ks * FT_W_COLS;
+                        const uint64_t d0 = desc(lo), d1 = d0 + PX, d2 = d1 + PX;       // the planes
+                        const bool seg_end = u == units - 1 || in_seg == seg - 1;
+                        if (u == 0) {                       // the corrections of the tile before have to be read first
+                            if (elect_one()) {
+                                mma_bf16_ts(g0, w, d0, idesc, 0u);
+                                if (two) mma_bf16_ts(g0, w + 8u, d0 + 2u, idesc, 1u);
+                            }
+                            __syncwarp();
                             ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->gx_empty), gph, abort_flag, p.status));
                             gph ^= 1u;
                             if (!ok) break;
                             tc_fence_after();
                         }
                         if (elect_one()) {
+                            if (u) {
+                                mma_bf16_ts(g0, w, d0, idesc, in_seg ? 1u : 0u);
+                                if (two) mma_bf16_ts(g0, w + 8u, d0 + 2u, idesc, 1u);
+                            }
                             mma_bf16_ts(gx, w, d1, idesc, u ? 1u : 0u);             // w0 x1
                             mma_bf16_ts(gx, w, d2, idesc, 1u);                      // w0 x2
                             mma_bf16_ts(gx, w + 16u, d0, idesc, 1u);                // w1 x0
                             mma_bf16_ts(gx, w + 16u, d1, idesc, 1u);                // w1 x1
                             mma_bf16_ts(gx, w + 32u, d0, idesc, 1u);                // w2 x0
-                            if (steps == 2) {
+                            if (two) {
                                 mma_bf16_ts(gx, w + 8u, d1 + 2u, idesc, 1u);
                                 mma_bf16_ts(gx, w + 8u, d2 + 2u, idesc, 1u);
                                 mma_bf16_ts(gx, w + 24u, d0 + 2u, idesc, 1u);
                                 mma_bf16_ts(gx, w + 24u, d1 + 2u, idesc, 1u);
                                 mma_bf16_ts(gx, w + 40u, d0 + 2u, idesc, 1u);
                             }
-                            if (!p.kres) mma_commit(smem_u32(&sh->k_empty[ks]));
-                            if (tap == p.taps - 1) mma_commit(smem_u32(&sh->a_empty[s]));
-                            if (seg_end) mma_commit(smem_u32(&sh->seg_full[b]));
+                            mma_commit(done + 8u * (g & 3u));
+                            if (MODE == FT_PATCH && tap == p.taps - 1) mma_commit(smem_u32(&sh->a_empty[s]));
                         }
                         __syncwarp();
-                        if (p.kres) { if (++ks == units) ks = 0; }       // (unit u of a tile stays in slot u)
-                        else if (++ks == FT_KSLOTS) { ks = 0; kph ^= 1u; }
+                        if (p.kres) { if (++ks == (uint32_t)units) ks = 0; }    // (unit u of a tile stays in slot u)
+                        else { ks ^= 1u; kph ^= ks ^ 1u; }
                         if (seg_end) {
                             in_seg = 0;
-                            if (++b == 2) { b = 0; bph ^= 1u; }
+                            b ^= 1u; bph ^= b ^ 1u;
                         } else ++in_seg;
-                        ++tap_row;
-                        if (++kw == p.K) { kw = 0; tap_row += p.P - p.K; }
+                        if (MODE == FT_PATCH) {             // the next tap starts a row of the patch further, a kernel row P rows
+                            lo += FT_ROW >> 4;
+                            if (++kw == p.K) { kw = 0; lo += (uint32_t)(p.P - p.K) * (FT_ROW >> 4); }
+                        }
                     }
-                    if (++s == p.ra) { s = 0; ph ^= 1u; }
+                    if (++s == (uint32_t)p.ra) { s = 0; ph ^= 1u; }
                 }
             }
         } else if ((warp == FT_W_TMAX || warp == FT_W_TMAW) && lane == 0) {
@@ -803,14 +841,15 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
 
 template <int MODE>
 __global__ void __launch_bounds__(FT_THREADS, 1)
-conv_f32_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ F32TcParams p)
+conv_f32_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
+                   const __grid_constant__ CUtensorMap tmO, const __grid_constant__ F32TcParams p)
 {
-    conv_f32_tc_body<MODE>(tmX, tmW, p, (int)blockIdx.x);
+    conv_f32_tc_body<MODE>(tmX, tmW, tmO, p, (int)blockIdx.x);
 }
 
 // ------------------------------------------------------------------------------ host side
 struct F32TcPlan {
-    CUtensorMap x, w;
+    CUtensorMap x, w, o;
     F32TcParams p;
     size_t smem;
 };
@@ -846,7 +885,7 @@ size_t layout(F32TcParams& p)
         size_t cur = (size_t)p.ra * p.slot_a;
         p.off_sa = (unsigned)cur; cur += (size_t)p.sa * p.stage_a;
         p.off_sb = (unsigned)cur; cur += p.wsrc == FT_W_PACKED ? up1k((size_t)units * p.wrows * (p.khalf ? 96 : 192)) : (size_t)p.sb * 128 * 128;
-        p.off_epi = (unsigned)cur; cur += 8 * 2048;
+        p.off_epi = (unsigned)cur; cur += p.tstore ? (size_t)2 * ((p.n_step + 31) / 32) * p.tstore * 128 : 8 * 2048;
         p.off_tbl = (unsigned)cur; cur += tbl;
         p.off_ctl = (unsigned)cur; cur += 1024;
         if (cur + 1024 > FT_SMEM_LIMIT) continue;
@@ -899,6 +938,7 @@ int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
     if (vec && d.K == 1 && d.S == 1 && d.pad == 0) {
         p.mode = FT_FLAT;
         p.prow = FT_N;
+        p.tstore = !p.vec_store || d.Cout % 4 != 0 ? 0 : p.n_step <= 64 ? 64 : 32;      // (TMA writes whole 16-byte pieces)
         found = finish(d.Cin, M);
     } else if (vec && d.K > 1 && d.S == 1 && d.pad < d.K && p.P <= 256 && positions < 0x7fffffffLL - 2 * FT_N - (long long)d.K * (p.P + 1)) {
         p.mode = FT_PATCH;
@@ -908,6 +948,7 @@ int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
         found = finish(d.Cin, positions);
     }
     if (!found) {
+        p.tstore = 0;
         p.mode = FT_BOX;
         p.prow = FT_N;
         p.taps = 1;
@@ -964,6 +1005,12 @@ int encode_f32_maps(const ConvDesc& d, F32TcPlan* plan)
         const cuuint32_t box[5] = {FT_BK, (cuuint32_t)p.P, 1, 1, 1};
         if (!tmap_encode_f32(&plan->x, 5, d.in, dims, str, box, 0)) return SQN_ERR_CUDA;
     }
+    if (p.tstore) {
+        // this layer's slice of the output
+        const cuuint64_t dims[2] = {(cuuint64_t)d.Cout, (cuuint64_t)p.M}, str[1] = {(cuuint64_t)d.out_c_total * 4};
+        const cuuint32_t box[2] = {32, (cuuint32_t)p.tstore};
+        if (!tmap_encode_f32(&plan->o, 2, p.out + p.out_c_offset, dims, str, box, 0)) return SQN_ERR_CUDA;
+    }
     if (p.wsrc == FT_W_BOXES) {
         const cuuint64_t dims[2] = {(cuuint64_t)p.Kdim, (cuuint64_t)d.Cout}, str[1] = {(cuuint64_t)p.Kdim * 4};
         const cuuint32_t box[2] = {FT_BK, 128};
@@ -978,7 +1025,7 @@ cudaError_t launch_mode(const F32TcPlan& plan, cudaStream_t stream)
     static const cudaError_t attr_rc =
         cudaFuncSetAttribute(conv_f32_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FT_SMEM_LIMIT);
     if (attr_rc != cudaSuccess) return attr_rc;
-    return launch_chained(conv_f32_tc_kernel<MODE>, dim3((unsigned)plan.p.grid), dim3(FT_THREADS), plan.smem, stream, plan.x, plan.w, plan.p);
+    return launch_chained(conv_f32_tc_kernel<MODE>, dim3((unsigned)plan.p.grid), dim3(FT_THREADS), plan.smem, stream, plan.x, plan.w, plan.o, plan.p);
 }
 
 // Microseconds this kernel takes, fitted to SqueezeNet's layers at batch 1 .. 256 (within 25 %): start and end of a launch,

@@ -52,13 +52,14 @@ def test_tensor_core_kernel_within_rounding(shape):
     assert (np.abs(got.astype(np.float64) - exp) <= bound(x, w, b, S, pad, K, C)).all()
 
 
-@pytest.mark.parametrize("offset,total", [(8, 160), (3, 135)])     # 16-byte stores, 4-byte stores
-def test_tensor_core_kernel_writes_its_slice_only(offset, total):
-    x, w, b = synth.conv_layer_case(8, 12, 128, 128, 29, 3)
-    exp = ref.conv2d(x, w, b, S=1, pad=1, relu=True)
-    got = G.gpu_conv(x, w, b, 1, 1, True, F32, c_offset=offset, c_total=total, fill=-7.0)
-    assert (np.abs(got[:, offset:offset + 128].astype(np.float64) - exp) <= bound(x, w, b, 1, 1, 3, 128)).all()
-    assert (got[:, :offset] == -7.0).all() and (got[:, offset + 128:] == -7.0).all()
+@pytest.mark.parametrize("offset,total", [(8, 160), (3, 135)])     # 16-byte stores or TMA boxes, 4-byte stores
+@pytest.mark.parametrize("N,M,K", [(12, 128, 3), (40, 128, 1), (40, 62, 1)])
+def test_tensor_core_kernel_writes_its_slice_only(N, M, K, offset, total):
+    x, w, b = synth.conv_layer_case(8, N, 128, M, 29, K)
+    exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=True)
+    got = G.gpu_conv(x, w, b, 1, K // 2, True, F32, c_offset=offset, c_total=total, fill=-7.0)
+    assert (np.abs(got[:, offset:offset + M].astype(np.float64) - exp) <= bound(x, w, b, 1, K // 2, K, 128)).all()
+    assert (got[:, :offset] == -7.0).all() and (got[:, offset + M:] == -7.0).all()
 
 
 @pytest.mark.parametrize("K", [1, 3])
