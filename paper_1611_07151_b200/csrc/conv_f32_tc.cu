@@ -28,9 +28,9 @@
 // What bounds it (clock traces and ablations at batch 256): instructions.  28 warps in six roles run straight-line code that
 // does not stay in the schedulers' instruction caches, some six clocks per instruction and warp, so a unit costs what the
 // slowest role's instructions for it cost: the issuing warp 1300 clocks (its 12 MMAs: 830), the splitting groups 1000 to 1350,
-// the epilogue 1100; and once per tile 3200 to 4200 for bias, ReLU and stores, during which the two segment accumulators
-// cover two units.  Against the FFMA kernel, batch 256: conv1 1011 us (2687), fire2's expand-3x3 230 (373), fire4's 381
-// (1296), fire6's 294 (675), fire8's 345 (1237), conv10 315 (1256), fire8's squeeze 114 (234), fire4's expand-1x1 89 (204).
+// the epilogue 1000; and once per tile 3200 to 4200 for bias, ReLU and stores, during which the two segment accumulators
+// cover two units.  Against the FFMA kernel, batch 256: conv1 996 us (2687), fire2's expand-3x3 229 (373), fire4's 354
+// (1296), fire6's 292 (675), fire8's 311 (1237), conv10 281 (1256), fire8's squeeze 109 (234), fire4's expand-1x1 89 (204).
 // Warps (one persistent CTA per SM, all of its tiles in one column of output layers):
 //   0..7    two groups of four split pixels into bf16 planes, written as swizzled K-major operand tiles (FLAT, BOX: the
 //           groups take the chunks of 32 reduction elements in turn; PATCH: each takes half of the patch's rows)
@@ -133,15 +133,25 @@ struct F32TcShared {
 
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
+// Two fp32 differences (the bits of all operands), one instruction
+__device__ __forceinline__ void sub2(uint32_t ax, uint32_t ay, uint32_t bx, uint32_t by, uint32_t& dx, uint32_t& dy)
+{
+    asm("{\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%2, %3};\n\t"
+        "mov.b64 b, {%4, %5};\n\t"
+        "sub.rn.f32x2 a, a, b;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "=r"(dx), "=r"(dy) : "r"(ax), "r"(ay), "r"(bx), "r"(by));
+}
 // Two values as three packed bf16 pairs whose sums are the values (see the head of the file).
 __device__ __forceinline__ void split_pair(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l)
 {
     h = pack_x2(x, y, 0);
-    const float rx = x - __uint_as_float(h << 16), ry = y - __uint_as_float(h & 0xffff0000u);       // at most 16 significant bits
-    const uint32_t ux = __float_as_uint(rx), uy = __float_as_uint(ry);
-    m = __byte_perm(ux, uy, 0x7632);
-    const float sx = rx - __uint_as_float(ux & 0xffff0000u), sy = ry - __uint_as_float(uy & 0xffff0000u);      // at most 8
-    l = __byte_perm(__float_as_uint(sx), __float_as_uint(sy), 0x7632);
+    uint32_t rx, ry, sx, sy;
+    sub2(__float_as_uint(x), __float_as_uint(y), h << 16, h & 0xffff0000u, rx, ry);         // at most 16 significant bits
+    m = __byte_perm(rx, ry, 0x7632);
+    sub2(rx, ry, rx & 0xffff0000u, ry & 0xffff0000u, sx, sy);                               // at most 8
+    l = __byte_perm(sx, sy, 0x7632);
 }
 
 // Four consecutive reduction elements -> the three planes (plane pitch in bytes), at address a of the first
@@ -204,6 +214,19 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+
+// a + (a * c + b) for two fp32 numbers at a time, each operation rounded to nearest (half the instructions of the segments'
+// sums: batch 256, fire8's expand-3x3 342 -> 314 us, conv10 316 -> 284)
+__device__ __forceinline__ void add_cut2(float& ax, float& ay, uint64_t c, uint32_t bx, uint32_t by)
+{
+    asm("{\n\t.reg .b64 a, b, t;\n\t"
+        "mov.b64 a, {%0, %1};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "fma.rn.f32x2 t, a, %2, b;\n\t"
+        "add.rn.f32x2 a, a, t;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(ax), "+f"(ay) : "l"(c), "r"(bx), "r"(by));
 }
 
 // One output pixel m and layer n with fp32 multiply-adds in the order of the reduction index.
@@ -616,7 +639,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                     if (!ok) break;
                     tc_fence_after();
                 }
-                const float cut = corr ? FT_CUT : 0.f;      // (one copy of the unrolled code below: two of them spill)
+                const uint64_t cut = corr ? (uint64_t)__float_as_uint(FT_CUT) * 0x100000001ull : 0ull;      // (one copy of the unrolled code below: two of them spill)
                 const uint32_t src = ta + (corr ? FT_COL_GX : (uint32_t)(b * FT_N));
 #pragma unroll
                 for (int c = 0; c < 64; c += 16) {
@@ -624,7 +647,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                     tmem_ld_x16(src + c, v);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[c + j] += fmaf(acc[c + j], cut, __uint_as_float(v[j]));
+                    for (int j = 0; j < 16; j += 2) add_cut2(acc[c + j], acc[c + j + 1], cut, v[j], v[j + 1]);
                 }
                 tc_fence_before();
                 __syncwarp();
