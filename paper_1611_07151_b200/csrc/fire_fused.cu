@@ -697,9 +697,9 @@ int fire_layout(FireParams& p, int R, int patches, int BKc_in, size_t* smem_byte
     return *smem_bytes <= FF_SMEM_LIMIT ? 1 + stages : 0;
 }
 
-// Band heights to try, best first: SQN_FIRE_BAND in the environment (tuning aid, read at every call) names one;
-// else 14 rows for maps of 40 rows and more (four equal bands for 55 rows), 8 for 20 rows and more, else the whole
-// image; with so few images that this leaves SMs idle, one tile.  A band is a whole number of expand tiles.
+// Band heights to try, best first: SQN_FIRE_BAND in the environment (tuning aid, read at every call) names one; else by
+// the number of bands per CTA (see below), the table, and 14 rows for maps of 40 rows and more (four equal bands for 55
+// rows), 8 for 20 rows and more, else the whole image.  A band is a whole number of expand tiles.
 // Winners of the band-height sweep at batch 256 (`bench.py --kernel fireN` under SQN_FIRE_BAND = 4 ... 28), frozen per
 // layer shape: {H, Cin, s, e1 + e3, rows}.  Shapes not listed take the rule below.
 struct BandChoice { int H, Cin, s, e, R; };
@@ -709,7 +709,8 @@ const BandChoice kBandTable[] = {
     {27, 256, 32, 256, 16},     // fire5: 51.5 us (8 rows: 51.9, 12 rows: 59.7)
 };
 
-int band_candidates(int H, int RT, int N, int Cin, int s, int e, int* out)
+// jobs: of a tile of the fused layer, 0 for the expands on a stored map.
+int band_candidates(int H, int RT, int N, int Cin, int s, int e, int jobs, int* out)
 {
     int n = 0;
     auto add = [&](int R) {
@@ -723,12 +724,31 @@ int band_candidates(int H, int RT, int N, int Cin, int s, int e, int* out)
         const int r = std::atoi(v);
         if (r > 0) { add(r); return n; }
     }
-    // few images: bands of one tile, so that as many CTAs as possible have work (the layer is latency-bound then)
     const int pref = H >= 40 ? 14 : H >= 20 ? 8 : H;
-    if ((long long)N * ((H + pref - 1) / pref) < sm_count()) { add(RT); add(2 * RT); }
-    else
-        for (const BandChoice& c : kBandTable)
-            if (c.H == H && c.Cin == Cin && c.s == s && c.e == e) add(c.R);
+    int listed = 0;
+    for (const BandChoice& c : kBandTable)
+        if (c.H == H && c.Cin == Cin && c.s == s && c.e == e) listed = c.R;
+    auto rounds = [&](int R) { return ((long long)N * ((H + R - 1) / R) + sm_count() - 1) / sm_count(); };     // bands of the busiest CTA
+    if (jobs == 1 && rounds(listed ? listed : pref) <= 3) {
+        // A CTA's time is its bands' rows, half a row of hand-overs per band, and the first band's squeeze, which nothing
+        // hides.  fire2: 16 images, 4 rows (two bands a CTA) 13.4 us, 2 rows (four) 14.3, 14 rows (one band on half of the
+        // SMs) 17.2; 50 images, 4 rows (five bands) 22.1, 14 rows (two) 26.4; 110 images, 14 rows 33.5, 4 rows 36.9.
+        int best = RT;
+        double least = 1e30;
+        for (int R = RT; R <= 14; R += RT) {
+            const double cost = (double)rounds(R) * (R + 0.5) + (R + 2) * Cin / 480.0;
+            if (cost < least) { least = cost; best = R; }
+        }
+        add(best);
+    } else if (jobs == 2 && rounds(RT) <= 4) {
+        // Two jobs per tile: the expands are the longer part, and bands of one tile let them start first.  fire5, 50 images: 4
+        // rows (three bands a CTA) 20.0 us, 16 rows (one) 22.4; 110 images: 30.2 and 31.0, 8 rows 29.3.
+        add(RT);
+        add(2 * RT);
+    } else if ((long long)N * ((H + pref - 1) / pref) < sm_count()) {      // few images: as many CTAs as possible have work
+        add(RT);
+        add(2 * RT);
+    } else if (listed) add(listed);
     if (H >= 40) { add(14); add(8); }
     else if (H >= 20) { add(8); add(12); add(16); }
     else add(H);
@@ -810,7 +830,7 @@ int build_fire_plan(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3,
         // two patches with (if there is one) an input ring of 32 KB or more and three slots or more, else one patch
         // under the same condition, else whatever fits
         int cand[8];
-        const int nc = band_candidates(H, p.RT, N, Cin, s, e1 + e3, cand);
+        const int nc = band_candidates(H, p.RT, N, Cin, s, e1 + e3, dsq ? p.njobs : 0, cand);
         // (flat expands: a third patch first -- the box of band j + 2 can only be requested once band j's MMAs are
         // done, and with two patches the request's latency shows in the issuers' waits; SQN_FIRE_PATCHES=2 tuning aid)
         const char* pv = std::getenv("SQN_FIRE_PATCHES");
