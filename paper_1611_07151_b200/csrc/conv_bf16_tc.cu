@@ -105,7 +105,7 @@ struct TcParams {
     int PW_out, PH_out;              // pooled extents
     int pool_ctot;                   // layers per pixel of the pooled tensor
     __nv_bfloat16* pool_out;
-    int npix;                        // conv_pool_kernel: pixels per tile, 256 or 128
+    int npix;                        // conv_pool_kernel: pixels per tile, 256, 144 or 128
     int two_issuers;                 // ... 1 (no rider): warp 18 issues the odd tiles' MMAs (the ring then has an even number of slots)
     int f16;                         // 1: the 16-bit type is fp16, 0: bf16
     // conv_pool_kernel: a second layer, 1x1 on the same input with as many output layers, that rides on this layer's
@@ -642,16 +642,16 @@ constexpr int POOLT_RIDER_WARP = 18;           // issues the rider's MMAs (idle 
 __host__ __device__ constexpr int poolt_rows(int npix) { return npix / 8; }                 // output rows per tile
 __host__ __device__ constexpr int poolt_prows(int npix) { return (npix / 8 - 2) / 2; }      // pooled rows per strip
 
-// NPIX = 256 (8 x 32 pixels per tile, 15 pooled rows per strip) where the layer's kernels leave room for the larger
-// patches, else 128 (8 x 16 pixels, 7 pooled rows).
+// NPIX = 256 (8 x 32 pixels per tile, 15 pooled rows per strip), 144 (8 x 18, 8 rows) or 128 (8 x 16, 7 rows): see build_plan.
 // CTOT: the layers per pixel of the pooled tensor as a compile-time constant (0: read from the parameters) -- the
 // four stores of a pooled row then differ by immediate offsets.
 template <int NPIX, bool F16, int CTOT>
 __device__ __forceinline__ void conv_pool_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB2,
                                                const TcParams& p, const int bid)
 {
-    constexpr int PROWS = poolt_prows(NPIX);          // 15 or 7
+    constexpr int PROWS = poolt_prows(NPIX);          // 15, 8 or 7
     constexpr int PR = (PROWS + 3) / 4;               // pooled rows per epilogue group: 4 or 2
+    constexpr int ACC = NPIX == 144 ? 256 : NPIX;     // TMEM columns from one accumulator to the next
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -796,7 +796,7 @@ __device__ __forceinline__ void conv_pool_body(const CUtensorMap& tmA, const CUt
             ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->full[s]), ph, abort_flag, p.status));
             if (!ok) break;
             tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)(as * NPIX);
+            const uint32_t d_tmem = tmem_base + (uint32_t)(as * ACC);
             const uint32_t x_base = smA16 + (uint32_t)s * a_tile16;
             if (elect_one()) {
                 uint32_t acc = 0u;
@@ -838,7 +838,7 @@ __device__ __forceinline__ void conv_pool_body(const CUtensorMap& tmA, const CUt
                 ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->full[s]), ph, abort_flag, p.status));
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d2 = tmem_base + (uint32_t)(ar * NPIX);
+                const uint32_t d2 = tmem_base + (uint32_t)(ar * ACC);
                 const uint32_t x_base = smA16 + (uint32_t)s * a_tile16;
                 if (elect_one()) {
                     uint32_t acc = 0u;
@@ -858,7 +858,7 @@ __device__ __forceinline__ void conv_pool_body(const CUtensorMap& tmA, const CUt
         }
     } else if (warp < POOLT_RIDER_WARP) {
         // -------------------------------------------------------------------- epilogue: pool in registers
-        // group g = (warp - 2) / 4 takes the pooled rows PR*g .. PR*g + PR-1 of the strip (group 3: one fewer), i.e.
+        // group g = (warp - 2) / 4 takes the pooled rows PR*g .. PR*g + PR-1 of the strip (group 3: what is left), i.e.
         // the rows 2*PR*g .. 2*PR*g + 2*PR of the tile = accumulator columns 16*PR*g .. 16*PR*g + 16*PR + 7
         const int q = warp & 3, grp = (warp - 2) >> 2;
         const int m = q * 32 + lane;
@@ -880,7 +880,7 @@ __device__ __forceinline__ void conv_pool_body(const CUtensorMap& tmA, const CUt
             ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->tmem_full[as]), aph, abort_flag, p.status));
             if (!ok) return;
             tc_fence_after();
-            const uint32_t taddr = tmem_base + lane_base + (uint32_t)(as * NPIX) + (uint32_t)(grp * 16 * PR);
+            const uint32_t taddr = tmem_base + lane_base + (uint32_t)(as * ACC) + (uint32_t)(grp * 16 * PR);
             const int pw0 = tc.tw * 4 - 1, ph0 = tc.th * PROWS + grp * PR;
             unsigned short* dst0 = reinterpret_cast<unsigned short*>(p.pool_out) +
                                    (((size_t)tc.ti * p.PH_out + ph0) * p.PW_out + pw0) * ctot + c_off + m;
@@ -890,8 +890,8 @@ __device__ __forceinline__ void conv_pool_body(const CUtensorMap& tmA, const CUt
             // One pooled row per step: its three tile rows are the last row of the step before (still in registers) and
             // two new ones (16 accumulator columns).  The load of step r + 1 is issued before the maxima of step r are
             // taken, so that only the first load's latency is exposed; three buffers rotate (the step before, this one,
-            // the one in flight).  The last group has one pooled row -- one step -- fewer.
-            const int nsteps = grp == 3 ? PR - 1 : PR;
+            // the one in flight).  The last group may have one pooled row -- one step -- fewer.
+            const int nsteps = grp == 3 ? PROWS - 3 * PR : PR;
             uint32_t row0[8], buf[3][16];
             tmem_ld_x8(taddr, row0);
             tmem_ld_x16(taddr + 8u, buf[0]);
@@ -965,7 +965,7 @@ __device__ __forceinline__ void pool_body(const CUtensorMap& tmA, const CUtensor
 {
     if (p.f16) conv_pool_body<NPIX, true, 0>(tmA, tmB, tmB2, p, bid);
     else if (p.pool_ctot == 256) conv_pool_body<NPIX, false, 256>(tmA, tmB, tmB2, p, bid);
-    else if (NPIX == 256 && p.pool_ctot == 96) conv_pool_body<NPIX, false, 96>(tmA, tmB, tmB2, p, bid);
+    else if (p.pool_ctot == 96) conv_pool_body<NPIX, false, 96>(tmA, tmB, tmB2, p, bid);
     else if (NPIX == 128 && p.pool_ctot == 512) conv_pool_body<NPIX, false, 512>(tmA, tmB, tmB2, p, bid);
     else conv_pool_body<NPIX, false, 0>(tmA, tmB, tmB2, p, bid);
 }
@@ -975,6 +975,7 @@ conv_pool_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                  const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ TcParams p)
 {
     if (p.npix == 256) pool_body<256>(tmA, tmB, tmB2, p, (int)blockIdx.x);
+    else if (p.npix == 144) pool_body<144>(tmA, tmB, tmB2, p, (int)blockIdx.x);
     else pool_body<128>(tmA, tmB, tmB2, p, (int)blockIdx.x);
 }
 
@@ -1204,7 +1205,7 @@ int num_sms()
 // Shared-memory layout for one candidate (store chunk width, staging slots); returns the number
 // of A stages that fit (0 if the candidate does not fit at all).
 thread_local size_t t_smem_limit = SMEM_LIMIT;   // budget the layout search below works against
-thread_local int t_pool_npix = 256;              // conv_pool_kernel: pixels per tile the plan is built for (256 or 128)
+thread_local int t_pool_npix = 256;              // conv_pool_kernel: pixels per tile the plan is built for
 thread_local const ConvDesc* t_rider = nullptr;  // conv_pool_kernel: the 1x1 layer that rides on the plan's layer (see TcParams::rider)
 thread_local int t_force_cw = 0;                 // != 0: only layouts with this store chunk width (see launch_conv_bf16_pair)
 
@@ -1353,7 +1354,7 @@ int build_plan_cfg(const ConvDesc& d, bool stem, const void* a_ptr, const void* 
         // belong to whatever follows in shared memory
         p.npix = t_pool_npix;
         if (p.rider && p.npix != 128) return SQN_ERR_UNSUPPORTED;      // (three accumulators for the layer, one for the rider: 4 x 128 columns)
-        p.tmem_cols = (p.rider ? 4u : 2u) * (unsigned)p.npix;
+        p.tmem_cols = p.npix == 144 ? 512u : (p.rider ? 4u : 2u) * (unsigned)p.npix;
         p.b_tile = (unsigned)p.BN * row_bytes;
     }
 
@@ -1546,11 +1547,25 @@ int build_plan(const ConvDesc& d, bool stem, const void* a_ptr, const void* w_pt
         const TcParams& p = plan->p;
         if ((p.patch && p.BN <= 64) || (!p.patch && p.taps == 1 && p.stages >= 3)) return SQN_OK;
     }
-    if (d.pool) {       // the larger tiles where the layer's kernels leave room for their patches
-        t_pool_npix = 256;
-        int rc = build_plan_cfg(d, stem, a_ptr, w_ptr, Hp, Wp, 2, plan);
-        if (rc != SQN_OK) {
-            t_pool_npix = 128;
+    if (d.pool) {
+        // A CTA's time is its strips times a strip's rows (npix / 8) and some six rows of hand-overs per row of tiles.  Many
+        // images: the larger tiles; few: the size whose strips leave no CTA with one more than the others, or without one.  The
+        // stem, its repack and pool1, 256-pixel tiles against the size chosen here: 16 images 27.8 us, 21.8 with 128; 19 images
+        // 27.9, 21.9 with 144; 40 images 44.2, 33.5 with 144; 80 images 67.0, 58.6 with 144; 128 images 89.8, 92.1 with 128 (not
+        // chosen).  A size whose patches do not fit beside the layer's kernels is passed over.
+        const int ph = (d.OH - 3) / 2 + 1, sizes[3] = {256, 144, 128};
+        long long cost[3];
+        for (int i = 0; i < 3; ++i) {
+            const long long strips = (long long)d.N * ((ph + poolt_prows(sizes[i]) - 1) / poolt_prows(sizes[i]));
+            cost[i] = (strips + num_sms() - 1) / num_sms() * (sizes[i] + 48);
+        }
+        int rc = SQN_ERR_UNSUPPORTED;
+        for (int turn = 0; turn < 3 && rc != SQN_OK; ++turn) {
+            int best = 0;
+            for (int i = 1; i < 3; ++i)
+                if (cost[i] < cost[best]) best = i;
+            cost[best] = 0x7fffffffffffffffLL;
+            t_pool_npix = sizes[best];
             rc = build_plan_cfg(d, stem, a_ptr, w_ptr, Hp, Wp, 2, plan);
             t_pool_npix = 256;
         }
@@ -1733,7 +1748,7 @@ int launch_conv_bf16_pair(const ConvDesc& small, const ConvDesc& big, cudaStream
     if (rc != SQN_OK) return rc;
     rc = cached_plan(small, false, small.in, small.w, 0, 0, nullptr, &ps);
     if (rc != SQN_OK) return rc;
-    if (big.pool && ps->p.npix != pb->p.npix) {          // both with the smaller tiles
+    if (big.pool && (ps->p.npix != pb->p.npix || pb->p.npix == 144)) {       // both with the smallest tiles
         if (cached_plan(big, false, big.in, big.w, 0, 0, nullptr, &pb, 2, -128) != SQN_OK ||
             cached_plan(small, false, small.in, small.w, 0, 0, nullptr, &ps, 2, -128) != SQN_OK)
             return SQN_ERR_UNSUPPORTED;
