@@ -1340,15 +1340,17 @@ int build_plan_cfg(const ConvDesc& d, bool stem, const void* a_ptr, const void* 
     }
     const unsigned row_bytes = (unsigned)p.BKc * 2u;
 
-    p.BN = d.Cout <= 256 ? d.Cout : 256;
-    p.n_tiles = (d.Cout + p.BN - 1) / p.BN;
-    p.bn_pad = (p.BN + 31) / 32 * 32;
-    unsigned cols = 32;
-    while (cols < 2u * (unsigned)p.bn_pad) cols *= 2;
-    p.tmem_cols = cols;
-    if (halves == 1 && (cols > 256 || d.pool)) return SQN_ERR_UNSUPPORTED;   // two CTAs share the SM's 512 TMEM columns
-    p.b_tile = ((unsigned)p.BN * row_bytes + 1023u) / 1024u * 1024u;
-    p.b_bytes = (unsigned)p.BN * row_bytes;
+    auto set_width = [&](int bn) {              // output layers per tile
+        p.BN = bn;
+        p.n_tiles = (d.Cout + bn - 1) / bn;
+        p.bn_pad = (bn + 31) / 32 * 32;
+        p.tmem_cols = 32;
+        while (p.tmem_cols < 2u * (unsigned)p.bn_pad) p.tmem_cols *= 2;
+        p.b_tile = ((unsigned)bn * row_bytes + 1023u) / 1024u * 1024u;
+        p.b_bytes = (unsigned)bn * row_bytes;
+    };
+    set_width(d.Cout <= 256 ? d.Cout : 256);
+    if (halves == 1 && (p.tmem_cols > 256 || d.pool)) return SQN_ERR_UNSUPPORTED;   // two CTAs share the SM's 512 TMEM columns
     if (p.pool) {
         // conv_pool_kernel: the kernels are the M = 128 operand; their tiles hold Cout rows and the rows past them
         // belong to whatever follows in shared memory
@@ -1411,6 +1413,12 @@ int build_plan_cfg(const ConvDesc& d, bool stem, const void* a_ptr, const void* 
         if (flat) { p.BW = OW < TILE_M ? OW : TILE_M; p.BH = 1; p.BI = 1; }
         else choose_box(OW, OH, NI, &p.BW, &p.BH, &p.BI);
         p.a_bytes = (unsigned)(p.BW * p.BH * p.BI) * row_bytes;
+        // Few tiles: narrower ones, as long as they still are one wave of CTAs.  A CTA then streams half of the kernels and an MMA of
+        // half the layers takes half the time down to 64 layers (48 clocks; 256 layers 128).  17 images of a bottleneck's
+        // layers: 256 -> 256 3x3 at 14 x 14 16.1 -> 13.8 us, 512 -> 512 3x3 at 7 x 7 27.1 -> 22.5, 512 -> 2048 1x1 10.8 -> 7.7.
+        const long long px_tiles = (long long)((OW + p.BW - 1) / p.BW) * ((OH + p.BH - 1) / p.BH) * ((NI + p.BI - 1) / p.BI);
+        for (int bn = 128; bn >= 64; bn /= 2)
+            if (p.BN > bn && px_tiles * ((d.Cout + bn - 1) / bn) <= num_sms()) set_width(bn);
         const size_t a_tile = (size_t)TILE_M * row_bytes;
         if (!choose_layout(p, a_tile, true, 3, false, &plan->smem) && !choose_layout(p, a_tile, false, 3, false, &plan->smem) &&
             !choose_layout(p, a_tile, false, 2, false, &plan->smem))
