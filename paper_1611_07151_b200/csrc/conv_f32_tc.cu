@@ -586,7 +586,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
         const uint32_t stg0 = base + p.off_epi + (uint32_t)(quad * 2 + half) * (MODE == FT_FLAT && p.tstore ? (uint32_t)p.tstore * 128u : 2048u);
         if (!p.early) chain_wait();
         const float bias = lane < wl ? __ldg(p.bias + nw + lane) : 0.f;
-        const float least = p.relu ? 0.f : -INFINITY;
+        const float least = p.relu ? 0.f : bias != bias ? bias : -INFINITY;     // (fmaxf drops a NaN that only one operand has)
         // 16 staged pixels -> memory; lane l of mc has the output pixel of staged row l - first
         auto copy_out = [&](uint32_t stg, int mc, int first) {
             const int l4 = 4 * (lane & 7);

@@ -78,3 +78,17 @@ def test_exact_sums_stay_exact_and_infinities_come_through(K):
     with np.errstate(invalid="ignore"):
         exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=False)
     np.testing.assert_array_equal(G.gpu_conv(x, w, b, 1, K // 2, False, F32), exp)
+
+
+@pytest.mark.parametrize("relu", [True, False])
+def test_a_bias_that_is_not_finite(relu):
+    """The sum is finite, the bias is not: NaN stays NaN without ReLU and becomes 0 with it, as max(0, .) has it everywhere."""
+    x, w, b = synth.conv_layer_case(6, 32, 64, 128, 27, 1)
+    b[[7, 40, 100]] = np.nan, np.inf, -np.inf
+    exp = ref.conv2d(x, w, np.where(np.isfinite(b), b, 0).astype(np.float32), S=1, pad=0, relu=relu)
+    got = G.gpu_conv(x, w, b, 1, 0, relu, F32)
+    special = {7: 0.0 if relu else np.nan, 40: np.inf, 100: 0.0 if relu else -np.inf}
+    for m, v in special.items():
+        np.testing.assert_array_equal(got[:, m], np.full_like(got[:, m], v))
+    rest = np.isfinite(b)
+    assert (np.abs(got.astype(np.float64) - exp) <= bound(x, w, np.nan_to_num(b, posinf=0, neginf=0), 1, 0, 1, 64))[:, rest].all()
