@@ -92,3 +92,20 @@ def test_a_bias_that_is_not_finite(relu):
         np.testing.assert_array_equal(got[:, m], np.full_like(got[:, m], v))
     rest = np.isfinite(b)
     assert (np.abs(got.astype(np.float64) - exp) <= bound(x, w, np.nan_to_num(b, posinf=0, neginf=0), 1, 0, 1, 64))[:, rest].all()
+
+
+@pytest.mark.parametrize("ex,ew", [(-139, 120), (-130, 120), (120, -130), (124, -135), (-100, -20), (75, -60), (-60, 75), (113, -100), (60, 40)])
+@pytest.mark.parametrize("K", [1, 3])
+def test_operands_of_any_magnitude_keep_their_bits(K, ex, ew):
+    """Multiples of 2^-10 and 2^-14 times powers of two, subnormal numbers and ones that the scaled split cannot hold among
+    them: the outputs are those of the unscaled operands times the same power, within the same bound."""
+    x, w, b = synth.conv_layer_case(9, 20, 64, 128, 27, K)
+    x, w = np.round(x * 2 ** 10) / np.float32(2 ** 10), np.round(w * 2 ** 14) / np.float32(2 ** 14)
+    b[:] = 0
+    x[:, 3] *= -1
+    exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=False)
+    xs, ws = np.ldexp(x, ex), np.ldexp(w, ew)
+    assert (np.ldexp(xs.astype(np.float64), -ex) == x).all() and (np.ldexp(ws.astype(np.float64), -ew) == w).all()
+    got = np.ldexp(G.gpu_conv(xs, ws, b, 1, K // 2, False, F32).astype(np.float64), -ex - ew)
+    # (the last term: half a unit of the smallest fp32 output)
+    assert (np.abs(got - exp) <= bound(x, w, b, 1, K // 2, K, 64) + 2.0 ** (-150 - ex - ew)).all()
