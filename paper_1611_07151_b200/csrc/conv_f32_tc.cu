@@ -241,21 +241,77 @@ __device__ __forceinline__ void add_cut2(float& ax, float& ay, uint64_t c, uint3
         : "+f"(ax), "+f"(ay) : "l"(c), "r"(bx), "r"(by));
 }
 
-// One output pixel m and layer n with fp32 multiply-adds in the order of the reduction index.
-__device__ __noinline__ float plain_dot(const F32TcParams& p, int m, int n)
+// Called by an epilogue warp, lane l with output layer n = (the first one's) + l (also past the last one).  m < 0: the sum of the
+// absolute values of the layer's kernel.  Else output pixel m: as it is stored where the sums of the absolute values of its operands
+// (ws: the kernel's) bound every partial sum, else with fp32 multiply-adds.  All lanes work on one pixel, four layers at a time, so
+// that kernels are read in whole lines.  64 images of 128 -> 128 3x3 at 27 x 27 (90 us): with one infinity in all 513 us, in each image
+// 780, while every output of such a warp was computed again 10030 and 14380 us (the FFMA kernel: 384).  A mask of the outputs made in the
+// epilogue, a call with more in it, or this done behind the epilogue's loop or by other warps makes that loop spill: the stem of 256
+// images 8 to 11 % slower.
+__device__ __noinline__ float redo_output(const F32TcParams& p, int m, int n, float ws)
 {
-    const int img = fast_div(m, p.div_ohw), r = m - img * p.OHW;
-    const int oh = fast_div(r, p.div_ow), ow = r - oh * p.OW;
-    const float* w = p.w + (size_t)n * p.Kdim;
-    float acc = 0.f;
-    for (int kh = 0; kh < p.K; ++kh)
-        for (int kw = 0; kw < p.K; ++kw) {
-            const int ih = oh * p.S - p.pad + kh, iw = ow * p.S - p.pad + kw;
-            const bool in = (unsigned)ih < (unsigned)p.H && (unsigned)iw < (unsigned)p.W;
-            const float* x = p.in + (((size_t)img * p.H + (in ? ih : 0)) * p.W + (in ? iw : 0)) * p.Cin;
-            for (int c = 0; c < p.Cin; ++c) acc = fmaf(in ? __ldg(x + c) : 0.f, __ldg(w++), acc);
+    const int lane = threadIdx.x & 31, first = n - lane;
+    const int end = (first / p.n_step + 1) * p.n_step, left = (end < p.Cout ? end : p.Cout) - first;
+    auto warp_sum = [](float v) {
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) v += __shfl_xor_sync(0xffffffffu, v, h);
+        return v;
+    };
+    const int row_len = p.K * p.Cin, map_row = p.W * p.Cin;
+    float mine = 0.f;
+    unsigned mask = left < 32 ? (1u << left) - 1u : 0xffffffffu;
+    const float* x = p.in;
+    int ih0 = 0, col0 = 0;                              // first row of the window, its first column in elements
+    if (m >= 0) {
+        const int img = fast_div(m, p.div_ohw), r = m - img * p.OHW, oh = fast_div(r, p.div_ow);
+        ih0 = oh * p.S - p.pad; col0 = ((r - oh * p.OW) * p.S - p.pad) * p.Cin;
+        x += (size_t)img * p.H * map_row;
+        float xs = 0.f;
+        for (int kh = 0; kh < p.K; ++kh) {
+            if ((unsigned)(ih0 + kh) >= (unsigned)p.H) continue;
+            const float* row = x + (size_t)(ih0 + kh) * map_row;
+#pragma unroll 4
+            for (int f = col0 + lane; f < col0 + row_len; f += 32) xs += (unsigned)f < (unsigned)map_row ? fabsf(__ldg(row + f)) : 0.f;
         }
-    return acc;
+        __syncwarp();
+        xs = warp_sum(xs);
+        if (lane < left) mine = __ldcg(p.out + (size_t)m * p.out_c_total + p.out_c_offset + n);      // (not through the L1: TMA may have stored it)
+        mask &= __ballot_sync(0xffffffffu, !(xs < 0x1p111f && ws < 0x1p111f && xs * ws < 0x1p95f));
+    }
+    while (mask) {
+        int l[4];
+        float s[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            l[i] = mask ? __ffs(mask) - 1 : l[0];
+            mask &= mask - 1u;
+            s[i] = 0.f;
+        }
+        const float* w = p.w + (size_t)first * p.Kdim;
+        for (int kh = 0; kh < p.K; ++kh, w += row_len) {
+            const bool in = m >= 0 && (unsigned)(ih0 + kh) < (unsigned)p.H;
+            const float* row = x + (size_t)(in ? ih0 + kh : 0) * map_row + col0;
+#pragma unroll 2
+            for (int f = lane; f < row_len; f += 32) {
+                const float q = in && (unsigned)(col0 + f) < (unsigned)map_row ? __ldg(row + f) : 0.f;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float v = __ldg(w + (size_t)l[i] * p.Kdim + f);
+                    s[i] = m < 0 ? s[i] + fabsf(v) : fmaf(q, v, s[i]);
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float v = warp_sum(s[i]);
+            if (lane != l[i]) continue;
+            mine = v;
+            if (m >= 0) mine += __ldg(p.bias + n);
+            if (m >= 0 && p.relu) mine = fmaxf(mine, 0.f);
+        }
+    }
+    return mine;
 }
 
 // MODE is a compile-time constant so that a kernel's code stays small: six roles run different code at the same time, and
@@ -703,11 +759,13 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             if (__any_sync(0xffffffffu, lane < wl && nan != 0.f)) {      // something was not finite: this warp's outputs with fp32 multiply-adds
                 if (MODE == FT_FLAT && p.tstore && lane == 0) tma_store_wait_all();
                 __syncwarp();
-                for (int c = 0; c < 64; ++c) {
-                    const int m = pixel_of(mt0 + t * p.m_step, half * 64 + c);
-                    if (m < 0 || lane >= wl) continue;
-                    const float v = plain_dot(p, m, nw + lane) + __ldg(p.bias + nw + lane);
-                    out_w[(size_t)m * p.out_c_total + lane] = p.relu ? fmaxf(v, 0.f) : v;
+                float ws = 0.f;
+                for (int c = -1; c < 64; ++c) {
+                    const int m = c < 0 ? -1 : pixel_of(mt0 + t * p.m_step, half * 64 + c);
+                    if (m < 0 && c >= 0) continue;
+                    const float v = redo_output(p, m, nw + lane, ws);
+                    if (c < 0) ws = v;
+                    else if (lane < wl) out_w[(size_t)m * p.out_c_total + lane] = v;
                 }
             }
         }

@@ -109,3 +109,49 @@ def test_operands_of_any_magnitude_keep_their_bits(K, ex, ew):
     got = np.ldexp(G.gpu_conv(xs, ws, b, 1, K // 2, False, F32).astype(np.float64), -ex - ew)
     # (the last term: half a unit of the smallest fp32 output)
     assert (np.abs(got - exp) <= bound(x, w, b, 1, K // 2, K, 64) + 2.0 ** (-150 - ex - ew)).all()
+
+
+# (N, Cin, Cout, H, K, S, pad): a 1x1 layer with and without TMA stores, a patch, staged windows
+@pytest.mark.parametrize("shape", [(30, 300, 96, 27, 1, 1, 0), (30, 300, 70, 27, 1, 1, 0), (16, 130 * 2, 100, 20, 3, 1, 1),
+                                   (16, 64, 128, 56, 3, 2, 1)], ids=lambda s: "x".join(map(str, s)))
+def test_sums_that_are_not_finite(shape):
+    """Infinities and NaN in pixels and kernels, single ones and whole rows of them: outputs that they reach are those of
+    multiply-adds, all others stay within the bound; and one infinity per image costs a few times the finite layer (up to 12
+    measured), not a hundred times: only the outputs that it reaches are computed again."""
+    import torch
+    N, C, M, H, K, S, pad = shape
+    rng = np.random.default_rng(sum(shape))
+    x = rng.standard_normal((N, C, H, H)).astype(np.float32)
+    w, b = synth.draw_conv_params(rng, C, M, K)
+
+    def time_of(x):
+        xd, wd, bd = G.dev_act(x, F32), G.dev_w(w, F32), G.dev_b(b)
+        OH = (H + 2 * pad - K) // S + 1
+        out = B.empty_device((N, OH, OH, M), F32)
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        for i in range(6):
+            if i == 1:
+                ev[0].record()
+            B.conv_forward_ex(xd, wd, bd, out, C, M, H, H, K, S, pad, N, dtype=F32)
+        ev[1].record()
+        torch.cuda.synchronize()
+        return ev[0].elapsed_time(ev[1])
+
+    finite = time_of(x)
+    x[:, C // 2, H // 2, H // 2] = np.inf
+    assert time_of(x) < 40 * finite
+    x[0, 1, :, 3], x[1, :, 2, 2], x[2, 0, 5, :], x[3] = -np.inf, np.nan, np.float32(3e38), np.inf
+    # (the middle of the window: a padding zero times an infinity, which the oracle leaves out, does not occur)
+    w[M - 1, 3, K // 2, K // 2], w[5, C - 1, K // 2, K // 2] = np.inf, np.nan
+    with np.errstate(invalid="ignore", over="ignore"):
+        exp = ref.conv2d(x, w, b, S=S, pad=pad, relu=False)
+        got = G.gpu_conv(x, w, b, S, pad, False, F32)
+        # (3e38 times a kernel value: a sum that overflows or not by the order of its terms is left out)
+        unsure = np.isinf(ref.conv2d(np.abs(np.nan_to_num(x, nan=0, posinf=0, neginf=0)), np.abs(np.nan_to_num(w, nan=0, posinf=0)), np.abs(b),
+                                     S=S, pad=pad, relu=False))
+    fin = np.isfinite(exp)
+    np.testing.assert_array_equal(got[~fin & ~unsure], exp[~fin & ~unsure])
+    xf, wf = np.nan_to_num(x, nan=0, posinf=0, neginf=0), np.nan_to_num(w, nan=0, posinf=0)
+    ok = fin & ~unsure
+    # (outputs computed again are chains of K*K*C/32 multiply-adds and a tree of five: covered by the bound)
+    assert (np.abs(got[ok].astype(np.float64) - exp[ok]) <= bound(xf, wf, b, S, pad, K, C)[ok]).all()
