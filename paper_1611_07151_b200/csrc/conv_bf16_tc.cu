@@ -30,6 +30,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -39,6 +40,7 @@
 
 #include "plan_cache.h"
 #include "ptx_sm100.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
 #include "tc_host.h"
@@ -1190,13 +1192,12 @@ struct Plan {
 
 int num_sms()
 {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
+    static std::atomic<int> known[64];           // per device; 0: not asked yet
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+    if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+    if (dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
@@ -1585,10 +1586,9 @@ int build_plan(const ConvDesc& d, bool stem, const void* a_ptr, const void* w_pt
 template <int SPLIT, int HC>
 cudaError_t launch_variant(const Plan& plan, cudaStream_t stream)
 {
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(conv_tc_kernel<SPLIT, HC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT));
-    if (attr_rc != cudaSuccess) return attr_rc;
+    static SmemAttr attr;
+    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel<SPLIT, HC>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
+    if (arc != cudaSuccess) return arc;
     return launch_chained(conv_tc_kernel<SPLIT, HC>, dim3((unsigned)plan.grid), dim3(threads_for(SPLIT)), plan.smem,
                           stream, plan.a, plan.b, plan.o, plan.p);
 }
@@ -1598,11 +1598,11 @@ int launch_plan(const Plan& plan, cudaStream_t stream)
     cudaError_t rc;
     const int hc = plan.p.CW / 2;
     if (plan.p.pool) {
-        static const cudaError_t attr_rc =
-            cudaFuncSetAttribute(conv_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT);
-        rc = attr_rc != cudaSuccess ? attr_rc
-           : launch_chained(conv_pool_kernel, dim3((unsigned)plan.grid), dim3(POOLT_THREADS), plan.smem, stream, plan.a, plan.b, plan.r,
-                            plan.p);
+        static SmemAttr attr;
+        rc = attr.allow((const void*)conv_pool_kernel, SMEM_LIMIT);
+        if (rc == cudaSuccess)
+            rc = launch_chained(conv_pool_kernel, dim3((unsigned)plan.grid), dim3(POOLT_THREADS), plan.smem, stream, plan.a, plan.b, plan.r,
+                                plan.p);
     }
     else if (plan.split == 1)
         rc = hc == 32 ? launch_variant<1, 32>(plan, stream)
@@ -1618,10 +1618,9 @@ int launch_plan(const Plan& plan, cudaStream_t stream)
 template <int SPLIT, int HC>
 cudaError_t launch_variant2(const Plan& a, const Plan& b, cudaStream_t stream)
 {
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(conv_tc_kernel2<SPLIT, HC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT));
-    if (attr_rc != cudaSuccess) return attr_rc;
+    static SmemAttr attr;
+    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel2<SPLIT, HC>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
+    if (arc != cudaSuccess) return arc;
     return launch_chained(conv_tc_kernel2<SPLIT, HC>, dim3((unsigned)(a.grid + b.grid)), dim3(threads_for(SPLIT)),
                           a.smem > b.smem ? a.smem : b.smem, stream, a.a, a.b, a.o, a.p, b.a, b.b, b.o, b.p);
 }
@@ -1634,11 +1633,11 @@ int launch_plan2(const Plan& a, const Plan& b, cudaStream_t stream)
     if (a.p.pool != b.p.pool) return SQN_ERR_UNSUPPORTED;
     if (a.p.pool) {
         if (a.p.npix != b.p.npix) return SQN_ERR_UNSUPPORTED;
-        static const cudaError_t attr_rc =
-            cudaFuncSetAttribute(conv_pool_kernel2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT);
-        rc = attr_rc != cudaSuccess ? attr_rc
-           : launch_chained(conv_pool_kernel2, dim3((unsigned)(a.grid + b.grid)), dim3(POOLT_THREADS), smem, stream, a.a, a.b,
-                            a.r, a.p, b.a, b.b, b.r, b.p);
+        static SmemAttr attr;
+        rc = attr.allow((const void*)conv_pool_kernel2, SMEM_LIMIT);
+        if (rc == cudaSuccess)
+            rc = launch_chained(conv_pool_kernel2, dim3((unsigned)(a.grid + b.grid)), dim3(POOLT_THREADS), smem, stream, a.a, a.b,
+                                a.r, a.p, b.a, b.b, b.r, b.p);
     } else {
         const int hc = a.p.CW / 2;
         if (a.split != b.split || a.p.CW != b.p.CW) return SQN_ERR_UNSUPPORTED;
@@ -1781,9 +1780,8 @@ int launch_conv_bf16_pool4(const ConvDesc* d, cudaStream_t stream)
         if (pl[i]->smem > smem) smem = pl[i]->smem;
         grid += pl[i]->grid;
     }
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(conv_pool_kernel4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT);
-    if (attr_rc != cudaSuccess) return SQN_ERR_CUDA;
+    static SmemAttr attr;
+    if (attr.allow((const void*)conv_pool_kernel4, SMEM_LIMIT) != cudaSuccess) return SQN_ERR_CUDA;
     const cudaError_t rc = launch_chained(conv_pool_kernel4, dim3((unsigned)grid), dim3(POOLT_THREADS), smem, stream, pl[0]->a, pl[0]->b,
                                           pl[0]->p, pl[1]->a, pl[1]->b, pl[1]->p, pl[2]->a, pl[2]->b, pl[2]->p, pl[3]->a, pl[3]->b, pl[3]->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;

@@ -11,6 +11,7 @@
 #include <cstring>
 
 #include "f32_common.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 
 namespace sqn {
@@ -234,9 +235,9 @@ template <int TY, int RM, int SL, int ST, bool VEC>
 cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
 {
     constexpr size_t smem = (size_t)SL * ST * (RM * TY + 128 / TY) * SPITCH * 4;
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(conv_f32_small_kernel<TY, RM, SL, ST, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (attr_rc != cudaSuccess) return attr_rc;
+    static SmemAttr attr;
+    const cudaError_t arc = attr.allow((const void*)conv_f32_small_kernel<TY, RM, SL, ST, VEC>, smem);
+    if (arc != cudaSuccess) return arc;
     return launch_chained(conv_f32_small_kernel<TY, RM, SL, ST, VEC>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
 }
 

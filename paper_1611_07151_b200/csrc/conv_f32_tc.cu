@@ -45,6 +45,7 @@
 
 #include "f32_common.cuh"
 #include "ptx_sm100.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
 #include "tc_host.h"
@@ -1115,9 +1116,9 @@ int encode_f32_maps(const ConvDesc& d, F32TcPlan* plan)
 template <int MODE>
 cudaError_t launch_mode(const F32TcPlan& plan, cudaStream_t stream)
 {
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(conv_f32_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FT_SMEM_LIMIT);
-    if (attr_rc != cudaSuccess) return attr_rc;
+    static SmemAttr attr;
+    const cudaError_t arc = attr.allow((const void*)conv_f32_tc_kernel<MODE>, FT_SMEM_LIMIT);
+    if (arc != cudaSuccess) return arc;
     return launch_chained(conv_f32_tc_kernel<MODE>, dim3((unsigned)plan.p.grid), dim3(FT_THREADS), plan.smem, stream, plan.x, plan.w, plan.o, plan.p);
 }
 

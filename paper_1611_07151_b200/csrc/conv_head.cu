@@ -20,6 +20,7 @@
 
 #include "plan_cache.h"
 #include "ptx_sm100.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
 #include "tc_host.h"
@@ -322,9 +323,8 @@ int launch_conv_avgpool_bf16(const ConvDesc& d, float* logits, cudaStream_t stre
     std::shared_ptr<const HeadPlan> plan;
     const int prc = g_head_plans.get(k, &plan, [&](HeadPlan* p) { return build_head_plan(d, logits, p); });
     if (prc != SQN_OK) return prc;
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(conv_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM_LIMIT);
-    if (attr_rc != cudaSuccess) return SQN_ERR_CUDA;
+    static SmemAttr attr;
+    if (attr.allow((const void*)conv_head_kernel, CH_SMEM_LIMIT) != cudaSuccess) return SQN_ERR_CUDA;
     const cudaError_t rc = launch_chained(conv_head_kernel, dim3((unsigned)plan->grid), dim3(CH_THREADS), plan->smem, stream, plan->x,
                                           plan->w, plan->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;

@@ -11,6 +11,7 @@
 #include <cstring>
 
 #include "f32_common.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
 
@@ -195,9 +196,9 @@ template <bool F16, int SL, int ST>
 cudaError_t launch(const MmaSmallParams& a, const MmaSmallParams& b, cudaStream_t stream)
 {
     constexpr size_t smem = (size_t)SL * ST * MSLOT;
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(conv_mma_small_kernel<F16, SL, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (attr_rc != cudaSuccess) return attr_rc;
+    static SmemAttr attr;
+    const cudaError_t arc = attr.allow((const void*)conv_mma_small_kernel<F16, SL, ST>, smem);
+    if (arc != cudaSuccess) return arc;
     return launch_chained(conv_mma_small_kernel<F16, SL, ST>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
 }
 

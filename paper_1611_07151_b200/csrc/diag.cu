@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include "ptx_sm100.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
 
@@ -120,8 +121,8 @@ int launch_mma_rate_selftest(int n, int row_bytes, int issuers, int iters, long 
 {
     int* status = device_status_word();
     if (!status) return SQN_ERR_CUDA;
-    static const cudaError_t attr_rc = cudaFuncSetAttribute(mma_rate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-    if (attr_rc != cudaSuccess) return SQN_ERR_CUDA;
+    static SmemAttr attr;
+    if (attr.allow((const void*)mma_rate_kernel, 100 * 1024) != cudaSuccess) return SQN_ERR_CUDA;
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -34,6 +34,7 @@
 
 #include "plan_cache.h"
 #include "ptx_sm100.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
 #include "tc_host.h"
@@ -983,12 +984,10 @@ int launch_fire(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, cud
     const int prc = fire_plan(dsq, d1, d3, &plan);
     if (prc != SQN_OK) return prc;
     // (the 16-bit type is a compile-time constant of the kernel: the epilogues' conversion loops are straight-line code)
-    static const cudaError_t attr_rc0 =
-        cudaFuncSetAttribute(fire_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FF_SMEM_LIMIT);
-    static const cudaError_t attr_rc1 =
-        cudaFuncSetAttribute(fire_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FF_SMEM_LIMIT);
-    if (attr_rc0 != cudaSuccess || attr_rc1 != cudaSuccess) return SQN_ERR_CUDA;
-    const cudaError_t rc = launch_chained(plan->p.f16 ? fire_fused_kernel<true> : fire_fused_kernel<false>, dim3((unsigned)plan->p.grid),
+    static SmemAttr attr[2];
+    const auto kernel = plan->p.f16 ? fire_fused_kernel<true> : fire_fused_kernel<false>;
+    if (attr[plan->p.f16 ? 1 : 0].allow((const void*)kernel, FF_SMEM_LIMIT) != cudaSuccess) return SQN_ERR_CUDA;
+    const cudaError_t rc = launch_chained(kernel, dim3((unsigned)plan->p.grid),
                                           dim3(FF_THREADS), plan->smem, stream, plan->x, plan->wsq, plan->w3, plan->w1, plan->o, plan->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
     note_launch();

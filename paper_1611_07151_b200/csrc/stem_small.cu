@@ -10,6 +10,7 @@
 #include <cstring>
 
 #include "f32_common.cuh"
+#include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
 #include "tc_host.h"
@@ -187,9 +188,9 @@ __global__ void __launch_bounds__(256) stem_small_kernel(const __grid_constant__
 template <bool F16, bool RAW>
 cudaError_t launch(const StemSmallParams& p, int blocks, cudaStream_t stream)
 {
-    static const cudaError_t attr_rc =
-        cudaFuncSetAttribute(stem_small_kernel<F16, RAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, S_SMEM);
-    if (attr_rc != cudaSuccess) return attr_rc;
+    static SmemAttr attr;
+    const cudaError_t arc = attr.allow((const void*)stem_small_kernel<F16, RAW>, S_SMEM);
+    if (arc != cudaSuccess) return arc;
     return launch_chained(stem_small_kernel<F16, RAW>, dim3((unsigned)blocks), dim3(256), (size_t)S_SMEM, stream, p);
 }
 
