@@ -123,11 +123,10 @@ def current_stream():
         import torch
         torch.cuda.current_stream()         # (initialises CUDA)
         # the address itself: building the Stream object around it costs 3 us a call, a third of a small convolution's call
-        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
         _current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
-        if _raw_stream is None:
-            def _raw_stream(device):
-                return torch.cuda.current_stream(device).cuda_stream
+        # (assigned last: it tells other threads that both are there)
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+            (lambda device: torch.cuda.current_stream(device).cuda_stream)
     return _raw_stream(_current_device())
 
 
