@@ -315,6 +315,14 @@ int sqn_selftest_mma_rate(int n, int row_bytes, int issuers, int iters, void* ou
 /* Static, human-readable name of a status code. */
 const char* sqn_status_string(int status);
 
+/*
+ * Names the kernels that this thread's calls launch: from here on every launch made by the calling thread appends a line to
+ * text (HOST memory of `size` bytes, kept zero-terminated, whole lines only), e.g. "conv_f32_small 32x32 vec, 8 warps, 3
+ * slots".  text = NULL ends it; the buffer must stay valid until then.  The names are for reading and for tests of the choice
+ * between kernels, and change with them.  (Diagnostic: the paper has no counterpart.)
+ */
+int sqn_trace_launches(char* text, size_t size);
+
 /* Number of kernel launches the library has enqueued since it was loaded (host counter). */
 unsigned long long sqn_launch_count(void);
 

@@ -69,6 +69,7 @@ SIGNATURES = {
     "sqn_selftest_wait_timeout": (_c_int, [ctypes.c_longlong, _c_vp]),
     "sqn_selftest_mma_rate": (_c_int, [_c_int, _c_int, _c_int, _c_int, _c_vp, ctypes.POINTER(_c_int), _c_vp]),
     "sqn_status_string": (ctypes.c_char_p, [_c_int]),
+    "sqn_trace_launches": (_c_int, [_c_vp, _c_sz]),
     "sqn_launch_count": (ctypes.c_ulonglong, []),
 }
 
@@ -296,6 +297,11 @@ def sqn_selftest_mma_rate(n, row_bytes=128, issuers=1, iters=2000):
 
 def sqn_status_string(status):
     return lib().sqn_status_string(status).decode()
+
+
+def sqn_trace_launches(text, size=0):
+    """text: a ctypes string buffer that outlives the trace, or None to end it."""
+    _check(lib().sqn_trace_launches(text, size), "sqn_trace_launches")
 
 
 def sqn_launch_count():

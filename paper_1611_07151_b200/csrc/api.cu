@@ -1,6 +1,8 @@
 // C-ABI entry points: argument validation, dispatch, the fire layer and the SqueezeNet v1.0
 // forward composition, host-side layout helpers.  No device memory is allocated here.
 #include <atomic>
+#include <cstdarg>
+#include <cstdio>
 #include <cstdlib>
 #include <cmath>
 #include <cstring>
@@ -16,7 +18,26 @@
 namespace sqn {
 
 static std::atomic<unsigned long long> g_launches{0};
-void note_launch(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
+
+// sqn_trace_launches: this thread's buffer
+thread_local char* t_trace = nullptr;
+thread_local size_t t_trace_left = 0;
+
+void note_launch(const char* kernel, ...)
+{
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (!t_trace) return;
+    va_list args;
+    va_start(args, kernel);
+    const int n = std::vsnprintf(t_trace, t_trace_left, kernel, args);
+    va_end(args);
+    if (n < 0 || (size_t)n + 1 >= t_trace_left) { t_trace[0] = 0; t_trace = nullptr; return; }       // (full: whole lines only)
+    t_trace[n] = '\n';
+    t_trace[n + 1] = 0;
+    t_trace += n + 1;
+    t_trace_left -= (size_t)n + 1;
+}
+
 bool tuning_env_present()
 {
     for (char** e = environ; e && *e; ++e)
@@ -1035,6 +1056,15 @@ extern "C" const char* sqn_status_string(int status)
         case SQN_ERR_DEBUG: return "index check of the debug build failed";
         default: return "unknown status";
     }
+}
+
+extern "C" int sqn_trace_launches(char* text, size_t size)
+{
+    if (text && size == 0) return SQN_ERR_BADARG;
+    t_trace = text;
+    t_trace_left = size;
+    if (text) text[0] = 0;
+    return SQN_OK;
 }
 
 extern "C" unsigned long long sqn_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }

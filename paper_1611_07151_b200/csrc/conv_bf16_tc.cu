@@ -1611,7 +1611,7 @@ int launch_plan(const Plan& plan, cudaStream_t stream)
         rc = hc == 32 ? launch_variant<2, 32>(plan, stream)
            : hc == 16 ? launch_variant<2, 16>(plan, stream) : launch_variant<2, 8>(plan, stream);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
+    note_launch(plan.p.pool ? "conv_pool, %d pixels" : "conv_tc, %d layers", plan.p.pool ? plan.p.npix : plan.p.BN);
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 
@@ -1649,7 +1649,7 @@ int launch_plan2(const Plan& a, const Plan& b, cudaStream_t stream)
                : hc == 16 ? launch_variant2<2, 16>(a, b, stream) : launch_variant2<2, 8>(a, b, stream);
     }
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
+    note_launch(a.p.pool ? "conv_pool x 2, %d pixels" : "conv_tc x 2, %d layers", a.p.pool ? a.p.npix : a.p.BN);
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 
@@ -1785,7 +1785,7 @@ int launch_conv_bf16_pool4(const ConvDesc* d, cudaStream_t stream)
     const cudaError_t rc = launch_chained(conv_pool_kernel4, dim3((unsigned)grid), dim3(POOLT_THREADS), smem, stream, pl[0]->a, pl[0]->b,
                                           pl[0]->p, pl[1]->a, pl[1]->b, pl[1]->p, pl[2]->a, pl[2]->b, pl[2]->p, pl[3]->a, pl[3]->b, pl[3]->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
+    note_launch("conv_pool x 4, 128 pixels");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 
@@ -1860,7 +1860,7 @@ int launch_stem_pack_bf16(const ConvDesc& d, void* workspace, size_t workspace_b
                                          (size_t)PACK_ROWS * pitch * 2, stream, static_cast<const __nv_bfloat16*>(d.in), pin,
                                          d.N, d.H, d.W, Hp, Wp, (long long)d.N * d.H * d.W * 3, pitch, row_blocks,
                                          static_cast<const unsigned short*>(d.w), pw, d.Cout, d.bias, d.f16);
-    note_launch(1);
+    note_launch("stem_pack");
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

@@ -302,7 +302,7 @@ int launch_cfg(const F32Params& p, bool vec, cudaStream_t stream)
     dim3 grid((p.M + BM - 1) / BM, (p.Cout + BN - 1) / BN, 1);
     if (vec) conv_f32_kernel<BM, BN, VN, QN, true><<<grid, NTHREADS, 0, stream>>>(p);
     else conv_f32_kernel<BM, BN, VN, QN, false><<<grid, NTHREADS, 0, stream>>>(p);
-    note_launch();
+    note_launch("conv_f32 %dx%d%s%s", BM, BN, vec ? " vec" : "", !vec && p.Kdim > TBL_MAX ? " no table" : "");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

@@ -238,7 +238,10 @@ cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_
     static SmemAttr attr;
     const cudaError_t arc = attr.allow((const void*)conv_f32_small_kernel<TY, RM, SL, ST, VEC>, smem);
     if (arc != cudaSuccess) return arc;
-    return launch_chained(conv_f32_small_kernel<TY, RM, SL, ST, VEC>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
+    const cudaError_t rc =
+        launch_chained(conv_f32_small_kernel<TY, RM, SL, ST, VEC>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
+    if (rc == cudaSuccess) note_launch("conv_f32_small%s %dx%d%s, %d warps, %d slots", b.blocks ? " x 2" : "", RM * TY, 128 / TY, VEC ? " vec" : "", SL, ST);
+    return rc;
 }
 
 // Tile, warps and ring for a layer (or two) of so many tiles; measured on SqueezeNet's layers at batch 1 and 4:
@@ -301,7 +304,6 @@ int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
     else rc = c.narrow ? (vec ? launch_ty<8, 4, true>(p[0], p[1], stream) : launch_ty<8, 4, false>(p[0], p[1], stream))
                        : (vec ? launch_ty<4, 4, true>(p[0], p[1], stream) : launch_ty<4, 4, false>(p[0], p[1], stream));
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

@@ -1142,7 +1142,10 @@ int launch_conv_f32_tc(const ConvDesc& d, float limit_us, cudaStream_t stream)
     const cudaError_t e = plan.p.mode == FT_FLAT ? launch_mode<FT_FLAT>(plan, stream)
                         : plan.p.mode == FT_PATCH ? launch_mode<FT_PATCH>(plan, stream) : launch_mode<FT_BOX>(plan, stream);
     if (e != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
+    const F32TcParams& p = plan.p;
+    note_launch("conv_f32_tc %s, kernels %s, %d %s%s", p.mode == FT_FLAT ? "flat" : p.mode == FT_PATCH ? "patch" : "box",
+                p.wsrc == FT_W_PACKED ? "packed" : p.wsrc == FT_W_BOXES ? "by boxes" : "by copies", p.mode == FT_BOX ? p.nb : 1,
+                p.mode == FT_BOX && p.nb > 1 ? "blocks" : "block", p.mode == FT_BOX && p.S > p.K ? ", apart" : "");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

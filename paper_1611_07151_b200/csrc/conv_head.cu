@@ -328,7 +328,7 @@ int launch_conv_avgpool_bf16(const ConvDesc& d, float* logits, cudaStream_t stre
     const cudaError_t rc = launch_chained(conv_head_kernel, dim3((unsigned)plan->grid), dim3(CH_THREADS), plan->smem, stream, plan->x,
                                           plan->w, plan->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
+    note_launch("conv_head");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

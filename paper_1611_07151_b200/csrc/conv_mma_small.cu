@@ -199,7 +199,10 @@ cudaError_t launch(const MmaSmallParams& a, const MmaSmallParams& b, cudaStream_
     static SmemAttr attr;
     const cudaError_t arc = attr.allow((const void*)conv_mma_small_kernel<F16, SL, ST>, smem);
     if (arc != cudaSuccess) return arc;
-    return launch_chained(conv_mma_small_kernel<F16, SL, ST>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
+    const cudaError_t rc =
+        launch_chained(conv_mma_small_kernel<F16, SL, ST>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
+    if (rc == cudaSuccess) note_launch("conv_mma_small%s, %d warps, %d slots", b.blocks ? " x 2" : "", SL, ST);
+    return rc;
 }
 
 // Warps that share a tile's reduction and ring slots per warp: no more warps than chunks, and as many slots as let all CTAs
@@ -243,7 +246,6 @@ int launch_conv_mma_small(const ConvDesc* d, int n, cudaStream_t stream)
     if (n == 1) { p[1] = p[0]; p[1].blocks = 0; }
     const cudaError_t rc = d[0].f16 ? launch_shape<true>(p[0], p[1], stream) : launch_shape<false>(p[0], p[1], stream);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

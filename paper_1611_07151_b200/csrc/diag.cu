@@ -112,7 +112,7 @@ int launch_wait_timeout_selftest(long long limit_cycles, cudaStream_t stream)
     int* status = device_status_word();
     if (!status) return SQN_ERR_CUDA;
     wait_timeout_kernel<<<1, 64, 0, stream>>>(limit_cycles, status);
-    note_launch();
+    note_launch("wait_timeout");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 
@@ -128,7 +128,7 @@ int launch_mma_rate_selftest(int n, int row_bytes, int issuers, int iters, long 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms <= 0) return SQN_ERR_CUDA;
     mma_rate_kernel<<<sms, 128, 98 * 1024, stream>>>(iters, n, row_bytes, issuers, out, status);
-    note_launch();
+    note_launch("mma_rate");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

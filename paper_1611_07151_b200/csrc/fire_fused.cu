@@ -990,7 +990,7 @@ int launch_fire(const ConvDesc* dsq, const ConvDesc& d1, const ConvDesc& d3, cud
     const cudaError_t rc = launch_chained(kernel, dim3((unsigned)plan->p.grid),
                                           dim3(FF_THREADS), plan->smem, stream, plan->x, plan->wsq, plan->w3, plan->w1, plan->o, plan->p);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
+    note_launch("%s", dsq ? "fire_fused" : "fire_expands");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

@@ -337,7 +337,7 @@ int launch_maxpool3x3s2(const void* in, void* out, int C, int H, int W, int N, i
                                 static_cast<__nv_bfloat16*>(out), C, H, W, OH, OW, total);
         }
     }
-    note_launch();
+    note_launch("maxpool");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 
@@ -356,7 +356,7 @@ int launch_avgpool_softmax(const void* in, float* logits, float* probs, int C, i
             launch_chained(global_avgpool_bf16_v8<Bf16>, grid, dim3(256), 0, stream, static_cast<const uint4*>(in), logits, C, H * W);
     } else if (dtype == SQN_F16) launch_chained(global_avgpool_kernel<2>, grid, dim3(256), 0, stream, in, logits, C, H * W);
     else launch_chained(global_avgpool_kernel<1>, grid, dim3(256), 0, stream, in, logits, C, H * W);
-    note_launch();
+    note_launch("global_avgpool");
     if (cudaGetLastError() != cudaSuccess) return SQN_ERR_CUDA;
     if (probs) return launch_softmax(logits, probs, C, N, stream);
     return SQN_OK;
@@ -365,7 +365,7 @@ int launch_avgpool_softmax(const void* in, float* logits, float* probs, int C, i
 int launch_softmax(const float* logits, float* probs, int C, int N, cudaStream_t stream)
 {
     launch_chained(softmax_kernel, dim3((unsigned)N), dim3(256), (size_t)C * sizeof(float), stream, logits, probs, C);
-    note_launch();
+    note_launch("softmax");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

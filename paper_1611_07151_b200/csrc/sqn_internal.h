@@ -24,8 +24,8 @@ struct ConvDesc {
     int stem_prepacked;   // 1 (stem only): in and w already have the stem kernel's own layouts, see sqn_pack_stem_input
 };
 
-// Launch counter (host side): every kernel launch goes through note_launch().
-void note_launch(int n = 1);
+// Host side: every kernel launch is counted here, and its kernel named (printf style) for sqn_trace_launches.
+void note_launch(const char* kernel, ...);
 
 // False when no variable of the environment starts with SQN_: none of the tuning aids need be asked for.
 bool tuning_env_present();

@@ -222,7 +222,7 @@ int launch_stem_small(const ConvDesc& d, void* pool, cudaStream_t stream)
     const cudaError_t rc = d.stem_prepacked ? (d.f16 ? launch<true, false>(p, blocks, stream) : launch<false, false>(p, blocks, stream))
                                             : (d.f16 ? launch<true, true>(p, blocks, stream) : launch<false, true>(p, blocks, stream));
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch();
+    note_launch("stem_small");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

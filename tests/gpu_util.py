@@ -1,5 +1,8 @@
 """Helpers for the GPU parity tests: move oracle-layout arrays through the library's
 pack helpers, call the C ABI via the binding, and bring results back as NCHW float32."""
+import contextlib
+import ctypes
+
 import numpy as np
 
 from paper_1611_07151_b200 import binding as B
@@ -51,3 +54,15 @@ def gpu_conv(x, w, b, S, pad, relu=True, dtype=B.SQN_F32, c_offset=0, c_total=0,
                       out_c_total=c_total, workspace=ws, workspace_bytes=ws_bytes, fuse_maxpool=fuse_maxpool)
     assert B.sqn_check() == B.SQN_OK
     return host_act(out, dtype)
+
+
+@contextlib.contextmanager
+def traced():
+    """The kernels launched by the calls inside, as a list of names that is filled at the end."""
+    buf, names = ctypes.create_string_buffer(1 << 16), []
+    B.sqn_trace_launches(buf, len(buf))
+    try:
+        yield names
+    finally:
+        B.sqn_trace_launches(None)
+        names += buf.value.decode().splitlines()

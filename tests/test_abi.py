@@ -1,5 +1,6 @@
 """CPU-side checks of the boundary: the library loads, exports what include/sqn.h declares,
 validates arguments before touching the GPU, and its host layout helpers are exact."""
+import ctypes
 import os
 import re
 
@@ -152,3 +153,12 @@ def test_fp16_rounding_is_nearest_even():
     np.testing.assert_array_equal(got, exp)
     back = B.sqn_unpack_nhwc_to_nchw(got.reshape(1, 1, 1, -1), B.SQN_F16).ravel()
     np.testing.assert_array_equal(back, torch.from_numpy(x.ravel()).to(torch.float16).float().numpy())
+
+
+def test_trace_takes_a_buffer_or_nothing():
+    l = B.lib()
+    assert l.sqn_trace_launches(None, 0) == B.SQN_OK
+    buf = ctypes.create_string_buffer(b"x" * 16, 16)
+    assert l.sqn_trace_launches(buf, 0) == B.SQN_ERR_BADARG and buf.raw == b"x" * 16
+    assert l.sqn_trace_launches(buf, 16) == B.SQN_OK and buf.value == b""
+    assert l.sqn_trace_launches(None, 0) == B.SQN_OK
