@@ -149,7 +149,8 @@ int make_conv_desc(const void* in, const void* w, const void* bias, void* out, i
 inline bool is_stem_shape(const ConvDesc& d) { return d.K == 7 && d.S == 2 && d.pad == 0 && d.Cin == 3; }
 
 // A single 16-bit layer on the small-layer kernel?  Where its estimate is clearly below that of a tcgen05 kernel with no more
-// tiles than SMs, 3.6 us and 5 ns per reduction element (3.8 where its tiles of more than 64 layers can be made narrower).  One
+// tiles than SMs, 3.6 us and 4.2 ns per reduction element (3.8 where its tiles of more than 64 layers can be made narrower; with 5
+// the 5x5 layer 96 -> 16 at 62 x 12, 11 images, came here for 13.5 us in the place of 12.3).  One
 // image of a bottleneck's 512 -> 512 3x3 layer at 7 x 7: 10.7 us against 26.4 (22 with narrow tiles); 256 -> 256 at 14 x 14: 6.6
 // against 15.3 (13); 512 -> 1000 1x1 at 13 x 13: 4.8 against 8.5; eight images of 384 -> 48 at 27 x 27: 6.3 against 5.5.
 // Layers that the pooled kernels take as well (up to 128 output layers, in groups of 32) keep the kernels whose sums add up
@@ -157,7 +158,7 @@ inline bool is_stem_shape(const ConvDesc& d) { return d.K == 7 && d.S == 2 && d.
 bool small_conv(const ConvDesc& d)
 {
     if (d.pool || (d.Cout <= 128 && d.Cout % 32 == 0)) return false;
-    const float tc = 3.6f + (d.Cout > 64 ? 0.0038f : 0.005f) * d.K * d.K * d.Cin;
+    const float tc = 3.6f + (d.Cout > 64 ? 0.0038f : 0.0042f) * d.K * d.K * d.Cin;
     return mma_small_estimate(&d, 1) < 0.92f * tc && !(tuning_env_present() && std::getenv("SQN_TC_VARIANT"));
 }
 

@@ -340,7 +340,7 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
     // idle, the tile with the least estimated time is taken instead: rounds of CTAs per SM x tile area / relative
     // FFMA efficiency of the thread tile (8 x TN: fewer output layers per thread mean more shared-memory loads per
     // FFMA).  The sum over the reduction index runs in the same order for every tile shape, so the values do not
-    // depend on this choice.
+    // depend on the tile; they do depend on which of the three kernels is chosen below.
     const int sms = sm_count();
     auto ctas_of = [&](int tm, int tn) { return ((M + tm - 1) / tm) * (long long)((d.Cout + tn - 1) / tn); };
     int bm = best <= 32 ? 256 : 128, bn = best;
@@ -356,20 +356,31 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
         }
     }
     {
-        // Which of the three fp32 kernels: by estimated time.  This one: rounds of CTAs at 0.6 of the FFMA rate (0.45 with
-        // 4-byte loads), the latency of the reduction loop, or bytes.  Measured, this kernel / the small layers' / the tensor
-        // cores' -- batch 1: fire9's squeeze 19.6 / 4.7 / 18.0 us, fire6's expand-3x3 16.4 / 6.4 / 15.5, fire4's 14.5 / 11.3 /
-        // 12.6, conv1 25.7 / 31 / 17.4; batch 16: fire4's expand-3x3 99 / 109 / 33, its expand-1x1 17.2 / 34 / 11.5, fire2's
-        // expand-1x1 6.9 / 15.6 / 10.0; batch 256: conv1 2687 / - / 996, fire4's expand-3x3 1296 / - / 354, conv10 1256 / - /
-        // 281, fire2's squeeze 132 / - / 133, fire3's 141 / - / 164, fire2's expand-1x1 88 / - / 78.
+        // Which of the three fp32 kernels: by estimated time.  This one: rounds of CTAs at 0.6 of the FFMA rate (with 4-byte loads
+        // 0.4, the 256-pixel tiles 0.24, and 1.9 us for the start and end of every two CTAs on an SM: 450 random layers 0.9 to 1.1 of
+        // it in eight of ten), the latency of the reduction loop, or bytes.  Over 990 random layers the kernel chosen takes 0.7 %
+        // longer than the best of the three on average, 30 % or more in four.  Measured, this kernel / the small layers' / the
+        // tensor cores' -- batch 1: fire9's squeeze 19.6 / 4.7 / 18.0 us, fire6's expand-3x3 16.4 / 6.4 / 15.5, fire4's 14.5 /
+        // 11.3 / 12.6, conv1 25.7 / 31 / 17.4; batch 16: fire4's expand-3x3 99 / 109 / 33, its expand-1x1 17.2 / 34 / 11.5,
+        // fire2's expand-1x1 6.9 / 15.6 / 10.0; batch 256: conv1 2687 / - / 1050, fire4's expand-3x3 1296 / - / 354, conv10
+        // 1256 / - / 281, fire2's squeeze 132 / - / 133, fire3's 141 / - / 164, fire2's expand-1x1 88 / - / 78.
         const double eff = bm == 128 ? (bn == 128 ? 1.0 : bn == 96 ? 0.95 : bn == 64 ? 0.85 : 0.75)
                          : bm == 256 ? (bn == 32 ? 0.85 : 0.6) : (bn == 128 ? 0.85 : bn == 64 ? 0.6 : 0.4);
         const double area = (double)((ctas_of(bm, bn) + sms - 1) / sms) * bm * bn / eff;
-        float us = (float)(area * (double)Kdim / (128.0 * 1965.0 * (vec ? 0.6 : 0.45)));
-        const float lat_us = 0.035f * (float)Kdim, mem_us = 4.f * ((float)d.N * d.H * d.W * d.Cin + (float)M * d.Cout) / 2.7e6f;
+        const float pairs = (float)((ctas_of(bm, bn) + 2 * sms - 1) / (2 * sms));       // rounds of two CTAs per SM
+        const float mem_us = 4.f * ((float)d.N * d.H * d.W * d.Cin + (float)M * d.Cout) / 2.7e6f;
+        float us, lat_us;
+        if (vec) {
+            us = (float)(area * (double)Kdim / (128.0 * 1965.0 * 0.6));
+            lat_us = 0.035f * (float)Kdim;
+        } else {
+            const float slow = Kdim > TBL_MAX ? 1.65f : 1.f;        // (two divisions per element)
+            us = slow * (float)(area * (double)Kdim / (128.0 * 1965.0 * (bm == 256 ? 0.24 : 0.4)));
+            lat_us = slow * 0.0175f * (float)Kdim * pairs;
+        }
         if (lat_us > us) us = lat_us;
         if (mem_us > us) us = mem_us;
-        us += 2.f;
+        us += vec ? (d.S == 1 ? 2.f : 2.f + pairs) : 2.8f + 1.9f * pairs;
         const float small_us = f32_small_estimate(d), other_us = small_us < us ? small_us : us;
         if (6.1f + 0.45f * (float)((Kdim + 31) / 32) < other_us) {      // (one tile of the tensor-core kernel: not worth a plan if above)
             const int rc = launch_conv_f32_tc(d, other_us, stream);

@@ -277,14 +277,17 @@ cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, cudaStre
 
 }  // namespace
 
-// Microseconds, fitted to SqueezeNet's layers at batch 1 and 4 (within 25 %): a launch, then the busiest SM's tiles at 260
-// clocks per chunk (150 with the smaller tile; 750 where the operands come in pieces of 4 bytes).
+// Microseconds: a launch, then the busiest SM's tiles at 260 clocks per chunk (150 with the smaller tile), fitted to SqueezeNet's
+// layers at batch 1 and 4; where the operands come in pieces of 4 bytes 500 clocks (450 with the smaller tile, 900 for the narrow
+// one) and more for a tile's start, fitted to 450 random layers (0.85 to 1.15 of it in eight of ten; 750 for all of them gave 0.46).
 float f32_small_estimate(const ConvDesc& d)
 {
     const SmallConfig c = config_of(&d, 1);
     const long long blocks = (((long long)d.N * d.OH * d.OW + c.tm - 1) / c.tm) * ((d.Cout + c.tn - 1) / c.tn);
     const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
-    const float us = (float)((blocks + 147) / 148) * (chunks * (d.Cin % 4 != 0 ? 750.f : c.rm == 4 ? 150.f : 260.f) + 450.f) / 1965.f;
+    const float rounds = (float)((blocks + 147) / 148);
+    if (d.Cin % 4 != 0) return 2.7f + rounds * (chunks * (c.rm == 4 ? 450.f : c.narrow ? 900.f : 500.f) + 1650.f) / 1965.f;
+    const float us = rounds * (chunks * (c.rm == 4 ? 150.f : 260.f) + 450.f) / 1965.f;
     return 2.2f + (blocks > 296 ? 1.2f * us : us);
 }
 

@@ -1122,10 +1122,20 @@ cudaError_t launch_mode(const F32TcPlan& plan, cudaStream_t stream)
     return launch_chained(conv_f32_tc_kernel<MODE>, dim3((unsigned)plan.p.grid), dim3(FT_THREADS), plan.smem, stream, plan.x, plan.w, plan.o, plan.p);
 }
 
-// Microseconds this kernel takes, fitted to SqueezeNet's layers at batch 1 .. 256 (within 25 %): start and end of a launch,
-// then per tile of the busiest CTA its epilogue and its units of 32 (or 16) reduction elements.
+// Microseconds this kernel takes: start and end of a launch, then per tile of the busiest CTA its epilogue and its units of 32
+// (or 16) reduction elements.  FLAT and PATCH: fitted to SqueezeNet's layers at batch 1 .. 256 (500 random layers: 0.85 to 1.2
+// of it in nine of ten).  BOX: the copies of a tile's windows, a thread's share one after the other (0.05 us each where a window
+// row is one run of memory, else 0.1) and 0.4 us for every block of layers, and the kernels' split, once; fitted to 890 random
+// layers with a stride or odd layer counts (0.9 to 1.15 of it in eight of ten, 1.7 at most; without these terms 1.0 to 6.5, and a
+// 1x1/3 layer of 28 images, 151 -> 53 at 57 x 49, went here for 40 us in the place of 15).
 float f32_tc_estimate(const F32TcParams& p)
 {
+    if (p.mode == FT_BOX) {
+        const int copies = ceil_div(p.rh, 8) * ceil_div((long long)p.rc * p.cb, p.box_vec ? 128 : 32);
+        const float unit = p.wsrc == FT_W_COPIES ? 1.24f : 0.8f, packed = p.wsrc == FT_W_PACKED ? (float)(p.chunks * p.wrows) / 128.f : 0.f;
+        const float tile = 2.f + unit * (float)p.chunks + (float)p.nb * (0.4f + (p.nb == 1 && p.S <= p.K ? 0.047f : 0.1f) * (float)copies);
+        return 3.5f + 1.5f * (p.khalf ? 0.5f : 1.f) * packed + (float)ceil_div(p.m_tiles, p.m_step) * ceil_div(p.grid, sm_count()) * tile;
+    }
     const float unit = p.wsrc != FT_W_PACKED && p.mode != FT_PATCH ? 0.9f : p.khalf ? 0.45f : 0.63f;
     return 4.5f + (float)ceil_div(p.m_tiles, p.m_step) * ceil_div(p.grid, sm_count()) * (1.6f + unit * (float)(p.chunks * p.taps));
 }
