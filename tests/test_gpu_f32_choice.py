@@ -19,6 +19,8 @@ CASES = [
     ((19, 125, 373, 13, 11, 3, 2, 0), "conv_f32_small",),                   # 96 / 38 / 100
     ((51, 145, 6, 75, 52, 5, 1, 0), "conv_f32_tc", "conv_f32_small"),       # 1770 / 2040 / 3150
     ((50, 285, 17, 61, 56, 3, 3, 0), "conv_f32_small",),                    # 577 / 199 / 661
+    ((25, 96, 16, 55, 55, 1, 1, 0), "conv_f32 "),                          # 18 / 17 / 15
+    ((71, 96, 16, 55, 55, 1, 1, 0), "conv_f32 "),                          # 44 / 42 / 37
     ((16, 64, 128, 56, 56, 3, 2, 1), "conv_f32_tc",),                       # 38 / - / 65
     ((64, 3, 96, 227, 227, 7, 2, 0), "conv_f32_tc",),                       # 265 / - / 690
 ]
