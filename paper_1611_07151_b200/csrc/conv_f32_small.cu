@@ -278,9 +278,10 @@ cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, cudaStre
 }  // namespace
 
 // Microseconds: a launch, then the busiest SM's tiles at 260 clocks per chunk (150 with the smaller tile), fitted to SqueezeNet's
-// layers at batch 1 and 4, and 345 with the narrow one (42 random layers of up to 16 output layers 314 to 375, half of them; with 260
-// fire2's squeeze of 25 images came here for 16.9 us, FFMA 14.6); where the operands come in pieces of 4 bytes 500 clocks (450 with the smaller tile, 900 for the narrow
-// one) and more for a tile's start, fitted to 450 random layers (0.85 to 1.15 of it in eight of ten; 750 for all of them gave 0.46).
+// layers at batch 1 and 4, and 375 with the narrow one (42 random layers of up to 16 output layers: 257 to 414, fire2's squeezes
+// 390; with 260 fire2's squeeze of 25 images came here for 16.9 us, FFMA 14.6).  Where the operands come in pieces of 4 bytes
+// 500 clocks (450 with the smaller tile, 900 with the narrow one) and more for a tile's start, fitted to 450 random layers (0.85
+// to 1.15 of it in eight of ten; 750 for all of them gave 0.46).
 float f32_small_estimate(const ConvDesc& d)
 {
     const SmallConfig c = config_of(&d, 1);
@@ -288,7 +289,7 @@ float f32_small_estimate(const ConvDesc& d)
     const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
     const float rounds = (float)((blocks + 147) / 148);
     if (d.Cin % 4 != 0) return 2.7f + rounds * (chunks * (c.rm == 4 ? 450.f : c.narrow ? 900.f : 500.f) + 1650.f) / 1965.f;
-    const float us = rounds * (chunks * (c.rm == 4 ? 150.f : c.narrow ? 345.f : 260.f) + 450.f) / 1965.f;
+    const float us = rounds * (chunks * (c.rm == 4 ? 150.f : c.narrow ? 375.f : 260.f) + 450.f) / 1965.f;
     return 2.2f + (blocks > 296 ? 1.2f * us : us);
 }
 
