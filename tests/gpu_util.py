@@ -36,8 +36,9 @@ def out_extent(H, K, S, pad):
     return (H + 2 * pad - K) // S + 1
 
 
-def gpu_conv(x, w, b, S, pad, relu=True, dtype=B.SQN_F32, c_offset=0, c_total=0, fill=None, fuse_maxpool=False):
-    """Run one convolution through conv_forward_ex; returns the full output tensor as NCHW."""
+def gpu_conv(x, w, b, S, pad, relu=True, dtype=B.SQN_F32, c_offset=0, c_total=0, fill=None, fuse_maxpool=False, kernel=None):
+    """Run one convolution through conv_forward_ex; returns the full output tensor as NCHW.  kernel: the name (or its start)
+    of the one kernel that has to run."""
     import torch
     N, C, H, W = x.shape
     M, _, K, _ = w.shape
@@ -50,9 +51,11 @@ def gpu_conv(x, w, b, S, pad, relu=True, dtype=B.SQN_F32, c_offset=0, c_total=0,
     ws_bytes = B.conv_workspace_bytes(C, M, H, W, K, S, pad, N, dtype)
     ws = torch.empty(max(ws_bytes, 16), dtype=torch.uint8, device="cuda")
     xd, wd, bd = dev_act(x, dtype), dev_w(w, dtype), dev_b(b)
-    B.conv_forward_ex(xd, wd, bd, out, C, M, H, W, K, S, pad, N, dtype=dtype, relu=relu, out_c_offset=c_offset,
-                      out_c_total=c_total, workspace=ws, workspace_bytes=ws_bytes, fuse_maxpool=fuse_maxpool)
+    with traced() as names:
+        B.conv_forward_ex(xd, wd, bd, out, C, M, H, W, K, S, pad, N, dtype=dtype, relu=relu, out_c_offset=c_offset,
+                          out_c_total=c_total, workspace=ws, workspace_bytes=ws_bytes, fuse_maxpool=fuse_maxpool)
     assert B.sqn_check() == B.SQN_OK
+    assert kernel is None or (len(names) == 1 and names[0].startswith(kernel)), names
     return host_act(out, dtype)
 
 

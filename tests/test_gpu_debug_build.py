@@ -21,6 +21,10 @@ SMALL_SHAPE_TESTS = [
     "tests/test_gpu_bf16.py::test_conv_with_fused_global_average",
     "tests/test_gpu_bf16.py::test_full_forward_bf16_small_batch_keeps_every_map",
     "tests/test_gpu_f32.py::test_awkward_shapes",
+    "tests/test_gpu_f32_small.py",
+    "tests/test_gpu_f32_ffma.py",
+    "tests/test_gpu_f32_tensor.py",
+    "tests/test_gpu_mma_small.py",
     "tests/test_gpu_f32.py::test_config2_full_forward_batch1",
 ]
 

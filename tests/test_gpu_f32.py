@@ -34,22 +34,22 @@ def test_plain_conv_forward_entry_point():
     assert G.rel_err(G.host_act(out, F32), exp) <= TOL
 
 
-# (N, Cin, Cout, H, K, S, pad): tiles with ragged tails, layer counts off the vector widths,
-# every output-tile configuration, strides and paddings beyond SqueezeNet's
+# (N, Cin, Cout, H, K, S, pad): small layers with ragged tails, layer counts off the vector widths, strides and paddings
+# beyond SqueezeNet's, whichever kernel they run on (test_gpu_f32_small, _ffma and _tensor name the kernel's variant)
 AWKWARD = [
     (1, 3, 96, 37, 7, 2, 0),      # stem shape, small map
     (3, 3, 5, 11, 3, 1, 1),       # scalar path, tiny layer count
     (2, 5, 7, 9, 2, 1, 0),        # even kernel, odd everything
     (2, 4, 16, 13, 3, 2, 1),      # vector path, Kdim = 36 (not a multiple of the k tile)
     (1, 12, 33, 10, 1, 1, 0),     # Cout one past a tile
-    (3, 16, 48, 14, 3, 1, 1),     # 48-wide tile
-    (2, 32, 192, 9, 1, 1, 0),     # 96-wide tiles
-    (1, 64, 256, 13, 3, 1, 1),    # 128-wide tiles, Kdim 576
+    (3, 16, 48, 14, 3, 1, 1),     # 48 layers
+    (2, 32, 192, 9, 1, 1, 0),     # 192 layers
+    (1, 64, 256, 13, 3, 1, 1),    # 256 layers, Kdim 576
     (1, 48, 130, 7, 3, 1, 2),     # pad larger than SqueezeNet's, ragged Cout
     (5, 20, 17, 6, 5, 3, 2),      # stride 3, 5x5
     (1, 8, 8, 1, 1, 1, 0),        # 1x1 map
     (1, 7, 9, 5, 5, 1, 0),        # window == input: single output pixel
-    (2, 515, 10, 4, 3, 1, 1),     # long scalar reduction (table does not fit)
+    (2, 515, 10, 4, 3, 1, 1),     # long reduction in 4-byte pieces
 ]
 
 

@@ -1,5 +1,5 @@
 """The exact path's tensor-core kernel (every fp32 operand as three bf16 numbers) against the oracle, at the sizes where its
-tiles, chunks and dispatch branches end.  The shapes are large enough for the dispatch to take it.
+tiles, chunks and dispatch branches end.  That a shape really runs on it, and in which variant, is asserted by name.
 
 Bound per output, S = sum of |kernel * input| over the window: the products left out are below 2^-22 of the operands'
 product; a segment of 32 products is cut to 24 bits in two steps of at most 2^-23 of what it holds, the segments are added
@@ -15,24 +15,32 @@ import gpu_util as G
 pytestmark = pytest.mark.gpu
 F32 = B.SQN_F32
 
-# (N, Cin, Cout, H, K, S, pad)
+# (N, Cin, Cout, H, K, S, pad), the variant that runs
 SHAPES = [
-    (40, 128, 32, 55, 1, 1, 0),     # kernels kept in shared memory, a quarter of the MMA rows live
-    (11, 260, 130, 27, 1, 1, 0),    # streamed kernels, last chunk of 4, two columns of tiles, ragged everywhere
-    (3, 512, 1000, 13, 1, 1, 0),    # eight columns of tiles
-    (24, 16, 64, 55, 3, 1, 1),      # patch, units of 16 reduction elements
-    (9, 48, 192, 27, 3, 1, 1),      # patch, last chunk of 16, 96 layers per column
-    (8, 64, 130, 33, 3, 1, 1),      # patch, streamed kernels
-    (6, 36, 70, 40, 5, 1, 2),       # 5x5 patch, chunk of 4
-    (4, 32, 64, 60, 3, 1, 0),       # no padding
-    (6, 32, 96, 41, 2, 1, 1),       # even kernel, output larger than the input
-    (2, 3, 96, 111, 7, 2, 0),       # staged windows, layers not a multiple of 4
-    (8, 64, 128, 33, 3, 2, 1),      # staged windows in 16-byte pieces, several blocks of layers
-    (4, 35, 72, 45, 3, 2, 1),       # ... in 4-byte pieces, kernels by copies
-    (12, 130, 128, 28, 1, 2, 0),    # windows apart from one another
-    (1, 64, 64, 300, 3, 1, 1),      # rows too long for the patch
+    ((40, 128, 32, 55, 1, 1, 0), "flat, kernels packed"),           # a quarter of the MMA rows live
+    ((11, 260, 130, 27, 1, 1, 0), "flat, kernels by boxes"),        # last chunk of 4, two columns of tiles, ragged everywhere
+    ((3, 512, 1000, 13, 1, 1, 0), "flat, kernels by boxes"),        # eight columns of tiles
+    ((24, 16, 64, 55, 3, 1, 1), "patch, kernels packed"),           # units of 16 reduction elements
+    ((9, 48, 192, 27, 3, 1, 1), "patch, kernels by boxes"),         # last chunk of 16, 96 layers per column
+    ((8, 64, 130, 33, 3, 1, 1), "patch, kernels by boxes"),
+    ((6, 36, 70, 40, 5, 1, 2), "patch, kernels by boxes"),          # 5x5, chunk of 4
+    ((4, 32, 64, 60, 3, 1, 0), "patch, kernels by boxes"),          # no padding
+    ((6, 32, 96, 41, 2, 1, 1), "patch, kernels packed"),            # even kernel, output larger than the input
+    ((5, 3, 96, 111, 7, 2, 0), "box, kernels packed, 1 block"),     # layers not a multiple of 4
+    ((46, 8, 323, 31, 2, 2, 1), "box, kernels packed, 1 block"),    # ... a multiple of 4
+    ((34, 16, 496, 50, 1, 2, 0), "box, kernels packed, 1 block, apart"),        # windows apart from one another
+    ((42, 122, 124, 18, 1, 1, 0), "box, kernels packed, 4 blocks"),
+    ((40, 124, 128, 58, 1, 2, 0), "box, kernels packed, 4 blocks, apart"),
+    ((1, 64, 64, 300, 3, 1, 1), "box, kernels by boxes, 1 block"),  # rows too long for the patch
+    ((30, 47, 308, 7, 2, 1, 1), "box, kernels by boxes, 1 block"),
+    ((43, 24, 353, 26, 2, 3, 0), "box, kernels by boxes, 1 block, apart"),
+    ((60, 11, 2, 38, 7, 2, 0), "box, kernels by copies, 1 block"),  # two output layers
+    ((25, 95, 109, 60, 1, 2, 0), "box, kernels by copies, 1 block, apart"),
+    ((16, 64, 128, 56, 3, 2, 1), "box, kernels by copies, 4 blocks"),           # 16-byte pieces
+    ((23, 36, 304, 30, 2, 2, 0), "box, kernels by copies, 3 blocks"),           # ... the last block of 4 layers
+    ((20, 77, 133, 21, 3, 1, 1), "box, kernels by copies, 3 blocks"),           # 4-byte pieces
+    ((60, 206, 97, 25, 1, 2, 0), "box, kernels by copies, 7 blocks, apart"),
 ]
-
 
 def bound(x, w, b, S, pad, K, C):
     z = np.zeros_like(b)
@@ -40,14 +48,14 @@ def bound(x, w, b, S, pad, K, C):
     return (2.0 ** -22 + 2 * 2.0 ** -23 + (K * K * C / 32 + 4) * 2.0 ** -24) * (terms + np.abs(b)[None, :, None, None])
 
 
-@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
-def test_tensor_core_kernel_within_rounding(shape):
+@pytest.mark.parametrize("shape,variant", SHAPES, ids=["x".join(map(str, s)) for s, _ in SHAPES])
+def test_tensor_core_kernel_within_rounding(shape, variant):
     N, C, M, H, K, S, pad = shape
     rng = np.random.default_rng(sum(shape))
     x = rng.standard_normal((N, C, H, H - 2)).astype(np.float32)
     w, b = synth.draw_conv_params(rng, C, M, K)
     exp = ref.conv2d(x, w, b, S=S, pad=pad, relu=False)
-    got = G.gpu_conv(x, w, b, S, pad, False, F32)
+    got = G.gpu_conv(x, w, b, S, pad, False, F32, kernel="conv_f32_tc " + variant)
     assert got.shape == exp.shape
     assert (np.abs(got.astype(np.float64) - exp) <= bound(x, w, b, S, pad, K, C)).all()
 
@@ -57,7 +65,7 @@ def test_tensor_core_kernel_within_rounding(shape):
 def test_tensor_core_kernel_writes_its_slice_only(N, M, K, offset, total):
     x, w, b = synth.conv_layer_case(8, N, 128, M, 29, K)
     exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=True)
-    got = G.gpu_conv(x, w, b, 1, K // 2, True, F32, c_offset=offset, c_total=total, fill=-7.0)
+    got = G.gpu_conv(x, w, b, 1, K // 2, True, F32, c_offset=offset, c_total=total, fill=-7.0, kernel="conv_f32_tc ")
     assert (np.abs(got[:, offset:offset + M].astype(np.float64) - exp) <= bound(x, w, b, 1, K // 2, K, 128)).all()
     assert (got[:, :offset] == -7.0).all() and (got[:, offset + M:] == -7.0).all()
 
@@ -73,11 +81,11 @@ def test_exact_sums_stay_exact_and_infinities_come_through(K):
     w[np.arange(C), rng.permutation(C), K // 2, K // 2] = 1.0
     b = np.zeros(C, np.float32)
     exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=False)
-    np.testing.assert_array_equal(G.gpu_conv(x, w, b, 1, K // 2, False, F32), exp)
+    np.testing.assert_array_equal(G.gpu_conv(x, w, b, 1, K // 2, False, F32, kernel="conv_f32_tc "), exp)
     x[1, 5, 3, 4], x[2, 7, 20, 20], x[3, 9, 0, 0] = np.inf, np.nan, np.finfo(np.float32).max
     with np.errstate(invalid="ignore"):
         exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=False)
-    np.testing.assert_array_equal(G.gpu_conv(x, w, b, 1, K // 2, False, F32), exp)
+    np.testing.assert_array_equal(G.gpu_conv(x, w, b, 1, K // 2, False, F32, kernel="conv_f32_tc "), exp)
 
 
 @pytest.mark.parametrize("relu", [True, False])
@@ -86,7 +94,7 @@ def test_a_bias_that_is_not_finite(relu):
     x, w, b = synth.conv_layer_case(6, 32, 64, 128, 27, 1)
     b[[7, 40, 100]] = np.nan, np.inf, -np.inf
     exp = ref.conv2d(x, w, np.where(np.isfinite(b), b, 0).astype(np.float32), S=1, pad=0, relu=relu)
-    got = G.gpu_conv(x, w, b, 1, 0, relu, F32)
+    got = G.gpu_conv(x, w, b, 1, 0, relu, F32, kernel="conv_f32_tc ")
     special = {7: 0.0 if relu else np.nan, 40: np.inf, 100: 0.0 if relu else -np.inf}
     for m, v in special.items():
         np.testing.assert_array_equal(got[:, m], np.full_like(got[:, m], v))
@@ -106,7 +114,7 @@ def test_operands_of_any_magnitude_keep_their_bits(K, ex, ew):
     exp = ref.conv2d(x, w, b, S=1, pad=K // 2, relu=False)
     xs, ws = np.ldexp(x, ex), np.ldexp(w, ew)
     assert (np.ldexp(xs.astype(np.float64), -ex) == x).all() and (np.ldexp(ws.astype(np.float64), -ew) == w).all()
-    got = np.ldexp(G.gpu_conv(xs, ws, b, 1, K // 2, False, F32).astype(np.float64), -ex - ew)
+    got = np.ldexp(G.gpu_conv(xs, ws, b, 1, K // 2, False, F32, kernel="conv_f32_tc ").astype(np.float64), -ex - ew)
     # (the last term: half a unit of the smallest fp32 output)
     assert (np.abs(got - exp) <= bound(x, w, b, 1, K // 2, K, 64) + 2.0 ** (-150 - ex - ew)).all()
 
@@ -145,7 +153,7 @@ def test_sums_that_are_not_finite(shape):
     w[M - 1, 3, K // 2, K // 2], w[5, C - 1, K // 2, K // 2] = np.inf, np.nan
     with np.errstate(invalid="ignore", over="ignore"):
         exp = ref.conv2d(x, w, b, S=S, pad=pad, relu=False)
-        got = G.gpu_conv(x, w, b, S, pad, False, F32)
+        got = G.gpu_conv(x, w, b, S, pad, False, F32, kernel="conv_f32_tc ")
         # (3e38 times a kernel value: a sum that overflows or not by the order of its terms is left out)
         unsure = np.isinf(ref.conv2d(np.abs(np.nan_to_num(x, nan=0, posinf=0, neginf=0)), np.abs(np.nan_to_num(w, nan=0, posinf=0)), np.abs(b),
                                      S=S, pad=pad, relu=False))

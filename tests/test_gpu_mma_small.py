@@ -16,20 +16,17 @@ import gpu_util as G
 pytestmark = pytest.mark.gpu
 ULP = {B.SQN_BF16: 2.0 ** -8, B.SQN_F16: 2.0 ** -11}
 
-# (N, Cin, Cout, H, W, K, pad)
+# (N, Cin, Cout, H, W, K, pad), the variant that runs
 SHAPES = [
-    (1, 32, 264, 9, 7, 1, 0),       # one chunk, layers past a tile
-    (1, 48, 144, 12, 8, 1, 0),      # two chunks, the last of 16
-    (1, 112, 160, 5, 13, 1, 0),     # four chunks
-    (1, 512, 1000, 13, 13, 1, 0),   # 192 tiles, 8 pixels past a tile, 8 layers past a tile
-    (2, 512, 1000, 13, 13, 1, 0),   # 352 tiles: four warps, three slots
-    (3, 512, 1000, 13, 13, 1, 0),   # 512 tiles: two slots
-    (1, 512, 512, 7, 7, 3, 1),      # 144 chunks
-    (1, 16, 48, 1, 1, 3, 1),        # one pixel
-    (1, 176, 256, 3, 10, 5, 2),
-    (1, 64, 256, 13, 13, 3, 0),
+    ((1, 32, 264, 9, 7, 1, 0), "1 warps, 2 slots"),         # one chunk, layers past a tile
+    ((1, 48, 144, 12, 8, 1, 0), "2 warps, 2 slots"),        # two chunks, the last of 16
+    ((1, 112, 160, 5, 13, 1, 0), "4 warps, 2 slots"),       # four chunks
+    ((1, 512, 1000, 13, 13, 1, 0), "8 warps, 2 slots"),     # 192 tiles, 8 pixels past a tile, 8 layers past a tile
+    ((1, 512, 512, 7, 7, 3, 1), "8 warps, 3 slots"),        # 144 chunks
+    ((1, 16, 48, 1, 1, 3, 1), "8 warps, 3 slots"),          # one pixel
+    ((1, 176, 256, 3, 10, 5, 2), "8 warps, 3 slots"),
+    ((1, 64, 256, 13, 13, 3, 0), "8 warps, 3 slots"),
 ]
-
 
 def check(got, x, w, b, pad, relu, dtype):
     exp = ref.conv2d(x, w, b, S=1, pad=pad, relu=relu).astype(np.float64)
@@ -46,30 +43,39 @@ def rounded(a, dtype):
     return (t.half() if dtype == B.SQN_F16 else t.bfloat16()).float().numpy()
 
 
-@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("shape,variant", SHAPES, ids=["x".join(map(str, s)) for s, _ in SHAPES])
 @pytest.mark.parametrize("dtype", [B.SQN_BF16, B.SQN_F16], ids=["bf16", "f16"])
-def test_single_layers(shape, dtype):
+def test_single_layers(shape, variant, dtype):
     N, C, M, H, W, K, pad = shape
     rng = np.random.default_rng(sum(shape))
     x = rounded(rng.standard_normal((N, C, H, W)), dtype)
     w, b = synth.draw_conv_params(rng, C, M, K)
     w = rounded(w, dtype)
     for relu in (True, False):
-        check(G.gpu_conv(x, w, b, 1, pad, relu, dtype), x, w, b, pad, relu, dtype)
+        check(G.gpu_conv(x, w, b, 1, pad, relu, dtype, kernel="conv_mma_small, " + variant), x, w, b, pad, relu, dtype)
 
 
-@pytest.mark.parametrize("cin,s,e1,e3,h", [(512, 64, 256, 256, 13), (384, 48, 192, 192, 27), (64, 80, 32, 48, 6)])
+@pytest.mark.parametrize("cin,s,e1,e3,h,batch,variant", [
+    (512, 64, 256, 256, 13, 1, "8 warps, 3 slots"),
+    (512, 64, 256, 256, 13, 2, "8 warps, 2 slots"),         # 208 tiles of both expands
+    (512, 64, 256, 256, 13, 4, "4 warps, 3 slots"),         # 400
+    (512, 64, 256, 256, 13, 6, "4 warps, 2 slots"),         # 592
+    (384, 48, 192, 192, 27, 1, "4 warps, 3 slots"),
+    (64, 80, 32, 48, 6, 1, "8 warps, 3 slots")])
 @pytest.mark.parametrize("dtype", [B.SQN_BF16, B.SQN_F16], ids=["bf16", "f16"])
-def test_fire_layers(cin, s, e1, e3, h, dtype):
+def test_fire_layers(cin, s, e1, e3, h, batch, variant, dtype):
     rng = np.random.default_rng(cin + s)
-    x = rounded(np.abs(rng.standard_normal((1, cin, h, h + 2))), dtype)
+    x = rounded(np.abs(rng.standard_normal((batch, cin, h, h + 2))), dtype)
     sq, x1, x3 = ((rounded(w, dtype), b) for w, b in
                   (synth.draw_conv_params(rng, *a) for a in ((cin, s, 1), (s, e1, 1), (s, e3, 3))))
-    scratch = B.empty_device((1, h, h + 2, s), dtype)
-    out = B.empty_device((1, h, h + 2, e1 + e3), dtype)
+    scratch = B.empty_device((batch, h, h + 2, s), dtype)
+    out = B.empty_device((batch, h, h + 2, e1 + e3), dtype)
     out.fill_(float("nan"))
-    B.fire_forward(G.dev_act(x, dtype), G.dev_w(sq[0], dtype), G.dev_b(sq[1]), G.dev_w(x1[0], dtype), G.dev_b(x1[1]),
-                   G.dev_w(x3[0], dtype), G.dev_b(x3[1]), scratch, out, cin, s, e1, e3, h, h + 2, 1, dtype)
+    args = (G.dev_act(x, dtype), G.dev_w(sq[0], dtype), G.dev_b(sq[1]), G.dev_w(x1[0], dtype), G.dev_b(x1[1]), G.dev_w(x3[0], dtype),
+            G.dev_b(x3[1]), scratch, out, cin, s, e1, e3, h, h + 2, batch, dtype)
+    with G.traced() as names:
+        B.fire_forward(*args)
+    assert len(names) == 2 and names[0].startswith("conv_mma_small, ") and names[1] == "conv_mma_small x 2, " + variant, names
     assert B.sqn_check() == B.SQN_OK
     squeezed = G.host_act(scratch, dtype)
     check(squeezed, x, *sq, 0, True, dtype)
