@@ -13,6 +13,7 @@
 #include "f32_common.cuh"
 #include "smem_attr.h"
 #include "sqn_internal.h"
+#include "tc_host.h"
 
 namespace sqn {
 namespace {
@@ -260,7 +261,7 @@ SmallConfig config_of(const ConvDesc* d, int n)
     long long blocks = 0;
     for (int i = 0; i < n; ++i)
         blocks += (((long long)d[i].N * d[i].OH * d[i].OW + (c.narrow ? 63 : 31)) / (c.narrow ? 64 : 32)) * ((d[i].Cout + c.tn - 1) / c.tn);
-    if (blocks <= 74) c.rm = 4;
+    if (blocks <= sm_count() / 2) c.rm = 4;
     c.tm = (c.narrow ? 8 : 4) * c.rm;
     return c;
 }
@@ -268,10 +269,10 @@ SmallConfig config_of(const ConvDesc* d, int n)
 template <int TY, int RM, bool VEC>
 cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
 {
-    const int blocks = a.blocks + b.blocks;
+    const int blocks = a.blocks + b.blocks, sms = sm_count();
     const bool deep = a.chunks > 2 || (b.blocks && b.chunks > 2);       // (more than two warps have chunks)
-    if (deep && blocks <= 148) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
-    if (deep && blocks <= 296) return launch<TY, RM, 8, 2, VEC>(a, b, stream);
+    if (deep && blocks <= sms) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
+    if (deep && blocks <= 2 * sms) return launch<TY, RM, 8, 2, VEC>(a, b, stream);
     return launch<TY, RM, 4, 3, VEC>(a, b, stream);
 }
 
@@ -287,10 +288,11 @@ float f32_small_estimate(const ConvDesc& d)
     const SmallConfig c = config_of(&d, 1);
     const long long blocks = (((long long)d.N * d.OH * d.OW + c.tm - 1) / c.tm) * ((d.Cout + c.tn - 1) / c.tn);
     const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
-    const float rounds = (float)((blocks + 147) / 148);
+    const int sms = sm_count();
+    const float rounds = (float)((blocks + sms - 1) / sms);
     if (d.Cin % 4 != 0) return 2.7f + rounds * (chunks * (c.rm == 4 ? 450.f : c.narrow ? 900.f : 500.f) + 1650.f) / 1965.f;
     const float us = rounds * (chunks * (c.rm == 4 ? 150.f : c.narrow ? 375.f : 260.f) + 450.f) / 1965.f;
-    return 2.2f + (blocks > 296 ? 1.2f * us : us);
+    return 2.2f + (blocks > 2 * sms ? 1.2f * us : us);
 }
 
 int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)

@@ -14,6 +14,7 @@
 #include "smem_attr.h"
 #include "sqn_internal.h"
 #include "tc_common.cuh"
+#include "tc_host.h"
 
 namespace sqn {
 namespace {
@@ -211,12 +212,12 @@ cudaError_t launch(const MmaSmallParams& a, const MmaSmallParams& b, cudaStream_
 template <bool F16>
 cudaError_t launch_shape(const MmaSmallParams& a, const MmaSmallParams& b, cudaStream_t stream)
 {
-    const int chunks = b.blocks && b.chunks > a.chunks ? b.chunks : a.chunks, blocks = a.blocks + b.blocks;
+    const int chunks = b.blocks && b.chunks > a.chunks ? b.chunks : a.chunks, blocks = a.blocks + b.blocks, sms = sm_count();
     if (chunks == 1) return launch<F16, 1, 2>(a, b, stream);
     if (chunks == 2) return launch<F16, 2, 2>(a, b, stream);
-    if (chunks <= 4 || blocks > 444) return launch<F16, 4, 2>(a, b, stream);
-    if (blocks > 296) return launch<F16, 4, 3>(a, b, stream);
-    if (blocks > 148) return launch<F16, 8, 2>(a, b, stream);
+    if (chunks <= 4 || blocks > 3 * sms) return launch<F16, 4, 2>(a, b, stream);
+    if (blocks > 2 * sms) return launch<F16, 4, 3>(a, b, stream);
+    if (blocks > sms) return launch<F16, 8, 2>(a, b, stream);
     return launch<F16, 8, 3>(a, b, stream);
 }
 
