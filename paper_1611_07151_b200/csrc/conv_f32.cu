@@ -381,7 +381,7 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
         if (lat_us > us) us = lat_us;
         if (mem_us > us) us = mem_us;
         us += vec ? (d.S == 1 ? 2.f : 2.f + pairs) : 2.8f + 1.9f * pairs;
-        const float small_us = f32_small_estimate(d), other_us = small_us < us ? small_us : us;
+        const float small_us = f32_small_estimate(d, sms), other_us = small_us < us ? small_us : us;
         if (6.1f + 0.45f * (float)((Kdim + 31) / 32) < other_us) {      // (one tile of the tensor-core kernel: not worth a plan if above)
             const int rc = launch_conv_f32_tc(d, other_us, stream);
             if (rc != SQN_ERR_UNSUPPORTED) return rc;
@@ -411,7 +411,8 @@ int launch_conv_f32_pair(const ConvDesc& a, const ConvDesc& b, cudaStream_t stre
 {
     if (paired) *paired = false;
     int rc = SQN_ERR_UNSUPPORTED;
-    if (f32_small_estimate(a) < 14.f && f32_small_estimate(b) < 14.f) {
+    const int sms = sm_count();
+    if (f32_small_estimate(a, sms) < 14.f && f32_small_estimate(b, sms) < 14.f) {
         const ConvDesc two[2] = {b, a};             // the longer reduction's tiles first
         rc = launch_conv_f32_small(two, 2, stream);
         if (rc == SQN_OK && paired) *paired = true;

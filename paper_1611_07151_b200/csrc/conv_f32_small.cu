@@ -252,7 +252,7 @@ cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_
 //    wave (fire8's expand-3x3 at batch 1, 184 tiles: 14.1 -> 12.5 us), else four warps and three slots.
 struct SmallConfig { bool narrow; int rm, tm, tn; };
 
-SmallConfig config_of(const ConvDesc* d, int n)
+SmallConfig config_of(const ConvDesc* d, int n, int sms)
 {
     SmallConfig c;
     c.narrow = d[0].Cout <= 16 && (n == 1 || d[1].Cout <= 16);
@@ -261,15 +261,15 @@ SmallConfig config_of(const ConvDesc* d, int n)
     long long blocks = 0;
     for (int i = 0; i < n; ++i)
         blocks += (((long long)d[i].N * d[i].OH * d[i].OW + (c.narrow ? 63 : 31)) / (c.narrow ? 64 : 32)) * ((d[i].Cout + c.tn - 1) / c.tn);
-    if (blocks <= sm_count() / 2) c.rm = 4;
+    if (blocks <= sms / 2) c.rm = 4;
     c.tm = (c.narrow ? 8 : 4) * c.rm;
     return c;
 }
 
 template <int TY, int RM, bool VEC>
-cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
+cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, int sms, cudaStream_t stream)
 {
-    const int blocks = a.blocks + b.blocks, sms = sm_count();
+    const int blocks = a.blocks + b.blocks;
     const bool deep = a.chunks > 2 || (b.blocks && b.chunks > 2);       // (more than two warps have chunks)
     if (deep && blocks <= sms) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
     if (deep && blocks <= 2 * sms) return launch<TY, RM, 8, 2, VEC>(a, b, stream);
@@ -283,12 +283,11 @@ cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, cudaStre
 // 390; with 260 fire2's squeeze of 25 images came here for 16.9 us, FFMA 14.6).  Where the operands come in pieces of 4 bytes
 // 500 clocks (450 with the smaller tile, 900 with the narrow one) and more for a tile's start, fitted to 450 random layers (0.85
 // to 1.15 of it in eight of ten; 750 for all of them gave 0.46).
-float f32_small_estimate(const ConvDesc& d)
+float f32_small_estimate(const ConvDesc& d, int sms)
 {
-    const SmallConfig c = config_of(&d, 1);
+    const SmallConfig c = config_of(&d, 1, sms);
     const long long blocks = (((long long)d.N * d.OH * d.OW + c.tm - 1) / c.tm) * ((d.Cout + c.tn - 1) / c.tn);
     const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
-    const int sms = sm_count();
     const float rounds = (float)((blocks + sms - 1) / sms);
     if (d.Cin % 4 != 0) return 2.7f + rounds * (chunks * (c.rm == 4 ? 450.f : c.narrow ? 900.f : 500.f) + 1650.f) / 1965.f;
     const float us = rounds * (chunks * (c.rm == 4 ? 150.f : c.narrow ? 375.f : 260.f) + 450.f) / 1965.f;
@@ -297,7 +296,8 @@ float f32_small_estimate(const ConvDesc& d)
 
 int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
 {
-    const SmallConfig c = config_of(d, n);
+    const int sms = sm_count();
+    const SmallConfig c = config_of(d, n, sms);
     bool vec = true;
     F32SmallParams p[2];
     for (int i = 0; i < n; ++i) {
@@ -306,10 +306,10 @@ int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
     }
     if (n == 1) { p[1] = p[0]; p[1].blocks = 0; }
     cudaError_t rc;
-    if (c.rm == 8) rc = c.narrow ? (vec ? launch_ty<8, 8, true>(p[0], p[1], stream) : launch_ty<8, 8, false>(p[0], p[1], stream))
-                                 : (vec ? launch_ty<4, 8, true>(p[0], p[1], stream) : launch_ty<4, 8, false>(p[0], p[1], stream));
-    else rc = c.narrow ? (vec ? launch_ty<8, 4, true>(p[0], p[1], stream) : launch_ty<8, 4, false>(p[0], p[1], stream))
-                       : (vec ? launch_ty<4, 4, true>(p[0], p[1], stream) : launch_ty<4, 4, false>(p[0], p[1], stream));
+    if (c.rm == 8) rc = c.narrow ? (vec ? launch_ty<8, 8, true>(p[0], p[1], sms, stream) : launch_ty<8, 8, false>(p[0], p[1], sms, stream))
+                                 : (vec ? launch_ty<4, 8, true>(p[0], p[1], sms, stream) : launch_ty<4, 8, false>(p[0], p[1], sms, stream));
+    else rc = c.narrow ? (vec ? launch_ty<8, 4, true>(p[0], p[1], sms, stream) : launch_ty<8, 4, false>(p[0], p[1], sms, stream))
+                       : (vec ? launch_ty<4, 4, true>(p[0], p[1], sms, stream) : launch_ty<4, 4, false>(p[0], p[1], sms, stream));
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }

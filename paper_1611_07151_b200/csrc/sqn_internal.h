@@ -44,7 +44,7 @@ int launch_conv_f32_tc(const ConvDesc& d, float limit_us, cudaStream_t stream);
 // n (1 or 2) small layers in one launch, the reduction split over a CTA's warps (SQN_ERR_UNSUPPORTED: sizes beyond its
 // 32-bit offsets), and its time in microseconds.
 int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream);
-float f32_small_estimate(const ConvDesc& d);
+float f32_small_estimate(const ConvDesc& d, int sms);
 
 // bf16 path: tcgen05/TMEM implicit GEMM fed by TMA.
 // Returns SQN_ERR_UNSUPPORTED for shapes outside its family.
