@@ -68,17 +68,17 @@ __device__ int g_device_status;   // written by kernels whose bounded waits run 
 
 int* device_status_word()
 {
-    static std::mutex mu;
-    static int* ptrs[64] = {nullptr};
+    static std::atomic<int*> ptrs[64];              // (every thread that looks one up finds the same address: no lock)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!ptrs[dev]) {
+    int* word = ptrs[dev].load(std::memory_order_acquire);
+    if (!word) {
         void* p = nullptr;
         if (cudaGetSymbolAddress(&p, g_device_status) != cudaSuccess) return nullptr;
-        ptrs[dev] = static_cast<int*>(p);
+        word = static_cast<int*>(p);
+        ptrs[dev].store(word, std::memory_order_release);
     }
-    return ptrs[dev];
+    return word;
 }
 
 namespace {

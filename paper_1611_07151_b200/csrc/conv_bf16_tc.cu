@@ -1192,12 +1192,13 @@ struct Plan {
 
 int num_sms()
 {
-    static std::atomic<int> known[64];           // per device; 0: not asked yet
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-    if (dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
+    // Of the device that is asked for first: grid sizes and estimates go by it, no kernel's correctness does, and asking for the
+    // current device at every call is 0.06 us of a small layer's 6.8.
+    static std::atomic<int> known{0};
+    int n = known.load(std::memory_order_relaxed), dev = 0;
+    if (n > 0) return n;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+    known.store(n, std::memory_order_relaxed);
     return n;
 }
 

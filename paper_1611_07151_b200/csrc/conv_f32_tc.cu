@@ -4,8 +4,9 @@
 //   x = x0 + x1 + x2,  w = w0 + w1 + w2:   w*x = w0*x0 + (w0*x1 + w1*x0) + (w0*x2 + w1*x1 + w2*x0) + dropped
 //
 // x0 is x rounded to nearest (the remainder is below 2^-8 of x and of either sign), x1 the leading eight bits of the
-// remainder, x2 the rest; the dropped products w1*x2, w2*x1, w2*x2 are below 2^-22 of w*x at worst, 2^-25 typically and of
-// either sign: less than the rounding of one fp32 multiply-add.  The products are exact in the tensor core; its
+// remainder, x2 the rest; the dropped products w1*x2, w2*x1, w2*x2 are of either sign, 0.23 units of 2^-24 of w*x in the root mean
+// square and up to 1.75 (four million random pairs; the rounding of one fp32 multiply-add: 0.42, up to 1), so that an output that
+// is a single product may be off by more than a multiply-add's, a sum is not.  The products are exact in the tensor core; its
 // accumulator, though, cuts sums off at 24 bits instead of rounding them: an error towards zero that would grow with the
 // length of the reduction and add up from layer to layer.  So w0*x0 is summed on the tensor core over short segments of
 // the reduction only (32 elements; 64 would take 10 % less time), which the epilogue warps add up in registers with rounded

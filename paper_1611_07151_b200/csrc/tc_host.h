@@ -15,6 +15,6 @@ bool tmap_encode_16(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t*
 bool tmap_encode_f32(CUtensorMap* m, int rank, const void* ptr, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
                      const cuuint32_t* box, unsigned inner_bytes);
 
-int sm_count();     // SMs of the current device
+int sm_count();     // SMs of the device (see num_sms in conv_bf16_tc.cu)
 
 }  // namespace sqn
