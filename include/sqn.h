@@ -12,7 +12,13 @@
  *    (The paper, Section III-B/C, reorders data so that values of consecutive
  *    layers at one pixel are adjacent and has every layer write its output in
  *    that order; NHWC/OHWI is the same idea carried to all layers of a pixel.)
- *  - dtype SQN_F32: activations and kernels fp32, fp32 FFMA accumulation.
+ *  - dtype SQN_F32: activations and kernels fp32, sums in fp32.  Three kernels share the layers, by estimated time:
+ *    multiply-adds in sequence, multiply-adds split over warps, and the tensor cores with every operand as the exact
+ *    sum of three bf16 numbers (relative 2-norm error of a layer against 64-bit arithmetic 0.7e-7 to 2e-7, of
+ *    multiply-adds up to 1e-6).  They add in different orders: which one runs depends on the layer and the batch, so
+ *    the result for one image may differ in the last bits between batches.  No operand loses bits, whatever its
+ *    magnitude; layers with infinities, NaN, operands of 2^112 and more or sums of 2^96 and more take longer on the
+ *    tensor cores (their outputs are computed again with multiply-adds).
  *    dtype SQN_BF16: activations and kernels bf16, fp32 accumulation on the
  *    tensor cores, bias/ReLU/pooling arithmetic in fp32, outputs rounded to
  *    bf16 (round to nearest even).  Logits and probabilities are always fp32.
@@ -208,7 +214,8 @@ int avgpool_softmax_forward(const void* in, void* logits_f32, void* probs_f32, i
  *   computes conv1+pool1, fire4+pool4 and fire8+pool8 in fused kernels and never stores the maps of conv1, fire4
  *   and fire8: asking for one of those then returns SQN_ERR_UNSUPPORTED.  A bf16 net also runs the fire layers whose
  *   kernels fit in shared memory (fire2, fire3, fire5; fire4 too below a batch of 16) as one kernel each, without
- *   storing their squeeze maps, and takes conv10, its ReLU and the global average in one kernel without storing
+ *   storing their squeeze maps (at one image, where two launches may be faster, the map is refused as well),
+ *   and takes conv10, its ReLU and the global average in one kernel without storing
  *   conv10's map: "fireN_sq" of those layers and "conv10" then return SQN_ERR_UNSUPPORTED as well.  With
  *   SQN_FUSED_FIRE=0 and SQN_FUSED_HEAD=0 in the environment (read at every call) these layers run as separate
  *   launches and their maps can be read.

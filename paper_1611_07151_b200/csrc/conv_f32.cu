@@ -362,8 +362,8 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
         // longer than the best of the three on average, 30 % or more in four.  Measured, this kernel / the small layers' / the
         // tensor cores' -- batch 1: fire9's squeeze 19.6 / 4.7 / 18.0 us, fire6's expand-3x3 16.4 / 6.4 / 15.5, fire4's 14.5 /
         // 11.3 / 12.6, conv1 25.7 / 31 / 17.4; batch 16: fire4's expand-3x3 99 / 109 / 33, its expand-1x1 17.2 / 34 / 11.5,
-        // fire2's expand-1x1 6.9 / 15.6 / 10.0; batch 256: conv1 2687 / - / 1050, fire4's expand-3x3 1296 / - / 354, conv10
-        // 1256 / - / 281, fire2's squeeze 132 / - / 133, fire3's 141 / - / 164, fire2's expand-1x1 88 / - / 78.
+        // fire2's expand-1x1 6.9 / 15.6 / 10.0; batch 256: conv1 2687 / - / 1053, fire4's expand-3x3 1296 / - / 359, conv10
+        // 1256 / - / 290, fire2's squeeze 132 / - / 121, fire3's 141 / - / 154, fire2's expand-1x1 88 / - / 80.
         const double eff = bm == 128 ? (bn == 128 ? 1.0 : bn == 96 ? 0.95 : bn == 64 ? 0.85 : 0.75)
                          : bm == 256 ? (bn == 32 ? 0.85 : 0.6) : (bn == 128 ? 0.85 : bn == 64 ? 0.6 : 0.4);
         const double area = (double)((ctas_of(bm, bn) + sms - 1) / sms) * bm * bn / eff;

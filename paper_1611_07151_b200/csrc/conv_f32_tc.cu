@@ -31,8 +31,8 @@
 // does not stay in the schedulers' instruction caches, some six clocks per instruction and warp, so a unit costs what the
 // slowest role's instructions for it cost: the issuing warp 1300 clocks (its 12 MMAs: 830), the splitting groups 1000 to 1350,
 // the epilogue 1000; and once per tile 3200 to 4200 for bias, ReLU and stores, during which the two segment accumulators
-// cover two units.  Against the FFMA kernel, batch 256: conv1 996 us (2687), fire2's expand-3x3 229 (373), fire4's 354
-// (1296), fire6's 292 (675), fire8's 311 (1237), conv10 281 (1256), fire8's squeeze 109 (234), fire4's expand-1x1 89 (204).
+// cover two units.  Against the FFMA kernel, batch 256: conv1 1053 us (2687), fire2's expand-3x3 234 (373), fire4's 359
+// (1296), fire6's 299 (675), fire8's 316 (1237), conv10 290 (1256), fire8's squeeze 112 (234), fire4's expand-1x1 89 (204).
 // Warps (one persistent CTA per SM, all of its tiles in one column of output layers):
 //   0..7    two groups of four split pixels into bf16 planes, written as swizzled K-major operand tiles (FLAT, BOX: the
 //           groups take the chunks of 32 reduction elements in turn; PATCH: each takes half of the patch's rows)
