@@ -266,14 +266,16 @@ __device__ __noinline__ float redo_output(const F32TcParams& p, int m, int n, fl
     int ih0 = 0, col0 = 0;                              // first row of the window, its first column in elements
     if (m >= 0) {
         const int img = fast_div(m, p.div_ohw), r = m - img * p.OHW, oh = fast_div(r, p.div_ow);
-        ih0 = oh * p.S - p.pad; col0 = ((r - oh * p.OW) * p.S - p.pad) * p.Cin;
+        const int iw0 = (r - oh * p.OW) * p.S - p.pad;
+        ih0 = oh * p.S - p.pad;
+        col0 = (iw0 < -p.K ? -p.K : iw0 < p.W ? iw0 : p.W) * p.Cin;        // (outside the map all the same: padding may be any number)
         x += (size_t)img * p.H * map_row;
         float xs = 0.f;
         for (int kh = 0; kh < p.K; ++kh) {
             if ((unsigned)(ih0 + kh) >= (unsigned)p.H) continue;
             const float* row = x + (size_t)(ih0 + kh) * map_row;
 #pragma unroll 4
-            for (int f = col0 + lane; f < col0 + row_len; f += 32) xs += (unsigned)f < (unsigned)map_row ? fabsf(__ldg(row + f)) : 0.f;
+            for (int f = lane; f < row_len; f += 32) xs += (unsigned)col0 + (unsigned)f < (unsigned)map_row ? fabsf(__ldg(row + col0 + f)) : 0.f;
         }
         __syncwarp();
         xs = warp_sum(xs);
@@ -295,7 +297,7 @@ __device__ __noinline__ float redo_output(const F32TcParams& p, int m, int n, fl
             const float* row = x + (size_t)(in ? ih0 + kh : 0) * map_row + col0;
 #pragma unroll 2
             for (int f = lane; f < row_len; f += 32) {
-                const float q = in && (unsigned)(col0 + f) < (unsigned)map_row ? __ldg(row + f) : 0.f;
+                const float q = in && (unsigned)col0 + (unsigned)f < (unsigned)map_row ? __ldg(row + f) : 0.f;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float v = __ldg(w + (size_t)l[i] * p.Kdim + f);
