@@ -372,7 +372,8 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
         float us, lat_us;
         if (vec) {
             us = (float)(area * (double)Kdim / (128.0 * 1965.0 * 0.6));
-            lat_us = 0.035f * (float)Kdim;
+            // (256 x 16, by fire2's and fire3's squeezes: one CTA on an SM 10.5 us at K = 96, every two 14.5, at K = 128 18.6)
+            lat_us = bn == 16 ? (ctas_of(bm, bn) <= sms ? 0.088f : 0.13f * pairs) * (float)Kdim : 0.035f * (float)Kdim;
         } else {
             const float slow = Kdim > TBL_MAX ? 1.65f : 1.f;        // (two divisions per element)
             us = slow * (float)(area * (double)Kdim / (128.0 * 1965.0 * (bm == 256 ? 0.24 : 0.4)));

@@ -8,6 +8,7 @@
 // in a fixed order.  Operand rows are stored as they lie in memory (reduction index contiguous, 80-byte pitch): a thread
 // takes four reduction elements of its 8 pixels and 4 layers with twelve 16-byte reads, free of bank conflicts, for 128
 // multiply-adds.  Two layers that read the same input (the expands of a fire layer) go out as one grid.
+#include <cmath>
 #include <cstring>
 
 #include "f32_common.cuh"
@@ -279,10 +280,11 @@ cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, int sms,
 }  // namespace
 
 // Microseconds: a launch, then the busiest SM's tiles at 260 clocks per chunk (150 with the smaller tile), fitted to SqueezeNet's
-// layers at batch 1 and 4, and 375 with the narrow one (42 random layers of up to 16 output layers: 257 to 414, fire2's squeezes
-// 390; with 260 fire2's squeeze of 25 images came here for 16.9 us, FFMA 14.6).  Where the operands come in pieces of 4 bytes
-// 500 clocks (450 with the smaller tile, 900 with the narrow one) and more for a tile's start, fitted to 450 random layers (0.85
-// to 1.15 of it in eight of ten; 750 for all of them gave 0.46).
+// layers at batch 1 and 4.  With the narrow tile 300 clocks per chunk, and where warps take several, as if every warp had as many
+// as the one with the most: fire2's squeeze, 6 chunks for 4 warps, 12.9 us at 19 images, 16.5 at 25, 40 at 71 (FFMA 14.5, 14.5, 37),
+// fire3's, 8 chunks, 14.3 at 19, 67 at 116 (FFMA 18.6, 76).  Where the operands come in pieces of 4 bytes 500 clocks (450 with the
+// smaller tile, 900 with the narrow one) and more for a tile's start, fitted to 450 random layers (0.85 to 1.15 of it in eight
+// of ten; 750 for all of them gave 0.46).
 float f32_small_estimate(const ConvDesc& d, int sms)
 {
     const SmallConfig c = config_of(&d, 1, sms);
@@ -290,7 +292,9 @@ float f32_small_estimate(const ConvDesc& d, int sms)
     const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
     const float rounds = (float)((blocks + sms - 1) / sms);
     if (d.Cin % 4 != 0) return 2.7f + rounds * (chunks * (c.rm == 4 ? 450.f : c.narrow ? 900.f : 500.f) + 1650.f) / 1965.f;
-    const float us = rounds * (chunks * (c.rm == 4 ? 150.f : c.narrow ? 375.f : 260.f) + 450.f) / 1965.f;
+    const float warps = blocks > 2 * sms ? 4.f : 8.f;           // (see launch_ty)
+    const float narrow = 300.f * (chunks > warps ? warps * ceilf(chunks / warps) : chunks);
+    const float us = rounds * ((c.rm == 4 ? 150.f * chunks : c.narrow ? narrow : 260.f * chunks) + 450.f) / 1965.f;
     return 2.2f + (blocks > 2 * sms ? 1.2f * us : us);
 }
 

@@ -21,6 +21,9 @@ CASES = [
     ((50, 285, 17, 61, 56, 3, 3, 0), "conv_f32_small",),                    # 577 / 199 / 661
     ((25, 96, 16, 55, 55, 1, 1, 0), "conv_f32 "),                          # 18 / 17 / 15
     ((71, 96, 16, 55, 55, 1, 1, 0), "conv_f32 "),                          # 44 / 42 / 37
+    ((8, 96, 16, 55, 55, 1, 1, 0), "conv_f32_small"),                      # - / 8.4 / 10.5
+    ((19, 128, 16, 55, 55, 1, 1, 0), "conv_f32_small"),                    # - / 14 / 19
+    ((116, 128, 16, 55, 55, 1, 1, 0), "conv_f32_small"),                   # - / 67 / 76
     ((16, 64, 128, 56, 56, 3, 2, 1), "conv_f32_tc",),                       # 38 / - / 65
     ((64, 3, 96, 227, 227, 7, 2, 0), "conv_f32_tc",),                       # 265 / - / 690
 ]

@@ -24,7 +24,7 @@ SHAPES = [
     ((9, 9, 40, 41, 3, 1, 1), "128x48"),
     ((6, 12, 28, 59, 1, 1, 0), "256x32 vec"),
     ((28, 3, 19, 40, 1, 1, 0), "256x32"),
-    ((9, 20, 7, 55, 3, 1, 1), "256x16 vec"),
+    ((71, 96, 16, 55, 1, 1, 0), "256x16 vec"),
     ((16, 3, 13, 26, 1, 1, 0), "256x16"),
     ((1, 4, 12800, 7, 1, 1, 0), "64x128 vec"),
     ((1, 3, 12800, 7, 1, 1, 0), "64x128"),
