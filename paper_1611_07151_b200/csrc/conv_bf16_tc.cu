@@ -75,6 +75,7 @@ struct TcParams {
     int Cout;
     int taps, taps_w, pad;           // kernel taps, taps per kernel row, zero padding
     int chunks, BKc;                 // reduction chunks per tap, elements per chunk (16/32/64)
+    int ksteps_last;                 // MMAs (16 reduction elements each) of a tap's last chunk, BKc / 16 for the others
     int k_per_tap;                   // reduction elements per tap in the kernel matrix
     int patch;                       // 1: one input patch per tile serves every tap (see below)
     int taps_h;                      // kernel rows
@@ -438,22 +439,23 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
                 if (++s == p.stages) { s = 0; ph ^= 1u; }
             } else {
                 uint32_t bres16 = smB16;
+                int ch = 0;
                 for (int i = 0; i < items; ++i, bres16 += b_tile16) {
+                    const int ks = ++ch == p.chunks ? p.ksteps_last : ksteps;
+                    if (ch == p.chunks) ch = 0;
                     ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->full[s]), ph, abort_flag, p.status));
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t a16 = smA16 + (uint32_t)s * a_tile16;
                     const uint32_t b16 = p.b_resident ? bres16 : smB16 + (uint32_t)s * b_tile16;
                     if (elect_one()) {
-                        // ksteps MMAs of K = 16 (32 bytes = 2 address units along the row)
+                        // ks MMAs of K = 16 (32 bytes = 2 address units along the row)
                         const uint64_t da = ((uint64_t)hiA << 32) | (uint64_t)(a16 | 0x10000u);
                         const uint64_t db = ((uint64_t)hiB << 32) | (uint64_t)(b16 | 0x10000u);
                         mma_bf16_ss(d_tmem, da, db, idesc, i > 0 ? 1u : 0u);
-                        if (ksteps >= 2) mma_bf16_ss(d_tmem, da + 2, db + 2, idesc, 1u);
-                        if (ksteps == 4) {
-                            mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
-                            mma_bf16_ss(d_tmem, da + 6, db + 6, idesc, 1u);
-                        }
+                        if (ks >= 2) mma_bf16_ss(d_tmem, da + 2, db + 2, idesc, 1u);
+                        if (ks >= 3) mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
+                        if (ks == 4) mma_bf16_ss(d_tmem, da + 6, db + 6, idesc, 1u);
                         mma_commit(smem_u32(&sh->empty[s]));        // slot free once these MMAs have read it
                         if (i == items - 1) {
                             mma_bf16_ss(d_tmem, bias_da, bias_db, idesc, 1u);
@@ -1340,7 +1342,8 @@ int build_plan_cfg(const ConvDesc& d, bool stem, const void* a_ptr, const void* 
         p.chunks = d.Cin / p.BKc;
         p.k_per_tap = d.Cin;
     }
-    const unsigned row_bytes = (unsigned)p.BKc * 2u;
+    unsigned row_bytes = (unsigned)p.BKc * 2u;
+    p.ksteps_last = p.BKc / 16;
 
     auto set_width = [&](int bn) {              // output layers per tile
         p.BN = bn;
@@ -1412,6 +1415,16 @@ int build_plan_cfg(const ConvDesc& d, bool stem, const void* a_ptr, const void* 
         if (stem || p.pool) return SQN_ERR_UNSUPPORTED;
         p.patch = 0;
         p.h_mul = 1;
+        if (d.Cin % 64 != 0 && d.Cin > 32) {
+            // Without a patch every chunk is a ring slot with its barriers and boxes, some 250 clocks of the issuing thread
+            // whatever it holds: 64 layers to a chunk, and only the MMAs that the last chunk has layers for (TMA fills what lies
+            // past the last layer; the same MMAs in the same order).  240 -> 128 3x3 at 19 x 18, four images: 34.4 -> 12.8 us; 112 -> 96 5x5 at 40 x 30, 16 images: 86 -> 32.
+            p.BKc = 64;
+            p.chunks = (d.Cin + 63) / 64;
+            p.ksteps_last = (d.Cin % 64) / 16;
+            row_bytes = 128u;
+            set_width(p.BN);
+        }
         if (flat) { p.BW = OW < TILE_M ? OW : TILE_M; p.BH = 1; p.BI = 1; }
         else choose_box(OW, OH, NI, &p.BW, &p.BH, &p.BI);
         p.a_bytes = (unsigned)(p.BW * p.BH * p.BI) * row_bytes;
