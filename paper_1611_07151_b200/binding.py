@@ -1,4 +1,4 @@
-"""ctypes binding of libsqn.so (declared in include/sqn.h).
+"""ctypes binding of libsqn.so (declared in include/sqn.h), with the two calls made once per layer marshalled in C.
 
 Argument marshalling only: every function here has the name and argument order
 of the C entry point it calls; tensors are passed as device addresses and
@@ -74,6 +74,11 @@ SIGNATURES = {
 }
 
 _lib = None
+try:
+    from . import _native               # the marshalling of conv_forward_ex and fire_forward in C (csrc/binding_native.c)
+except ImportError:                     # (not built, or for another Python: ctypes marshals all calls)
+    _native = None
+_conv_forward_ex_at = _fire_forward_at = None       # addresses of the library's functions
 
 
 class SqnError(RuntimeError):
@@ -85,7 +90,7 @@ class SqnError(RuntimeError):
 
 def lib():
     """Load libsqn.so (once).  Raises if it has not been built: there is no other path."""
-    global _lib
+    global _lib, _conv_forward_ex_at, _fire_forward_at
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError("libsqn.so is missing (%s): build it with "
@@ -95,6 +100,8 @@ def lib():
             fn = getattr(l, name)
             fn.restype = res
             fn.argtypes = args
+        _conv_forward_ex_at = ctypes.cast(l.conv_forward_ex, _c_vp).value
+        _fire_forward_at = ctypes.cast(l.fire_forward, _c_vp).value
         _lib = l
     return _lib
 
@@ -142,8 +149,17 @@ def conv_forward(inp, weights, bias, out, numInputLayers, numOutputLayers, H, W,
 def conv_forward_ex(inp, weights, bias, out, numInputLayers, numOutputLayers, H, W, K, S, pad, batch, dtype=SQN_F32,
                     relu=True, out_c_offset=0, out_c_total=0, stream=None, workspace=None, workspace_bytes=0,
                     fuse_maxpool=False, fuse_global_avgpool=False):
-    opts = sqn_conv_opts(dtype, 1 if relu else 0, out_c_offset, out_c_total,
-                         current_stream() if stream is None else stream, _p(workspace), workspace_bytes,
+    if stream is None:
+        stream = current_stream()
+    if _native is not None:
+        if _lib is None:
+            lib()
+        rc = _native.conv_forward_ex(_conv_forward_ex_at, inp, weights, bias, out, numInputLayers, numOutputLayers, H, W, K, S, pad,
+                                     batch, dtype, relu, out_c_offset, out_c_total, stream, workspace, workspace_bytes,
+                                     fuse_maxpool, fuse_global_avgpool)
+        if rc is not None:
+            return _check(rc, "conv_forward_ex")
+    opts = sqn_conv_opts(dtype, 1 if relu else 0, out_c_offset, out_c_total, stream, _p(workspace), workspace_bytes,
                          1 if fuse_maxpool else 0, 1 if fuse_global_avgpool else 0)
     _check(lib().conv_forward_ex(_p(inp), _p(weights), _p(bias), _p(out), numInputLayers, numOutputLayers, H, W, K, S,
                                  pad, batch, ctypes.byref(opts)), "conv_forward_ex")
@@ -158,9 +174,17 @@ def conv_workspace_bytes(numInputLayers, numOutputLayers, H, W, K, S, pad, batch
 
 def fire_forward(inp, w_sq, b_sq, w_e1, b_e1, w_e3, b_e3, squeeze_scratch, out, Cin, s, e1, e3, H, W, batch, dtype,
                  stream=None):
+    if stream is None:
+        stream = current_stream()
+    if _native is not None:
+        if _lib is None:
+            lib()
+        rc = _native.fire_forward(_fire_forward_at, inp, w_sq, b_sq, w_e1, b_e1, w_e3, b_e3, squeeze_scratch, out, Cin, s, e1, e3, H,
+                                  W, batch, dtype, stream)
+        if rc is not None:
+            return _check(rc, "fire_forward")
     _check(lib().fire_forward(_p(inp), _p(w_sq), _p(b_sq), _p(w_e1), _p(b_e1), _p(w_e3), _p(b_e3),
-                              _p(squeeze_scratch), _p(out), Cin, s, e1, e3, H, W, batch, dtype,
-                              current_stream() if stream is None else stream), "fire_forward")
+                              _p(squeeze_scratch), _p(out), Cin, s, e1, e3, H, W, batch, dtype, stream), "fire_forward")
 
 
 def fire_forward_static(inp, w_sq, b_sq, w_e1, b_e1, w_e3, b_e3, out, Cin, s, e1, e3, H, W, batch, dtype, stream=None):

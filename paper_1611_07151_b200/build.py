@@ -6,6 +6,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -13,6 +14,9 @@ CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libsqn.so")
 LIB_DEBUG = os.path.join(PKG, "libsqn_debug.so")      # the same sources with -DSQN_DEBUG: index checks in the kernels
 OBJ_DIR = os.path.join(PKG, "_build")
+
+NATIVE_SRC = os.path.join(CSRC, "binding_native.c")
+NATIVE = os.path.join(PKG, "_native.so")              # the binding's marshalling (see binding.py)
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -34,9 +38,21 @@ def up_to_date(lib=LIB):
     return all(os.path.getmtime(f) <= t for f in _deps())
 
 
+def build_native(force=False):
+    """Compile the binding's marshalling module (plain C against Python.h)."""
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= os.path.getmtime(NATIVE_SRC):
+        return NATIVE
+    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(ROOT, "include"), NATIVE_SRC, "-o", tmp], check=True)
+    os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 def build(force=False, verbose=False, debug=False):
     """Compile every .cu under csrc/ and link them into libsqn.so (debug=True: libsqn_debug.so, with -DSQN_DEBUG)."""
     lib = LIB_DEBUG if debug else LIB
+    build_native(force)
     if not force and up_to_date(lib):
         return lib
     nvcc = os.environ.get("NVCC", "nvcc")
