@@ -13,7 +13,7 @@
 // fp32 additions, and what a segment loses on average is added back (FT_CUT); the other five products are 2^-8 smaller and
 // stay in an accumulator of their own for the whole tile.  Relative 2-norm error of a layer against 64-bit arithmetic: 0.7e-7
 // to 2e-7 (multiply-adds in sequence: 2e-7 to 1e-6); of SqueezeNet's logits at batch 160: 1.05e-7 (1.13e-7).
-// Operands are scaled by 2^16 before the split (FT_SCALE), so that it is exact for every number below 2^112.
+// Operands are scaled by 2^16 before the split (SPLIT_SCALE; SqueezeNet in fp32, 256 images: 5458 us without it, 5478 with), so that it is exact for every number below 2^112.
 // Outputs that are not finite, or too large for the scaled sums, are computed again with fp32 multiply-adds.
 //
 // GEMM view: D[layer][pixel] = sum_k W[layer][k] * X[pixel][k].  The kernels are the M = 128 operand and sit in TMEM, the
@@ -68,11 +68,6 @@ constexpr int FT_MAX_RA = 4, FT_MAX_SA = 4, FT_MAX_SB = 3;
 // both signs, up to 4e-8 on sums of one sign); added back with the corrections.  Less than half a unit in the last place of
 // any sum, so a sum that was exact stays as it is.
 constexpr float FT_CUT = 1.6e-8f;
-// Operands are multiplied by this before they are split: the last bit of the smallest fp32 number, 2^-149, is then bf16's
-// smallest subnormal number, 2^-133, so that all three parts of any number are exact (without it a number of 1e-36 kept 14 bits,
-// one of 1e-40 one).  Sums carry its square.  What overflows by it (operands from 2^112, sums from 2^96) is not finite and
-// computed again.  SqueezeNet in fp32, 256 images: 5458 us without it, 5478 with; kernels by copies of 4 bytes up to 10 %.
-constexpr float FT_SCALE = 0x1p16f, FT_UNSCALE = 0x1p-32f;
 constexpr int FT_KSLOTS = 2;                // kernel slots in TMEM, one per kernel group
 constexpr unsigned FT_COL_GX = 256, FT_COL_W = 384, FT_W_COLS = 48;     // TMEM: two segment accumulators, corrections, kernel slots
 constexpr int FT_TBL_MAX = 2048;            // BOX: reduction elements per block of layers
@@ -103,7 +98,7 @@ struct F32TcParams {
     int chunks, ksteps_last;    // pixel chunks of a tile, MMA k-steps of the last one
     int seg;                    // (chunk, tap) units whose w0*x0 products are summed on the tensor core before they are added in registers
     int kres;                   // 1: at most FT_KSLOTS units: the kernels stay in TMEM
-    int tstore;                 // FLAT where vec_store holds and Cout is a multiple of 4: pixels per TMA store of the epilogue (0: no TMA)
+    int tstore;                 // FLAT and BOX where vec_store holds and Cout is a multiple of 4: pixels per TMA store of the epilogue (0: no TMA)
     int vec_store;              // 1: output rows and this layer's slice are 16-byte aligned
     int early;                  // 1: kernels and bias may be read before the wait for the grid ahead
     int ra, sa, sb;             // slots: split pixels, pixel boxes, kernel boxes
@@ -139,34 +134,20 @@ struct F32TcShared {
     volatile int abort_flag;
 };
 
+// The same question as mbar_try_wait's, answered at once
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
-
-// Two fp32 differences (the bits of all operands), one instruction
-__device__ __forceinline__ void sub2(uint32_t ax, uint32_t ay, uint32_t bx, uint32_t by, uint32_t& dx, uint32_t& dy)
-{
-    asm("{\n\t.reg .b64 a, b;\n\t"
-        "mov.b64 a, {%2, %3};\n\t"
-        "mov.b64 b, {%4, %5};\n\t"
-        "sub.rn.f32x2 a, a, b;\n\t"
-        "mov.b64 {%0, %1}, a;\n\t}"
-        : "=r"(dx), "=r"(dy) : "r"(ax), "r"(ay), "r"(bx), "r"(by));
-}
-// Two values as three packed bf16 pairs whose sums are FT_SCALE times the values (see the head of the file).
-__device__ __forceinline__ void split_pair(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l)
-{
-    asm("{\n\t.reg .b64 a, b;\n\t"
-        "mov.b64 a, {%0, %1};\n\t"
-        "mov.b64 b, {%2, %2};\n\t"
-        "mul.rn.f32x2 a, a, b;\n\t"
-        "mov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(x), "+f"(y) : "f"(FT_SCALE));
-    h = pack_x2(x, y, 0);
-    uint32_t rx, ry, sx, sy;
-    sub2(__float_as_uint(x), __float_as_uint(y), h << 16, h & 0xffff0000u, rx, ry);         // at most 16 significant bits
-    m = __byte_perm(rx, ry, 0x7632);
-    sub2(rx, ry, rx & 0xffff0000u, ry & 0xffff0000u, sx, sy);                               // at most 8
-    l = __byte_perm(sx, sy, 0x7632);
-}
 
 // Four consecutive reduction elements -> the three planes (plane pitch in bytes), at address a of the first
 __device__ __forceinline__ void store_split(uint32_t a, uint32_t pitch, float4 v)
@@ -351,7 +332,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
         fence_mbar_init();
         if (p.sa) prefetch_tensormap(&tmX);
         if (p.wsrc == FT_W_BOXES) prefetch_tensormap(&tmW);
-        if (MODE == FT_FLAT && p.tstore) prefetch_tensormap(&tmO);
+        if (MODE != FT_PATCH && p.tstore) prefetch_tensormap(&tmO);
     }
     if (warp == FT_W_MMA) {
         tmem_alloc(smem_u32(&sh->tmem_base), 512);
@@ -655,7 +636,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
         const int wl = n_live - quad * 32 < 32 ? n_live - quad * 32 : 32;       // output layers of this warp
         const bool vec = p.vec_store && wl % 4 == 0;
         float* out_w = p.out + p.out_c_offset + nw;
-        const uint32_t stg0 = base + p.off_epi + (uint32_t)(quad * 2 + half) * (MODE == FT_FLAT && p.tstore ? (uint32_t)p.tstore * 128u : 2048u);
+        const uint32_t stg0 = base + p.off_epi + (uint32_t)(quad * 2 + half) * (MODE != FT_PATCH && p.tstore ? (uint32_t)p.tstore * 128u : 2048u);
         if (!p.early) chain_wait();
         const float bias = lane < wl ? __ldg(p.bias + nw + lane) : 0.f;
         const float least = p.relu ? 0.f : bias != bias ? bias : -INFINITY;     // (fmaxf drops a NaN that only one operand has)
@@ -728,8 +709,9 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             }
             if (!ok) break;
             // bias and ReLU here, where a thread has one layer and 64 independent pixels, then 16 pixels at a time through a
-            // staging tile (a pixel's 32 layers are a row) and in 16-byte pieces, eight lanes per pixel, to memory; FLAT, whose
-            // pixels are consecutive: 32 or 64 pixels, then a TMA store.  Only two warps per 32 layers have rows to store, so
+            // staging tile (a pixel's 32 layers are a row) and in 16-byte pieces, eight lanes per pixel, to memory; FLAT and BOX, whose
+            // pixels are consecutive or boxes of the map: 32 or 64 pixels, then a TMA store, which leaves out what lies outside the map
+            // (BOX: conv1 at batch 256 1021 -> 975 us).  Only two warps per 32 layers have rows to store, so
             // the length of this chain is a tile's time where the reduction is short (fire2's 1x1 expand at batch 256 with
             // bias and ReLU after the staging tile and no TMA 107 us, so 80; a bulk copy per pixel instead of the 16-byte
             // pieces: fire2's expand-3x3 310 us instead of 230, conv1 1358 instead of 1011)
@@ -737,21 +719,27 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 16) {
                 // (TMA: a staging tile of 32 or 64 pixels, free again when the store before has read it)
-                const uint32_t stg = stg0 + (MODE == FT_FLAT && p.tstore ? (uint32_t)(c0 & (p.tstore - 1)) * 128u : 0u);
-                if (MODE == FT_FLAT && lane == 0 && p.tstore && (c0 & (p.tstore - 1)) == 0) tma_store_wait_read();
+                const uint32_t stg = stg0 + (MODE != FT_PATCH && p.tstore ? (uint32_t)(c0 & (p.tstore - 1)) * 128u : 0u);
+                if (MODE != FT_PATCH && lane == 0 && p.tstore && (c0 & (p.tstore - 1)) == 0) tma_store_wait_read();
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     nan = fmaf(acc[c0 + j], 0.f, nan);
-                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(stg + (uint32_t)(128 * j + 4 * lane)), "f"(fmaxf(fmaf(acc[c0 + j], FT_UNSCALE, bias), least)) : "memory");
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(stg + (uint32_t)(128 * j + 4 * lane)), "f"(fmaxf(fmaf(acc[c0 + j], SPLIT_UNSCALE, bias), least)) : "memory");
                 }
-                if (MODE == FT_FLAT && p.tstore) {
+                if (MODE != FT_PATCH && p.tstore) {
                     if (((c0 + 16) & (p.tstore - 1)) == 0) {
                         fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) {
-                            const int m = (mt0 + t * p.m_step) * FT_N + half * 64 + c0 + 16 - p.tstore;
-                            if (m < p.M) tma_store_2d(&tmO, stg0, nw, m);
+                            const int c = half * 64 + c0 + 16 - p.tstore, tile = mt0 + t * p.m_step;
+                            if (MODE == FT_FLAT) {
+                                if (tile * FT_N + c < p.M) tma_store_2d(&tmO, stg0, nw, tile * FT_N + c);
+                            } else {
+                                const int tt = fast_div(tile, p.div_tw), tx = tile - tt * p.tiles_w, img = fast_div(tt, p.div_th), ty = tt - img * p.tiles_h;
+                                const int y = ty * p.bh + (c >> p.bw_shift), x = (tx << p.bw_shift) + (c & ((1 << p.bw_shift) - 1));
+                                if (y < p.OH && x < p.OW) tma_store_4d(&tmO, stg0, nw, x, y, img);
+                            }
                             tma_store_commit();
                         }
                     }
@@ -761,7 +749,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                 }
             }
             if (__any_sync(0xffffffffu, lane < wl && nan != 0.f)) {      // something was not finite: this warp's outputs with fp32 multiply-adds
-                if (MODE == FT_FLAT && p.tstore && lane == 0) tma_store_wait_all();
+                if (MODE != FT_PATCH && p.tstore && lane == 0) tma_store_wait_all();
                 __syncwarp();
                 float ws = 0.f;
                 for (int c = -1; c < 64; ++c) {
@@ -773,7 +761,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                 }
             }
         }
-        if (MODE == FT_FLAT && p.tstore && lane == 0) tma_store_wait_all();
+        if (MODE != FT_PATCH && p.tstore && lane == 0) tma_store_wait_all();
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");       // (of 28 x 32 x 72 registers: 104 for the epilogue, 64 for the groups that split)
         if (warp == FT_W_MMA) {
@@ -791,6 +779,73 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             bool ok = true;
             uint32_t s = 0, ks = 0, b = 0, g = 0;
             uint32_t ph = 0, kph = 0, bph = 1, gph = 1;
+            if (MODE == FT_BOX && units > 2) {
+                // The last three MMAs of a unit go out behind a look at the next unit's barriers, so that the tensor pipe has work
+                // meanwhile (it holds some four MMAs): conv1 at batch 256 1056 -> 1021 us.  (Not so with a patch: fire4's expand-3x3 368
+                // -> 392; with one or two units to a tile fire4's expand-1x1 90 -> 94, 8 -> 323 2x2/2 13.5 -> 13.9; flat reductions of
+                // more units gain 3 %, less than those lose.)
+                const int total = my_tiles * units;
+                int u = 0, in_seg = 0;
+                bool ready = false;
+                for (int i = 0; i < total; ++i) {
+                    if (!ready) {
+                        ok = wait_bar(a_full + 8u * s, ph, abort_flag, p.status);
+                        ok = ok && (in_seg != 0 || wait_bar(seg_empty + 8u * b, bph, abort_flag, p.status));
+                        ok = __all_sync(0xffffffffu, ok && wait_bar(k_full + 8u * ks, kph, abort_flag, p.status));
+                        if (!ok) break;
+                    }
+                    tc_fence_after();
+                    const uint32_t g0 = tmem_base + b * FT_N, w = tmem_base + FT_COL_W + ks * FT_W_COLS;
+                    const uint64_t d0 = desc((base + s * p.slot_a) >> 4);       // the first plane; the others PX and 2 * PX further
+                    const bool two = u != units - 1 || p.ksteps_last == 2;
+                    if (elect_one()) {
+                        mma_bf16_ts(g0, w, d0, idesc, in_seg ? 1u : 0u);
+                        if (two) mma_bf16_ts(g0, w + 8u, d0 + 2u, idesc, 1u);
+                    }
+                    __syncwarp();
+                    if (u == 0) {                           // the corrections of the tile before have to be read first
+                        ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->gx_empty), gph, abort_flag, p.status));
+                        gph ^= 1u;
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    if (elect_one()) {
+                        mma_bf16_ts(gx, w, d0 + PX, idesc, u ? 1u : 0u);            // w0 x1
+                        mma_bf16_ts(gx, w, d0 + 2u * PX, idesc, 1u);                // w0 x2
+                        if (two) {
+                            mma_bf16_ts(gx, w + 16u, d0, idesc, 1u);                // w1 x0
+                            mma_bf16_ts(gx, w + 16u, d0 + PX, idesc, 1u);           // w1 x1
+                            mma_bf16_ts(gx, w + 32u, d0, idesc, 1u);                // w2 x0
+                            mma_bf16_ts(gx, w + 8u, d0 + PX + 2u, idesc, 1u);
+                            mma_bf16_ts(gx, w + 8u, d0 + 2u * PX + 2u, idesc, 1u);
+                        }
+                    }
+                    __syncwarp();
+                    const uint32_t wl = two ? w + 8u : w;
+                    const uint64_t dl = two ? d0 + 2u : d0;
+                    ks ^= 1u; kph ^= ks ^ 1u;
+                    if (u == units - 1 || in_seg == seg - 1) {
+                        in_seg = 0;
+                        b ^= 1u; bph ^= b ^ 1u;
+                    } else ++in_seg;
+                    if (++u == units) u = 0;
+                    if (++s == (uint32_t)p.ra) { s = 0; ph ^= 1u; }
+                    ready = false;
+                    if (i + 1 < total) {
+                        ready = mbar_test_wait(a_full + 8u * s, ph);
+                        ready &= in_seg != 0 || mbar_test_wait(seg_empty + 8u * b, bph);
+                        ready &= mbar_test_wait(k_full + 8u * ks, kph);
+                        ready = __all_sync(0xffffffffu, ready);
+                    }
+                    if (elect_one()) {
+                        mma_bf16_ts(gx, wl + 16u, dl, idesc, 1u);
+                        mma_bf16_ts(gx, wl + 16u, dl + PX, idesc, 1u);
+                        mma_bf16_ts(gx, wl + 32u, dl, idesc, 1u);
+                        mma_commit(done + 8u * ((uint32_t)i & 3u));
+                    }
+                    __syncwarp();
+                }
+            } else
             for (int t = 0; t < my_tiles && ok; ++t) {
                 int in_seg = 0, u = 0;
                 for (int ch = 0; ch < p.chunks && ok; ++ch) {
@@ -1045,7 +1100,7 @@ int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
         found = finish(d.Cin, positions);
     }
     if (!found) {
-        p.tstore = 0;
+        p.tstore = p.vec_store && d.Cout % 4 == 0 ? 32 : 0;
         p.mode = FT_BOX;
         p.prow = FT_N;
         p.taps = 1;
@@ -1104,9 +1159,18 @@ int encode_f32_maps(const ConvDesc& d, F32TcPlan* plan)
     }
     if (p.tstore) {
         // this layer's slice of the output
-        const cuuint64_t dims[2] = {(cuuint64_t)d.Cout, (cuuint64_t)p.M}, str[1] = {(cuuint64_t)d.out_c_total * 4};
-        const cuuint32_t box[2] = {32, (cuuint32_t)p.tstore};
-        if (!tmap_encode_f32(&plan->o, 2, p.out + p.out_c_offset, dims, str, box, 0)) return SQN_ERR_CUDA;
+        const cuuint64_t s1 = (cuuint64_t)d.out_c_total * 4;
+        if (p.mode == FT_FLAT) {
+            const cuuint64_t dims[2] = {(cuuint64_t)d.Cout, (cuuint64_t)p.M}, str[1] = {s1};
+            const cuuint32_t box[2] = {32, (cuuint32_t)p.tstore};
+            if (!tmap_encode_f32(&plan->o, 2, p.out + p.out_c_offset, dims, str, box, 0)) return SQN_ERR_CUDA;
+        } else {
+            const cuuint64_t dims[4] = {(cuuint64_t)d.Cout, (cuuint64_t)d.OW, (cuuint64_t)d.OH, (cuuint64_t)d.N};
+            const cuuint64_t str[3] = {s1, s1 * d.OW, s1 * d.OW * d.OH};
+            const cuuint32_t bw = 1u << p.bw_shift, w = bw < (cuuint32_t)p.tstore ? bw : (cuuint32_t)p.tstore;
+            const cuuint32_t box[4] = {32, w, (cuuint32_t)p.tstore / w, 1};
+            if (!tmap_encode_f32(&plan->o, 4, p.out + p.out_c_offset, dims, str, box, 0)) return SQN_ERR_CUDA;
+        }
     }
     if (p.wsrc == FT_W_BOXES) {
         const cuuint64_t dims[2] = {(cuuint64_t)p.Kdim, (cuuint64_t)d.Cout}, str[1] = {(cuuint64_t)p.Kdim * 4};
