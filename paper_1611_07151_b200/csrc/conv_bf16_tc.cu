@@ -222,8 +222,8 @@ __device__ __forceinline__ void fill_bias_rows(const TcParams& p, unsigned char*
 }
 
 // HC: output layers per epilogue piece (8, 16 or 32; a store chunk CW is two pieces), fixed at compile time so
-// that the conversion loop is straight-line code.
-template <int SPLIT, int HC, bool F16>
+// that the conversion loop is straight-line code.  TURN: the two groups of epilogue warps take chunks in turn (see there).
+template <int SPLIT, int HC, bool F16, bool TURN>
 __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO,
                                              const TcParams& p, const int bid)
 {
@@ -263,7 +263,7 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
             mbar_init(smem_u32(&sh->tmem_empty[a]), EPI_WARPS);
         }
         for (int b = 0; b < p.nstg; ++b) {
-            mbar_init(smem_u32(&sh->stg_full[b]), EPI_WARPS);
+            mbar_init(smem_u32(&sh->stg_full[b]), TURN ? 4 : EPI_WARPS);
             mbar_init(smem_u32(&sh->stg_free[b]), 1);
         }
         sh->abort_flag = 0;
@@ -472,13 +472,17 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
     } else if (warp < 2 + EPI_WARPS) {
         // -------------------------------------------------------------------- epilogue
         // 4*SPLIT warps: warp w reads TMEM lane quadrant w % 4 (one output pixel per thread) and, of
-        // every chunk of CW layers, the piece(s) given by (w - 2) / 4.  TMEM -> registers (bias already added by the last MMA), ReLU, -> bf16,
+        // every chunk of CW layers, the piece(s) given by (w - 2) / 4; TURN: every second chunk, all of it.  A chunk is a chain of
+        // latencies of some 1000 clocks whatever its width, so that tiles of three chunks and more gain by two of them at a time:
+        // 64 -> 256 1x1 at 56 x 56, 64 images, 23.8 -> 22.6 us, 48 -> 192 at 27 x 27, 37 images, 6.5 -> 6.0, 256 -> 1024 at 14 x 14,
+        // 125 images, 22.8 -> 22.3; with one or two chunks it loses 1 to 2 % (384 -> 64 at 27 x 27: 6.8 -> 6.9).  TMEM -> registers (bias already added by the last MMA), ReLU, -> bf16,
         // into a slot of the staging ring (TMA-swizzled rows); the store warp sends the slot to
         // global memory while the next chunk is converted.
         const int q = warp & 3;
         constexpr int PIECES = SPLIT < 2 ? 2 : SPLIT;  // a chunk is converted in this many pieces
-        constexpr int NH = PIECES / SPLIT;             // pieces each thread converts per chunk (2 when SPLIT == 1)
-        const int half0 = ((warp - 2) >> 2) * NH;      // first piece of this warp
+        constexpr int NH = TURN ? PIECES : PIECES / SPLIT;     // pieces each thread converts per chunk (2 when SPLIT == 1)
+        const int half0 = TURN ? 0 : ((warp - 2) >> 2) * NH;   // first piece of this warp
+        int turn = (warp - 2) >> 2;                    // TURN: chunks until this warp's next one
         const int row = q * 32 + lane;
         const uint32_t cw_bytes = (uint32_t)p.CW * 2u;
         const uint32_t slot_bytes = (uint32_t)TILE_M * cw_bytes;
@@ -499,6 +503,14 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
             for (int chunk = 0; chunk < nchunks; ++chunk) {
                 const int c0 = chunk * p.CW;
                 if (n0 + c0 >= p.Cout) break;
+                if (TURN) {
+                    const bool mine = turn == 0;
+                    turn ^= 1;
+                    if (!mine) {
+                        if (++sb == p.nstg) { sb = 0; sph ^= 1u; }
+                        continue;
+                    }
+                }
                 uint32_t v[NH][32];
 #pragma unroll
                 for (int h = 0; h < NH; ++h) {
@@ -596,14 +608,14 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
 // One layer per launch, or two independent layers that read the same input (the two expands of a fire layer):
 // the first p0.grid CTAs work on the first, the others on the second, so the second fills the tail of the first
 // and the pair costs one launch.
-template <int SPLIT, int HC>
+template <int SPLIT, int HC, bool TURN>
 __global__ void __launch_bounds__(threads_for(SPLIT), SPLIT == 1 ? 2 : 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmO, const __grid_constant__ TcParams p)
 {
     // (the 16-bit type is a compile-time constant of the body: the epilogue's conversion loop is straight-line code)
-    if (p.f16) conv_tc_body<SPLIT, HC, true>(tmA, tmB, tmO, p, (int)blockIdx.x);
-    else conv_tc_body<SPLIT, HC, false>(tmA, tmB, tmO, p, (int)blockIdx.x);
+    if (p.f16) conv_tc_body<SPLIT, HC, true, TURN>(tmA, tmB, tmO, p, (int)blockIdx.x);
+    else conv_tc_body<SPLIT, HC, false, TURN>(tmA, tmB, tmO, p, (int)blockIdx.x);
 }
 
 template <int SPLIT, int HC>
@@ -614,11 +626,11 @@ conv_tc_kernel2(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
                 const __grid_constant__ CUtensorMap tmO1, const __grid_constant__ TcParams p1)
 {
     if (p0.f16) {
-        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, true>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
-        else conv_tc_body<SPLIT, HC, true>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
+        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, true, false>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
+        else conv_tc_body<SPLIT, HC, true, false>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
     } else {
-        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, false>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
-        else conv_tc_body<SPLIT, HC, false>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
+        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, false, false>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
+        else conv_tc_body<SPLIT, HC, false, false>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
     }
 }
 
@@ -1597,13 +1609,13 @@ int build_plan(const ConvDesc& d, bool stem, const void* a_ptr, const void* w_pt
     return build_plan_cfg(d, stem, a_ptr, w_ptr, Hp, Wp, 2, plan);
 }
 
-template <int SPLIT, int HC>
+template <int SPLIT, int HC, bool TURN>
 cudaError_t launch_variant(const Plan& plan, cudaStream_t stream)
 {
     static SmemAttr attr;
-    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel<SPLIT, HC>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
+    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel<SPLIT, HC, TURN>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
     if (arc != cudaSuccess) return arc;
-    return launch_chained(conv_tc_kernel<SPLIT, HC>, dim3((unsigned)plan.grid), dim3(threads_for(SPLIT)), plan.smem,
+    return launch_chained(conv_tc_kernel<SPLIT, HC, TURN>, dim3((unsigned)plan.grid), dim3(threads_for(SPLIT)), plan.smem,
                           stream, plan.a, plan.b, plan.o, plan.p);
 }
 
@@ -1619,11 +1631,14 @@ int launch_plan(const Plan& plan, cudaStream_t stream)
                                 plan.p);
     }
     else if (plan.split == 1)
-        rc = hc == 32 ? launch_variant<1, 32>(plan, stream)
-           : hc == 16 ? launch_variant<1, 16>(plan, stream) : launch_variant<1, 8>(plan, stream);
+        rc = hc == 32 ? launch_variant<1, 32, false>(plan, stream)
+           : hc == 16 ? launch_variant<1, 16, false>(plan, stream) : launch_variant<1, 8, false>(plan, stream);
+    else if (plan.p.BN >= 3 * plan.p.CW)
+        rc = hc == 32 ? launch_variant<2, 32, true>(plan, stream)
+           : hc == 16 ? launch_variant<2, 16, true>(plan, stream) : launch_variant<2, 8, true>(plan, stream);
     else
-        rc = hc == 32 ? launch_variant<2, 32>(plan, stream)
-           : hc == 16 ? launch_variant<2, 16>(plan, stream) : launch_variant<2, 8>(plan, stream);
+        rc = hc == 32 ? launch_variant<2, 32, false>(plan, stream)
+           : hc == 16 ? launch_variant<2, 16, false>(plan, stream) : launch_variant<2, 8, false>(plan, stream);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
     note_launch(plan.p.pool ? "conv_pool, %d pixels" : "conv_tc, %d layers", plan.p.pool ? plan.p.npix : plan.p.BN);
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
