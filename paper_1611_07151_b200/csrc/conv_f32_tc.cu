@@ -589,6 +589,10 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
                     src = boxes + (uint32_t)sl * (128u * 128u) + (uint32_t)row * 128u;
                     sl ^= 1;
                 } else {
+                    // An odd number of slots: the box before in this slot, unit u - sb's, was the other group's.  It has to be here first (its
+                    // unit's MMAs are done), or this unit's, whose phase has the parity of the one before that, would look as if it
+                    // were: where unit 1's box came later than unit 2's and unit 0's MMAs, unit 4 took its slot and gave it back twice.
+                    if ((p.sb & 1) && !wait_done(u - p.sb)) break;
                     if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&sh->sb_full[st]), sph, abort_flag, p.status))) break;
                     src = base + p.off_sb + (uint32_t)st * (128u * 128u) + (uint32_t)row * 128u;
                 }
