@@ -641,13 +641,12 @@ extern "C" int squeezenet_forward(sqn_net* net, const void* in_nhwc, void* logit
     } else {
         rc = make_conv_desc(in_nhwc, net->w[0], net->b[0], buf(net->i_conv1), 3, 96, IMG, IMG, 7, 2, 0, batch, 1, 0, 0, &d);
         if (rc != SQN_OK) return rc;
-        rc = SQN_ERR_UNSUPPORTED;
-        if (is16(dt)) {                         // one image: convolution and pool in one launch
+        {                                       // one image: convolution and pool in one launch
             ConvDesc sd = d;
             sd.params_static = 1;
             sd.f16 = f16;
             sd.stem_prepacked = net->stem_prepacked;
-            rc = launch_stem_small(sd, buf(net->i_pool1), st);
+            rc = is16(dt) ? launch_stem_small(sd, buf(net->i_pool1), st) : launch_stem_small_f32(sd, buf(net->i_pool1), st);
         }
         if (rc == SQN_OK) mark("conv1+pool1");
         else if (rc != SQN_ERR_UNSUPPORTED) return rc;

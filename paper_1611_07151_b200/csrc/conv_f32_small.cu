@@ -7,13 +7,15 @@
 // chunks asynchronously into a ring of its own, waits for nobody else, and the warps' partial sums are added once at the end,
 // in a fixed order.  Operand rows are stored as they lie in memory (reduction index contiguous, 80-byte pitch): a thread
 // takes four reduction elements of its 8 pixels and 4 layers with twelve 16-byte reads, free of bank conflicts, for 128
-// multiply-adds.  Two layers that read the same input (the expands of a fire layer) go out as one grid.
+// multiply-adds.  Layers with 16-byte pieces and tiles of 32 layers or more do the same on the matrix instructions (further down).  Two layers that read the same input (the expands of a fire layer) go out as one grid.
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "f32_common.cuh"
 #include "smem_attr.h"
 #include "sqn_internal.h"
+#include "tc_common.cuh"
 #include "tc_host.h"
 
 namespace sqn {
@@ -202,6 +204,208 @@ __device__ __forceinline__ void conv_f32_small_body(const F32SmallParams& p, con
     }
 }
 
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_shared_f1(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+// The same layer on the warp-level matrix instructions at fp32 precision: every operand as three bf16 numbers (split_pair), six
+// of the nine products (see conv_f32_tc.cu), w0*x0 of 16 reduction elements at a time, added up in registers with rounded
+// additions.  Tiles of 16*MF pixels x 8*NF layers; chunks of 16 reduction elements lie in shared memory as in global memory,
+// rows of 64 bytes.  The order of a chunk's elements in the MMA's reduction is free: lane t of four takes elements 4t .. 4t+3 of
+// its rows with one 16-byte read, free of bank conflicts.  A chunk of a 32 x 32 tile is 48 MMAs of 8 clocks per scheduler against 512
+// multiply-adds of 1.45 and six times the reads; what bounds it is the chain of a chunk (read, split, products) in every warp.
+// Multiply-adds against this kernel, one image: fire8's expand-3x3 12.5 -> 10.8 us, fire9's 6.9 -> 5.3, fire8's squeeze 5.4 -> 3.9,
+// conv10 11.5 -> 9.8; 256 -> 256 3x3 at 14 x 14, 3 images: 42.2 -> 35.0.  Error against 64 bits 0.7e-7 to 1.3e-7 (0.9e-7 to 4.0e-7).
+// A tile with a sum that is not finite is computed again with multiply-adds.
+template <int MF, int NF, int SL, int ST>
+__device__ __forceinline__ void conv_f32_small_tc_body(const F32SmallParams& p, const int bid)
+{
+    constexpr int TM = 16 * MF, TN = 8 * NF, SLOT = (TM + TN) * SK * 4;      // (bytes of a ring slot)
+    extern __shared__ __align__(16) float sm_small[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int mt = bid / p.n_tiles, n0 = (bid - mt * p.n_tiles) * TN, m0 = mt * TM;
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(sm_small) + (uint32_t)(warp * ST * SLOT);
+
+    // this lane's copies: piece q (4 reduction elements) of rows r0 + 8 * j
+    const int q = lane & 3, r0 = lane >> 2;
+    __shared__ int4 rows[TM];                   // {offset, first row, first column} of every pixel's window
+    if (tid < TM) {
+        const int m = m0 + tid;
+        int4 v = make_int4(0, -(1 << 30), 0, 0);
+        if (m < p.M) {
+            const int img = fast_div(m, p.div_ohw), r = m - img * p.OHW;
+            const int oh = fast_div(r, p.div_ow), ow = r - oh * p.OW;
+            v.y = oh * p.S - p.pad; v.z = ow * p.S - p.pad;
+            v.x = ((img * p.H + v.y) * p.W + v.z) * p.Cin;
+        }
+        rows[tid] = v;
+    }
+    __syncthreads();
+    const uint32_t my_piece = (uint32_t)(16 * lane);
+    auto load_w = [&](int ch, int slot) {
+        const uint32_t dst = ring + (uint32_t)(slot * SLOT + TM * SK * 4) + my_piece;
+        const int k = ch * SK + 4 * q;
+#pragma unroll
+        for (int j = 0; j < NF; ++j) {
+            const bool ok = k < p.Kdim && n0 + r0 + 8 * j < p.Cout;
+            cp_async_16(dst + (uint32_t)(512 * j), ok ? p.w + (size_t)(n0 + r0 + 8 * j) * p.Kdim + k : p.w, ok);
+        }
+    };
+    auto load_x = [&](int ch, int slot) {
+        const uint32_t dst = ring + (uint32_t)(slot * SLOT) + my_piece;
+        const int k = ch * SK + 4 * q;
+        const int t = fast_div(k, p.div_cin), c = k - t * p.Cin, kh = fast_div(t, p.div_k), kw = t - kh * p.K;
+        const int off = (kh * p.W + kw) * p.Cin + c;
+#pragma unroll
+        for (int j = 0; j < 2 * MF; ++j) {
+            const int4 v = rows[r0 + 8 * j];
+            const bool ok = k < p.Kdim && (unsigned)(v.y + kh) < (unsigned)p.H && (unsigned)(v.z + kw) < (unsigned)p.W;
+            cp_async_16(dst + (uint32_t)(512 * j), ok ? p.in + (v.x + off) : p.in, ok);
+        }
+    };
+    const int mine = p.chunks > warp ? (p.chunks - warp + SL - 1) / SL : 0;
+    const int g = lane >> 2, t4 = lane & 3;
+    const uint32_t xr = ring + (uint32_t)(g * 64 + t4 * 16), wr = xr + (uint32_t)(TM * 64);
+    constexpr int RP = TN + 4;
+    static_assert(TM * RP * 4 <= ST * SLOT, "the partial sums fit the ring");
+    // the first chunks' kernels may be fetched before the grid ahead has finished (a net's own parameters)
+    if (!p.early) chain_wait();
+    for (bool exact = false;; exact = true) {
+#pragma unroll
+        for (int i = 0; i < ST - 1; ++i)
+            if (i < mine) load_w(warp + SL * i, i);
+        if (p.early && !exact) chain_wait();
+#pragma unroll
+        for (int i = 0; i < ST - 1; ++i) {
+            if (i < mine) load_x(warp + SL * i, i);
+            cp_async_commit();
+        }
+        float acc[NF][MF][4];
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+#pragma unroll
+            for (int e = 0; e < MF; ++e)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[f][e][i] = 0.f;
+        for (int i = 0, slot = 0; i < mine; ++i) {
+            cp_async_wait<ST - 2>();
+            __syncwarp();               // chunk i is here for every lane, and every lane has done with chunk i - 1's slot
+            {
+                const int nx = i + ST - 1, ns = slot == 0 ? ST - 1 : slot - 1;
+                if (nx < mine) { load_w(warp + SL * nx, ns); load_x(warp + SL * nx, ns); }
+                cp_async_commit();
+            }
+            const uint32_t xs = xr + (uint32_t)(slot * SLOT), ws = wr + (uint32_t)(slot * SLOT);
+            if (!exact) {
+                uint32_t xh[MF][4], xm[MF][4], xl[MF][4];
+#pragma unroll
+                for (int e = 0; e < MF; ++e)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {           // rows g and g + 8
+                        const float4 v = ld_shared_f4(xs + (uint32_t)((16 * e + 8 * h) * 64));
+                        split_pair(v.x, v.y, xh[e][h], xm[e][h], xl[e][h]);
+                        split_pair(v.z, v.w, xh[e][2 + h], xm[e][2 + h], xl[e][2 + h]);
+                    }
+                auto layers = [&](auto count, int f0) {     // tiles of 8 layers f0 ..
+                    constexpr int F = decltype(count)::value;
+                    uint32_t wh[F][2], wm[F][2], wl[F][2];
+#pragma unroll
+                    for (int f = 0; f < F; ++f) {
+                        const float4 v = ld_shared_f4(ws + (uint32_t)(8 * (f0 + f) * 64));
+                        split_pair(v.x, v.y, wh[f][0], wm[f][0], wl[f][0]);
+                        split_pair(v.z, v.w, wh[f][1], wm[f][1], wl[f][1]);
+                    }
+                    mma_split(&acc[f0], xh, xm, xl, wh, wm, wl);
+                };
+#pragma unroll
+                for (int f = 0; f + 2 <= NF; f += 2) layers(std::integral_constant<int, 2>(), f);
+                if (NF % 2) layers(std::integral_constant<int, 1>(), NF - 1);
+            } else {
+                const uint32_t x0 = xs - (uint32_t)(t4 * 16), w0 = ws - (uint32_t)(t4 * 16 + g * 64) + (uint32_t)(2 * t4 * 64);
+#pragma unroll 1
+                for (int k = 0; k < SK; ++k) {
+                    float w[NF][2];
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) { w[f][0] = ld_shared_f1(w0 + 4u * k + (uint32_t)(8 * f * 64)); w[f][1] = ld_shared_f1(w0 + 4u * k + (uint32_t)(8 * f * 64 + 64)); }
+#pragma unroll
+                    for (int e = 0; e < MF; ++e) {
+                        const float xa = ld_shared_f1(x0 + 4u * k + (uint32_t)(16 * e * 64)), xb = ld_shared_f1(x0 + 4u * k + (uint32_t)((16 * e + 8) * 64));
+#pragma unroll
+                        for (int f = 0; f < NF; ++f) {
+                            acc[f][e][0] = fmaf(xa, w[f][0], acc[f][e][0]); acc[f][e][1] = fmaf(xa, w[f][1], acc[f][e][1]);
+                            acc[f][e][2] = fmaf(xb, w[f][0], acc[f][e][2]); acc[f][e][3] = fmaf(xb, w[f][1], acc[f][e][3]);
+                        }
+                    }
+                }
+            }
+            if (++slot == ST) slot = 0;
+        }
+        cp_async_wait<0>();
+        __syncwarp();
+        // partial sums into the warp's own ring, then all warps' sums in order
+        float* part = sm_small + warp * (ST * SLOT / 4);
+#pragma unroll
+        for (int e = 0; e < MF; ++e)
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+                float* d = part + (16 * e + g) * RP + 8 * f + 2 * t4;
+                *reinterpret_cast<float2*>(d) = make_float2(acc[f][e][0], acc[f][e][1]);
+                *reinterpret_cast<float2*>(d + 8 * RP) = make_float2(acc[f][e][2], acc[f][e][3]);
+            }
+        __syncthreads();
+        const float unscale = exact ? 1.f : SPLIT_UNSCALE;
+        bool finite = true;
+#pragma unroll
+        for (int i0 = 0; i0 < TM * TN / 4; i0 += 32 * SL) {
+            const int i = tid + i0;
+            if (i >= TM * TN / 4) break;
+            const int r = i / (TN / 4), l4 = 4 * (i % (TN / 4));
+            const int m = m0 + r, n = n0 + l4;
+            if (m >= p.M || n >= p.Cout) continue;
+            float4 v = *reinterpret_cast<const float4*>(sm_small + r * RP + l4);
+#pragma unroll
+            for (int s = 1; s < SL; ++s) {
+                const float4 u = *reinterpret_cast<const float4*>(sm_small + s * (ST * SLOT / 4) + r * RP + l4);
+                v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+            }
+            finite = finite && fabsf(v.x) < INFINITY && fabsf(v.y) < INFINITY && fabsf(v.z) < INFINITY && fabsf(v.w) < INFINITY;
+            const float* bias = p.bias + n;
+            v.x = fmaf(v.x, unscale, __ldg(bias));
+            if (n + 1 < p.Cout) v.y = fmaf(v.y, unscale, __ldg(bias + 1));
+            if (n + 2 < p.Cout) v.z = fmaf(v.z, unscale, __ldg(bias + 2));
+            if (n + 3 < p.Cout) v.w = fmaf(v.w, unscale, __ldg(bias + 3));
+            if (p.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+            if (!sqn_dbg_ok(m >= 0 && p.out_c_offset + n < p.out_c_total, p.status)) continue;
+            float* dst = p.out + (size_t)m * p.out_c_total + p.out_c_offset + n;
+            if (p.vec_store && n + 4 <= p.Cout) *reinterpret_cast<float4*>(dst) = v;
+            else {
+                dst[0] = v.x;
+                if (n + 1 < p.Cout) dst[1] = v.y;
+                if (n + 2 < p.Cout) dst[2] = v.z;
+                if (n + 3 < p.Cout) dst[3] = v.w;
+            }
+        }
+        if (exact || !__syncthreads_or(!finite)) break;     // (the rings are free again)
+    }
+}
+
+template <int MF, int NF, int SL, int ST>
+__global__ void __launch_bounds__(32 * SL, 16 / SL)
+conv_f32_small_tc_kernel(const __grid_constant__ F32SmallParams p0, const __grid_constant__ F32SmallParams p1)
+{
+    chain_release();
+    if ((int)blockIdx.x < p0.blocks) conv_f32_small_tc_body<MF, NF, SL, ST>(p0, (int)blockIdx.x);
+    else conv_f32_small_tc_body<MF, NF, SL, ST>(p1, (int)blockIdx.x - p0.blocks);
+}
+
 template <int TY, int RM, int SL, int ST, bool VEC>
 __global__ void __launch_bounds__(32 * SL, 16 / SL)
 conv_f32_small_kernel(const __grid_constant__ F32SmallParams p0, const __grid_constant__ F32SmallParams p1)
@@ -233,6 +437,20 @@ bool fill(const ConvDesc& d, int tm, int tn, F32SmallParams* p)
     return true;
 }
 
+// 16-byte pieces: on the matrix instructions
+template <int MF, int NF, int SL, int ST>
+cudaError_t launch_tc(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
+{
+    constexpr size_t smem = (size_t)SL * ST * (16 * MF + 8 * NF) * SK * 4;
+    static SmemAttr attr;
+    const cudaError_t arc = attr.allow((const void*)conv_f32_small_tc_kernel<MF, NF, SL, ST>, smem);
+    if (arc != cudaSuccess) return arc;
+    const cudaError_t rc =
+        launch_chained(conv_f32_small_tc_kernel<MF, NF, SL, ST>, dim3((unsigned)(a.blocks + b.blocks)), dim3(32 * SL), smem, stream, a, b);
+    if (rc == cudaSuccess) note_launch("conv_f32_small%s %dx%d vec, %d warps, %d slots, products", b.blocks ? " x 2" : "", 16 * MF, 8 * NF, SL, ST);
+    return rc;
+}
+
 template <int TY, int RM, int SL, int ST, bool VEC>
 cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
 {
@@ -246,14 +464,25 @@ cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_
     return rc;
 }
 
+// Tiles of 32 layers with 16-byte pieces go to the matrix instructions, see launch_ty.
+template <int TY, int RM, int SL, int ST, bool VEC>
+cudaError_t launch_any(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
+{
+    if constexpr (VEC && TY == 4) return launch_tc<TY * RM / 16, 16 / TY, SL, ST>(a, b, stream);
+    else return launch<TY, RM, SL, ST, VEC>(a, b, stream);
+}
+
 // Tile, warps and ring for a layer (or two) of so many tiles; measured on SqueezeNet's layers at batch 1 and 4:
 //  - half as many pixels per thread where the larger tiles would leave half of the SMs without a CTA (fire9's squeeze 6.9 ->
 //    4.7 us, fire5's 4.2 -> 3.2);
 //  - eight warps and three slots per warp where every SM gets one CTA at most, two slots where two CTAs per SM make it one
 //    wave (fire8's expand-3x3 at batch 1, 184 tiles: 14.1 -> 12.5 us), else four warps and three slots.
+//  - a single layer with 16-byte pieces and more tiles than SMs: tiles of 40 or 48 layers where they compute an eighth less than those
+//    of 32 and are two waves of CTAs at most (20 -> 36 5x5/2, nine images of 61 x 47, half of the 32-layer tiles' work for nothing:
+//    18.1 -> 13.1 us).
 struct SmallConfig { bool narrow; int rm, tm, tn; };
 
-SmallConfig config_of(const ConvDesc* d, int n, int sms)
+SmallConfig config_of(const ConvDesc* d, int n, int sms, bool wide)
 {
     SmallConfig c;
     c.narrow = d[0].Cout <= 16 && (n == 1 || d[1].Cout <= 16);
@@ -263,6 +492,11 @@ SmallConfig config_of(const ConvDesc* d, int n, int sms)
     for (int i = 0; i < n; ++i)
         blocks += (((long long)d[i].N * d[i].OH * d[i].OW + (c.narrow ? 63 : 31)) / (c.narrow ? 64 : 32)) * ((d[i].Cout + c.tn - 1) / c.tn);
     if (blocks <= sms / 2) c.rm = 4;
+    else if (wide && blocks > sms && !c.narrow && n == 1 && d[0].Cin % 4 == 0)
+        for (int tn = 40; tn <= 48; tn += 8) {
+            const int cols = (d[0].Cout + tn - 1) / tn;
+            if (cols * tn * 8LL <= (d[0].Cout + c.tn - 1) / c.tn * c.tn * 7LL && blocks / ((d[0].Cout + 31) / 32) * cols <= 2 * sms) c.tn = tn;
+        }
     c.tm = (c.narrow ? 8 : 4) * c.rm;
     return c;
 }
@@ -272,9 +506,21 @@ cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, int sms,
 {
     const int blocks = a.blocks + b.blocks;
     const bool deep = a.chunks > 2 || (b.blocks && b.chunks > 2);       // (more than two warps have chunks)
-    if (deep && blocks <= sms) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
-    if (deep && blocks <= 2 * sms) return launch<TY, RM, 8, 2, VEC>(a, b, stream);
+    if constexpr (VEC && TY == 4 && RM == 8)
+        // One CTA of eight warps per SM: a chunk on the matrix instructions is a longer chain for a warp (split, products, sums) than its
+        // multiply-adds, and two warps to a scheduler do not cover it; so only where a warp has two chunks at most (128 -> 32 1x1
+        // at 55 x 55: 3.8 -> 3.4 us; 48 -> 192 3x3 at 27 x 27, 27 chunks: 6.2 and 7.8; 1024 -> 256 1x1, 64 chunks: 12.4 and 14.9).
+        if (deep && blocks <= sms && (a.chunks > 16 || (b.blocks && b.chunks > 16))) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
+    if (deep && blocks <= sms) return launch_any<TY, RM, 8, 3, VEC>(a, b, stream);
+    if (deep && blocks <= 2 * sms) return launch_any<TY, RM, 8, 2, VEC>(a, b, stream);
+    // (CTAs of four warps: multiply-adds, fire4's expand-3x3 at one image 10.5 us and 10.9, 12 -> 100 3x3/2 at 40 x 40 6.5 and 6.8)
     return launch<TY, RM, 4, 3, VEC>(a, b, stream);
+}
+
+template <int NF>
+cudaError_t launch_wide(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
+{
+    return launch_tc<2, NF, 8, 2>(a, b, stream);
 }
 
 }  // namespace
@@ -287,7 +533,7 @@ cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, int sms,
 // of ten; 750 for all of them gave 0.46).
 float f32_small_estimate(const ConvDesc& d, int sms)
 {
-    const SmallConfig c = config_of(&d, 1, sms);
+    const SmallConfig c = config_of(&d, 1, sms, false);
     const long long blocks = (((long long)d.N * d.OH * d.OW + c.tm - 1) / c.tm) * ((d.Cout + c.tn - 1) / c.tn);
     const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
     const float rounds = (float)((blocks + sms - 1) / sms);
@@ -301,7 +547,7 @@ float f32_small_estimate(const ConvDesc& d, int sms)
 int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
 {
     const int sms = sm_count();
-    const SmallConfig c = config_of(d, n, sms);
+    const SmallConfig c = config_of(d, n, sms, true);
     bool vec = true;
     F32SmallParams p[2];
     for (int i = 0; i < n; ++i) {
@@ -310,7 +556,8 @@ int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
     }
     if (n == 1) { p[1] = p[0]; p[1].blocks = 0; }
     cudaError_t rc;
-    if (c.rm == 8) rc = c.narrow ? (vec ? launch_ty<8, 8, true>(p[0], p[1], sms, stream) : launch_ty<8, 8, false>(p[0], p[1], sms, stream))
+    if (c.tn > 32) rc = c.tn == 40 ? launch_wide<5>(p[0], p[1], stream) : launch_wide<6>(p[0], p[1], stream);
+    else if (c.rm == 8) rc = c.narrow ? (vec ? launch_ty<8, 8, true>(p[0], p[1], sms, stream) : launch_ty<8, 8, false>(p[0], p[1], sms, stream))
                                  : (vec ? launch_ty<4, 8, true>(p[0], p[1], sms, stream) : launch_ty<4, 8, false>(p[0], p[1], sms, stream));
     else rc = c.narrow ? (vec ? launch_ty<8, 4, true>(p[0], p[1], sms, stream) : launch_ty<8, 4, false>(p[0], p[1], sms, stream))
                        : (vec ? launch_ty<4, 4, true>(p[0], p[1], sms, stream) : launch_ty<4, 4, false>(p[0], p[1], sms, stream));

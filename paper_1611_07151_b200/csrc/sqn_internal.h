@@ -70,6 +70,7 @@ int launch_stem_conv_bf16(const ConvDesc& d, void* workspace, size_t workspace_b
 int launch_stem_conv_bf16_prepacked(const ConvDesc& d, cudaStream_t stream);
 // The stem and its max-pool for few images, one launch that stores both maps (see stem_small.cu).
 int launch_stem_small(const ConvDesc& d, void* pool, cudaStream_t stream);
+int launch_stem_small_f32(const ConvDesc& d, void* pool, cudaStream_t stream);       // (the same in fp32: stem_small_f32.cu)
 inline int stem_packed_rows(int H) { return (H + 1) / 2 * 2; }
 inline int stem_packed_cols(int W) { return (W + 2) / 2 * 2; }
 

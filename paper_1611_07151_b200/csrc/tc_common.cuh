@@ -113,4 +113,67 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
                      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// c += a * b for bf16 operands; free to be moved among other instructions (FIRST: c = a * b)
+template <bool FIRST>
+__device__ __forceinline__ void mma_bf16_free(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
+{
+    if (FIRST)
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+            : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.f));
+    else
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+            : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+// Of what the matrix instructions cut off a sum of 16 products on average (1.1e-8 of it, kernels of one sign 1.6e-8), added back with the
+// corrections: an error of one sign adds up from layer to layer.  Chosen so that none is left in SqueezeNet's logits at 1, 2 and 5
+// images (-6.4e-8 of them at one image without it, +8.3e-8 with 1e-8).  The corrections have to be summed apart: with all six products in
+// one sum 3.9e-8 of it were cut off, 5.5e-7 of the logits.
+constexpr float MMA_CUT = 4.5e-9f;
+
+// a += c + (c * MMA_CUT + r) for two numbers at a time, each operation rounded to nearest
+__device__ __forceinline__ void add_products2(float& a0, float& a1, float c0, float c1, float r0, float r1)
+{
+    asm("{\n\t.reg .b64 a, c, r, k;\n\t"
+        "mov.b64 a, {%0, %1};\n\t"
+        "mov.b64 c, {%2, %3};\n\t"
+        "mov.b64 r, {%4, %5};\n\t"
+        "mov.b64 k, {%6, %6};\n\t"
+        "fma.rn.f32x2 r, c, k, r;\n\t"
+        "add.rn.f32x2 r, c, r;\n\t"
+        "add.rn.f32x2 a, a, r;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(c0), "f"(c1), "f"(r0), "f"(r1), "f"(MMA_CUT));
+}
+
+// One step of 16 reduction elements of fp32 products, operands split into three bf16 numbers each (f32_common.cuh), for F tiles of 8
+// layers x N tiles of 16 pixels: the product of the first numbers and, summed on their own, the five next ones of the nine; both added
+// to acc with rounded additions (the matrix instructions cut their sums off).  The tiles take every product in turn: an MMA's
+// result is there after some 33 clocks, four of them take 32 to issue.
+template <int F, int N>
+__device__ __forceinline__ void mma_split(float (*acc)[N][4], const uint32_t (&xh)[N][4], const uint32_t (&xm)[N][4], const uint32_t (&xl)[N][4],
+                                          const uint32_t (&wh)[F][2], const uint32_t (&wm)[F][2], const uint32_t (&wl)[F][2])
+{
+    float c[F][N][4], r[F][N][4];
+#pragma unroll
+    for (int p = 0; p < 6; ++p)
+#pragma unroll
+        for (int f = 0; f < F; ++f)
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                if (p == 0) mma_bf16_free<true>(r[f][e], xl[e], wh[f]);
+                else if (p == 1) mma_bf16_free<false>(r[f][e], xm[e], wm[f]);
+                else if (p == 2) mma_bf16_free<false>(r[f][e], xh[e], wl[f]);
+                else if (p == 3) mma_bf16_free<true>(c[f][e], xh[e], wh[f]);
+                else if (p == 4) mma_bf16_free<false>(r[f][e], xm[e], wh[f]);
+                else mma_bf16_free<false>(r[f][e], xh[e], wm[f]);
+            }
+#pragma unroll
+    for (int f = 0; f < F; ++f)
+#pragma unroll
+        for (int e = 0; e < N; ++e)
+#pragma unroll
+            for (int k = 0; k < 4; k += 2) add_products2(acc[f][e][k], acc[f][e][k + 1], c[f][e][k], c[f][e][k + 1], r[f][e][k], r[f][e][k + 1]);
+}
+
 }  // namespace sqn

@@ -1,0 +1,101 @@
+"""The fp32 kernels of small layers on the matrix instructions (three bf16 numbers per operand): operands of any magnitude, sums
+that are not finite, and the stem with its max-pool in one launch, against the oracle.
+
+Bound per output, S = the sum of |kernel * input| over the window: the products left out are below 2^-22 of the operands'
+product, K*K*Cin + 9 additions of at most 2^-23 of what they hold."""
+import numpy as np
+import pytest
+
+from oracle import ref
+from paper_1611_07151_b200 import binding as B
+from paper_1611_07151_b200 import synth
+import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+F32 = B.SQN_F32
+
+
+def bound(x, w, b, S, pad):
+    terms = ref.conv2d(np.abs(x), np.abs(w), np.abs(b), S=S, pad=pad, relu=False).astype(np.float64)
+    return (2.0 ** -22 + (w.shape[1] * w.shape[2] ** 2 + 9) * 2.0 ** -23) * terms
+
+
+@pytest.mark.parametrize("ex,ew", [(-139, 120), (120, -130), (-100, -20), (75, -60), (113, -100), (60, 40)])
+def test_operands_of_any_magnitude(ex, ew):
+    """Multiples of 2^-10 and 2^-14 times powers of two: the outputs are those of the unscaled operands times the same power."""
+    x, w, b = synth.conv_layer_case(9, 1, 64, 256, 27, 3)
+    x, w = np.round(x * 2 ** 10) / np.float32(2 ** 10), np.round(w * 2 ** 14) / np.float32(2 ** 14)
+    b[:] = 0
+    x[:, 3] *= -1
+    exp = ref.conv2d(x, w, b, S=1, pad=1, relu=False)
+    got = G.gpu_conv(np.ldexp(x, ex), np.ldexp(w, ew), b, 1, 1, False, F32, kernel="conv_f32_small 32x32 vec, 8 warps, 2 slots, products")
+    got = np.ldexp(got.astype(np.float64), -ex - ew)
+    # (the last term: half a unit of the smallest fp32 output)
+    assert (np.abs(got - exp) <= bound(x, w, b, 1, 1) + 2.0 ** (-150 - ex - ew)).all()
+
+
+# (N, Cin, Cout, H, K, S, pad), the variant that runs
+VARIANTS = [((1, 64, 256, 27, 3, 1, 1), "32x32 vec, 8 warps, 2 slots"), ((1, 128, 32, 55, 1, 1, 0), "32x32 vec, 8 warps, 3 slots"),
+            ((2, 20, 33, 17, 3, 2, 1), "16x32 vec, 8 warps, 3 slots"), ((8, 64, 128, 33, 3, 2, 1), "32x32 vec, 8 warps, 2 slots"),
+            ((9, 20, 36, 44, 5, 2, 2), "32x40 vec, 8 warps, 2 slots"), ((6, 12, 48, 50, 3, 2, 1), "32x48 vec, 8 warps, 2 slots")]
+
+
+@pytest.mark.parametrize("shape,variant", VARIANTS, ids=lambda s: "x".join(map(str, s)) if isinstance(s, tuple) else s)
+def test_sums_finite_and_not(shape, variant):
+    N, C, M, H, K, S, pad = shape
+    rng = np.random.default_rng(sum(shape))
+    x = rng.standard_normal((N, C, H, H)).astype(np.float32)
+    w, b = synth.draw_conv_params(rng, C, M, K)
+    for special in (False, True):
+        if special:
+            x[0, 1, :, 3], x[0, 2, 9, 9], x[N - 1, 0, 5, 5] = np.inf, np.nan, -np.inf
+            w[M - 1, 3, K // 2, K // 2], w[5, C - 1, K // 2, K // 2] = np.inf, np.nan
+        with np.errstate(invalid="ignore", over="ignore"):
+            exp = ref.conv2d(x, w, b, S=S, pad=pad, relu=False)
+        got = G.gpu_conv(x, w, b, S, pad, False, F32, kernel="conv_f32_small %s, products" % variant)
+        fin = np.isfinite(exp)
+        np.testing.assert_array_equal(got[~fin], exp[~fin])
+        xf, wf = np.where(np.isfinite(x), x, 0), np.where(np.isfinite(w), w, 0)
+        assert (np.abs(got[fin].astype(np.float64) - exp[fin]) <= bound(xf, wf, b, S, pad)[fin]).all()
+
+
+@pytest.mark.parametrize("special", [False, True])
+def test_stem_of_one_image(special):
+    import torch
+    x, params = synth.squeezenet_case(37, 1)
+    if special:
+        x[0, 1, 100, 50], x[0, 2, 226, 226], x[0, 0, 0, 30] = np.inf, np.nan, np.float32(3e38)
+    names = [n for n, *_ in synth.SQUEEZENET_CONVS]
+    ws, bs = [G.dev_w(params[n][0], F32) for n in names], [G.dev_b(params[n][1]) for n in names]
+    net = B.squeezenet_create(ws, bs, F32, 1)
+    work = torch.empty(B.squeezenet_workspace_bytes(net, 1), dtype=torch.uint8, device="cuda")
+    logits = torch.empty((1, 1000), device="cuda")
+    with G.traced() as launched:
+        B.squeezenet_forward(net, G.dev_act(x, F32), logits, None, work, 1)
+    assert B.sqn_check() == B.SQN_OK
+    assert launched[0] == "stem_small_f32", launched
+    maps = []
+    for name in ("conv1", "pool1"):
+        ptr, C, H, W = B.squeezenet_layer_output(net, name, work, 1)
+        off = (ptr - work.data_ptr()) // 4
+        maps.append(work.view(torch.float32)[off:off + C * H * W].view(H, W, C).permute(2, 0, 1)[None].cpu().numpy())
+    B.squeezenet_destroy(net)
+    w, b = params["conv1"]
+    with np.errstate(invalid="ignore", over="ignore"):
+        exp = ref.conv2d(x, w, b, S=2, pad=0, relu=False)
+        low = ref.conv2d(np.abs(np.where(np.isfinite(x), x, 0)), np.abs(w), np.abs(b), S=2, pad=0, relu=False)
+    exp = np.where(np.isnan(exp), 0, np.maximum(exp, 0)).astype(np.float64)          # (max(0, NaN) = 0)
+    fin = np.isfinite(exp) & np.isfinite(low)
+    np.testing.assert_array_equal(maps[0][np.isposinf(exp) & np.isfinite(low)], np.inf)
+    assert (np.abs(maps[0][fin] - exp[fin]) <= (2.0 ** -22 + 156 * 2.0 ** -23) * low[fin].astype(np.float64)).all()
+    # the pooled map: the maximum of the stored one, exactly; where a tile was computed again and its neighbours, which share pixels
+    # with it, were not, up to both tiles' bounds
+    windows = lambda a: np.max([a[:, i:i + 109:2, j:j + 109:2] for i in range(3) for j in range(3)], axis=0)
+    pooled, most = windows(maps[0][0]), windows(low[0].astype(np.float64))
+    if special:
+        same = pooled == maps[1][0]
+        with np.errstate(invalid="ignore"):
+            near = np.abs(pooled - maps[1][0]) <= 2 * (2.0 ** -22 + 156 * 2.0 ** -23) * most
+        assert (same | near).all() and same.mean() > 0.99
+    else:
+        np.testing.assert_array_equal(maps[1][0], pooled)
