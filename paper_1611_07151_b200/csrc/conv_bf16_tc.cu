@@ -441,8 +441,8 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
                 uint32_t bres16 = smB16;
                 int ch = 0;
                 for (int i = 0; i < items; ++i, bres16 += b_tile16) {
-                    const int ks = ++ch == p.chunks ? p.ksteps_last : ksteps;
-                    if (ch == p.chunks) ch = 0;
+                    int ks = ksteps;
+                    if (++ch == p.chunks) { ch = 0; ks = p.ksteps_last; }
                     ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->full[s]), ph, abort_flag, p.status));
                     if (!ok) break;
                     tc_fence_after();
@@ -454,8 +454,10 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
                         const uint64_t db = ((uint64_t)hiB << 32) | (uint64_t)(b16 | 0x10000u);
                         mma_bf16_ss(d_tmem, da, db, idesc, i > 0 ? 1u : 0u);
                         if (ks >= 2) mma_bf16_ss(d_tmem, da + 2, db + 2, idesc, 1u);
-                        if (ks >= 3) mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
-                        if (ks == 4) mma_bf16_ss(d_tmem, da + 6, db + 6, idesc, 1u);
+                        if (ks == 4) {
+                            mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
+                            mma_bf16_ss(d_tmem, da + 6, db + 6, idesc, 1u);
+                        } else if (ks == 3) mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
                         mma_commit(smem_u32(&sh->empty[s]));        // slot free once these MMAs have read it
                         if (i == items - 1) {
                             mma_bf16_ss(d_tmem, bias_da, bias_db, idesc, 1u);

@@ -513,8 +513,7 @@ cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, int sms,
         if (deep && blocks <= sms && (a.chunks > 16 || (b.blocks && b.chunks > 16))) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
     if (deep && blocks <= sms) return launch_any<TY, RM, 8, 3, VEC>(a, b, stream);
     if (deep && blocks <= 2 * sms) return launch_any<TY, RM, 8, 2, VEC>(a, b, stream);
-    // (CTAs of four warps: multiply-adds, fire4's expand-3x3 at one image 10.5 us and 10.9, 12 -> 100 3x3/2 at 40 x 40 6.5 and 6.8)
-    return launch<TY, RM, 4, 3, VEC>(a, b, stream);
+    return launch_any<TY, RM, 4, 3, VEC>(a, b, stream);
 }
 
 template <int NF>
