@@ -382,6 +382,7 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
         // single diverged thread reading a shared-memory table needs about 100).
         const uint32_t idesc = make_idesc_bf16(TILE_M, (uint32_t)p.BN, (uint32_t)p.f16);
         const int ksteps = p.BKc / 16;
+        const bool ragged = p.ksteps_last != ksteps;
         const uint32_t hiA = p.a_lines ? (uint32_t)(make_kmajor_desc_plain(0, 16u, p.sbo_bytes) >> 32)
                                        : (uint32_t)(make_kmajor_desc(0, row_bytes, p.patch ? p.sbo_bytes : 8u * row_bytes) >> 32);
         const uint32_t hiB = (uint32_t)(make_kmajor_desc(0, row_bytes, 8u * row_bytes) >> 32);
@@ -441,23 +442,26 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
                 uint32_t bres16 = smB16;
                 int ch = 0;
                 for (int i = 0; i < items; ++i, bres16 += b_tile16) {
-                    int ks = ksteps;
-                    if (++ch == p.chunks) { ch = 0; ks = p.ksteps_last; }
                     ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&sh->full[s]), ph, abort_flag, p.status));
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t a16 = smA16 + (uint32_t)s * a_tile16;
                     const uint32_t b16 = p.b_resident ? bres16 : smB16 + (uint32_t)s * b_tile16;
                     if (elect_one()) {
-                        // ks MMAs of K = 16 (32 bytes = 2 address units along the row)
+                        // ksteps MMAs of K = 16 (32 bytes = 2 address units along the row), fewer for a tap's shorter last chunk
                         const uint64_t da = ((uint64_t)hiA << 32) | (uint64_t)(a16 | 0x10000u);
                         const uint64_t db = ((uint64_t)hiB << 32) | (uint64_t)(b16 | 0x10000u);
                         mma_bf16_ss(d_tmem, da, db, idesc, i > 0 ? 1u : 0u);
-                        if (ks >= 2) mma_bf16_ss(d_tmem, da + 2, db + 2, idesc, 1u);
-                        if (ks == 4) {
-                            mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
-                            mma_bf16_ss(d_tmem, da + 6, db + 6, idesc, 1u);
-                        } else if (ks == 3) mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
+                        if (ragged && ch == p.chunks - 1) {
+                            if (p.ksteps_last >= 2) mma_bf16_ss(d_tmem, da + 2, db + 2, idesc, 1u);
+                            if (p.ksteps_last >= 3) mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
+                        } else {
+                            if (ksteps >= 2) mma_bf16_ss(d_tmem, da + 2, db + 2, idesc, 1u);
+                            if (ksteps == 4) {
+                                mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
+                                mma_bf16_ss(d_tmem, da + 6, db + 6, idesc, 1u);
+                            }
+                        }
                         mma_commit(smem_u32(&sh->empty[s]));        // slot free once these MMAs have read it
                         if (i == items - 1) {
                             mma_bf16_ss(d_tmem, bias_da, bias_db, idesc, 1u);
@@ -466,6 +470,7 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
                     }
                     __syncwarp();
                     if (++s == p.stages) { s = 0; ph ^= 1u; }
+                    if (ragged && ++ch == p.chunks) ch = 0;
                 }
                 if (!ok) break;
             }
