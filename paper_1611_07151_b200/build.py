@@ -40,7 +40,8 @@ def up_to_date(lib=LIB):
 
 def build_native(force=False):
     """Compile the binding's marshalling module (plain C against Python.h)."""
-    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= os.path.getmtime(NATIVE_SRC):
+    deps = [NATIVE_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h"))       # (it fills sqn_conv_opts in)
+    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(NATIVE) >= os.path.getmtime(f) for f in deps):
         return NATIVE
     tmp = NATIVE + ".tmp.%d" % os.getpid()
     subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
