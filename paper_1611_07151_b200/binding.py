@@ -78,6 +78,8 @@ try:
     from . import _native               # the marshalling of conv_forward_ex and fire_forward in C (csrc/binding_native.c)
 except ImportError:                     # (not built, or for another Python: ctypes marshals all calls)
     _native = None
+if getattr(_native, "sizeof_conv_opts", 0) != ctypes.sizeof(sqn_conv_opts):     # (built against another sqn.h)
+    _native = None
 _conv_forward_ex_at = _fire_forward_at = None       # addresses of the library's functions
 
 

@@ -16,7 +16,8 @@ LIB_DEBUG = os.path.join(PKG, "libsqn_debug.so")      # the same sources with -D
 OBJ_DIR = os.path.join(PKG, "_build")
 
 NATIVE_SRC = os.path.join(CSRC, "binding_native.c")
-NATIVE = os.path.join(PKG, "_native.so")              # the binding's marshalling (see binding.py)
+# the binding's marshalling (see binding.py), under a name that only the interpreter it is built for imports
+NATIVE = os.path.join(PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]

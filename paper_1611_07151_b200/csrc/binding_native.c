@@ -110,5 +110,7 @@ static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", NULL, -1, 
 PyMODINIT_FUNC PyInit__native(void)
 {
     s_data_ptr = PyUnicode_InternFromString("data_ptr");
-    return s_data_ptr ? PyModule_Create(&module) : NULL;
+    PyObject* m = s_data_ptr ? PyModule_Create(&module) : NULL;
+    if (m && PyModule_AddIntConstant(m, "sizeof_conv_opts", (long)sizeof(sqn_conv_opts)) < 0) Py_CLEAR(m);
+    return m;
 }

@@ -1,6 +1,9 @@
 """The build of the binding's marshalling module."""
 import os
 import shutil
+import subprocess
+import sys
+import sysconfig
 
 import pytest
 
@@ -29,3 +32,43 @@ def test_built_again_when_a_source_or_the_header_is_newer(tree, changed):
     os.utime(tree / changed, (2000, 2000))
     build.build_native()
     assert os.path.getmtime(build.NATIVE) > 2000
+
+
+IMPORT = """
+import sys
+sys.path.insert(0, %r)
+from paper_1611_07151_b200 import binding
+print(binding._native is not None)
+"""
+
+
+def imported(package_parent):
+    r = subprocess.run([sys.executable, "-c", IMPORT % str(package_parent)], capture_output=True, text=True, check=True)
+    return r.stdout.strip() == "True"
+
+
+def test_only_the_interpreter_it_is_built_for_takes_the_module(tree):
+    """A plain .so is imported by every Python version, whatever its C API."""
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert os.path.basename(build.NATIVE) == "_native" + suffix
+    package = tree / "paper_1611_07151_b200"
+    package.mkdir()
+    for f in ("__init__.py", "binding.py"):
+        shutil.copy(os.path.join(build.PKG, f), package / f)
+    shutil.copy(build.NATIVE, package / ("_native" + suffix))
+    assert imported(tree)
+    os.rename(package / ("_native" + suffix), package / "_native.cpython-39-x86_64-linux-gnu.so")
+    assert not imported(tree)
+
+
+def test_a_module_for_another_options_struct_is_left_alone(tree):
+    header = tree / "include" / "sqn.h"
+    header.write_text(header.read_text().replace("int fuse_global_avgpool;", "int fuse_global_avgpool; double more;"))
+    assert "double more" in header.read_text()
+    build.build_native(force=True)
+    package = tree / "paper_1611_07151_b200"
+    package.mkdir()
+    for f in ("__init__.py", "binding.py"):
+        shutil.copy(os.path.join(build.PKG, f), package / f)
+    shutil.copy(build.NATIVE, package)
+    assert not imported(tree)
