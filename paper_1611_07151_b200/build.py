@@ -7,6 +7,7 @@ import os
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -40,13 +41,20 @@ def up_to_date(lib=LIB):
 
 
 def build_native(force=False):
-    """Compile the binding's marshalling module (plain C against Python.h)."""
+    """Compile the binding's marshalling module (plain C against Python.h).  Where that is not possible a warning says so, and the
+    binding does without it: ctypes marshals every call."""
     deps = [NATIVE_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h"))       # (it fills sqn_conv_opts in)
     if not force and os.path.exists(NATIVE) and all(os.path.getmtime(NATIVE) >= os.path.getmtime(f) for f in deps):
         return NATIVE
     tmp = NATIVE + ".tmp.%d" % os.getpid()
-    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
-                    "-I", os.path.join(ROOT, "include"), NATIVE_SRC, "-o", tmp], check=True)
+    try:
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                        "-I", os.path.join(ROOT, "include"), NATIVE_SRC, "-o", tmp], check=True)
+    except (OSError, subprocess.CalledProcessError) as e:
+        if os.path.exists(NATIVE):
+            os.remove(NATIVE)               # (older than what it depends on)
+        warnings.warn("the marshalling module was not built (%s): ctypes marshals the calls" % e)
+        return None
     os.replace(tmp, NATIVE)
     return NATIVE
 

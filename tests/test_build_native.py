@@ -72,3 +72,14 @@ def test_a_module_for_another_options_struct_is_left_alone(tree):
         shutil.copy(os.path.join(build.PKG, f), package / f)
     shutil.copy(build.NATIVE, package)
     assert not imported(tree)
+
+
+@pytest.mark.parametrize("compiler", ["false", "/nowhere/gcc"])
+def test_the_library_builds_without_the_module(tree, monkeypatch, compiler):
+    """No compiler or no Python.h: ctypes marshals the calls, and a module older than its sources does not stay."""
+    monkeypatch.setenv("CC", compiler)
+    monkeypatch.setattr(build, "up_to_date", lambda lib=None: True)
+    os.utime(tree / "include" / "sqn.h", (2000, 2000))
+    with pytest.warns(UserWarning, match="marshalling module"):
+        assert build.build() == build.LIB
+    assert not os.path.exists(build.NATIVE)
