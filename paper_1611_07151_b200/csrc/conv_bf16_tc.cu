@@ -223,7 +223,8 @@ __device__ __forceinline__ void fill_bias_rows(const TcParams& p, unsigned char*
 
 // HC: output layers per epilogue piece (8, 16 or 32; a store chunk CW is two pieces), fixed at compile time so
 // that the conversion loop is straight-line code.  TURN: the two groups of epilogue warps take chunks in turn (see there).
-template <int SPLIT, int HC, bool F16, bool TURN>
+// RAGGED: a tap's last chunk may be shorter than the others (see the MMA issuer).
+template <int SPLIT, int HC, bool F16, bool TURN, bool RAGGED>
 __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO,
                                              const TcParams& p, const int bid)
 {
@@ -382,7 +383,6 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
         // single diverged thread reading a shared-memory table needs about 100).
         const uint32_t idesc = make_idesc_bf16(TILE_M, (uint32_t)p.BN, (uint32_t)p.f16);
         const int ksteps = p.BKc / 16;
-        const bool ragged = p.ksteps_last != ksteps;
         const uint32_t hiA = p.a_lines ? (uint32_t)(make_kmajor_desc_plain(0, 16u, p.sbo_bytes) >> 32)
                                        : (uint32_t)(make_kmajor_desc(0, row_bytes, p.patch ? p.sbo_bytes : 8u * row_bytes) >> 32);
         const uint32_t hiB = (uint32_t)(make_kmajor_desc(0, row_bytes, 8u * row_bytes) >> 32);
@@ -448,11 +448,13 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
                     const uint32_t a16 = smA16 + (uint32_t)s * a_tile16;
                     const uint32_t b16 = p.b_resident ? bres16 : smB16 + (uint32_t)s * b_tile16;
                     if (elect_one()) {
-                        // ksteps MMAs of K = 16 (32 bytes = 2 address units along the row), fewer for a tap's shorter last chunk
+                        // ksteps MMAs of K = 16 (32 bytes = 2 address units along the row), fewer for a tap's shorter last chunk.  (Kernels
+                        // of their own for layers that have one: the question in every layer's loop cost the streamed ones 2 to 6 %,
+                        // 512 -> 512 3x3 at 7 x 7, ten images, 21.9 -> 23.2 us, 384 -> 48 1x1 at 27 x 27, 115 images, 10.8 -> 11.2.)
                         const uint64_t da = ((uint64_t)hiA << 32) | (uint64_t)(a16 | 0x10000u);
                         const uint64_t db = ((uint64_t)hiB << 32) | (uint64_t)(b16 | 0x10000u);
                         mma_bf16_ss(d_tmem, da, db, idesc, i > 0 ? 1u : 0u);
-                        if (ragged && ch == p.chunks - 1) {
+                        if (RAGGED && ch == p.chunks - 1) {
                             if (p.ksteps_last >= 2) mma_bf16_ss(d_tmem, da + 2, db + 2, idesc, 1u);
                             if (p.ksteps_last >= 3) mma_bf16_ss(d_tmem, da + 4, db + 4, idesc, 1u);
                         } else {
@@ -470,7 +472,7 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
                     }
                     __syncwarp();
                     if (++s == p.stages) { s = 0; ph ^= 1u; }
-                    if (ragged && ++ch == p.chunks) ch = 0;
+                    if (RAGGED && ++ch == p.chunks) ch = 0;
                 }
                 if (!ok) break;
             }
@@ -615,17 +617,17 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
 // One layer per launch, or two independent layers that read the same input (the two expands of a fire layer):
 // the first p0.grid CTAs work on the first, the others on the second, so the second fills the tail of the first
 // and the pair costs one launch.
-template <int SPLIT, int HC, bool TURN>
+template <int SPLIT, int HC, bool TURN, bool RAGGED>
 __global__ void __launch_bounds__(threads_for(SPLIT), SPLIT == 1 ? 2 : 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmO, const __grid_constant__ TcParams p)
 {
     // (the 16-bit type is a compile-time constant of the body: the epilogue's conversion loop is straight-line code)
-    if (p.f16) conv_tc_body<SPLIT, HC, true, TURN>(tmA, tmB, tmO, p, (int)blockIdx.x);
-    else conv_tc_body<SPLIT, HC, false, TURN>(tmA, tmB, tmO, p, (int)blockIdx.x);
+    if (p.f16) conv_tc_body<SPLIT, HC, true, TURN, RAGGED>(tmA, tmB, tmO, p, (int)blockIdx.x);
+    else conv_tc_body<SPLIT, HC, false, TURN, RAGGED>(tmA, tmB, tmO, p, (int)blockIdx.x);
 }
 
-template <int SPLIT, int HC>
+template <int SPLIT, int HC, bool RAGGED>
 __global__ void __launch_bounds__(threads_for(SPLIT), SPLIT == 1 ? 2 : 1)
 conv_tc_kernel2(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                 const __grid_constant__ CUtensorMap tmO0, const __grid_constant__ TcParams p0,
@@ -633,11 +635,11 @@ conv_tc_kernel2(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
                 const __grid_constant__ CUtensorMap tmO1, const __grid_constant__ TcParams p1)
 {
     if (p0.f16) {
-        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, true, false>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
-        else conv_tc_body<SPLIT, HC, true, false>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
+        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, true, false, RAGGED>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
+        else conv_tc_body<SPLIT, HC, true, false, RAGGED>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
     } else {
-        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, false, false>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
-        else conv_tc_body<SPLIT, HC, false, false>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
+        if ((int)blockIdx.x < p0.grid) conv_tc_body<SPLIT, HC, false, false, RAGGED>(tmA0, tmB0, tmO0, p0, (int)blockIdx.x);
+        else conv_tc_body<SPLIT, HC, false, false, RAGGED>(tmA1, tmB1, tmO1, p1, (int)blockIdx.x - p0.grid);
     }
 }
 
@@ -1616,20 +1618,33 @@ int build_plan(const ConvDesc& d, bool stem, const void* a_ptr, const void* w_pt
     return build_plan_cfg(d, stem, a_ptr, w_ptr, Hp, Wp, 2, plan);
 }
 
-template <int SPLIT, int HC, bool TURN>
+template <int SPLIT, int HC, bool TURN, bool RAGGED>
 cudaError_t launch_variant(const Plan& plan, cudaStream_t stream)
 {
     static SmemAttr attr;
-    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel<SPLIT, HC, TURN>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
+    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel<SPLIT, HC, TURN, RAGGED>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
     if (arc != cudaSuccess) return arc;
-    return launch_chained(conv_tc_kernel<SPLIT, HC, TURN>, dim3((unsigned)plan.grid), dim3(threads_for(SPLIT)), plan.smem,
+    return launch_chained(conv_tc_kernel<SPLIT, HC, TURN, RAGGED>, dim3((unsigned)plan.grid), dim3(threads_for(SPLIT)), plan.smem,
                           stream, plan.a, plan.b, plan.o, plan.p);
+}
+
+inline bool ragged(const TcParams& p) { return p.ksteps_last != p.BKc / 16; }
+inline bool in_turn(const Plan& plan) { return plan.split == 2 && plan.p.BN >= 3 * plan.p.CW; }
+
+template <int SPLIT, bool TURN>
+cudaError_t launch_chunks(const Plan& plan, cudaStream_t stream)
+{
+    const int hc = plan.p.CW / 2;
+    if (ragged(plan.p))
+        return hc == 32 ? launch_variant<SPLIT, 32, TURN, true>(plan, stream)
+             : hc == 16 ? launch_variant<SPLIT, 16, TURN, true>(plan, stream) : launch_variant<SPLIT, 8, TURN, true>(plan, stream);
+    return hc == 32 ? launch_variant<SPLIT, 32, TURN, false>(plan, stream)
+         : hc == 16 ? launch_variant<SPLIT, 16, TURN, false>(plan, stream) : launch_variant<SPLIT, 8, TURN, false>(plan, stream);
 }
 
 int launch_plan(const Plan& plan, cudaStream_t stream)
 {
     cudaError_t rc;
-    const int hc = plan.p.CW / 2;
     if (plan.p.pool) {
         static SmemAttr attr;
         rc = attr.allow((const void*)conv_pool_kernel, SMEM_LIMIT);
@@ -1637,28 +1652,34 @@ int launch_plan(const Plan& plan, cudaStream_t stream)
             rc = launch_chained(conv_pool_kernel, dim3((unsigned)plan.grid), dim3(POOLT_THREADS), plan.smem, stream, plan.a, plan.b, plan.r,
                                 plan.p);
     }
-    else if (plan.split == 1)
-        rc = hc == 32 ? launch_variant<1, 32, false>(plan, stream)
-           : hc == 16 ? launch_variant<1, 16, false>(plan, stream) : launch_variant<1, 8, false>(plan, stream);
-    else if (plan.p.BN >= 3 * plan.p.CW)
-        rc = hc == 32 ? launch_variant<2, 32, true>(plan, stream)
-           : hc == 16 ? launch_variant<2, 16, true>(plan, stream) : launch_variant<2, 8, true>(plan, stream);
-    else
-        rc = hc == 32 ? launch_variant<2, 32, false>(plan, stream)
-           : hc == 16 ? launch_variant<2, 16, false>(plan, stream) : launch_variant<2, 8, false>(plan, stream);
+    else if (plan.split == 1) rc = launch_chunks<1, false>(plan, stream);
+    else if (in_turn(plan)) rc = launch_chunks<2, true>(plan, stream);
+    else rc = launch_chunks<2, false>(plan, stream);
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch(plan.p.pool ? "conv_pool, %d pixels" : "conv_tc, %d layers", plan.p.pool ? plan.p.npix : plan.p.BN);
+    if (plan.p.pool) note_launch("conv_pool, %d pixels", plan.p.npix);
+    else note_launch("conv_tc, %d layers%s%s", plan.p.BN, in_turn(plan) ? ", chunks in turn" : "", ragged(plan.p) ? ", a shorter last chunk" : "");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 
-template <int SPLIT, int HC>
+template <int SPLIT, int HC, bool RAGGED>
 cudaError_t launch_variant2(const Plan& a, const Plan& b, cudaStream_t stream)
 {
     static SmemAttr attr;
-    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel2<SPLIT, HC>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
+    const cudaError_t arc = attr.allow((const void*)conv_tc_kernel2<SPLIT, HC, RAGGED>, SPLIT == 1 ? SMEM_LIMIT_2CTA : SMEM_LIMIT);
     if (arc != cudaSuccess) return arc;
-    return launch_chained(conv_tc_kernel2<SPLIT, HC>, dim3((unsigned)(a.grid + b.grid)), dim3(threads_for(SPLIT)),
+    return launch_chained(conv_tc_kernel2<SPLIT, HC, RAGGED>, dim3((unsigned)(a.grid + b.grid)), dim3(threads_for(SPLIT)),
                           a.smem > b.smem ? a.smem : b.smem, stream, a.a, a.b, a.o, a.p, b.a, b.b, b.o, b.p);
+}
+
+template <int SPLIT>
+cudaError_t launch_chunks2(const Plan& a, const Plan& b, cudaStream_t stream)
+{
+    const int hc = a.p.CW / 2;
+    if (ragged(a.p) || ragged(b.p))
+        return hc == 32 ? launch_variant2<SPLIT, 32, true>(a, b, stream)
+             : hc == 16 ? launch_variant2<SPLIT, 16, true>(a, b, stream) : launch_variant2<SPLIT, 8, true>(a, b, stream);
+    return hc == 32 ? launch_variant2<SPLIT, 32, false>(a, b, stream)
+         : hc == 16 ? launch_variant2<SPLIT, 16, false>(a, b, stream) : launch_variant2<SPLIT, 8, false>(a, b, stream);
 }
 
 // Two plans of the same kernel variant in one launch: the first a.grid CTAs run `a`, the others `b`.
@@ -1675,17 +1696,12 @@ int launch_plan2(const Plan& a, const Plan& b, cudaStream_t stream)
             rc = launch_chained(conv_pool_kernel2, dim3((unsigned)(a.grid + b.grid)), dim3(POOLT_THREADS), smem, stream, a.a, a.b,
                                 a.r, a.p, b.a, b.b, b.r, b.p);
     } else {
-        const int hc = a.p.CW / 2;
         if (a.split != b.split || a.p.CW != b.p.CW) return SQN_ERR_UNSUPPORTED;
-        if (a.split == 1)
-            rc = hc == 32 ? launch_variant2<1, 32>(a, b, stream)
-               : hc == 16 ? launch_variant2<1, 16>(a, b, stream) : launch_variant2<1, 8>(a, b, stream);
-        else
-            rc = hc == 32 ? launch_variant2<2, 32>(a, b, stream)
-               : hc == 16 ? launch_variant2<2, 16>(a, b, stream) : launch_variant2<2, 8>(a, b, stream);
+        rc = a.split == 1 ? launch_chunks2<1>(a, b, stream) : launch_chunks2<2>(a, b, stream);
     }
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
-    note_launch(a.p.pool ? "conv_pool x 2, %d pixels" : "conv_tc x 2, %d layers", a.p.pool ? a.p.npix : a.p.BN);
+    if (a.p.pool) note_launch("conv_pool x 2, %d pixels", a.p.npix);
+    else note_launch("conv_tc x 2, %d layers%s", a.p.BN, ragged(a.p) || ragged(b.p) ? ", a shorter last chunk" : "");
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

@@ -57,3 +57,14 @@ def test_ragged_chunks(shape, dtype):
         assert fin.sum() == fin.size - (fin.size // M if inf else 0)
         np.testing.assert_array_equal(mine[~fin], exp[~fin])
         assert (np.abs(mine[fin] - exp[fin]) <= (err + ULP[dtype] * (np.abs(exp) + err) + 2.0 ** -25)[fin]).all()
+
+
+@pytest.mark.parametrize("C,M,HW,K", [(512, 512, 7, 3), (384, 48, 27, 1), (64, 256, 28, 1), (256, 256, 14, 3), (112, 96, 20, 3), (96, 64, 27, 1)])
+def test_only_layers_with_a_shorter_last_chunk_ask_for_it(C, M, HW, K):
+    """The kernels that count MMAs per slot are slower on the layers that need not."""
+    x, w, b = (B.empty_device(n, t) for n, t in (((10, HW, HW, C), B.SQN_BF16), ((M, K, K, C), B.SQN_BF16), ((M,), B.SQN_F32)))
+    with G.traced() as names:
+        B.conv_forward_ex(x, w, b, B.empty_device((10, HW, HW, M), B.SQN_BF16), C, M, HW, HW, K, 1, K // 2, 10, dtype=B.SQN_BF16)
+    assert B.sqn_check() == B.SQN_OK
+    assert len(names) == 1 and names[0].startswith("conv_tc, "), names
+    assert names[0].endswith(", a shorter last chunk") == (C % 64 != 0), names
