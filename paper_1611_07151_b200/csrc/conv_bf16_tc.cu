@@ -482,9 +482,10 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmA, const CUten
         // -------------------------------------------------------------------- epilogue
         // 4*SPLIT warps: warp w reads TMEM lane quadrant w % 4 (one output pixel per thread) and, of
         // every chunk of CW layers, the piece(s) given by (w - 2) / 4; TURN: every second chunk, all of it.  A chunk is a chain of
-        // latencies of some 1000 clocks whatever its width, so that tiles of three chunks and more gain by two of them at a time:
-        // 64 -> 256 1x1 at 56 x 56, 64 images, 23.8 -> 22.6 us, 48 -> 192 at 27 x 27, 37 images, 6.5 -> 6.0, 256 -> 1024 at 14 x 14,
-        // 125 images, 22.8 -> 22.3; with one or two chunks it loses 1 to 2 % (384 -> 64 at 27 x 27: 6.8 -> 6.9).  TMEM -> registers (bias already added by the last MMA), ReLU, -> bf16,
+        // latencies of some 1000 clocks whatever its width, so that tiles of three chunks and more gain by two of them at a time
+        // where the epilogue is what a tile waits for (see in_turn):
+        // 64 -> 256 1x1 at 56 x 56, 33 images, 13.4 -> 12.6 us, 48 -> 192 at 27 x 27, 56 images, 7.4 -> 6.8, 128 -> 512 at 28 x 28,
+        // 31 images, 9.2 -> 8.9; with one or two chunks it loses 1 to 2 % (384 -> 64 at 27 x 27: 6.8 -> 6.9).  TMEM -> registers (bias already added by the last MMA), ReLU, -> bf16,
         // into a slot of the staging ring (TMA-swizzled rows); the store warp sends the slot to
         // global memory while the next chunk is converted.
         const int q = warp & 3;
@@ -1629,7 +1630,20 @@ cudaError_t launch_variant(const Plan& plan, cudaStream_t stream)
 }
 
 inline bool ragged(const TcParams& p) { return p.ksteps_last != p.BKc / 16; }
-inline bool in_turn(const Plan& plan) { return plan.split == 2 && plan.p.BN >= 3 * plan.p.CW; }
+
+// Whether the epilogue's two groups of warps take chunks in turn (tiles of three chunks or more, see there).  Several tiles per CTA: a
+// tile's epilogue runs behind the next tile's MMAs and is seen only where they are fewer than it takes, 1x1 layers of less than 256
+// input layers (46 layers timed both ways, geometric mean 0.971, the longest of them by more than 1 % a single one; with longer
+// reductions 85 layers 1.002, 288 -> 384 1x1 at 11 x 28, 52 images, 9.6 and 9.8 us).  One tile per CTA: the epilogue comes after all
+// MMAs and is 0 to 4 % of the layer shorter (90 layers, 0.995), but with fewer than eight MMAs 0 to 4 % longer (80 -> 384 1x1 at 21 x 12,
+// 28 images, 6.0 and 6.2).
+inline bool in_turn(const Plan& plan)
+{
+    const TcParams& p = plan.p;
+    if (plan.split != 2 || p.BN < 3 * p.CW) return false;
+    const int steps = p.taps * p.k_per_tap / 16;
+    return p.total_tiles > plan.grid ? p.taps == 1 && steps < 16 : steps >= 8;
+}
 
 template <int SPLIT, bool TURN>
 cudaError_t launch_chunks(const Plan& plan, cudaStream_t stream)
