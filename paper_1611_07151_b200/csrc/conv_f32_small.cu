@@ -223,7 +223,7 @@ __device__ __forceinline__ float ld_shared_f1(uint32_t a)
 // its rows with one 16-byte read, free of bank conflicts.  A chunk of a 32 x 32 tile is 48 MMAs of 8 clocks per scheduler against 512
 // multiply-adds of 1.45 and six times the reads; what bounds it is the chain of a chunk (read, split, products) in every warp.
 // Multiply-adds against this kernel, one image: fire8's expand-3x3 12.5 -> 10.8 us, fire9's 6.9 -> 5.3, fire8's squeeze 5.4 -> 3.9,
-// conv10 11.5 -> 9.8; 256 -> 256 3x3 at 14 x 14, 3 images: 42.2 -> 35.0.  Error against 64 bits 0.7e-7 to 1.3e-7 (0.9e-7 to 4.0e-7).
+// conv10 11.5 -> 9.8; 256 -> 256 3x3 at 14 x 14, 3 images: 42.2 -> 35.0.  Which layers take it: launch_ty.  Error against 64 bits 0.7e-7 to 1.3e-7 (0.9e-7 to 4.0e-7).
 // A tile with a sum that is not finite is computed again with multiply-adds.
 template <int MF, int NF, int SL, int ST>
 __device__ __forceinline__ void conv_f32_small_tc_body(const F32SmallParams& p, const int bid)
@@ -464,22 +464,15 @@ cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_
     return rc;
 }
 
-// Tiles of 32 layers with 16-byte pieces go to the matrix instructions, see launch_ty.
-template <int TY, int RM, int SL, int ST, bool VEC>
-cudaError_t launch_any(const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
-{
-    if constexpr (VEC && TY == 4) return launch_tc<TY * RM / 16, 16 / TY, SL, ST>(a, b, stream);
-    else return launch<TY, RM, SL, ST, VEC>(a, b, stream);
-}
-
 // Tile, warps and ring for a layer (or two) of so many tiles; measured on SqueezeNet's layers at batch 1 and 4:
 //  - half as many pixels per thread where the larger tiles would leave half of the SMs without a CTA (fire9's squeeze 6.9 ->
 //    4.7 us, fire5's 4.2 -> 3.2);
 //  - eight warps and three slots per warp where every SM gets one CTA at most, two slots where two CTAs per SM make it one
 //    wave (fire8's expand-3x3 at batch 1, 184 tiles: 14.1 -> 12.5 us), else four warps and three slots.
-//  - a single layer with 16-byte pieces and more tiles than SMs: tiles of 40 or 48 layers where they compute an eighth less than those
-//    of 32 and are two waves of CTAs at most (20 -> 36 5x5/2, nine images of 61 x 47, half of the 32-layer tiles' work for nothing:
-//    18.1 -> 13.1 us).
+//  - a single layer with 16-byte pieces, more than six chunks and more tiles than two per SM: tiles of 40 or 48 layers where they
+//    compute an eighth less than those of 32 and then are two per SM at most (20 -> 36 5x5/2, nine images of 61 x 47, half of the
+//    32-layer tiles' work for nothing: 18.0 -> 13.1 us; 50 such layers 0.81, with six chunks or fewer 1.0).  Fewer tiles of 32 run two
+//    to an SM at once and are the faster ones (150 layers, the wider tiles 1.03 to 1.24; 12 -> 48 3x3/2, six images of 50 x 50, 4.7 and 5.7 us).
 struct SmallConfig { bool narrow; int rm, tm, tn; };
 
 SmallConfig config_of(const ConvDesc* d, int n, int sms, bool wide)
@@ -492,7 +485,7 @@ SmallConfig config_of(const ConvDesc* d, int n, int sms, bool wide)
     for (int i = 0; i < n; ++i)
         blocks += (((long long)d[i].N * d[i].OH * d[i].OW + (c.narrow ? 63 : 31)) / (c.narrow ? 64 : 32)) * ((d[i].Cout + c.tn - 1) / c.tn);
     if (blocks <= sms / 2) c.rm = 4;
-    else if (wide && blocks > sms && !c.narrow && n == 1 && d[0].Cin % 4 == 0)
+    else if (wide && blocks > 2 * sms && !c.narrow && n == 1 && d[0].Cin % 4 == 0 && d[0].K * d[0].K * d[0].Cin > 6 * SK)
         for (int tn = 40; tn <= 48; tn += 8) {
             const int cols = (d[0].Cout + tn - 1) / tn;
             if (cols * tn * 8LL <= (d[0].Cout + c.tn - 1) / c.tn * c.tn * 7LL && blocks / ((d[0].Cout + 31) / 32) * cols <= 2 * sms) c.tn = tn;
@@ -504,16 +497,34 @@ SmallConfig config_of(const ConvDesc* d, int n, int sms, bool wide)
 template <int TY, int RM, bool VEC>
 cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, int sms, cudaStream_t stream)
 {
-    const int blocks = a.blocks + b.blocks;
-    const bool deep = a.chunks > 2 || (b.blocks && b.chunks > 2);       // (more than two warps have chunks)
-    if constexpr (VEC && TY == 4 && RM == 8)
-        // One CTA of eight warps per SM: a chunk on the matrix instructions is a longer chain for a warp (split, products, sums) than its
-        // multiply-adds, and two warps to a scheduler do not cover it; so only where a warp has two chunks at most (128 -> 32 1x1
-        // at 55 x 55: 3.8 -> 3.4 us; 48 -> 192 3x3 at 27 x 27, 27 chunks: 6.2 and 7.8; 1024 -> 256 1x1, 64 chunks: 12.4 and 14.9).
-        if (deep && blocks <= sms && (a.chunks > 16 || (b.blocks && b.chunks > 16))) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
-    if (deep && blocks <= sms) return launch_any<TY, RM, 8, 3, VEC>(a, b, stream);
-    if (deep && blocks <= 2 * sms) return launch_any<TY, RM, 8, 2, VEC>(a, b, stream);
-    return launch_any<TY, RM, 4, 3, VEC>(a, b, stream);
+    const int blocks = a.blocks + b.blocks, chunks = b.blocks && b.chunks > a.chunks ? b.chunks : a.chunks;
+    const bool deep = chunks > 2;               // (more than two warps have chunks)
+    if constexpr (VEC && TY == 4) {
+        // Where the matrix instructions are the faster ones; both timed on 1200 random layers and 600 fire layers' expands (geometric
+        // means, multiply-adds = 1).  A chunk on them is a longer chain for a warp (split, products, sums), so a warp needs some; but
+        // rings without padding let one CTA more live on an SM.
+        const bool pair = b.blocks != 0;
+        if (RM == 4) {
+            // CTAs on half the SMs: 12 to 64 chunks 0.95, more 0.87, 4 to 11 1.01, fewer 1.10; on more of them 4 to 8 0.96, 9 to 64 0.88, more
+            // 0.86, three 1.03.  Expands of 16 squeeze layers, nine chunks, 1.02, of 32 and more 0.91.
+            if (deep && blocks <= sms && chunks > (!pair && blocks > sms / 2 ? 3 : 11)) return launch_tc<1, 4, 8, 3>(a, b, stream);
+        } else if (blocks <= sms) {
+            // one CTA per SM: 1.03 to 1.09 at any number of chunks.  Except 1x1 layers of one column of tiles on three quarters of the SMs
+            // (0.77 to 0.97, 128 -> 32 at 55 x 55 3.7 -> 3.5 us; at 60 x 60 and more 0.91 to 1.07).
+            if (!pair && a.n_tiles == 1 && a.K == 1 && chunks > 4 && chunks <= 16 && blocks <= sms * 3 / 4) return launch_tc<2, 4, 8, 3>(a, b, stream);
+        } else if (blocks <= 2 * sms) {
+            // two CTAs per SM: 5 to 16 chunks 0.90, more 0.84, fewer 1.01; expands 0.87 (16 squeeze layers 0.93)
+            if (chunks > 4) return launch_tc<2, 4, 8, 2>(a, b, stream);
+        } else {
+            // Four warps: three CTAs per SM with multiply-adds, four with products.  Up to three per SM 0.99 to 1.05, up to four 0.67 to
+            // 0.75 (one wave instead of two), more 0.8.  Of a pair half the CTAs are short: up to 4 per SM 1.02, up to 4.75 1.05 (nine
+            // chunks 0.88), more 0.94 (0.85).
+            if (blocks > (pair ? (chunks > 9 ? 19 * sms / 4 : 4 * sms) : 3 * sms)) return launch_tc<2, 4, 4, 3>(a, b, stream);
+        }
+    }
+    if (deep && blocks <= sms) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
+    if (deep && blocks <= 2 * sms) return launch<TY, RM, 8, 2, VEC>(a, b, stream);
+    return launch<TY, RM, 4, 3, VEC>(a, b, stream);
 }
 
 template <int NF>

@@ -37,7 +37,9 @@ def test_operands_of_any_magnitude(ex, ew):
 # (N, Cin, Cout, H, K, S, pad), the variant that runs
 VARIANTS = [((1, 64, 256, 27, 3, 1, 1), "32x32 vec, 8 warps, 2 slots"), ((1, 128, 32, 55, 1, 1, 0), "32x32 vec, 8 warps, 3 slots"),
             ((2, 20, 33, 17, 3, 2, 1), "16x32 vec, 8 warps, 3 slots"), ((8, 64, 128, 33, 3, 2, 1), "32x32 vec, 8 warps, 2 slots"),
-            ((9, 20, 36, 44, 5, 2, 2), "32x40 vec, 8 warps, 2 slots"), ((6, 12, 48, 50, 3, 2, 1), "32x48 vec, 8 warps, 2 slots")]
+            ((13, 20, 36, 44, 5, 2, 2), "32x40 vec, 8 warps, 2 slots"), ((9, 12, 48, 50, 3, 2, 1), "32x48 vec, 8 warps, 2 slots"),
+            ((9, 20, 36, 44, 5, 2, 2), "32x32 vec, 8 warps, 2 slots"), ((6, 12, 48, 50, 3, 2, 1), "32x32 vec, 8 warps, 2 slots"),
+            ((17, 12, 96, 34, 3, 2, 1), "32x32 vec, 4 warps, 3 slots")]
 
 
 @pytest.mark.parametrize("shape,variant", VARIANTS, ids=lambda s: "x".join(map(str, s)) if isinstance(s, tuple) else s)
@@ -57,6 +59,24 @@ def test_sums_finite_and_not(shape, variant):
         np.testing.assert_array_equal(got[~fin], exp[~fin])
         xf, wf = np.where(np.isfinite(x), x, 0), np.where(np.isfinite(w), w, 0)
         assert (np.abs(got[fin].astype(np.float64) - exp[fin]) <= bound(xf, wf, b, S, pad)[fin]).all()
+
+
+# (N, Cin, Cout, H, W, K, S, pad), the variant that runs; microseconds with multiply-adds / products as measured
+MULTIPLY_ADDS = [((9, 64, 221, 19, 12, 1, 2, 0), "32x32 vec, 8 warps, 3 slots"),        # 2.7 / 3.3
+                 ((1, 128, 128, 30, 30, 1, 1, 0), "32x32 vec, 8 warps, 3 slots"),       # 3.3 / 3.6
+                 ((1, 4, 80, 53, 26, 1, 2, 0), "16x32 vec, 4 warps, 3 slots"),          # 1.9 / 2.1
+                 ((5, 476, 364, 13, 15, 1, 1, 0), "32x32 vec, 4 warps, 3 slots")]       # 15.8 / 17.2
+
+
+@pytest.mark.parametrize("shape,variant", MULTIPLY_ADDS, ids=lambda s: "x".join(map(str, s)) if isinstance(s, tuple) else s)
+def test_multiply_adds_where_they_are_faster(shape, variant):
+    N, C, M, H, W, K, S, pad = shape
+    x, w, b = B.empty_device((N, H, W, C)), B.empty_device((M, K, K, C)), B.empty_device((M,))
+    out = B.empty_device((N, (H + 2 * pad - K) // S + 1, (W + 2 * pad - K) // S + 1, M))
+    with G.traced() as names:
+        B.conv_forward_ex(x, w, b, out, C, M, H, W, K, S, pad, N)
+    assert B.sqn_check() == B.SQN_OK
+    assert names == ["conv_f32_small " + variant]
 
 
 @pytest.mark.parametrize("special", [False, True])
