@@ -42,6 +42,7 @@
 //           registers, then bias, ReLU and stores of 32 consecutive layers of a pixel per warp
 //   24, 25  TMA producers: pixels, kernels                 (26 idle: registers go by warpgroup)
 //   27      MMA issuer (one elected lane), on the scheduler with the least other work
+#include <cstdio>
 #include <cstring>
 
 #include "f32_common.cuh"
@@ -98,7 +99,7 @@ struct F32TcParams {
     int chunks, ksteps_last;    // pixel chunks of a tile, MMA k-steps of the last one
     int seg;                    // (chunk, tap) units whose w0*x0 products are summed on the tensor core before they are added in registers
     int kres;                   // 1: at most FT_KSLOTS units: the kernels stay in TMEM
-    int tstore;                 // FLAT and BOX where vec_store holds and Cout is a multiple of 4: pixels per TMA store of the epilogue (0: no TMA)
+    int tstore;                 // FLAT and BOX where vec_store holds and Cout is a multiple of 4: pixels per TMA store of the epilogue, 16, 32 or 64 (0: no TMA)
     int vec_store;              // 1: output rows and this layer's slice are 16-byte aligned
     int early;                  // 1: kernels and bias may be read before the wait for the grid ahead
     int ra, sa, sb;             // slots: split pixels, pixel boxes, kernel boxes
@@ -714,7 +715,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             if (!ok) break;
             // bias and ReLU here, where a thread has one layer and 64 independent pixels, then 16 pixels at a time through a
             // staging tile (a pixel's 32 layers are a row) and in 16-byte pieces, eight lanes per pixel, to memory; FLAT and BOX, whose
-            // pixels are consecutive or boxes of the map: 32 or 64 pixels, then a TMA store, which leaves out what lies outside the map
+            // pixels are consecutive or boxes of the map: 16, 32 or 64 pixels, then a TMA store, which leaves out what lies outside the map
             // (BOX: conv1 at batch 256 1021 -> 975 us).  Only two warps per 32 layers have rows to store, so
             // the length of this chain is a tile's time where the reduction is short (fire2's 1x1 expand at batch 256 with
             // bias and ReLU after the staging tile and no TMA 107 us, so 80; a bulk copy per pixel instead of the 16-byte
@@ -722,7 +723,7 @@ __device__ __forceinline__ void conv_f32_tc_body(const CUtensorMap& tmX, const C
             float nan = 0.f;                            // 0 as long as all outputs are finite
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 16) {
-                // (TMA: a staging tile of 32 or 64 pixels, free again when the store before has read it)
+                // (TMA: a staging tile of that many pixels, free again when the store before has read it)
                 const uint32_t stg = stg0 + (MODE != FT_PATCH && p.tstore ? (uint32_t)(c0 & (p.tstore - 1)) * 128u : 0u);
                 if (MODE != FT_PATCH && lane == 0 && p.tstore && (c0 & (p.tstore - 1)) == 0) tma_store_wait_read();
                 __syncwarp();
@@ -1032,7 +1033,14 @@ size_t layout(F32TcParams& p)
     p.khalf = p.chunks == 1 && p.ksteps_last == 1 ? 1 : 0;
     p.wrows = (p.n_step + 31) / 32 * 32;
     p.div_wrows = make_div(p.wrows); p.div_taps = make_div(p.taps);
-    for (int i = 0; i < n_packed + n; ++i) {
+    // BOX with TMA stores: 32 pixels per store before a second pair of pixel slots (conv1 at batch 256 970 us with two slots and 32 pixels,
+    // 1008 with four and 16), and 16 pixels, in the room that the stores without TMA take (1 to 2 % slower than with), before the kernels'
+    // source or the number of blocks: 18 -> 348 3x3/2 at 43 x 42, 48 images, 79 us with 16, 130 with 32 in three blocks; 33 -> 276 7x7 at
+    // 29 x 110, four images, 237 and 338.
+    const int widths = p.mode == FT_BOX && p.tstore ? 2 : 1;
+    for (int j = 0; j < (n_packed + n) * widths; ++j) {
+        const int i = widths == 1 ? j : j / 4 * 2 + j % 2;
+        if (widths == 2) p.tstore = j % 4 < 2 ? 32 : 16;
         const int* c = cand[i < n_packed ? i : i - n_packed];
         p.wsrc = i < n_packed ? FT_W_PACKED : streamed;
         p.ra = c[0];
@@ -1041,7 +1049,7 @@ size_t layout(F32TcParams& p)
         size_t cur = (size_t)p.ra * p.slot_a;
         p.off_sa = (unsigned)cur; cur += (size_t)p.sa * p.stage_a;
         p.off_sb = (unsigned)cur; cur += p.wsrc == FT_W_PACKED ? up1k((size_t)units * p.wrows * (p.khalf ? 96 : 192)) : (size_t)p.sb * 128 * 128;
-        p.off_epi = (unsigned)cur; cur += p.tstore ? (size_t)2 * ((p.n_step + 31) / 32) * p.tstore * 128 : 8 * 2048;
+        p.off_epi = (unsigned)cur; cur += p.tstore > 16 ? (size_t)2 * ((p.n_step + 31) / 32) * p.tstore * 128 : 8 * 2048;
         p.off_tbl = (unsigned)cur; cur += tbl;
         p.off_ctl = (unsigned)cur; cur += 1024;
         if (cur + 1024 > FT_SMEM_LIMIT) continue;
@@ -1104,7 +1112,7 @@ int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
         found = finish(d.Cin, positions);
     }
     if (!found) {
-        p.tstore = p.vec_store && d.Cout % 4 == 0 ? 32 : 0;
+        const int tstore = p.vec_store && d.Cout % 4 == 0 ? 32 : 0;
         p.mode = FT_BOX;
         p.prow = FT_N;
         p.taps = 1;
@@ -1130,6 +1138,7 @@ int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
                 p.div_cb = make_div(cb);
                 const long long cost = tiles * 1000000 + (long long)p.rh * p.rc * cb;
                 if (best >= 0 && cost >= best) break;
+                p.tstore = tstore;          // (layout() may take it down to 16)
                 if (!finish(d.K * d.K * cb, 0)) continue;
                 best = cost;
                 bp = *plan;
@@ -1224,9 +1233,11 @@ int launch_conv_f32_tc(const ConvDesc& d, float limit_us, cudaStream_t stream)
                         : plan.p.mode == FT_PATCH ? launch_mode<FT_PATCH>(plan, stream) : launch_mode<FT_BOX>(plan, stream);
     if (e != cudaSuccess) return SQN_ERR_CUDA;
     const F32TcParams& p = plan.p;
-    note_launch("conv_f32_tc %s, kernels %s, %d %s%s", p.mode == FT_FLAT ? "flat" : p.mode == FT_PATCH ? "patch" : "box",
+    char stores[32] = "";
+    if (p.mode == FT_BOX && p.tstore) std::snprintf(stores, sizeof(stores), ", %d pixels per store", p.tstore);
+    note_launch("conv_f32_tc %s, kernels %s, %d %s%s%s", p.mode == FT_FLAT ? "flat" : p.mode == FT_PATCH ? "patch" : "box",
                 p.wsrc == FT_W_PACKED ? "packed" : p.wsrc == FT_W_BOXES ? "by boxes" : "by copies", p.mode == FT_BOX ? p.nb : 1,
-                p.mode == FT_BOX && p.nb > 1 ? "blocks" : "block", p.mode == FT_BOX && p.S > p.K ? ", apart" : "");
+                p.mode == FT_BOX && p.nb > 1 ? "blocks" : "block", p.mode == FT_BOX && p.S > p.K ? ", apart" : "", stores);
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 

@@ -28,3 +28,25 @@ def test_boxes_of_pixels(shape, offset, total):
     mine = got[ends][:, offset:offset + M].astype(np.float64)
     assert (np.abs(mine - exp) <= bound(x[ends], w, b, S, pad, K, C)).all()
     assert not np.isnan(got).any()
+
+
+# (N, Cin, Cout, H, W, K, S, pad), the variant that runs: what the stores stage must not cost the kernels' source or more blocks of
+# layers (microseconds with those / without)
+PLANS = [((16, 3, 96, 227, 227, 7, 2, 0), "kernels packed, 1 block, 32 pixels per store"),
+         ((32, 20, 256, 112, 112, 3, 2, 1), "kernels by boxes, 1 block, 32 pixels per store"),      # 246 / 104
+         ((48, 18, 348, 43, 42, 3, 2, 1), "kernels by copies, 1 block, 16 pixels per store"),       # 131 / 80
+         ((4, 33, 276, 29, 110, 7, 1, 3), "kernels by copies, 1 block, 16 pixels per store"),       # 339 / 237
+         ((64, 20, 256, 28, 28, 5, 2, 2), "kernels by boxes, 1 block, 16 pixels per store")]        # 70 / 40
+
+
+@pytest.mark.parametrize("shape,variant", PLANS, ids=lambda s: "x".join(map(str, s)) if isinstance(s, tuple) else s)
+def test_staging_takes_nothing_from_the_plan(shape, variant):
+    N, C, M, H, W, K, S, pad = shape
+    rng = np.random.default_rng(sum(shape))
+    x = rng.standard_normal((N, C, H, W)).astype(np.float32)
+    w, b = synth.draw_conv_params(rng, C, M, K)
+    got = G.gpu_conv(x, w, b, S, pad, False, F32, c_offset=8, c_total=M + 12, fill=-7.0, kernel="conv_f32_tc box, " + variant)
+    assert (got[:, :8] == -7.0).all() and (got[:, 8 + M:] == -7.0).all()
+    exp = ref.conv2d(x[-1:], w, b, S=S, pad=pad, relu=False)
+    assert (np.abs(got[-1:, 8:8 + M].astype(np.float64) - exp) <= bound(x[-1:], w, b, S, pad, K, C)).all()
+    assert not np.isnan(got).any()
