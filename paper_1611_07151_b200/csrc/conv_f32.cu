@@ -358,8 +358,8 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
     {
         // Which of the three fp32 kernels: by estimated time.  This one: rounds of CTAs at 0.6 of the FFMA rate (with 4-byte loads
         // 0.4, the 256-pixel tiles 0.24, and 1.9 us for the start and end of every two CTAs on an SM: 450 random layers 0.9 to 1.1 of
-        // it in eight of ten), the latency of the reduction loop, or bytes.  Over 990 random layers the kernel chosen takes 0.7 %
-        // longer than the best of the three on average, 30 % or more in four.  Measured, this kernel / the small layers' / the
+        // it in eight of ten), the latency of the reduction loop, or bytes.  Over 1200 random layers, most of them small, the kernel
+        // chosen takes 2.5 % longer than the best of the three on average, 30 % or more in 19.  Measured, this kernel / the small layers' / the
         // tensor cores' -- batch 1: fire9's squeeze 19.6 / 4.7 / 18.0 us, fire6's expand-3x3 16.4 / 6.4 / 15.5, fire4's 14.5 /
         // 11.3 / 12.6, conv1 25.7 / 31 / 17.4; batch 16: fire4's expand-3x3 99 / 109 / 33, its expand-1x1 17.2 / 34 / 11.5,
         // fire2's expand-1x1 6.9 / 15.6 / 10.0; batch 256: conv1 2687 / - / 1053, fire4's expand-3x3 1296 / - / 359, conv10

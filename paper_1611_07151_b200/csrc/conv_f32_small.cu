@@ -223,7 +223,7 @@ __device__ __forceinline__ float ld_shared_f1(uint32_t a)
 // its rows with one 16-byte read, free of bank conflicts.  A chunk of a 32 x 32 tile is 48 MMAs of 8 clocks per scheduler against 512
 // multiply-adds of 1.45 and six times the reads; what bounds it is the chain of a chunk (read, split, products) in every warp.
 // Multiply-adds against this kernel, one image: fire8's expand-3x3 12.5 -> 10.8 us, fire9's 6.9 -> 5.3, fire8's squeeze 5.4 -> 3.9,
-// conv10 11.5 -> 9.8; 256 -> 256 3x3 at 14 x 14, 3 images: 42.2 -> 35.0.  Which layers take it: launch_ty.  Error against 64 bits 0.7e-7 to 1.3e-7 (0.9e-7 to 4.0e-7).
+// conv10 11.5 -> 9.8; 256 -> 256 3x3 at 14 x 14, 3 images: 42.2 -> 35.0.  Which layers take it: variant_of.  Error against 64 bits 0.7e-7 to 1.3e-7 (0.9e-7 to 4.0e-7).
 // A tile with a sum that is not finite is computed again with multiply-adds.
 template <int MF, int NF, int SL, int ST>
 __device__ __forceinline__ void conv_f32_small_tc_body(const F32SmallParams& p, const int bid)
@@ -475,7 +475,7 @@ cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_
 //    to an SM at once and are the faster ones (150 layers, the wider tiles 1.03 to 1.24; 12 -> 48 3x3/2, six images of 50 x 50, 4.7 and 5.7 us).
 struct SmallConfig { bool narrow; int rm, tm, tn; };
 
-SmallConfig config_of(const ConvDesc* d, int n, int sms, bool wide)
+SmallConfig config_of(const ConvDesc* d, int n, int sms)
 {
     SmallConfig c;
     c.narrow = d[0].Cout <= 16 && (n == 1 || d[1].Cout <= 16);
@@ -485,7 +485,7 @@ SmallConfig config_of(const ConvDesc* d, int n, int sms, bool wide)
     for (int i = 0; i < n; ++i)
         blocks += (((long long)d[i].N * d[i].OH * d[i].OW + (c.narrow ? 63 : 31)) / (c.narrow ? 64 : 32)) * ((d[i].Cout + c.tn - 1) / c.tn);
     if (blocks <= sms / 2) c.rm = 4;
-    else if (wide && blocks > 2 * sms && !c.narrow && n == 1 && d[0].Cin % 4 == 0 && d[0].K * d[0].K * d[0].Cin > 6 * SK)
+    else if (blocks > 2 * sms && !c.narrow && n == 1 && d[0].Cin % 4 == 0 && (long long)d[0].K * d[0].K * d[0].Cin > 6 * SK)
         for (int tn = 40; tn <= 48; tn += 8) {
             const int cols = (d[0].Cout + tn - 1) / tn;
             if (cols * tn * 8LL <= (d[0].Cout + c.tn - 1) / c.tn * c.tn * 7LL && blocks / ((d[0].Cout + 31) / 32) * cols <= 2 * sms) c.tn = tn;
@@ -494,37 +494,50 @@ SmallConfig config_of(const ConvDesc* d, int n, int sms, bool wide)
     return c;
 }
 
-template <int TY, int RM, bool VEC>
-cudaError_t launch_ty(const F32SmallParams& a, const F32SmallParams& b, int sms, cudaStream_t stream)
+// Warps, slots and arithmetic of a launch of so many tiles (blocks) in so many columns (0: two layers), the longest of them with so many
+// chunks; shared: windows that overlap at every pixel.
+struct SmallVariant { int warps, slots; bool products; };
+
+SmallVariant variant_of(const SmallConfig& c, bool vec, long long blocks, int chunks, int columns, bool shared, int sms)
 {
-    const int blocks = a.blocks + b.blocks, chunks = b.blocks && b.chunks > a.chunks ? b.chunks : a.chunks;
+    const bool pair = columns == 0;
     const bool deep = chunks > 2;               // (more than two warps have chunks)
+    SmallVariant v = {deep && blocks <= 2 * sms ? 8 : 4, deep && blocks > sms && blocks <= 2 * sms ? 2 : 3, false};
+    if (c.tn > 32) return {8, 2, true};
+    if (!vec || c.narrow) return v;
+    // Where the matrix instructions are the faster ones; both timed on 1200 random layers and 600 fire layers' expands (geometric
+    // means, multiply-adds = 1).  A chunk on them is a longer chain for a warp (split, products, sums), so a warp needs some; but
+    // rings without padding let one CTA more live on an SM.
+    if (c.rm == 4)
+        // CTAs on half the SMs: 7 to 11 chunks 1.0, 12 to 64 0.95, more 0.87, 4 to 6 1.04, fewer 1.10; on more of them 4 to 8 0.96, 9 to 64
+        // 0.88, more 0.86, three 1.03.  Expands of 16 squeeze layers, nine chunks, 1.02, of 32 and more 0.91.
+        v.products = deep && blocks <= sms && chunks > (pair ? 9 : blocks > sms / 2 ? 3 : 6);
+    else if (blocks <= sms)
+        // one CTA per SM: 1.03 to 1.09 at any number of chunks.  Except one column of tiles on three quarters of the SMs: 0.94 with up to 16
+        // chunks (128 -> 32 1x1 at 55 x 55 3.7 -> 3.5 us; on more of them 1.01).
+        v.products = columns == 1 && deep && chunks <= 16 && blocks <= sms * 3 / 4;
+    else if (blocks <= 2 * sms)
+        // two CTAs per SM: 5 to 16 chunks 0.90, more 0.84, fewer 1.01; expands 0.87 (16 squeeze layers 0.93)
+        v.products = chunks > 4;
+    else
+        // Four warps: three CTAs per SM with multiply-adds, four with products.  Up to three per SM 0.92 with one column of tiles, 0.90 with
+        // a few of windows that overlap, else 0.99 to 1.07; up to four 0.67 to 0.75 (one wave instead of two), more 0.8.  Of a pair half
+        // the CTAs are short: up to 4 per SM 1.02, up to 4.75 1.05 (nine chunks 0.88), more 0.94 (0.85).
+        v.products = pair ? blocks > (chunks > 9 ? 19 * sms / 4 : 4 * sms) : blocks > 3 * sms || (deep && (columns == 1 || (shared && columns <= 6)));
+    return v;
+}
+
+template <int TY, int RM, bool VEC>
+cudaError_t launch_ty(const SmallVariant& v, const F32SmallParams& a, const F32SmallParams& b, cudaStream_t stream)
+{
     if constexpr (VEC && TY == 4) {
-        // Where the matrix instructions are the faster ones; both timed on 1200 random layers and 600 fire layers' expands (geometric
-        // means, multiply-adds = 1).  A chunk on them is a longer chain for a warp (split, products, sums), so a warp needs some; but
-        // rings without padding let one CTA more live on an SM.
-        const bool pair = b.blocks != 0;
-        if (RM == 4) {
-            // CTAs on half the SMs: 12 to 64 chunks 0.95, more 0.87, 4 to 11 1.01, fewer 1.10; on more of them 4 to 8 0.96, 9 to 64 0.88, more
-            // 0.86, three 1.03.  Expands of 16 squeeze layers, nine chunks, 1.02, of 32 and more 0.91.
-            if (deep && blocks <= sms && chunks > (!pair && blocks > sms / 2 ? 3 : 11)) return launch_tc<1, 4, 8, 3>(a, b, stream);
-        } else if (blocks <= sms) {
-            // one CTA per SM: 1.03 to 1.09 at any number of chunks.  Except 1x1 layers of one column of tiles on three quarters of the SMs
-            // (0.77 to 0.97, 128 -> 32 at 55 x 55 3.7 -> 3.5 us; at 60 x 60 and more 0.91 to 1.07).
-            if (!pair && a.n_tiles == 1 && a.K == 1 && chunks > 4 && chunks <= 16 && blocks <= sms * 3 / 4) return launch_tc<2, 4, 8, 3>(a, b, stream);
-        } else if (blocks <= 2 * sms) {
-            // two CTAs per SM: 5 to 16 chunks 0.90, more 0.84, fewer 1.01; expands 0.87 (16 squeeze layers 0.93)
-            if (chunks > 4) return launch_tc<2, 4, 8, 2>(a, b, stream);
-        } else {
-            // Four warps: three CTAs per SM with multiply-adds, four with products.  Up to three per SM 0.99 to 1.05, up to four 0.67 to
-            // 0.75 (one wave instead of two), more 0.8.  Of a pair half the CTAs are short: up to 4 per SM 1.02, up to 4.75 1.05 (nine
-            // chunks 0.88), more 0.94 (0.85).
-            if (blocks > (pair ? (chunks > 9 ? 19 * sms / 4 : 4 * sms) : 3 * sms)) return launch_tc<2, 4, 4, 3>(a, b, stream);
+        if (v.products) {
+            if constexpr (RM == 4) return launch_tc<1, 4, 8, 3>(a, b, stream);
+            else return v.warps == 4 ? launch_tc<2, 4, 4, 3>(a, b, stream) : v.slots == 2 ? launch_tc<2, 4, 8, 2>(a, b, stream) : launch_tc<2, 4, 8, 3>(a, b, stream);
         }
     }
-    if (deep && blocks <= sms) return launch<TY, RM, 8, 3, VEC>(a, b, stream);
-    if (deep && blocks <= 2 * sms) return launch<TY, RM, 8, 2, VEC>(a, b, stream);
-    return launch<TY, RM, 4, 3, VEC>(a, b, stream);
+    if (v.warps == 4) return launch<TY, RM, 4, 3, VEC>(a, b, stream);
+    return v.slots == 2 ? launch<TY, RM, 8, 2, VEC>(a, b, stream) : launch<TY, RM, 8, 3, VEC>(a, b, stream);
 }
 
 template <int NF>
@@ -535,20 +548,29 @@ cudaError_t launch_wide(const F32SmallParams& a, const F32SmallParams& b, cudaSt
 
 }  // namespace
 
-// Microseconds: a launch, then the busiest SM's tiles at 260 clocks per chunk (150 with the smaller tile), fitted to SqueezeNet's
-// layers at batch 1 and 4.  With the narrow tile 300 clocks per chunk, and where warps take several, as if every warp had as many
+// Microseconds: a launch, then the busiest SM's tiles by their chunks.  With 16-byte pieces: eight warps by the variant that would run, and
+// the wide tiles, fitted to 640 random layers (0.88 to 1.1 of it in nine of ten); four warps by the multiply-adds' 260 clocks per chunk
+// (150 with the smaller tile), of which products take two thirds to three quarters.  With the narrow tile 300 clocks per chunk, and where warps take several, as if every warp had as many
 // as the one with the most: fire2's squeeze, 6 chunks for 4 warps, 12.9 us at 19 images, 16.5 at 25, 40 at 71 (FFMA 14.5, 14.5, 37),
 // fire3's, 8 chunks, 14.3 at 19, 67 at 116 (FFMA 18.6, 76).  Where the operands come in pieces of 4 bytes 500 clocks (450 with the
 // smaller tile, 900 with the narrow one) and more for a tile's start, fitted to 450 random layers (0.85 to 1.15 of it in eight
 // of ten; 750 for all of them gave 0.46).
 float f32_small_estimate(const ConvDesc& d, int sms)
 {
-    const SmallConfig c = config_of(&d, 1, sms, false);
-    const long long blocks = (((long long)d.N * d.OH * d.OW + c.tm - 1) / c.tm) * ((d.Cout + c.tn - 1) / c.tn);
-    const float chunks = (float)(((long long)d.K * d.K * d.Cin + SK - 1) / SK);
+    const SmallConfig c = config_of(&d, 1, sms);
+    const int n_tiles = (d.Cout + c.tn - 1) / c.tn;
+    const long long blocks = (((long long)d.N * d.OH * d.OW + c.tm - 1) / c.tm) * n_tiles, Kdim = (long long)d.K * d.K * d.Cin;
+    const float chunks = (float)((Kdim + SK - 1) / SK);
     const float rounds = (float)((blocks + sms - 1) / sms);
     if (d.Cin % 4 != 0) return 2.7f + rounds * (chunks * (c.rm == 4 ? 450.f : c.narrow ? 900.f : 500.f) + 1650.f) / 1965.f;
-    const float warps = blocks > 2 * sms ? 4.f : 8.f;           // (see launch_ty)
+    if (c.tn > 32) return c.tn == 40 ? 2.9f + 0.285f * chunks : 3.3f + 0.316f * chunks;         // (two CTAs per SM)
+    const SmallVariant v = variant_of(c, true, blocks, Kdim < (1 << 20) ? (int)chunks : 1 << 16, n_tiles, d.K > 1 && d.S == 1, sms);
+    if (!c.narrow && v.warps == 8) {
+        if (c.rm == 4) return v.products ? 1.7f + 0.07f * chunks * (float)blocks / (float)sms + 0.53f * ceilf(chunks / 8.f) : 1.75f + 0.084f * chunks;
+        if (v.slots == 3) return 2.2f + 0.166f * chunks;
+        return v.products ? 2.55f + 0.228f * chunks : 2.65f + 0.21f * chunks;
+    }
+    const float warps = blocks > 2 * sms ? 4.f : 8.f;
     const float narrow = 300.f * (chunks > warps ? warps * ceilf(chunks / warps) : chunks);
     const float us = rounds * ((c.rm == 4 ? 150.f * chunks : c.narrow ? narrow : 260.f * chunks) + 450.f) / 1965.f;
     return 2.2f + (blocks > 2 * sms ? 1.2f * us : us);
@@ -557,7 +579,7 @@ float f32_small_estimate(const ConvDesc& d, int sms)
 int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
 {
     const int sms = sm_count();
-    const SmallConfig c = config_of(d, n, sms, true);
+    const SmallConfig c = config_of(d, n, sms);
     bool vec = true;
     F32SmallParams p[2];
     for (int i = 0; i < n; ++i) {
@@ -565,12 +587,14 @@ int launch_conv_f32_small(const ConvDesc* d, int n, cudaStream_t stream)
         vec = vec && d[i].Cin % 4 == 0;
     }
     if (n == 1) { p[1] = p[0]; p[1].blocks = 0; }
+    const int chunks = n == 2 && p[1].chunks > p[0].chunks ? p[1].chunks : p[0].chunks;
+    const SmallVariant v = variant_of(c, vec, (long long)p[0].blocks + p[1].blocks, chunks, n == 1 ? p[0].n_tiles : 0, d[0].K > 1 && d[0].S == 1, sms);
     cudaError_t rc;
     if (c.tn > 32) rc = c.tn == 40 ? launch_wide<5>(p[0], p[1], stream) : launch_wide<6>(p[0], p[1], stream);
-    else if (c.rm == 8) rc = c.narrow ? (vec ? launch_ty<8, 8, true>(p[0], p[1], sms, stream) : launch_ty<8, 8, false>(p[0], p[1], sms, stream))
-                                 : (vec ? launch_ty<4, 8, true>(p[0], p[1], sms, stream) : launch_ty<4, 8, false>(p[0], p[1], sms, stream));
-    else rc = c.narrow ? (vec ? launch_ty<8, 4, true>(p[0], p[1], sms, stream) : launch_ty<8, 4, false>(p[0], p[1], sms, stream))
-                       : (vec ? launch_ty<4, 4, true>(p[0], p[1], sms, stream) : launch_ty<4, 4, false>(p[0], p[1], sms, stream));
+    else if (c.rm == 8) rc = c.narrow ? (vec ? launch_ty<8, 8, true>(v, p[0], p[1], stream) : launch_ty<8, 8, false>(v, p[0], p[1], stream))
+                                 : (vec ? launch_ty<4, 8, true>(v, p[0], p[1], stream) : launch_ty<4, 8, false>(v, p[0], p[1], stream));
+    else rc = c.narrow ? (vec ? launch_ty<8, 4, true>(v, p[0], p[1], stream) : launch_ty<8, 4, false>(v, p[0], p[1], stream))
+                       : (vec ? launch_ty<4, 4, true>(v, p[0], p[1], stream) : launch_ty<4, 4, false>(v, p[0], p[1], stream));
     if (rc != cudaSuccess) return SQN_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }

@@ -26,6 +26,9 @@ CASES = [
     ((116, 128, 16, 55, 55, 1, 1, 0), "conv_f32_small"),                   # - / 67 / 76
     ((16, 64, 128, 56, 56, 3, 2, 1), "conv_f32_tc",),                       # 38 / - / 65
     ((64, 3, 96, 227, 227, 7, 2, 0), "conv_f32_tc",),                       # 265 / - / 690
+    ((7, 224, 40, 21, 54, 1, 1, 0), "conv_f32_small",),                     # 10.3 / 7.2 / 11.7
+    ((8, 24, 40, 42, 27, 7, 1, 3), "conv_f32_small",),                      # 37 / 24 / 52
+    ((12, 384, 48, 27, 27, 1, 1, 0), "conv_f32_small",),                    # 14.4 / 11.1 / 18.5
 ]
 
 
