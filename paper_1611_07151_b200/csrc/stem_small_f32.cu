@@ -7,7 +7,7 @@
 // fp32 precision (see conv_f32_small.cu).  Kernels and the input patch lie in shared memory as in global memory; lane t of four takes
 // the reduction elements 4t .. 4t+3 of every 16, those of a pixel's window by a table of offsets.  The matrix instructions bound
 // it: 10 blocks of 16 reduction elements, 72 MMAs of 8 clocks per scheduler and warp each, are 6 us.
-// A tile with a sum that is not finite is computed again with multiply-adds.
+// Sums that are not finite are computed again with multiply-adds, those alone: a pixel that two tiles compute has one value.
 #include <cstring>
 
 #include "f32_common.cuh"
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) stem_small_f32_kernel(const __grid_consta
         }
     float acc[6][2][4];
     bool finite = true;
-    auto store = [&](float unscale) {           // bias and ReLU, the convolution's pixels side by side
+    auto store = [&](float unscale, bool again) {       // bias and ReLU, the convolution's pixels side by side; NaN: to be computed again
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
             const int n = 48 * nh + 8 * j + 2 * t4;
@@ -106,9 +106,17 @@ __global__ void __launch_bounds__(256) stem_small_f32_kernel(const __grid_consta
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float s0 = acc[j][e][2 * h], s1 = acc[j][e][2 * h + 1];
-                    finite = finite && fabsf(s0) < INFINITY && fabsf(s1) < INFINITY;
-                    *reinterpret_cast<float2*>(sy + (32 * mg + 16 * e + 8 * h + g) * FYP + n) =
-                        make_float2(fmaxf(fmaf(s0, unscale, b.x), 0.f), fmaxf(fmaf(s1, unscale, b.y), 0.f));
+                    float2* dst = reinterpret_cast<float2*>(sy + (32 * mg + 16 * e + 8 * h + g) * FYP + n);
+                    float2 v = make_float2(fmaxf(fmaf(s0, unscale, b.x), 0.f), fmaxf(fmaf(s1, unscale, b.y), 0.f));     // (never NaN)
+                    if (again) {
+                        const float2 old = *dst;
+                        if (old.x == old.x) v.x = old.x;
+                        if (old.y == old.y) v.y = old.y;
+                    } else {
+                        if (!(fabsf(s0) < INFINITY)) { v.x = NAN; finite = false; }
+                        if (!(fabsf(s1) < INFINITY)) { v.y = NAN; finite = false; }
+                    }
+                    *dst = v;
                 }
         }
     };
@@ -142,7 +150,7 @@ __global__ void __launch_bounds__(256) stem_small_f32_kernel(const __grid_consta
             mma_split(&acc[j], xh, xm, xl, wh, wm, wl);
         }
     }
-    store(SPLIT_UNSCALE);
+    store(SPLIT_UNSCALE, false);
     if (__syncthreads_or(!finite)) {
 #pragma unroll
         for (int e = 0; e < 2; ++e)
@@ -164,7 +172,7 @@ __global__ void __launch_bounds__(256) stem_small_f32_kernel(const __grid_consta
                         for (int h = 0; h < 2; ++h) acc[j][e][2 * h + i] = fmaf(win[e][h][o], v, acc[j][e][2 * h + i]);
                 }
         }
-        store(1.f);
+        store(1.f, true);
         __syncthreads();
     }
     // the convolution's map (a tile's last row and column are also its neighbours' first)

@@ -79,8 +79,8 @@ def test_multiply_adds_where_they_are_faster(shape, variant):
     assert names == ["conv_f32_small " + variant]
 
 
-@pytest.mark.parametrize("special", [False, True])
-def test_stem_of_one_image(special):
+def stem_of_one_image(special):
+    """(image, kernels, bias, the stored convolution, the stored pooled map)."""
     import torch
     x, params = synth.squeezenet_case(37, 1)
     if special:
@@ -100,7 +100,12 @@ def test_stem_of_one_image(special):
         off = (ptr - work.data_ptr()) // 4
         maps.append(work.view(torch.float32)[off:off + C * H * W].view(H, W, C).permute(2, 0, 1)[None].cpu().numpy())
     B.squeezenet_destroy(net)
-    w, b = params["conv1"]
+    return (x,) + params["conv1"] + tuple(maps)
+
+
+@pytest.mark.parametrize("special", [False, True])
+def test_stem_of_one_image(special):
+    x, w, b, *maps = stem_of_one_image(special)
     with np.errstate(invalid="ignore", over="ignore"):
         exp = ref.conv2d(x, w, b, S=2, pad=0, relu=False)
         low = ref.conv2d(np.abs(np.where(np.isfinite(x), x, 0)), np.abs(w), np.abs(b), S=2, pad=0, relu=False)
@@ -119,3 +124,10 @@ def test_stem_of_one_image(special):
         assert (same | near).all() and same.mean() > 0.99
     else:
         np.testing.assert_array_equal(maps[1][0], pooled)
+
+
+def test_a_stem_with_an_infinity_pools_the_map_that_it_stores():
+    """Tiles share pixels: one that is computed again must not change the pixels whose sums were finite."""
+    *_, conv, pool = stem_of_one_image(True)
+    windows = np.max([conv[0][:, i:i + 109:2, j:j + 109:2] for i in range(3) for j in range(3)], axis=0)
+    np.testing.assert_array_equal(pool[0], windows)
