@@ -125,11 +125,13 @@ __device__ __forceinline__ void mma_bf16_free(float (&c)[4], const uint32_t (&a)
         asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
             : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// Of what the matrix instructions cut off a sum of 16 products on average (1.1e-8 of it, kernels of one sign 1.6e-8), added back with the
-// corrections: an error of one sign adds up from layer to layer.  Chosen so that none is left in SqueezeNet's logits at 1, 2 and 5
-// images (-6.4e-8 of them at one image without it, +8.3e-8 with 1e-8).  The corrections have to be summed apart: with all six products in
-// one sum 3.9e-8 of it were cut off, 5.5e-7 of the logits.
-constexpr float MMA_CUT = 4.5e-9f;
+// What the matrix instructions cut off a sum of 16 products on average, added back with the corrections: an error of one sign adds up
+// from layer to layer.  It grows with the number of products that are not zero.  Mean signed error of a layer without it (20 layers of
+// 256 to 576 products per output, inputs |N(0, 1)| of which a share is set to zero), kernels of both signs / of one: no zeros 1.14e-8 /
+// 1.65e-8 of the output, a quarter 8.1e-9 / 1.11e-8, half 5.0e-9 / 6.2e-9, three quarters 2.0e-9 / 2.1e-9, one product 0.  This is the value
+// for half, maps behind a ReLU, with kernels of both signs; dense inputs keep 6e-9 (one sign 1.1e-8) too little, few products up to
+// 5e-9 too much.  The corrections have to be summed apart: with all six products in one sum 3.9e-8 were cut off.
+constexpr float MMA_CUT = 5e-9f;
 
 // a += c + (c * MMA_CUT + r) for two numbers at a time, each operation rounded to nearest
 __device__ __forceinline__ void add_products2(float& a0, float& a1, float c0, float c1, float r0, float r1)

@@ -61,6 +61,53 @@ def test_sums_finite_and_not(shape, variant):
         assert (np.abs(got[fin].astype(np.float64) - exp[fin]) <= bound(xf, wf, b, S, pad)[fin]).all()
 
 
+def relu_map(rng, shape):
+    """Positive values and as many zeros, what a layer behind a ReLU reads."""
+    return np.maximum(rng.standard_normal(shape), 0).astype(np.float32)
+
+
+def exact(x, w, pad):
+    import torch
+    return torch.nn.functional.conv2d(torch.from_numpy(x).double(), torch.from_numpy(w).double(), padding=pad).numpy()
+
+
+def signed(got, exp):
+    """The error of one sign: its mean towards larger magnitudes over the mean magnitude."""
+    return float(((got.astype(np.float64) - exp) * np.sign(exp)).sum() / np.abs(exp).sum())
+
+
+# Products of sums that the matrix instructions cut off: without what is added back 5e-9 and 6.2e-9 (kernels of both signs, of one), with
+# 1e-8 added back 4.9e-9 and 3.8e-9 in the other direction; what is added back leaves less than half of either.  The mean of 46000 outputs
+# and more, each off by 0.8e-7 of the mean magnitude (0.5e-7), is itself within 4e-10 of its expectation.
+@pytest.mark.parametrize("signs,most", [("both", 2.5e-9), ("one", 2.7e-9)])
+def test_no_error_of_one_sign_on_maps_behind_a_relu(signs, most):
+    means = []
+    for seed, (N, C, M, H, K, variant) in enumerate([(1, 64, 256, 27, 3, "32x32 vec, 8 warps, 2 slots"), (1, 256, 128, 40, 1, "32x32 vec, 8 warps, 2 slots"),
+                                                     (2, 48, 96, 39, 3, "32x32 vec, 8 warps, 2 slots"), (4, 512, 64, 13, 1, "16x32 vec, 8 warps, 3 slots")]):
+        rng = np.random.default_rng(seed)
+        x = relu_map(rng, (N, C, H, H))
+        w, b = synth.draw_conv_params(rng, C, M, K)
+        w = np.abs(w) if signs == "one" else w
+        got = G.gpu_conv(x, w, np.zeros_like(b), 1, K // 2, False, F32, kernel="conv_f32_small %s, products" % variant)
+        means.append(signed(got, exact(x, w, K // 2)))
+    assert abs(np.mean(means)) <= most, means
+
+
+def test_a_chain_of_layers():
+    """Eight 3x3 layers with ReLU, one after the other: an error of one sign would add up (8 x 5e-9 without what is added back)."""
+    rng = np.random.default_rng(3)
+    x = relu_map(rng, (2, 48, 39, 39))
+    got, exp = x, x.astype(np.float64)
+    for i in range(8):
+        w, b = synth.draw_conv_params(rng, 48 if i == 0 else 96, 96, 3)
+        b[:] = 0
+        got = G.gpu_conv(got, w, b, 1, 1, True, F32, kernel="conv_f32_small 32x32 vec, 8 warps, 2 slots, products")
+        exp = np.maximum(exact(exp, w.astype(np.float64), 1), 0)
+    assert abs(signed(got, exp)) <= 8 * 2.5e-9, signed(got, exp)
+    err = np.linalg.norm(got - exp) / np.linalg.norm(exp)
+    assert err <= 3e-7, err                     # (each layer's own 1e-7, most of it averaged out by the next)
+
+
 # (N, Cin, Cout, H, W, K, S, pad), the variant that runs; microseconds with multiply-adds / products as measured
 MULTIPLY_ADDS = [((9, 64, 221, 19, 12, 1, 2, 0), "32x32 vec, 8 warps, 3 slots"),        # 2.7 / 3.3
                  ((1, 128, 128, 30, 30, 1, 1, 0), "32x32 vec, 8 warps, 3 slots"),       # 3.3 / 3.6
