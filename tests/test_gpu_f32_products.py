@@ -59,6 +59,57 @@ def test_sums_finite_and_not(shape, variant):
         np.testing.assert_array_equal(got[~fin], exp[~fin])
         xf, wf = np.where(np.isfinite(x), x, 0), np.where(np.isfinite(w), w, 0)
         assert (np.abs(got[fin].astype(np.float64) - exp[fin]) <= bound(xf, wf, b, S, pad)[fin]).all()
+        if not special:
+            check_precision(got, x, w, b, S, pad)
+
+
+def check_precision(got, x, w, b, S, pad):
+    """Against 64 bits.  2-norm: 0.7e-7 to 1.4e-7 measured; without the least of the five correction products (2^-17 of a product, in random
+    directions) it would be 1e-6.  Largest: the products left out, two cuts of 2^-23 of what a chunk of 16 holds, a rounding for every chunk, and
+    twelve for corrections, the warps' partial sums and the bias, on sums no larger than the sum of |kernel * input|."""
+    K = w.shape[2]
+    exp = exact(x, w, pad, S) + b[None, :, None, None].astype(np.float64)
+    terms = exact(np.abs(x), np.abs(w), pad, S) + np.abs(b)[None, :, None, None]
+    d = got.astype(np.float64) - exp
+    assert np.linalg.norm(d) <= 3e-7 * np.linalg.norm(exp), np.linalg.norm(d) / np.linalg.norm(exp)
+    assert (np.abs(d) <= (2.0 ** -22 + 2 * 2.0 ** -23 + (w.shape[1] * K * K / 16 + 12) * 2.0 ** -24) * terms).all()
+
+
+# (images, input, squeeze, expand layers, rows), the variant of both expands' launch
+PAIRS = [((1, 128, 32, 128, 55), "32x32 vec, 4 warps, 3 slots"), ((1, 256, 32, 128, 27), "32x32 vec, 8 warps, 2 slots"),
+         ((1, 256, 48, 64, 19), "16x32 vec, 8 warps, 3 slots")]
+
+
+@pytest.mark.parametrize("shape,variant", PAIRS, ids=lambda s: "x".join(map(str, s)) if isinstance(s, tuple) else s)
+@pytest.mark.parametrize("special", [False, True])
+def test_both_expands_finite_and_not(shape, variant, special):
+    N, cin, s, e, h = shape
+    rng = np.random.default_rng(sum(shape))
+    x = np.abs(rng.standard_normal((N, cin, h, h + 1))).astype(np.float32)
+    sq, x1, x3 = (synth.draw_conv_params(rng, *a) for a in ((cin, s, 1), (s, e, 1), (s, e, 3)))
+    if special:
+        x1[0][5, 2, 0, 0], x3[0][e - 1, 0, 1, 1], x3[0][3, 1, 1, 1] = np.inf, np.nan, -np.inf
+        x[0, 3, 4, 5] = np.inf
+    scratch, out = B.empty_device((N, h, h + 1, s), F32), B.empty_device((N, h, h + 1, 2 * e), F32)
+    with G.traced() as names:
+        B.fire_forward(G.dev_act(x, F32), G.dev_w(sq[0], F32), G.dev_b(sq[1]), G.dev_w(x1[0], F32), G.dev_b(x1[1]), G.dev_w(x3[0], F32),
+                       G.dev_b(x3[1]), scratch, out, cin, s, e, e, h, h + 1, N, F32)
+    assert B.sqn_check() == B.SQN_OK
+    assert len(names) == 2 and names[1] == "conv_f32_small x 2 %s, products" % variant, names
+    squeezed, got = G.host_act(scratch, F32), G.host_act(out, F32)
+    for part, (w, b), pad in ((got[:, :e], x1, 0), (got[:, e:], x3, 1)):
+        with np.errstate(invalid="ignore", over="ignore"):
+            exp = ref.conv2d(squeezed, w, b, S=1, pad=pad, relu=False)
+        fin = np.isfinite(exp)
+        assert special != fin.all()
+        exp = np.where(np.isnan(exp), 0, np.maximum(exp, 0))            # (max(0, NaN) = 0)
+        np.testing.assert_array_equal(part[~fin], exp[~fin])
+        xf, wf = np.where(np.isfinite(squeezed), squeezed, 0), np.where(np.isfinite(w), w, 0)
+        assert (np.abs(part[fin].astype(np.float64) - exp[fin]) <= bound(xf, wf, b, 1, pad)[fin]).all()
+        if not special:
+            full = exact(squeezed, w, pad) + b[None, :, None, None].astype(np.float64)
+            d = part.astype(np.float64) - np.maximum(full, 0)
+            assert np.linalg.norm(d) <= 3e-7 * np.linalg.norm(np.maximum(full, 0))
 
 
 def relu_map(rng, shape):
@@ -66,9 +117,9 @@ def relu_map(rng, shape):
     return np.maximum(rng.standard_normal(shape), 0).astype(np.float32)
 
 
-def exact(x, w, pad):
+def exact(x, w, pad, S=1):
     import torch
-    return torch.nn.functional.conv2d(torch.from_numpy(x).double(), torch.from_numpy(w).double(), padding=pad).numpy()
+    return torch.nn.functional.conv2d(torch.from_numpy(x).double(), torch.from_numpy(w).double(), stride=S, padding=pad).numpy()
 
 
 def signed(got, exp):
@@ -156,6 +207,9 @@ def test_stem_of_one_image(special):
     with np.errstate(invalid="ignore", over="ignore"):
         exp = ref.conv2d(x, w, b, S=2, pad=0, relu=False)
         low = ref.conv2d(np.abs(np.where(np.isfinite(x), x, 0)), np.abs(w), np.abs(b), S=2, pad=0, relu=False)
+    if not special:
+        full = np.maximum(exact(x, w, 0, 2) + b[None, :, None, None].astype(np.float64), 0)
+        assert np.linalg.norm(maps[0] - full) <= 3e-7 * np.linalg.norm(full)
     exp = np.where(np.isnan(exp), 0, np.maximum(exp, 0)).astype(np.float64)          # (max(0, NaN) = 0)
     fin = np.isfinite(exp) & np.isfinite(low)
     np.testing.assert_array_equal(maps[0][np.isposinf(exp) & np.isfinite(low)], np.inf)
