@@ -2,8 +2,12 @@
 the CPU: barriers as phase counters that answer a parity wait as the hardware does (true when the current phase's parity differs), boxes
 that land in any order, groups that run as far ahead as their other waits let them.  A group must never take a box that is not there."""
 import itertools
+import os
+import re
 
 import pytest
+
+SOURCE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_1611_07151_b200", "csrc", "conv_f32_tc.cu")
 
 
 def run(slots, units, order, guarded):
@@ -64,3 +68,13 @@ def test_no_box_is_taken_early(slots):
 def test_the_model_sees_what_an_odd_ring_does_without_the_guard():
     """Three slots, unit 2's box before unit 1's: unit 4 takes slot 1 while it is empty."""
     assert not run(3, 7, (0, 2, 1, 3, 4, 5, 6), guarded=False)
+
+
+def test_the_kernel_is_the_one_that_is_modelled():
+    """The slot counts of the kernel's rings are those above, and its guard stands before the wait for the box."""
+    text = open(SOURCE).read()
+    boxes = {int(n) for name in ("flat", "patch", "box") for n in re.findall(r"{\d, \d, (\d)}", re.search(r"\b%s\[\]\[3\] = {(.*?)}[,;]" % name, text).group(1) + "}")}
+    assert boxes and boxes <= {2, 3, 4}, boxes
+    guard = text.index("if ((p.sb & 1) && !wait_done(u - p.sb)) break;")
+    wait = text.index("wait_bar(smem_u32(&sh->sb_full[st]), sph")
+    assert 0 < wait - guard < 200 and text.count("sb_full[st]), sph") == 1
