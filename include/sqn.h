@@ -12,10 +12,15 @@
  *    (The paper, Section III-B/C, reorders data so that values of consecutive
  *    layers at one pixel are adjacent and has every layer write its output in
  *    that order; NHWC/OHWI is the same idea carried to all layers of a pixel.)
- *  - dtype SQN_F32: activations and kernels fp32, sums in fp32.  Three kernels share the layers, by estimated time:
+ *  - dtype SQN_F32: activations and kernels fp32, sums in fp32.  Several kernels share the layers, by estimated time:
  *    multiply-adds in sequence, multiply-adds split over warps, and the tensor cores with every operand as the exact
- *    sum of three bf16 numbers (relative 2-norm error of a layer against 64-bit arithmetic 0.7e-7 to 2e-7, of
- *    multiply-adds up to 1e-6).  They add in different orders: which one runs depends on the layer and the batch, so
+ *    sum of three bf16 numbers, for large layers and (warp-level, the stem of one image among them) for small ones.
+ *    Of the nine partial products the tensor cores take six; what is left out is up to 1.75 units of 2^-24 of a
+ *    product.  Relative 2-norm error of a layer against 64-bit arithmetic 0.7e-7 to 2e-7, of multiply-adds up to
+ *    1e-6; an output with one product that is not zero, which a multiply-add rounds once (6e-8 of it at most), is off
+ *    by 1.5e-7 of it at most (2-norm of a layer of such outputs 2.8e-8, multiply-adds 2.5e-8; of two products 3.8e-8
+ *    and 3.6e-8).
+ *    They add in different orders: which one runs depends on the layer and the batch, so
  *    the result for one image may differ in the last bits between batches.  No operand loses bits, whatever its
  *    magnitude; layers with infinities, NaN, operands of 2^112 and more or sums of 2^96 and more take longer on the
  *    tensor cores (their outputs are computed again with multiply-adds).

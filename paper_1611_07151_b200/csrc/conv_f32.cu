@@ -407,7 +407,7 @@ int launch_conv_f32(const ConvDesc& d, cudaStream_t stream)
 
 // One launch for two layers saves a launch's start and end (2 us of the squeezes' and expands' 3 to 12 at batch 1: fp32
 // forward of one image 168 -> 158 us, fire4 17.7 -> 15.4) as long as the small layers' kernel suits both; the line is where
-// its estimate meets the tensor-core kernel's on fire4's and fire8's expand-3x3.
+// the estimate of its multiply-adds meets the tensor-core kernel's on fire4's and fire8's expand-3x3.
 int launch_conv_f32_pair(const ConvDesc& a, const ConvDesc& b, cudaStream_t stream, bool* paired)
 {
     if (paired) *paired = false;

@@ -7,7 +7,8 @@
 // chunks asynchronously into a ring of its own, waits for nobody else, and the warps' partial sums are added once at the end,
 // in a fixed order.  Operand rows are stored as they lie in memory (reduction index contiguous, 80-byte pitch): a thread
 // takes four reduction elements of its 8 pixels and 4 layers with twelve 16-byte reads, free of bank conflicts, for 128
-// multiply-adds.  Layers with 16-byte pieces and tiles of 32 layers or more do the same on the matrix instructions (further down).  Two layers that read the same input (the expands of a fire layer) go out as one grid.
+// multiply-adds.  Layers with 16-byte pieces and tiles of 32 layers or more do the same on the matrix
+// instructions where that is faster (further down).  Two layers that read the same input (the expands of a fire layer) go out as one grid.
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -222,8 +223,10 @@ __device__ __forceinline__ float ld_shared_f1(uint32_t a)
 // rows of 64 bytes.  The order of a chunk's elements in the MMA's reduction is free: lane t of four takes elements 4t .. 4t+3 of
 // its rows with one 16-byte read, free of bank conflicts.  A chunk of a 32 x 32 tile is 48 MMAs of 8 clocks per scheduler against 512
 // multiply-adds of 1.45 and six times the reads; what bounds it is the chain of a chunk (read, split, products) in every warp.
-// Multiply-adds against this kernel, one image: fire8's expand-3x3 12.5 -> 10.8 us, fire9's 6.9 -> 5.3, fire8's squeeze 5.4 -> 3.9,
-// conv10 11.5 -> 9.8; 256 -> 256 3x3 at 14 x 14, 3 images: 42.2 -> 35.0.  Which layers take it: variant_of.  Error against 64 bits 0.7e-7 to 1.3e-7 (0.9e-7 to 4.0e-7).
+// Multiply-adds against this kernel, one image: fire8's expand-3x3 12.2 -> 10.5 us, fire9's 6.8 -> 5.0, fire8's squeeze 5.3 -> 4.1,
+// conv10 11.4 -> 9.4; 256 -> 256 3x3 at 14 x 14, 3 images: 42.0 -> 34.1.  Which layers take it: variant_of.  Error of a layer against 64 bits 0.5e-7 to 1.4e-7 (0.7e-7 to
+// 4.0e-7); of outputs with a single product that is not zero 2.8e-8 (2.5e-8), with two 3.8e-8 (3.6e-8): with eight products instead of
+// six 2.55e-8 and 3.6e-8, but fire4's pair 14.2 -> 15.9 us, conv10 9.5 -> 10.9.
 // A tile with a sum that is not finite is computed again with multiply-adds.
 template <int MF, int NF, int SL, int ST>
 __device__ __forceinline__ void conv_f32_small_tc_body(const F32SmallParams& p, const int bid)
@@ -471,7 +474,7 @@ cudaError_t launch(const F32SmallParams& a, const F32SmallParams& b, cudaStream_
 //    wave (fire8's expand-3x3 at batch 1, 184 tiles: 14.1 -> 12.5 us), else four warps and three slots.
 //  - a single layer with 16-byte pieces, more than six chunks and more tiles than two per SM: tiles of 40 or 48 layers where they
 //    compute an eighth less than those of 32 and then are two per SM at most (20 -> 36 5x5/2, nine images of 61 x 47, half of the
-//    32-layer tiles' work for nothing: 18.0 -> 13.1 us; 50 such layers 0.81, with six chunks or fewer 1.0).  Fewer tiles of 32 run two
+//    32-layer tiles' work for nothing: 17.8 -> 12.8 us; 50 such layers 0.81, with six chunks or fewer 1.0).  Fewer tiles of 32 run two
 //    to an SM at once and are the faster ones (150 layers, the wider tiles 1.03 to 1.24; 12 -> 48 3x3/2, six images of 50 x 50, 4.7 and 5.7 us).
 struct SmallConfig { bool narrow; int rm, tm, tn; };
 

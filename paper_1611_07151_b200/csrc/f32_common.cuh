@@ -51,7 +51,8 @@ __device__ __forceinline__ void sub2(uint32_t ax, uint32_t ay, uint32_t bx, uint
         "mov.b64 {%0, %1}, a;\n\t}"
         : "=r"(dx), "=r"(dy) : "r"(ax), "r"(ay), "r"(bx), "r"(by));
 }
-// Two values as three packed bf16 pairs whose sums are SPLIT_SCALE times the values.  The first is the value rounded to nearest
+// Two values as three packed bf16 pairs whose sums are SPLIT_SCALE times the values (the split of Henry, Tang and Heinecke, "Leveraging the
+// bfloat16 Artificial Intelligence Datatype For Higher-Precision Computations", 2019).  The first is the value rounded to nearest
 // (the remainder is below 2^-8 of it and of either sign), the second the leading eight bits of the remainder, the third the rest.
 __device__ __forceinline__ void split_pair(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l)
 {
