@@ -1033,14 +1033,7 @@ size_t layout(F32TcParams& p)
     p.khalf = p.chunks == 1 && p.ksteps_last == 1 ? 1 : 0;
     p.wrows = (p.n_step + 31) / 32 * 32;
     p.div_wrows = make_div(p.wrows); p.div_taps = make_div(p.taps);
-    // BOX with TMA stores: 32 pixels per store before a second pair of pixel slots (conv1 at batch 256 970 us with two slots and 32 pixels,
-    // 1008 with four and 16), and 16 pixels, in the room that the stores without TMA take (1 to 2 % slower than with), before the kernels'
-    // source or the number of blocks: 18 -> 348 3x3/2 at 43 x 42, 48 images, 79 us with 16, 130 with 32 in three blocks; 33 -> 276 7x7 at
-    // 29 x 110, four images, 237 and 338.
-    const int widths = p.mode == FT_BOX && p.tstore ? 2 : 1;
-    for (int j = 0; j < (n_packed + n) * widths; ++j) {
-        const int i = widths == 1 ? j : j / 4 * 2 + j % 2;
-        if (widths == 2) p.tstore = j % 4 < 2 ? 32 : 16;
+    for (int i = 0; i < n_packed + n; ++i) {
         const int* c = cand[i < n_packed ? i : i - n_packed];
         p.wsrc = i < n_packed ? FT_W_PACKED : streamed;
         p.ra = c[0];
@@ -1057,6 +1050,24 @@ size_t layout(F32TcParams& p)
         return cur + 1024;
     }
     return 0;
+}
+
+// Microseconds this kernel takes: start and end of a launch, then per tile of the busiest CTA its epilogue and its units of 32
+// (or 16) reduction elements.  FLAT and PATCH: fitted to SqueezeNet's layers at batch 1 .. 256 (500 random layers: 0.85 to 1.2
+// of it in nine of ten).  BOX: the copies of a tile's windows, a thread's share one after the other (0.05 us each where a window
+// row is one run of memory, else 0.1) and 0.4 us for every block of layers, and the kernels' split, once; fitted to 890 random
+// layers with a stride or odd layer counts (0.9 to 1.15 of it in eight of ten, 1.7 at most; without these terms 1.0 to 6.5, and a
+// 1x1/3 layer of 28 images, 151 -> 53 at 57 x 49, went here for 40 us in the place of 15).
+float f32_tc_estimate(const F32TcParams& p)
+{
+    if (p.mode == FT_BOX) {
+        const int copies = ceil_div(p.rh, 8) * ceil_div((long long)p.rc * p.cb, p.box_vec ? 128 : 32);
+        const float unit = p.wsrc == FT_W_COPIES ? 1.24f : 0.8f, packed = p.wsrc == FT_W_PACKED ? (float)(p.chunks * p.wrows) / 128.f : 0.f;
+        const float tile = 2.f + unit * (float)p.chunks + (float)p.nb * (0.4f + (p.nb == 1 && p.S <= p.K ? 0.047f : 0.1f) * (float)copies);
+        return 3.5f + 1.5f * (p.khalf ? 0.5f : 1.f) * packed + (float)ceil_div(p.m_tiles, p.m_step) * ceil_div(p.grid, sm_count()) * tile;
+    }
+    const float unit = p.wsrc != FT_W_PACKED && p.mode != FT_PATCH ? 0.9f : p.khalf ? 0.45f : 0.63f;
+    return 4.5f + (float)ceil_div(p.m_tiles, p.m_step) * ceil_div(p.grid, sm_count()) * (1.6f + unit * (float)(p.chunks * p.taps));
 }
 
 int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
@@ -1097,6 +1108,12 @@ int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
         plan->smem = layout(p);
         return plan->smem != 0;
     };
+    auto grid = [&](F32TcParams& q) {
+        q.m_step = sms / q.n_tiles;
+        if (q.m_step < 1) q.m_step = 1;
+        if (q.m_step > q.m_tiles) q.m_step = q.m_tiles;
+        q.grid = q.n_tiles * q.m_step;
+    };
     bool found = false;
     p.taps = 1;
     if (vec && d.K == 1 && d.S == 1 && d.pad == 0) {
@@ -1112,46 +1129,54 @@ int build_f32_plan(const ConvDesc& d, F32TcPlan* plan)
         found = finish(d.Cin, positions);
     }
     if (!found) {
-        const int tstore = p.vec_store && d.Cout % 4 == 0 ? 32 : 0;
         p.mode = FT_BOX;
         p.prow = FT_N;
         p.taps = 1;
         // tile shape with the fewest tiles (the smaller box on ties), layers per block as many as fit
-        long long best = -1;
-        F32TcPlan bp = *plan;
-        for (int sh = 7; sh >= 0; --sh) {
-            const int bw = 1 << sh, bh = 128 >> sh;
-            p.stepb = d.S < d.K ? d.S : d.K;
-            p.rh = (bh - 1) * p.stepb + d.K; p.rc = (bw - 1) * p.stepb + d.K;
-            p.bw_shift = sh; p.bh = bh;
-            p.tiles_w = ceil_div(d.OW, bw); p.tiles_h = ceil_div(d.OH, bh);
-            const long long tiles = (long long)p.tiles_w * p.tiles_h;
-            if (tiles * d.N > 0x3fffffffLL) continue;
-            p.div_tw = make_div(p.tiles_w); p.div_th = make_div(p.tiles_h);
-            for (int cb = d.Cin; cb > 0; cb = cb > 32 ? 32 : cb / 2 / 4 * 4) {
-                if ((long long)d.K * d.K * cb > FT_TBL_MAX || (long long)p.rh * p.rc * cb * 4 > 64 * 1024) continue;
-                p.cb = cb;
-                p.nb = ceil_div(d.Cin, cb);
-                p.cpb = ceil_div((long long)d.K * d.K * cb, FT_BK);
-                p.pitch = (p.rc * cb + 3) / 4 * 4;
-                p.box_vec = vec && cb % 4 == 0 ? 1 : 0;
-                p.div_cb = make_div(cb);
-                const long long cost = tiles * 1000000 + (long long)p.rh * p.rc * cb;
-                if (best >= 0 && cost >= best) break;
-                p.tstore = tstore;          // (layout() may take it down to 16)
-                if (!finish(d.K * d.K * cb, 0)) continue;
-                best = cost;
-                bp = *plan;
-                break;
+        auto search = [&](int tstore, F32TcPlan* found) {
+            long long best = -1;
+            p.tstore = tstore;
+            for (int sh = 7; sh >= 0; --sh) {
+                const int bw = 1 << sh, bh = 128 >> sh;
+                p.stepb = d.S < d.K ? d.S : d.K;
+                p.rh = (bh - 1) * p.stepb + d.K; p.rc = (bw - 1) * p.stepb + d.K;
+                p.bw_shift = sh; p.bh = bh;
+                p.tiles_w = ceil_div(d.OW, bw); p.tiles_h = ceil_div(d.OH, bh);
+                const long long tiles = (long long)p.tiles_w * p.tiles_h;
+                if (tiles * d.N > 0x3fffffffLL) continue;
+                p.div_tw = make_div(p.tiles_w); p.div_th = make_div(p.tiles_h);
+                for (int cb = d.Cin; cb > 0; cb = cb > 32 ? 32 : cb / 2 / 4 * 4) {
+                    if ((long long)d.K * d.K * cb > FT_TBL_MAX || (long long)p.rh * p.rc * cb * 4 > 64 * 1024) continue;
+                    p.cb = cb;
+                    p.nb = ceil_div(d.Cin, cb);
+                    p.cpb = ceil_div((long long)d.K * d.K * cb, FT_BK);
+                    p.pitch = (p.rc * cb + 3) / 4 * 4;
+                    p.box_vec = vec && cb % 4 == 0 ? 1 : 0;
+                    p.div_cb = make_div(cb);
+                    const long long cost = tiles * 1000000 + (long long)p.rh * p.rc * cb;
+                    if (best >= 0 && cost >= best) break;
+                    if (!finish(d.K * d.K * cb, 0)) continue;
+                    best = cost;
+                    *found = *plan;
+                    grid(found->p);
+                    break;
+                }
             }
-        }
-        if (best < 0) return SQN_ERR_UNSUPPORTED;
-        *plan = bp;
+            return best >= 0;
+        };
+        // TMA stores of 32 pixels need more staging than those of 16, which need no more than stores without TMA: other tiles, a poorer
+        // source of the kernels or more blocks.  The better plan by its estimate, 32 pixels where they are equal (conv1 at batch 256
+        // 970 us with two pixel slots and 32 pixels, 1008 with four and 16).  188 random layers, geometric mean, plain stores 1: this
+        // 0.975, always 32 0.981, 16 ahead of a poorer plan 0.983.  18 -> 348 3x3/2 at 43 x 42, 48 images, 79 us with 16, 130 with 32 in
+        // three blocks; 4 -> 164 7x7/2 at 56 x 53, 20 images, 21 with 32 and kernels by boxes, 28 with 16 and packed ones.
+        const bool tma = p.vec_store && d.Cout % 4 == 0;
+        F32TcPlan bp, other;
+        const bool a = search(tma ? 32 : 0, &bp), b = tma && search(16, &other);
+        if (!a && !b) return SQN_ERR_UNSUPPORTED;
+        *plan = !a || (b && f32_tc_estimate(other.p) < f32_tc_estimate(bp.p)) ? other : bp;
+        return SQN_OK;
     }
-    p.m_step = sms / p.n_tiles;
-    if (p.m_step < 1) p.m_step = 1;
-    if (p.m_step > p.m_tiles) p.m_step = p.m_tiles;
-    p.grid = p.n_tiles * p.m_step;
+    grid(p);
     return SQN_OK;
 }
 
@@ -1200,24 +1225,6 @@ cudaError_t launch_mode(const F32TcPlan& plan, cudaStream_t stream)
     const cudaError_t arc = attr.allow((const void*)conv_f32_tc_kernel<MODE>, FT_SMEM_LIMIT);
     if (arc != cudaSuccess) return arc;
     return launch_chained(conv_f32_tc_kernel<MODE>, dim3((unsigned)plan.p.grid), dim3(FT_THREADS), plan.smem, stream, plan.x, plan.w, plan.o, plan.p);
-}
-
-// Microseconds this kernel takes: start and end of a launch, then per tile of the busiest CTA its epilogue and its units of 32
-// (or 16) reduction elements.  FLAT and PATCH: fitted to SqueezeNet's layers at batch 1 .. 256 (500 random layers: 0.85 to 1.2
-// of it in nine of ten).  BOX: the copies of a tile's windows, a thread's share one after the other (0.05 us each where a window
-// row is one run of memory, else 0.1) and 0.4 us for every block of layers, and the kernels' split, once; fitted to 890 random
-// layers with a stride or odd layer counts (0.9 to 1.15 of it in eight of ten, 1.7 at most; without these terms 1.0 to 6.5, and a
-// 1x1/3 layer of 28 images, 151 -> 53 at 57 x 49, went here for 40 us in the place of 15).
-float f32_tc_estimate(const F32TcParams& p)
-{
-    if (p.mode == FT_BOX) {
-        const int copies = ceil_div(p.rh, 8) * ceil_div((long long)p.rc * p.cb, p.box_vec ? 128 : 32);
-        const float unit = p.wsrc == FT_W_COPIES ? 1.24f : 0.8f, packed = p.wsrc == FT_W_PACKED ? (float)(p.chunks * p.wrows) / 128.f : 0.f;
-        const float tile = 2.f + unit * (float)p.chunks + (float)p.nb * (0.4f + (p.nb == 1 && p.S <= p.K ? 0.047f : 0.1f) * (float)copies);
-        return 3.5f + 1.5f * (p.khalf ? 0.5f : 1.f) * packed + (float)ceil_div(p.m_tiles, p.m_step) * ceil_div(p.grid, sm_count()) * tile;
-    }
-    const float unit = p.wsrc != FT_W_PACKED && p.mode != FT_PATCH ? 0.9f : p.khalf ? 0.45f : 0.63f;
-    return 4.5f + (float)ceil_div(p.m_tiles, p.m_step) * ceil_div(p.grid, sm_count()) * (1.6f + unit * (float)(p.chunks * p.taps));
 }
 
 }  // namespace

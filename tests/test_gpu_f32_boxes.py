@@ -33,10 +33,11 @@ def test_boxes_of_pixels(shape, offset, total):
 # (N, Cin, Cout, H, W, K, S, pad), the variant that runs: what the stores stage must not cost the kernels' source or more blocks of
 # layers (microseconds with those / without)
 PLANS = [((16, 3, 96, 227, 227, 7, 2, 0), "kernels packed, 1 block, 32 pixels per store"),
-         ((32, 20, 256, 112, 112, 3, 2, 1), "kernels by boxes, 1 block, 32 pixels per store"),      # 246 / 104
+         ((32, 20, 256, 112, 112, 3, 2, 1), "kernels by boxes, 1 block, 16 pixels per store"),      # 246 / 104
          ((48, 18, 348, 43, 42, 3, 2, 1), "kernels by copies, 1 block, 16 pixels per store"),       # 131 / 80
          ((4, 33, 276, 29, 110, 7, 1, 3), "kernels by copies, 1 block, 16 pixels per store"),       # 339 / 237
-         ((64, 20, 256, 28, 28, 5, 2, 2), "kernels by boxes, 1 block, 16 pixels per store")]        # 70 / 40
+         ((64, 20, 256, 28, 28, 5, 2, 2), "kernels by boxes, 1 block, 16 pixels per store"),        # 70 / 40
+         ((20, 4, 164, 56, 53, 7, 2, 3), "kernels by boxes, 1 block, 32 pixels per store")]         # (packed, 16 pixels: 28) / 21
 
 
 @pytest.mark.parametrize("shape,variant", PLANS, ids=lambda s: "x".join(map(str, s)) if isinstance(s, tuple) else s)
