@@ -42,7 +42,6 @@
 //           registers, then bias, ReLU and stores of 32 consecutive layers of a pixel per warp
 //   24, 25  TMA producers: pixels, kernels                 (26 idle: registers go by warpgroup)
 //   27      MMA issuer (one elected lane), on the scheduler with the least other work
-#include <cstdio>
 #include <cstring>
 
 #include "f32_common.cuh"
@@ -1240,11 +1239,11 @@ int launch_conv_f32_tc(const ConvDesc& d, float limit_us, cudaStream_t stream)
                         : plan.p.mode == FT_PATCH ? launch_mode<FT_PATCH>(plan, stream) : launch_mode<FT_BOX>(plan, stream);
     if (e != cudaSuccess) return SQN_ERR_CUDA;
     const F32TcParams& p = plan.p;
-    char stores[32] = "";
-    if (p.mode == FT_BOX && p.tstore) std::snprintf(stores, sizeof(stores), ", %d pixels per store", p.tstore);
-    note_launch("conv_f32_tc %s, kernels %s, %d %s%s%s", p.mode == FT_FLAT ? "flat" : p.mode == FT_PATCH ? "patch" : "box",
+    const bool stores = p.mode == FT_BOX && p.tstore;
+    note_launch(stores ? "conv_f32_tc %s, kernels %s, %d %s%s, %d pixels per store" : "conv_f32_tc %s, kernels %s, %d %s%s",
+                p.mode == FT_FLAT ? "flat" : p.mode == FT_PATCH ? "patch" : "box",
                 p.wsrc == FT_W_PACKED ? "packed" : p.wsrc == FT_W_BOXES ? "by boxes" : "by copies", p.mode == FT_BOX ? p.nb : 1,
-                p.mode == FT_BOX && p.nb > 1 ? "blocks" : "block", p.mode == FT_BOX && p.S > p.K ? ", apart" : "", stores);
+                p.mode == FT_BOX && p.nb > 1 ? "blocks" : "block", p.mode == FT_BOX && p.S > p.K ? ", apart" : "", p.tstore);
     return cudaGetLastError() == cudaSuccess ? SQN_OK : SQN_ERR_CUDA;
 }
 
